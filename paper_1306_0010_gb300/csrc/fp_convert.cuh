@@ -32,13 +32,15 @@ __device__ __forceinline__ double f2d_exact(float f)
 }
 
 // Square root and reciprocal.  Split path: the hardware approximations (MUFU, about 1-2 ulp), well
-// inside the FP32 error budget of the fluxes.  FP64 path: IEEE square root; the reciprocal is the
-// hardware FP64 approximation refined by two Newton-Raphson steps r <- r + r (1 - x r), each of which
-// squares the relative error (from below 2^-20 to below 2^-40, then to rounding): within an ulp or
-// two of 1/x, not the correctly rounded quotient, which the FP64 path does not need (its bound
-// against the oracle is 1e-12) and which costs several more FP64 operations.  x = 0, +-inf and FP64
-// denormals (flushed) give NaN.
-__device__ __forceinline__ double sqrt_fast(double x) { return sqrt(x); }
+// inside the FP32 error budget of the fluxes.  FP64 path: the FP64 pipe of this part issues one warp
+// instruction per 64 cycles and SM sub-partition, so its instructions are what the FP64 kernels are made
+// of and every one counts: the hardware FP64 approximations (MUFU pipe, relative error below 2^-20) are
+// refined by one third-order step, r <- r (1 + e + e^2) with e = 1 - x r for the reciprocal (the error
+// becomes e^3 < 2^-60; three FP64 instructions against four for two Newton-Raphson steps), and
+// y <- y + y r (1/2 + 3/8 r) with r = 1 - x y^2 for the inverse square root (the dropped term is
+// 5/16 r^3 < 2^-58; five instructions against eight).  Results within an ulp or two, not correctly
+// rounded, which the FP64 path does not need (its bound against the oracle is 1e-12).  Reciprocal: x = 0,
+// +-inf and FP64 denormals (flushed) give NaN.
 __device__ __forceinline__ float sqrt_fast(float x)
 {
     float r;
@@ -49,22 +51,69 @@ __device__ __forceinline__ double rcp(double x)
 {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    double e = fma(-x, r, 1.0);
-    r = fma(r, e, r);
-    e = fma(-x, r, 1.0);
-    return fma(r, e, r);
+    const double e = __fma_rn(-x, r, 1.0);
+    return __fma_rn(r, __fma_rn(e, e, e), r);
 }
-// 1/sqrt(x) for normal x > 0, FP64: the hardware approximation refined by two Newton-Raphson steps for
-// f(y) = y^-2 - x, y <- y + (y/2)(1 - x y^2), each of which squares the relative error (within an ulp or
-// two of 1/sqrt(x); tested against CUDA's 1/sqrt).  x sqrt(x)^-1 is then the square root as well.
+// 1/sqrt(x) for normal x > 0, FP64 (within an ulp or two; tested against CUDA's 1/sqrt).  x sqrt(x)^-1 is
+// then the square root as well.
 __device__ __forceinline__ double rsqrt_nr(double x)
 {
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    double r = __fma_rn(-__dmul_rn(x, y), y, 1.0);
-    y = __fma_rn(__dmul_rn(0.5, y), r, y);
-    r = __fma_rn(-__dmul_rn(x, y), y, 1.0);
-    return __fma_rn(__dmul_rn(0.5, y), r, y);
+    const double r = __fma_rn(-__dmul_rn(x, y), y, 1.0);
+    return __fma_rn(__dmul_rn(y, r), __fma_rn(r, 0.375, 0.5), y);
+}
+// sqrt(x), FP64, by the same step on x y ~ sqrt(x) (five instructions; CUDA's correctly rounded sqrt takes
+// about twice as many and a slow path).  Zero and subnormal x give 0, +inf gives +inf, negative x NaN.
+__device__ __forceinline__ double sqrt_fast(double x)
+{
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double g = __dmul_rn(x, y);
+    const double r = __fma_rn(-g, y, 1.0);
+    const double s = __fma_rn(__dmul_rn(g, r), __fma_rn(r, 0.375, 0.5), g);
+    const int hi = __double2hiint(x);
+    return (hi & 0x7fffffff) < 0x00100000 ? 0.0 : (hi == 0x7ff00000 ? x : s);
+}
+
+// Comparisons of FP64 values by their bits, on the integer pipes (an FP64 comparison, minimum or maximum
+// occupies the FP64 pipe like an addition).  Values of one sign are ordered as the integers their bits
+// make; a NaN counts as larger than any number.
+__device__ __forceinline__ unsigned long long mag_bits(double x)
+{
+    return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
+}
+// max(a, b, 0) and min(a, b, 0)
+__device__ __forceinline__ double max0_d(double a, double b)
+{
+    const long long x = max(__double_as_longlong(a), 0ll), y = max(__double_as_longlong(b), 0ll);
+    return __longlong_as_double(max(x, y));
+}
+__device__ __forceinline__ double min0_d(double a, double b)
+{
+    const unsigned long long s = 0x8000000000000000ull;
+    const unsigned long long x = (unsigned long long)__double_as_longlong(a), y = (unsigned long long)__double_as_longlong(b);
+    return __longlong_as_double((long long)max(x >= s ? x : 0ull, y >= s ? y : 0ull));
+}
+// x > 0 (false for NaN)
+__device__ __forceinline__ bool pos_d(double x)
+{
+    const long long b = __double_as_longlong(x);
+    return b > 0 && b <= 0x7ff0000000000000ll;
+}
+__device__ __forceinline__ bool is_one_d(double x) { return __double_as_longlong(x) == 0x3ff0000000000000ll; }
+// x > 1 - 2^-50 (true for +inf, false for NaN)
+__device__ __forceinline__ bool reaches1_d(double x)
+{
+    const long long b = __double_as_longlong(x);
+    return b > 0x3ff0000000000000ll - 8 && b <= 0x7ff0000000000000ll;
+}
+// minmod(a, b): the one nearer zero if both have the same sign, else 0 (and 0 if either is NaN)
+__device__ __forceinline__ double minmod_d(double a, double b)
+{
+    const unsigned long long x = mag_bits(a), y = mag_bits(b);
+    const bool none = (__double2hiint(a) ^ __double2hiint(b)) < 0 || max(x, y) > 0x7ff0000000000000ull;
+    return none ? 0.0 : (x < y ? a : b);
 }
 __device__ __forceinline__ float rcp(float x)
 {

@@ -140,14 +140,8 @@ __device__ __forceinline__ ClosureScalars<R> closure_scalars(R E, R gx, R gy, R 
     }
     k.invE = invE;
     const R x4 = xfma(R(-3), f2, R(4));  // in [1, 4]
-    R inv_s;
-    if constexpr (sizeof(R) == 8) {
-        inv_s = rsqrt_nr(x4);  // s and 1/s from one refined inverse square root
-        k.s = xmul(x4, inv_s);
-    } else {
-        k.s = sqrt_fast(x4);
-        inv_s = rcp(k.s);
-    }
+    k.s = sqrt_fast(x4);
+    const R inv_s = rcp(k.s);
     k.inv2ps = rcp(xadd(R(2), k.s));
     k.cs = xmul(chat, inv_s);
     if (p1) {
@@ -485,45 +479,21 @@ struct ExchangeOut {
 __device__ __forceinline__ float exchange_delta_fp32(const GridParams& g, float chat, float dt, float rho, float kP,
                                                      float E, float T, ExchangeOut& o, float& qout);
 
-__device__ __forceinline__ ExchangeOut exchange_fp64(const GridParams& g, double chat, double dt, double rho,
-                                                     double kP, double& E, double& T)
+// The solve from delta = d0 with clamped FP64 Newton steps and the bisection fallback: the cells that the
+// two steps of exchange_fp64 do not settle (a seed outside the FP32 range).
+struct ExchangeGeneral {
+    double d;
+    int newton_fb, iters;
+};
+static __device__ __noinline__ ExchangeGeneral exchange_general(double A, double B, double C, double e, double c0,
+                                                                double d0)
 {
-    ExchangeOut o = {0, 0, 0};
-    // divisions as Newton-refined reciprocals times the numerator (within an ulp or two; the iteration
-    // below converges to its own rounding fixed point either way)
-    const double c = g.c;
-    const double q = g.gm1_mu * rcp(rho);
-    const double e = rho * T * g.inv_gm1_mu;
-    const double alpha = g.a_rad * (q * q) * (q * q);
-    const double eta = c * kP * dt;
-    const double r = chat * g.inv_c;
-    double th = g.theta_E;
-    double Ebar = e + E * rcp(r);
-    double e4 = (e * e) * (e * e);
-    double c0 = (1.0 - th) * eta * (alpha * e4 - E) - (e + r * eta * th * Ebar);
-    if (c0 > 0.0) {
-        th = 1.0;
-        o.theta_fb = 1;
-        c0 = -(e + r * eta * th * Ebar);
-    }
-    const double A = eta * th * alpha;
-    const double B = 1.0 + r * eta * th;
-    const double C = eta * ((1.0 - th) * alpha * e4 - E);
+    ExchangeGeneral o = {0.0, 0, 0};
     double b = fabs(c0 * rcp(B));
     if (A > 0.0) b = fmin(b, sqrt(sqrt(fabs(c0 * rcp(A)))));
     const double dhi = b - e;   // delta upper bound
     const double dlo = -e;      // x >= 0
-    // start from the same iteration in FP32 (within 2^-25 of the root, on the FP32 pipe; values outside
-    // the FP32 range give a non-finite seed and the start d = 0): one or two FP64 steps then reach the
-    // FP64 rounding fixed point, against up to about fifteen from d = 0 on states far from equilibrium
-    double d = 0.0;
-    {
-        ExchangeOut o32;
-        float q32;
-        const float d32 = exchange_delta_fp32(g, (float)chat, (float)dt, (float)rho, (float)kP, (float)E, (float)T,
-                                              o32, q32);
-        if (isfinite(d32) && !o32.newton_fb) d = fmin(fmax((double)d32, dlo), dhi);
-    }
+    double d = isfinite(d0) ? fmin(fmax(d0, dlo), dhi) : 0.0;
     bool conv = false;
     int it;
     for (it = 0; it < 100; ++it) {
@@ -555,7 +525,67 @@ __device__ __forceinline__ ExchangeOut exchange_fp64(const GridParams& g, double
         }
         d = lo;
     }
-    E = E - r * d;
+    o.d = d;
+    return o;
+}
+
+// FP64 solve.  The same iteration run in FP32 (exchange_delta_fp32, within 2^-25 of the root, on the FP32
+// pipe) gives the start; two Newton steps follow whose residual g is FP64 and whose 1/g' is FP32: each
+// multiplies the error by the relative error of 1/g' (2^-22 and the seed's own) and squares what is left,
+// so the second step is about 2^-47 of x and the result is at the rounding level of g, where the clamped
+// iteration ends as well.  A second step above 2^-36 of x, or anything not finite, sends the cell to
+// exchange_general.  About 30 FP64 instructions with theta = 1, against about 110 when the bracket of the
+// general solve was set up in every cell and each Newton step took its own FP64 reciprocal.
+__device__ __forceinline__ ExchangeOut exchange_fp64(const GridParams& g, double chat, double dt, double rho,
+                                                     double kP, double& E, double& T)
+{
+    ExchangeOut o = {0, 0, 2};
+    const double q = g.gm1_mu * rcp(rho);
+    const double e = rho * T * g.inv_gm1_mu;
+    const double q2 = q * q, alpha = g.a_rad * q2 * q2;
+    const double r = chat * g.inv_c;
+    const double eta = (g.c * dt) * kP;
+    const bool th1 = is_one_d(g.theta_E);
+    double th = g.theta_E, A, B, C;
+    if (th1) {
+        A = eta * alpha;
+        B = fma(r, eta, 1.0);
+        C = -eta * E;
+    } else {
+        const double e4 = (e * e) * (e * e), Ebar = e + E * rcp(r);
+        const double c0 = (1.0 - th) * eta * (alpha * e4 - E) - (e + r * eta * th * Ebar);
+        if (c0 > 0.0) {  // no feasible root (Section 3.4): the step is redone with theta = 1
+            th = 1.0;
+            o.theta_fb = 1;
+        }
+        A = eta * th * alpha;
+        B = 1.0 + r * eta * th;
+        C = eta * ((1.0 - th) * alpha * e4 - E);
+    }
+    ExchangeOut o32;
+    float q32;
+    const float d32 = exchange_delta_fp32(g, d2f_trunc(chat), d2f_trunc(dt), d2f_trunc(rho), d2f_trunc(kP), d2f_trunc(E),
+                                          d2f_trunc(T), o32, q32);
+    double d = f2d_exact(d32);
+    const double x1 = e + d, y1 = x1 * x1, Ay = A * y1;
+    const float x32 = d2f_trunc(x1), gp = 4.0f * d2f_trunc(Ay) * x32 + d2f_trunc(B);
+    const double ig = f2d_exact(rcp(gp));
+    d = fma(-fma(Ay, y1, fma(B, d, C)), ig, d);
+    const double x2 = e + d, y2 = x2 * x2;
+    const double gv = fma(A * y2, y2, fma(B, d, C));
+    const float s2 = d2f_trunc(gv) * d2f_trunc(ig);
+    if (fabsf(s2) <= 1.4551915228366852e-11f * x32 && gp < 1e37f && !o32.newton_fb && o32.theta_fb == o.theta_fb) {
+        d = fma(-gv, ig, d);
+    } else {
+        double c0;
+        if (th1) c0 = -(e + r * eta * (e + E * rcp(r)));
+        else c0 = (1.0 - th) * eta * (alpha * ((e * e) * (e * e)) - E) - (e + r * eta * th * (e + E * rcp(r)));
+        const ExchangeGeneral w = exchange_general(A, B, C, e, c0, isfinite(d32) && !o32.newton_fb ? f2d_exact(d32) : 0.0);
+        d = w.d;
+        o.newton_fb = w.newton_fb;
+        o.iters = w.iters;
+    }
+    E = fma(-r, d, E);
     T = (e + d) * q;
     return o;
 }
@@ -570,13 +600,13 @@ __device__ __forceinline__ void exchange_linear_fp64(const GridParams& g, double
     const double eps = g.linear_eps, c = g.c;
     const double T2 = T * T;
     double v = g.a_rad * T2 * T2;
-    const double dtau = eps * c * kP * dt;
+    const double dtau = (eps * c * dt) * kP;
     const double r = chat * g.inv_eps_c;  // chat / (eps c), 1/(eps c) from the host
     const double dv = -(v - E) * dtau * rcp(1.0 + g.theta_E * (1.0 + r) * dtau);
     E = E + (-r * dv);
     v = v + dv;
-    if (v < 0.0) v = 0.0;
-    T = sqrt(sqrt(v * g.inv_a_rad));
+    v = max0_d(v, 0.0);
+    T = sqrt_fast(sqrt_fast(v * g.inv_a_rad));
 }
 
 // FP32 Newton for delta with the same iteration, which also stops once a step is small enough that
@@ -971,10 +1001,11 @@ __device__ __forceinline__ void hll_stored(const R* base, int stride, int iL, in
 // ------------------------------------------------------------------------------------------------
 // one tile of one subcycle: planes [z0, z1) of the column tile at (x0, y0)
 // ------------------------------------------------------------------------------------------------
-template <typename R, int TX, int TY, int DIM, bool SPLIT>
+template <int TX, int TY, int DIM>
 __device__ __forceinline__ void subcycle_tile(const GridParams& g, const GridArrays& a, double chat_d, double dt_d,
-                                              int x0, int y0, int z0, int z1, R* sm, Counters& cnt)
+                                              int x0, int y0, int z0, int z1, float* sm, Counters& cnt)
 {
+    using R = float;
     using G = Geo<TX, TY, DIM>;
     const int t = threadIdx.x;
     R* Um = sm + G::P_UM;
@@ -1206,7 +1237,7 @@ __device__ __forceinline__ void subcycle_tile(const GridParams& g, const GridArr
                             div[qq] = nd[qq];
                         }
                     }
-                    GasCell<R> gc = load_gas<R, SPLIT>(g, a, x0 + lx, y0 + ly, p, needT_pred, false);
+                    GasCell<R> gc = load_gas<R, true>(g, a, x0 + lx, y0 + ly, p, needT_pred, false);
                     R S[4];
                     explicit_sources(g, gc, U0, chat, S);
                     R U[4];
@@ -1378,7 +1409,7 @@ __device__ __forceinline__ void subcycle_tile(const GridParams& g, const GridArr
 #pragma unroll
                 for (int qq = 0; qq < 4; ++qq) Uhk[qq] = Uk[qq * G::N2 + ih];
                 const bool full = g.exchange == EX_FULL, linear = g.exchange == EX_LINEAR;
-                GasCell<R> gc = load_gas<R, SPLIT>(g, a, gx, gy, k, false, full && !SPLIT);
+                GasCell<R> gc = load_gas<R, true>(g, a, gx, gy, k, false, false);
                 R S[4];
                 explicit_sources(g, gc, Uhk, chat, S);
                 long long li = lin(g, gx, gy, k);
@@ -1387,49 +1418,20 @@ __device__ __forceinline__ void subcycle_tile(const GridParams& g, const GridArr
                 double Un[4];
                 double Tn = needT_corr ? stC[4 * G::NT + t] : 0.0;
                 gc.T = Tn;
-                if constexpr (!SPLIT) {
-                    double U[4];
+                // FP32 increment relative to the FP64 state; the stiff sources in FP64
+                float d[4];
 #pragma unroll
-                    for (int qq = 0; qq < 4; ++qq) U[qq] = U0[qq] - dt_d * (double)div[qq] + dt_d * (double)S[qq];
-                    GasCell<double> gd;
-                    gd.kP = (double)gc.kP;
-                    gd.kF = (double)gc.kF;
-                    gd.T = gc.T;
-                    gd.rho = gc.rho;
-                    gd.j = (double)gc.j;
-                    gd.v[0] = (double)gc.v[0];
-                    gd.v[1] = (double)gc.v[1];
-                    gd.v[2] = (double)gc.v[2];
-                    theta_updates(g, gd, chat_d, dt_d, U);
-                    if (full) {
-                        // transport can leave E <= 0 (not positivity preserving); exchange on E >= E_floor
-                        if (U[0] < g.E_floor) U[0] = g.E_floor;
-                        ExchangeOut o = exchange_fp64(g, chat_d, dt_d, gc.rho, (double)gc.kP, U[0], Tn);
-                        cnt.theta += o.theta_fb;
-                        cnt.newton_fb += o.newton_fb;
-                        cnt.iter_max = max(cnt.iter_max, (unsigned)o.iters);
-                    } else if (linear) {
-                        exchange_linear_fp64(g, chat_d, dt_d, (double)gc.kP, U[0], Tn);
-                    }
-                    cnt.fix += realize(U, g.E_floor);
+                for (int qq = 0; qq < 4; ++qq) d[qq] = -dt * div[qq] + dt * S[qq];
+                split_stiff(g, a, sk, (float)chat, (float)dt, gc, U0, d, Tn, Un, cnt);
+                // realizability: cheap FP32 screen, exact FP64 test only near the limit
+                const float ef = d2f_trunc(Un[0]);
+                float g2f = 0.f;
 #pragma unroll
-                    for (int qq = 0; qq < 4; ++qq) Un[qq] = U[qq];
-                } else {
-                    // FP32 increment relative to the FP64 state; the stiff sources in FP64
-                    float d[4];
-#pragma unroll
-                    for (int qq = 0; qq < 4; ++qq) d[qq] = -dt * div[qq] + dt * S[qq];
-                    split_stiff(g, a, sk, (float)chat, (float)dt, gc, U0, d, Tn, Un, cnt);
-                    // realizability: cheap FP32 screen, exact FP64 test only near the limit
-                    const float ef = d2f_trunc(Un[0]);
-                    float g2f = 0.f;
-#pragma unroll
-                    for (int qq = 1; qq < 4; ++qq) {
-                        const float gq = d2f_trunc(Un[qq]);
-                        g2f += gq * gq;
-                    }
-                    if (!(ef > g.f_E_floor * 1.001f) || g2f > 0.9999f * ef * ef) cnt.fix += realize(Un, g.E_floor);
+                for (int qq = 1; qq < 4; ++qq) {
+                    const float gq = d2f_trunc(Un[qq]);
+                    g2f += gq * gq;
                 }
+                if (!(ef > g.f_E_floor * 1.001f) || g2f > 0.9999f * ef * ef) cnt.fix += realize(Un, g.E_floor);
                 bool bad = !(finite_d(Un[0]) && finite_d(Un[1]) && finite_d(Un[2]) && finite_d(Un[3]) &&
                              (!(full || linear) || finite_d(Tn)));
                 cnt.nonfinite += bad;
@@ -1451,6 +1453,7 @@ __device__ __forceinline__ void subcycle_tile(const GridParams& g, const GridArr
 
 }  // namespace rhd
 
+#include "subcycle_fp64.cuh"
 #include "subcycle_pair.cuh"
 #include "subcycle_twopass.cuh"
 
@@ -1479,7 +1482,8 @@ __global__ void __launch_bounds__(Geo<TX, TY, DIM>::NT,
         z1 = min(z0 + P.z_chunk, P.g.n[2]);
     }
     Counters cnt = {0, 0, 0, 0, 0, 0};
-    subcycle_tile<R, TX, TY, DIM, SPLIT>(P.g, P.a, P.chat, P.dt, x0, y0, z0, z1, sm, cnt);
+    if constexpr (SPLIT) subcycle_tile<TX, TY, DIM>(P.g, P.a, P.chat, P.dt, x0, y0, z0, z1, sm, cnt);
+    else subcycle_tile64<TX, TY, DIM>(P.g, P.a, P.chat, P.dt, x0, y0, z0, z1, sm, cnt);
     add_counter(&P.stats->n_fix, cnt.fix);
     add_counter(&P.stats->n_face, cnt.face);
     add_counter(&P.stats->n_theta, cnt.theta);
@@ -1523,7 +1527,8 @@ __global__ void __launch_bounds__(TX* TY, (TX * TY > 256 || (sizeof(R) == 8 && T
         int tz = (int)(local / ((long long)eg.tiles_x * eg.tiles_y));
         int x0 = (txy % eg.tiles_x) * TX, y0 = (txy / eg.tiles_x) * TY;
         int z0 = tz * P.z_chunk, z1 = min(z0 + P.z_chunk, eg.g.n[2]);
-        subcycle_tile<R, TX, TY, 3, SPLIT>(eg.g, eg.a, P.chat, eg.dt, x0, y0, z0, z1, sm, cnt);
+        if constexpr (SPLIT) subcycle_tile<TX, TY, 3>(eg.g, eg.a, P.chat, eg.dt, x0, y0, z0, z1, sm, cnt);
+        else subcycle_tile64<TX, TY, 3>(eg.g, eg.a, P.chat, eg.dt, x0, y0, z0, z1, sm, cnt);
         __syncthreads();
     }
     add_counter(&P.stats->n_fix, cnt.fix);
