@@ -32,15 +32,13 @@ __device__ __forceinline__ double f2d_exact(float f)
 }
 
 // Square root and reciprocal.  Split path: the hardware approximations (MUFU, about 1-2 ulp), well
-// inside the FP32 error budget of the fluxes.  FP64 path: the FP64 pipe of this part issues one warp
-// instruction per 64 cycles and SM sub-partition, so its instructions are what the FP64 kernels are made
-// of and every one counts: the hardware FP64 approximations (MUFU pipe, relative error below 2^-20) are
-// refined by one third-order step, r <- r (1 + e + e^2) with e = 1 - x r for the reciprocal (the error
-// becomes e^3 < 2^-60; three FP64 instructions against four for two Newton-Raphson steps), and
-// y <- y + y r (1/2 + 3/8 r) with r = 1 - x y^2 for the inverse square root (the dropped term is
-// 5/16 r^3 < 2^-58; five instructions against eight).  Results within an ulp or two, not correctly
-// rounded, which the FP64 path does not need (its bound against the oracle is 1e-12).  Reciprocal: x = 0,
-// +-inf and FP64 denormals (flushed) give NaN.
+// inside the FP32 error budget of the fluxes.  FP64 path: IEEE square root; the reciprocal is the
+// hardware FP64 approximation refined by two Newton-Raphson steps r <- r + r (1 - x r), each of which
+// squares the relative error (from below 2^-20 to below 2^-40, then to rounding): within an ulp or
+// two of 1/x, not the correctly rounded quotient, which the FP64 path does not need (its bound
+// against the oracle is 1e-12) and which costs several more FP64 operations.  x = 0, +-inf and FP64
+// denormals (flushed) give NaN.
+__device__ __forceinline__ double sqrt_fast(double x) { return sqrt(x); }
 __device__ __forceinline__ float sqrt_fast(float x)
 {
     float r;
@@ -51,21 +49,46 @@ __device__ __forceinline__ double rcp(double x)
 {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    double e = fma(-x, r, 1.0);
+    r = fma(r, e, r);
+    e = fma(-x, r, 1.0);
+    return fma(r, e, r);
+}
+// 1/sqrt(x) for normal x > 0, FP64: the hardware approximation refined by two Newton-Raphson steps for
+// f(y) = y^-2 - x, y <- y + (y/2)(1 - x y^2), each of which squares the relative error (within an ulp or
+// two of 1/sqrt(x); tested against CUDA's 1/sqrt).  x sqrt(x)^-1 is then the square root as well.
+__device__ __forceinline__ double rsqrt_nr(double x)
+{
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    double r = __fma_rn(-__dmul_rn(x, y), y, 1.0);
+    y = __fma_rn(__dmul_rn(0.5, y), r, y);
+    r = __fma_rn(-__dmul_rn(x, y), y, 1.0);
+    return __fma_rn(__dmul_rn(0.5, y), r, y);
+}
+// The FP64 kernels of two- and three-dimensional grids are bound by the FP64 pipe (one warp instruction per
+// 64 cycles and SM sub-partition), so they refine the same hardware approximations (MUFU pipe, relative
+// error below 2^-19) by one third-order step: r <- r (1 + e + e^2), e = 1 - x r, for the reciprocal (the
+// error becomes e^3; three FP64 instructions against four for two Newton-Raphson steps), and
+// y <- y + y r (1/2 + 3/8 r), r = 1 - x y^2, for the inverse square root (the dropped term is 5/16 r^3; five
+// against eight).  Within an ulp or two; the special cases of rcp.
+__device__ __forceinline__ double rcp3(double x)
+{
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
     const double e = __fma_rn(-x, r, 1.0);
     return __fma_rn(r, __fma_rn(e, e, e), r);
 }
-// 1/sqrt(x) for normal x > 0, FP64 (within an ulp or two; tested against CUDA's 1/sqrt).  x sqrt(x)^-1 is
-// then the square root as well.
-__device__ __forceinline__ double rsqrt_nr(double x)
+__device__ __forceinline__ double rsqrt3(double x)
 {
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     const double r = __fma_rn(-__dmul_rn(x, y), y, 1.0);
     return __fma_rn(__dmul_rn(y, r), __fma_rn(r, 0.375, 0.5), y);
 }
-// sqrt(x), FP64, by the same step on x y ~ sqrt(x) (five instructions; CUDA's correctly rounded sqrt takes
-// about twice as many and a slow path).  Zero and subnormal x give 0, +inf gives +inf, negative x NaN.
-__device__ __forceinline__ double sqrt_fast(double x)
+// sqrt(x) by the same step on x y ~ sqrt(x) (five instructions; CUDA's correctly rounded sqrt takes about
+// twice as many and a slow path).  Zero and subnormal x give 0, +inf gives +inf, negative x NaN.
+__device__ __forceinline__ double sqrt3(double x)
 {
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
@@ -102,7 +125,12 @@ __device__ __forceinline__ bool pos_d(double x)
     return b > 0 && b <= 0x7ff0000000000000ll;
 }
 __device__ __forceinline__ bool is_one_d(double x) { return __double_as_longlong(x) == 0x3ff0000000000000ll; }
-// x > 1 - 2^-50 (true for +inf, false for NaN)
+// x > 1, and x > 1 - 2^-50 (true for +inf, false for NaN)
+__device__ __forceinline__ bool above1_d(double x)
+{
+    const long long b = __double_as_longlong(x);
+    return b > 0x3ff0000000000000ll && b <= 0x7ff0000000000000ll;
+}
 __device__ __forceinline__ bool reaches1_d(double x)
 {
     const long long b = __double_as_longlong(x);

@@ -83,6 +83,118 @@ cudaError_t launch_subcycle_fp64(const StepParams& p, cudaStream_t s)
     }
 }
 
+// ------------------------------------------------------------------------------------------------ pair
+// FP64 instructions of a tile's plane in units of one warp, counted from subcycle_fp64_pair.cuh (own
+// cells, halo cells, faces beyond the edges; whole warps), and the share of a plane that starting a z
+// chunk costs.
+namespace {
+struct PairCost {
+    double own, halo, face, start;
+};
+constexpr PairCost kPred3 = {180.0, 40.0, 23.0, 0.6}, kPred2 = {140.0, 40.0, 23.0, 0.0};
+constexpr PairCost kCorr3 = {432.0, 56.0, 23.0, 0.4}, kCorr2 = {305.0, 56.0, 23.0, 0.0};
+
+double plane_cost(const PairCost& c, bool predictor, int w, int h)
+{
+    const int edge = (w + h + 31) / 32, halo = predictor ? (2 * (w + h) + 31) / 32 : 2 * edge;
+    return c.own * ((w * h + 31) / 32) + c.halo * halo + c.face * edge;
+}
+
+// Tile shape and planes per CTA for an ex x ey x ez range: the fewest FP64 instructions on the busiest SM.
+// An SM's time is the sum over its CTAs (the pipe is shared), with a tenth more where it has only one to
+// fill the gaps between its phases.  128^3: 16 x 16 x 19 (448 CTAs, three per SM), 3.05 ms a subcycle
+// for both kernels against 3.6 ms with 32 planes per CTA (256 CTAs: one SM in three has half the work).
+void best_split(const PairCost& c, bool predictor, int ex, int ey, int ez, int n_sms, int z_fixed, bool shared,
+                int* bw, int* bh, int* bz)
+{
+    double best = -1.0;
+    for (int w = 8; w <= 32; ++w)
+        for (int h = 8; h <= 32 && w * h <= 256; ++h) {
+            if (w * h < 192 && w < ex && h < ey) continue;
+            const long long tiles = (long long)((ex + w - 1) / w) * ((ey + h - 1) / h);
+            const double pc = plane_cost(c, predictor, w, h);
+            for (int nz = 1; nz <= ez; ++nz) {
+                const int z = z_fixed > 0 ? std::min(z_fixed, ez) : (ez + nz - 1) / nz;
+                const long long ctas = tiles * ((ez + z - 1) / z);
+                const long long per_sm = (ctas + n_sms - 1) / n_sms;
+                const double load = shared ? (double)ctas : (double)per_sm * (per_sm == 1 ? 1.1 : 1.0);
+                const double cost = load * pc * (z + c.start);
+                if (best < 0.0 || cost < best * 0.999) {
+                    best = cost;
+                    *bw = w;
+                    *bh = h;
+                    *bz = z;
+                }
+                if (z_fixed > 0 || z <= 4 || per_sm > 24) break;
+            }
+        }
+}
+}  // namespace
+
+Tile64 pair64_plan(const GridParams& g, int n_sms, int z_chunk, bool shared_queue)
+{
+    Tile64 s;
+    const bool d3 = g.nact == 3;
+    const int e[3] = {upad_extent(g, 0), upad_extent(g, 1), d3 ? upad_extent(g, 2) : 1};
+    best_split(d3 ? kPred3 : kPred2, true, e[0], e[1], e[2], n_sms, z_chunk, shared_queue, &s.pw, &s.ph, &s.pz);
+    best_split(d3 ? kCorr3 : kCorr2, false, g.n[0], g.n[1], d3 ? g.n[2] : 1, n_sms, z_chunk, shared_queue, &s.cw, &s.ch,
+               &s.cz);
+    s.ptx = (e[0] + s.pw - 1) / s.pw;
+    s.pty = (e[1] + s.ph - 1) / s.ph;
+    s.ctx = (g.n[0] + s.cw - 1) / s.cw;
+    s.cty = (g.n[1] + s.ch - 1) / s.ch;
+    return s;
+}
+
+template <typename K>
+static cudaError_t launch_pair64(K k, size_t smem, SmemLimitOnce& once, dim3 grid, const StepParams& p, cudaStream_t s)
+{
+    cudaError_t e = once.set(k, smem);
+    if (e != cudaSuccess) return e;
+    k<<<grid, P64_NT, smem, s>>>(p);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_predictor64(const StepParams& p, cudaStream_t s)
+{
+    static SmemLimitOnce once;
+    const Tile64& t = p.t64;
+    const int ez = p.g.nact == 3 ? upad_extent(p.g, 2) : 1;
+    const dim3 grid((unsigned)(t.ptx * t.pty), (unsigned)((ez + t.pz - 1) / t.pz));
+    return p.g.nact == 3 ? launch_pair64(predictor64_kernel<3>, pair64_pred_smem(), once, grid, p, s)
+                         : launch_pair64(predictor64_kernel<2>, pair64_pred_smem(), once, grid, p, s);
+}
+
+cudaError_t launch_corrector64(const StepParams& p, cudaStream_t s)
+{
+    static SmemLimitOnce once;
+    const Tile64& t = p.t64;
+    const int nz = p.g.nact == 3 ? p.g.n[2] : 1;
+    const dim3 grid((unsigned)(t.ctx * t.cty), (unsigned)((nz + t.cz - 1) / t.cz));
+    return p.g.nact == 3 ? launch_pair64(corrector64_kernel<3>, pair64_corr_smem(), once, grid, p, s)
+                         : launch_pair64(corrector64_kernel<2>, pair64_corr_smem(), once, grid, p, s);
+}
+
+cudaError_t launch_ensemble_pair64(const EnsembleParams& p, bool predictor, int n_ctas, cudaStream_t s)
+{
+    static SmemLimitOnce once;
+    const size_t smem = predictor ? pair64_pred_smem() : pair64_corr_smem();
+    auto k = predictor ? ensemble64_kernel<true> : ensemble64_kernel<false>;
+    cudaError_t e = once.set(k, smem);
+    if (e != cudaSuccess) return e;
+    k<<<n_ctas, P64_NT, smem, s>>>(p);
+    return cudaGetLastError();
+}
+
+int ensemble_ctas_per_sm_pair64()
+{
+    int n = 0;
+    auto k = ensemble64_kernel<false>;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pair64_corr_smem()) != cudaSuccess) return 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, P64_NT, pair64_corr_smem()) != cudaSuccess || n < 1) return 1;
+    return n;
+}
+
 cudaError_t launch_ensemble_fp64(const EnsembleParams& p, int n_ctas, cudaStream_t s)
 {
     return launch_ens_kernel<double, 16, 16, false>(p, n_ctas, s);
@@ -91,7 +203,7 @@ cudaError_t launch_ensemble_fp64(const EnsembleParams& p, int n_ctas, cudaStream
 int ensemble_ctas_per_sm_fp64() { return ens_occupancy<double, 16, 16, false>(); }
 
 // The stiff exchange integrated once per gas step (Section 3.1 step 2, the paper's placement of S_i): in
-// every cell, E floored at E_floor, then the FULL quartic theta scheme of the subcycles (exchange_fp64,
+// every cell, E floored at E_floor, then the FULL quartic theta scheme of the subcycles (exchange64,
 // Eqs. source:energyupdate - source:polynomial) over dt = Delta t_gas, then |G| <= E by rescaling G.
 // FP64 on every grid: it runs once per gas step, not per subcycle.  One thread per cell, grid-stride.
 __global__ void __launch_bounds__(256) gas_exchange_kernel(const __grid_constant__ GasExchangeParams P)
@@ -103,7 +215,7 @@ __global__ void __launch_bounds__(256) gas_exchange_kernel(const __grid_constant
         const double rho = P.rho[i];
         const double kP = P.kP ? P.kP[i] : kappa_law(g.kappa_P, g.kpow, rho);
         if (E < g.E_floor) E = g.E_floor;
-        const ExchangeOut o = exchange_fp64(g, P.chat, P.dt, rho, kP, E, T);
+        const ExchangeOut o = exchange64(g, P.chat, P.dt, rho, kP, E, T);
         cnt.theta += o.theta_fb;
         cnt.newton_fb += o.newton_fb;
         cnt.iter_max = max(cnt.iter_max, (unsigned)o.iters);

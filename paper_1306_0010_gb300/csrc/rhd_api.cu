@@ -78,6 +78,8 @@ struct GridState {
     float4* um32 = nullptr;       // two-pass: FP32 mirror of the current state (valid when um32_ok)
     float4* gas4 = nullptr;       // two-pass: interleaved FP32 (rho, v) (valid when gas4_ok)
     bool um32_ok = false, gas4_ok = false;
+    double* uhalf64 = nullptr;    // FP64 pair (2D, 3D): U^{m+1/2} with its ghost layers; NULL: the fused kernel
+    Tile64 t64 = {};              // its work split for the current z chunk
     CUtensorMap uh_map;           // its tensor map (staging RHD_STAGING_TMA), valid when uh_map_ok
     bool uh_map_ok = false;
     const double* dir_dev = nullptr;  // low x Dirichlet state in device memory (rhd_marshak_advance only)
@@ -132,6 +134,7 @@ struct rhd_ctx {
     unsigned long long* d_counter = nullptr;
     long long n_items = 0, n_pitems = 0;
     int ens_ctas = 0, ens_pctas = 0, ens_cctas = 0;  // fused / predictor / corrector persistent CTAs
+    bool ens_pair64 = false;       // FP64: every grid has the pair's U^{m+1/2}
 };
 
 namespace {
@@ -341,6 +344,7 @@ void free_grid(GridState& gs)
     dfree(gs.kF32);
     dfree(gs.j32);
     dfree(gs.uhalf);
+    dfree(gs.uhalf64);
     dfree(gs.um32);
     dfree(gs.gas4);
     for (int q = 0; q < 5; ++q) {
@@ -387,6 +391,25 @@ void free_twopass(GridState& gs)
     gs.um32_ok = gs.gas4_ok = false;
 }
 
+// FP64 grids of two or three dimensions: U^{m+1/2} of the kernel pair (32 bytes per stored cell).  A grid
+// that leaves no room for it runs the fused kernel, which needs none.
+void alloc_pair64(rhd_ctx* ctx, GridState& gs)
+{
+    if (gs.desc.precision != RHD_FP64 || gs.gp.nact < 2) return;
+    size_t np = (size_t)upad_extent(gs.gp, 0) * upad_extent(gs.gp, 1);
+    if (gs.gp.nact == 3) np *= (size_t)upad_extent(gs.gp, 2);
+    const std::string err = ctx->err;
+    if (dalloc(ctx, (void**)&gs.uhalf64, 4 * sizeof(double) * np)) ctx->err = err;
+}
+
+// The pair's work split: z_chunk planes per CTA, or its own choice (0), which then is the grid's z chunk
+void plan_pair64(rhd_ctx* ctx, GridState& gs, int z_chunk)
+{
+    if (!gs.uhalf64) return;
+    gs.t64 = pair64_plan(gs.gp, ctx->num_sms, z_chunk, ctx->ensemble);
+    if (z_chunk == 0) gs.z_chunk = gs.t64.cz;
+}
+
 rhd_status alloc_grid(rhd_ctx* ctx, GridState& gs)
 {
     size_t bytes = sizeof(double) * (size_t)gs.ncell;
@@ -404,6 +427,8 @@ rhd_status alloc_grid(rhd_ctx* ctx, GridState& gs)
         if (st) return st;
     }
     if (gs.variant == RHD_VARIANT_TWOPASS) return alloc_twopass(ctx, gs);
+    alloc_pair64(ctx, gs);
+    plan_pair64(ctx, gs, gs.desc.z_chunk);
     return RHD_OK;
 }
 
@@ -622,6 +647,8 @@ StepParams step_params(rhd_ctx* ctx, GridState& gs, int src, double chat, double
     p.f_chat = (float)chat;
     p.f_dt = (float)dt;
     p.uhalf = gs.uhalf;
+    p.uhalf64 = gs.uhalf64;
+    p.t64 = gs.t64;
     p.staging = gs.staging;
     p.wait_polls = ctx->wait_polls;
     if (gs.staging == RHD_STAGING_TMA) p.uh_map = gs.uh_map;
@@ -651,13 +678,16 @@ rhd_status check_dt(rhd_ctx* ctx, const GridState& gs, double chat, double dt)
 enum KernelId {
     K_FUSED_FP64 = 0, K_FUSED_SPLIT, K_PREDICTOR, K_CORRECTOR, K_ENS_FP64, K_ENS_SPLIT, K_ENS_PRED, K_ENS_CORR,
     K_GAS_PRED_FLUX, K_GAS_PRED_UPDATE, K_GAS_CORR_FLUX, K_GAS_CORR_UPDATE, K_GAS_CORRECT, K_GAS_EXCHANGE,
+    K_PRED64, K_CORR64, K_ENS_PRED64, K_ENS_CORR64,
     K_COUNT
 };
 const char* const kKernelNames[K_COUNT] = {"subcycle_fused_fp64", "subcycle_fused_split", "twopass_predictor_split",
                                            "twopass_corrector_split", "ensemble_fp64", "ensemble_split",
                                            "ensemble_predictor_split", "ensemble_corrector_split",
                                            "gas_predictor_flux", "gas_predictor_update", "gas_corrector_flux",
-                                           "gas_corrector_update", "gas_source_correction", "gas_step_exchange"};
+                                           "gas_corrector_update", "gas_source_correction", "gas_step_exchange",
+                                           "predictor_fp64", "corrector_fp64", "ensemble_predictor_fp64",
+                                           "ensemble_corrector_fp64"};
 
 // Algorithmic bytes per interior cell of one launch of kernel k: every array the kernel reads, read
 // once, and every array it writes, written once.  Fused kernels: U^m and U^{m+1} (4 FP64 each), the
@@ -676,6 +706,9 @@ double alg_bytes_per_cell(const GridState& gs, int k)
     switch (k) {
     case K_PREDICTOR: return 16.0 + 16.0 + opt + (ex == RHD_EX_FROZEN_T ? 8.0 : 0.0) + 16.0;
     case K_CORRECTOR: return 16.0 + 32.0 + 16.0 + opt + Tr + 32.0 + Tw + 16.0;
+    // the FP64 pair: U^{m+1/2} in FP64 (32 B) written by the predictor and read by the corrector
+    case K_PRED64: return 32.0 + gas + (ex == RHD_EX_FROZEN_T ? 8.0 : 0.0) + 32.0;
+    case K_CORR64: return 32.0 + 32.0 + gas + Tr + 32.0 + Tw;
     default: return 32.0 + gas + Tr + 32.0 + Tw;
     }
 }
@@ -731,6 +764,13 @@ rhd_status launch_one(rhd_ctx* ctx, GridState& gs, int src, double chat, double 
     StepParams p = step_params(ctx, gs, src, chat, dt);
     cudaStream_t s = ctx->stream;
     const double nc = (double)gs.ncell;
+    if (gs.uhalf64) {
+        rhd_status st = timed_launch(ctx, K_PRED64, nc * alg_bytes_per_cell(gs, K_PRED64),
+                                     [&] { return launch_predictor64(p, s); });
+        if (st) return st;
+        return timed_launch(ctx, K_CORR64, nc * alg_bytes_per_cell(gs, K_CORR64),
+                            [&] { return launch_corrector64(p, s); });
+    }
     if (gs.desc.precision != RHD_SPLIT)
         return timed_launch(ctx, K_FUSED_FP64, nc * alg_bytes_per_cell(gs, K_FUSED_FP64),
                             [&] { return launch_subcycle_fp64(p, s); });
@@ -830,6 +870,16 @@ rhd_status ens_prepare(rhd_ctx* ctx, double chat, const double* dt_per_grid, dou
             eg[i].tiles_x = (gs.desc.n[0] + etx - 1) / etx;
             eg[i].tiles_y = (gs.desc.n[1] + ety - 1) / ety;
             eg[i].tiles_z = (gs.desc.n[2] + gs.z_chunk - 1) / gs.z_chunk;
+            if (ctx->ens_pair64) {
+                const Tile64& t = gs.t64;
+                eg[i].uhalf64 = gs.uhalf64;
+                eg[i].t64 = t;
+                eg[i].tiles_x = t.ctx;
+                eg[i].tiles_y = t.cty;
+                eg[i].tiles_z = (gs.desc.n[2] + t.cz - 1) / t.cz;
+                eg[i].first_pitem = pfirst;
+                pfirst += (long long)t.ptx * t.pty * ((upad_extent(gs.gp, 2) + t.pz - 1) / t.pz);
+            }
             eg[i].first_item = first;
             first += (long long)eg[i].tiles_x * eg[i].tiles_y * eg[i].tiles_z;
             if (twopass) {  // predictor items: 32 x 8 tiles of the stored U^{m+1/2} (ghost layers included)
@@ -867,6 +917,21 @@ rhd_status ens_launch(rhd_ctx* ctx, double chat, int src)
     ep.z_chunk = ctx->grids[0].z_chunk;
     ep.limiter = ctx->grids[0].desc.limiter;
     ep.stats = ctx->dstats;
+    if (ctx->ens_pair64) {
+        double pb = 0.0, cb = 0.0;
+        for (auto& gs : ctx->grids) {
+            pb += (double)gs.ncell * alg_bytes_per_cell(gs, K_PRED64);
+            cb += (double)gs.ncell * alg_bytes_per_cell(gs, K_CORR64);
+        }
+        RHD_CUDA(ctx, cudaMemsetAsync(ctx->d_counter, 0, 2 * sizeof(unsigned long long), ctx->stream));
+        ep.counter = ctx->d_counter;
+        rhd_status st = timed_launch(ctx, K_ENS_PRED64, pb,
+                                     [&] { return launch_ensemble_pair64(ep, true, ctx->ens_pctas, ctx->stream); });
+        if (st) return st;
+        ep.counter = ctx->d_counter + 1;
+        return timed_launch(ctx, K_ENS_CORR64, cb,
+                            [&] { return launch_ensemble_pair64(ep, false, ctx->ens_cctas, ctx->stream); });
+    }
     if (!twopass) {
         double bytes = 0.0;
         for (auto& gs : ctx->grids) {
@@ -948,6 +1013,7 @@ rhd_status apply_config(rhd_ctx* ctx, GridState& gs, const rhd_launch_config& c)
     gs.tiles_x = (gs.desc.n[0] + gs.tx - 1) / gs.tx;
     gs.tiles_y = (gs.desc.n[1] + gs.ty - 1) / gs.ty;
     gs.z_chunk = std::max(1, std::min(c.z_chunk, gs.desc.n[2]));
+    plan_pair64(ctx, gs, gs.z_chunk);
     clear_graphs(ctx);
     return RHD_OK;
 }
@@ -1165,6 +1231,7 @@ rhd_status ens_apply(rhd_ctx* ctx, int v, int zc)
         gs.um32_ok = false;
         gs.variant = v;
         gs.z_chunk = zc;  // one chunk length for all grids, as at creation
+        plan_pair64(ctx, gs, zc);
     }
     clear_graphs(ctx);
     return RHD_OK;
@@ -1939,7 +2006,26 @@ rhd_status rhd_ensemble_create(rhd_ctx** out, int n_grids, const rhd_grid_desc* 
         }
         // one z chunk for all grids (the largest grid's automatic choice)
         int zc = descs[0].z_chunk > 0 ? descs[0].z_chunk : 32;
-        for (auto& gs : ctx->grids) gs.z_chunk = zc;
+        if (!st && descs[0].precision == RHD_FP64) {
+            ctx->ens_pair64 = true;
+            for (auto& gs : ctx->grids) ctx->ens_pair64 = ctx->ens_pair64 && gs.uhalf64;
+            if (!ctx->ens_pair64)
+                for (auto& gs : ctx->grids) dfree(gs.uhalf64);
+            // shorter chunks (each costs less than a plane more) until the items even out over the SMs
+            while (ctx->ens_pair64 && descs[0].z_chunk == 0) {
+                long long n = 0;
+                for (auto& gs : ctx->grids) {
+                    plan_pair64(ctx, gs, zc);
+                    n += (long long)gs.t64.ctx * gs.t64.cty * ((gs.desc.n[2] + zc - 1) / zc);
+                }
+                if (zc <= 8 || n >= 16LL * ctx->num_sms) break;
+                zc /= 2;
+            }
+        }
+        for (auto& gs : ctx->grids) {
+            gs.z_chunk = zc;
+            plan_pair64(ctx, gs, zc);
+        }
         for (auto& gs : ctx->grids)
             items += (long long)gs.tiles_x * gs.tiles_y * ((gs.desc.n[2] + zc - 1) / zc);
         ctx->n_items = items;
@@ -1949,6 +2035,7 @@ rhd_status rhd_ensemble_create(rhd_ctx** out, int n_grids, const rhd_grid_desc* 
         if (!st) {
             int per_sm = descs[0].precision == RHD_SPLIT ? ensemble_ctas_per_sm_split() : ensemble_ctas_per_sm_fp64();
             ctx->ens_ctas = per_sm * ctx->num_sms;
+            if (ctx->ens_pair64) ctx->ens_pctas = ctx->ens_cctas = ensemble_ctas_per_sm_pair64() * ctx->num_sms;
             if (descs[0].precision == RHD_SPLIT) {
                 ctx->ens_pctas = ensemble_ctas_per_sm_predictor() * ctx->num_sms;
                 ctx->ens_cctas = ensemble_ctas_per_sm_corrector() * ctx->num_sms;

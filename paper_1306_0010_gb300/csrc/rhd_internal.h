@@ -76,12 +76,21 @@ struct GridArrays {
                                 // written by a kernel before each subcycle (fused kernels; else NULL)
 };
 
+// Work split of the FP64 kernel pair (subcycle_fp64_pair.cuh): tile width and height, planes per CTA and
+// tiles in x and y of the predictor (p) and the corrector (c)
+struct Tile64 {
+    int pw, ph, pz, ptx, pty;
+    int cw, ch, cz, ctx, cty;
+};
+
 struct StepParams {
     GridParams g;
     GridArrays a;
     double chat, dt;
     float f_chat, f_dt;         // FP32 copies: FP32 code reads them as constant operands (no conversion)
     float4* uhalf;              // two-pass split path: U^{m+1/2} on the grid plus its ghost layers (pad[])
+    double* uhalf64;            // FP64 pair: U^{m+1/2}, 4 doubles per cell of the same extent
+    Tile64 t64;
     int z_chunk;                // planes per CTA
     int tx, ty;                 // tile shape (selects the kernel instantiation)
     int tiles_x, tiles_y;       // tile grid in x, y
@@ -117,6 +126,8 @@ struct EnsembleGrid {
     float4* uhalf;
     int ptiles_x, ptiles_y, ptiles_z;
     long long first_pitem;
+    double* uhalf64;            // FP64 pair: likewise, with its work split
+    Tile64 t64;
 };
 
 struct EnsembleParams {
@@ -175,6 +186,14 @@ cudaError_t launch_to_gas4(float4* dst, const float* rho32, const float* vx, con
 // missing or the encoding is refused.
 bool encode_uhalf_map(CUtensorMap* map, float4* uhalf, const GridParams& g);
 cudaError_t launch_ensemble_fp64(const EnsembleParams& p, int n_ctas, cudaStream_t s);
+// the FP64 kernel pair of 2D and 3D grids, and of ensembles
+cudaError_t launch_predictor64(const StepParams& p, cudaStream_t s);
+cudaError_t launch_corrector64(const StepParams& p, cudaStream_t s);
+cudaError_t launch_ensemble_pair64(const EnsembleParams& p, bool predictor, int n_ctas, cudaStream_t s);
+int ensemble_ctas_per_sm_pair64();
+// Work split of one grid on n_sms SMs; z_chunk > 0 fixes the planes per CTA of both kernels.  shared_queue:
+// the CTAs of many grids share the SMs (ensembles), so only the total work counts.
+Tile64 pair64_plan(const GridParams& g, int n_sms, int z_chunk, bool shared_queue);
 cudaError_t launch_gas_exchange(const GasExchangeParams& p, int num_sms, cudaStream_t s);
 cudaError_t launch_ensemble_split(const EnsembleParams& p, int n_ctas, cudaStream_t s);
 int ensemble_ctas_per_sm_fp64();

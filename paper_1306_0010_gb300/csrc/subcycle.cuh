@@ -140,8 +140,14 @@ __device__ __forceinline__ ClosureScalars<R> closure_scalars(R E, R gx, R gy, R 
     }
     k.invE = invE;
     const R x4 = xfma(R(-3), f2, R(4));  // in [1, 4]
-    k.s = sqrt_fast(x4);
-    const R inv_s = rcp(k.s);
+    R inv_s;
+    if constexpr (sizeof(R) == 8) {
+        inv_s = rsqrt_nr(x4);  // s and 1/s from one refined inverse square root
+        k.s = xmul(x4, inv_s);
+    } else {
+        k.s = sqrt_fast(x4);
+        inv_s = rcp(k.s);
+    }
     k.inv2ps = rcp(xadd(R(2), k.s));
     k.cs = xmul(chat, inv_s);
     if (p1) {
@@ -536,11 +542,11 @@ static __device__ __noinline__ ExchangeGeneral exchange_general(double A, double
 // iteration ends as well.  A second step above 2^-36 of x, or anything not finite, sends the cell to
 // exchange_general.  About 30 FP64 instructions with theta = 1, against about 110 when the bracket of the
 // general solve was set up in every cell and each Newton step took its own FP64 reciprocal.
-__device__ __forceinline__ ExchangeOut exchange_fp64(const GridParams& g, double chat, double dt, double rho,
+__device__ __forceinline__ ExchangeOut exchange64(const GridParams& g, double chat, double dt, double rho,
                                                      double kP, double& E, double& T)
 {
     ExchangeOut o = {0, 0, 2};
-    const double q = g.gm1_mu * rcp(rho);
+    const double q = g.gm1_mu * rcp3(rho);
     const double e = rho * T * g.inv_gm1_mu;
     const double q2 = q * q, alpha = g.a_rad * q2 * q2;
     const double r = chat * g.inv_c;
@@ -552,7 +558,7 @@ __device__ __forceinline__ ExchangeOut exchange_fp64(const GridParams& g, double
         B = fma(r, eta, 1.0);
         C = -eta * E;
     } else {
-        const double e4 = (e * e) * (e * e), Ebar = e + E * rcp(r);
+        const double e4 = (e * e) * (e * e), Ebar = e + E * rcp3(r);
         const double c0 = (1.0 - th) * eta * (alpha * e4 - E) - (e + r * eta * th * Ebar);
         if (c0 > 0.0) {  // no feasible root (Section 3.4): the step is redone with theta = 1
             th = 1.0;
@@ -578,14 +584,90 @@ __device__ __forceinline__ ExchangeOut exchange_fp64(const GridParams& g, double
         d = fma(-gv, ig, d);
     } else {
         double c0;
-        if (th1) c0 = -(e + r * eta * (e + E * rcp(r)));
-        else c0 = (1.0 - th) * eta * (alpha * ((e * e) * (e * e)) - E) - (e + r * eta * th * (e + E * rcp(r)));
+        if (th1) c0 = -(e + r * eta * (e + E * rcp3(r)));
+        else c0 = (1.0 - th) * eta * (alpha * ((e * e) * (e * e)) - E) - (e + r * eta * th * (e + E * rcp3(r)));
         const ExchangeGeneral w = exchange_general(A, B, C, e, c0, isfinite(d32) && !o32.newton_fb ? f2d_exact(d32) : 0.0);
         d = w.d;
         o.newton_fb = w.newton_fb;
         o.iters = w.iters;
     }
     E = fma(-r, d, E);
+    T = (e + d) * q;
+    return o;
+}
+
+// 1D grids: the clamped iteration from the FP32 seed, FP64 throughout.
+__device__ __forceinline__ ExchangeOut exchange_fp64(const GridParams& g, double chat, double dt, double rho,
+                                                     double kP, double& E, double& T)
+{
+    ExchangeOut o = {0, 0, 0};
+    // divisions as Newton-refined reciprocals times the numerator (within an ulp or two; the iteration
+    // below converges to its own rounding fixed point either way)
+    const double c = g.c;
+    const double q = g.gm1_mu * rcp(rho);
+    const double e = rho * T * g.inv_gm1_mu;
+    const double alpha = g.a_rad * (q * q) * (q * q);
+    const double eta = c * kP * dt;
+    const double r = chat * g.inv_c;
+    double th = g.theta_E;
+    double Ebar = e + E * rcp(r);
+    double e4 = (e * e) * (e * e);
+    double c0 = (1.0 - th) * eta * (alpha * e4 - E) - (e + r * eta * th * Ebar);
+    if (c0 > 0.0) {
+        th = 1.0;
+        o.theta_fb = 1;
+        c0 = -(e + r * eta * th * Ebar);
+    }
+    const double A = eta * th * alpha;
+    const double B = 1.0 + r * eta * th;
+    const double C = eta * ((1.0 - th) * alpha * e4 - E);
+    double b = fabs(c0 * rcp(B));
+    if (A > 0.0) b = fmin(b, sqrt(sqrt(fabs(c0 * rcp(A)))));
+    const double dhi = b - e;   // delta upper bound
+    const double dlo = -e;      // x >= 0
+    // start from the same iteration in FP32 (within 2^-25 of the root, on the FP32 pipe; values outside
+    // the FP32 range give a non-finite seed and the start d = 0): one or two FP64 steps then reach the
+    // FP64 rounding fixed point, against up to about fifteen from d = 0 on states far from equilibrium
+    double d = 0.0;
+    {
+        ExchangeOut o32;
+        float q32;
+        const float d32 = exchange_delta_fp32(g, (float)chat, (float)dt, (float)rho, (float)kP, (float)E, (float)T,
+                                              o32, q32);
+        if (isfinite(d32) && !o32.newton_fb) d = fmin(fmax((double)d32, dlo), dhi);
+    }
+    bool conv = false;
+    int it;
+    for (it = 0; it < 100; ++it) {
+        double x = e + d;
+        double x2 = x * x;
+        double gv = A * x2 * x2 + B * d + C;
+        double gp = 4.0 * A * x2 * x + B;
+        double dn = d - gv * rcp(gp);
+        if (dn > dhi) dn = dhi;
+        if (dn < dlo) dn = dlo;
+        if (it > 0 && !(dn < d)) {
+            conv = true;
+            break;
+        }
+        d = dn;
+    }
+    o.iters = it;
+    if (!conv) {
+        // bisection to adjacent doubles on [dlo, dhi]
+        o.newton_fb = 1;
+        double lo = dlo, hi = dhi;
+        for (int k = 0; k < 2200; ++k) {
+            double mid = lo + 0.5 * (hi - lo);
+            if (!(mid > lo && mid < hi)) break;
+            double x = e + mid;
+            double x2 = x * x;
+            double gv = A * x2 * x2 + B * mid + C;
+            if (gv <= 0.0) lo = mid; else hi = mid;
+        }
+        d = lo;
+    }
+    E = E - r * d;
     T = (e + d) * q;
     return o;
 }
@@ -606,7 +688,7 @@ __device__ __forceinline__ void exchange_linear_fp64(const GridParams& g, double
     E = E + (-r * dv);
     v = v + dv;
     v = max0_d(v, 0.0);
-    T = sqrt_fast(sqrt_fast(v * g.inv_a_rad));
+    T = sqrt3(sqrt3(v * g.inv_a_rad));
 }
 
 // FP32 Newton for delta with the same iteration, which also stops once a step is small enough that
@@ -1456,6 +1538,7 @@ __device__ __forceinline__ void subcycle_tile(const GridParams& g, const GridArr
 #include "subcycle_fp64.cuh"
 #include "subcycle_pair.cuh"
 #include "subcycle_twopass.cuh"
+#include "subcycle_fp64_pair.cuh"
 
 namespace rhd {
 

@@ -25,7 +25,7 @@ struct Closure64 {
 __device__ __forceinline__ Closure64 closure64(const double U[4], int p1)
 {
     Closure64 k;
-    const double invE = rcp(U[0]);
+    const double invE = rcp3(U[0]);
 #pragma unroll
     for (int d = 0; d < 3; ++d) k.f[d] = xmul(U[1 + d], invE);
     double f2 = xfma(k.f[2], k.f[2], xfma(k.f[1], k.f[1], xmul(k.f[0], k.f[0])));
@@ -33,15 +33,15 @@ __device__ __forceinline__ Closure64 closure64(const double U[4], int p1)
     // light cone to the rounding of f^2 (a rescaled one, a beam), whose 1 - f^2 of a few 2^-53 would
     // otherwise enter the speeds across G as its square root
     if (reaches1_d(f2)) {
-        const double q = rsqrt_nr(f2);
+        const double q = rsqrt3(f2);
 #pragma unroll
         for (int d = 0; d < 3; ++d) k.f[d] = xmul(k.f[d], q);
         f2 = 1.0;
     }
     const double x4 = xfma(-3.0, f2, 4.0);  // in [1, 4]
-    k.is = rsqrt_nr(x4);
+    k.is = rsqrt3(x4);
     k.s = xmul(x4, k.is);
-    k.i3 = rcp(xfma(k.s, 1.0 / 3.0, 2.0 / 3.0));
+    k.i3 = rcp3(xfma(k.s, 1.0 / 3.0, 2.0 / 3.0));
     k.k23 = xmul(xadd(k.s, -1.0), 2.0 / 3.0);
     if (p1) {
         k.a = xmul(U[0], 1.0 / 3.0);
@@ -63,7 +63,7 @@ __device__ __forceinline__ void speeds64(const Closure64& k, double fd, int fixe
         return;
     }
     const double rad = xmul(k.k23, xfma(-xmul(fd, fd), k.i3, k.s));
-    const double sr = sqrt_fast(max0_d(rad, 0.0));
+    const double sr = sqrt3(max0_d(rad, 0.0));
     const double m = xmul(fd, k.is);
     l1 = xfma(-sr, k.is, m);
     l3 = xfma(sr, k.is, m);
@@ -88,7 +88,7 @@ __device__ __forceinline__ void hll64(const double UL[4], const double UR[4], co
     const double den = xadd(SRp, -SLm);
     double wL = 0.5, wR = 0.5, wU = 0.0;
     if (mag_bits(den) != 0) {
-        const double inv = rcp(den);
+        const double inv = rcp3(den);
         wL = xmul(SRp, inv);
         wR = xmul(-SLm, inv);
         wU = xmul(wL, SLm);
@@ -182,17 +182,46 @@ __device__ __forceinline__ void sources64(const GridParams& g, const GasCell<dou
         for (int q = 0; q < 3; ++q) U[1 + q] = xfma(m, gc.v[q], U[1 + q]);
     }
     double fF;
-    if (is_one_d(g.theta_F)) fF = rcp(xadd(1.0, xF));
-    else fF = xfma(-(1.0 - g.theta_F), xF, 1.0) * rcp(xfma(g.theta_F, xF, 1.0));
+    if (is_one_d(g.theta_F)) fF = rcp3(xadd(1.0, xF));
+    else fF = xfma(-(1.0 - g.theta_F), xF, 1.0) * rcp3(xfma(g.theta_F, xF, 1.0));
 #pragma unroll
     for (int q = 1; q < 4; ++q) U[q] = xmul(U[q], fF);
     if (g.exchange == EX_ABSORB) {
         const double xP = chat_h * gc.kP;
-        U[0] *= (1.0 - (1.0 - g.theta_E) * xP) * rcp(1.0 + g.theta_E * xP);
+        U[0] *= (1.0 - (1.0 - g.theta_E) * xP) * rcp3(1.0 + g.theta_E * xP);
     } else if (g.exchange == EX_FROZEN_T) {
         const double xP = chat_h * gc.kP, T2 = gc.T * gc.T;
-        U[0] = (U[0] * (1.0 - (1.0 - g.theta_E) * xP) + xP * (g.a_rad * T2 * T2)) * rcp(1.0 + g.theta_E * xP);
+        U[0] = (U[0] * (1.0 - (1.0 - g.theta_E) * xP) + xP * (g.a_rad * T2 * T2)) * rcp3(1.0 + g.theta_E * xP);
     }
+}
+
+// The end of the corrector for one cell: U holds U^m plus its flux differences; the explicit sources from
+// U^{m+1/2} (Uhk), the theta updates, the exchange and realizability follow, then the stores at li.
+__device__ __forceinline__ void finish_cell64(const GridParams& g, const GridArrays& a, GasCell<double>& gc, double chat,
+                                              double dt, const double Uhk[4], double U[4], double Tn, bool has_j,
+                                              bool full, bool linear, long long li, Counters& cnt)
+{
+    gc.T = Tn;
+    sources64(g, gc, Uhk, chat * dt, chat * dt * g.inv_c, has_j, U);
+    if (full) {
+        // transport can leave E <= 0 (not positivity preserving); exchange on E >= E_floor
+        if (!(d2f_trunc(U[0]) > g.f_E_floor * 1.001f) && U[0] < g.E_floor) U[0] = g.E_floor;
+        const ExchangeOut o = exchange64(g, chat, dt, gc.rho, gc.kP, U[0], Tn);
+        cnt.theta += o.theta_fb;
+        cnt.newton_fb += o.newton_fb;
+        cnt.iter_max = max(cnt.iter_max, (unsigned)o.iters);
+    } else if (linear) {
+        exchange_linear_fp64(g, chat, dt, gc.kP, U[0], Tn);
+    }
+    cnt.fix += realize64(U, g.E_floor, g.f_E_floor);
+    const bool bad = !(finite_d(U[0]) && finite_d(U[1]) && finite_d(U[2]) && finite_d(U[3]) &&
+                       (!(full || linear) || finite_d(Tn)));
+    cnt.nonfinite += bad;
+    a.Eo[li] = U[0];
+    a.Go[0][li] = U[1];
+    a.Go[1][li] = U[2];
+    a.Go[2][li] = U[3];
+    if (full || linear) a.T[li] = Tn;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -527,27 +556,7 @@ __device__ __forceinline__ void subcycle_tile64(const GridParams& g, const GridA
                     if (DIM == 3) U[qq] = xfma(-cz, dz[qq], U[qq]);
                 }
                 double Tn = needT_corr ? stC[4 * G::NT + t] : 0.0;
-                gc.T = Tn;
-                sources64(g, gc, Uhk, chat * dt, chat * dt * g.inv_c, has_j, U);
-                if (full) {
-                    // transport can leave E <= 0 (not positivity preserving); exchange on E >= E_floor
-                    if (!(d2f_trunc(U[0]) > g.f_E_floor * 1.001f) && U[0] < g.E_floor) U[0] = g.E_floor;
-                    const ExchangeOut o = exchange_fp64(g, chat, dt, gc.rho, gc.kP, U[0], Tn);
-                    cnt.theta += o.theta_fb;
-                    cnt.newton_fb += o.newton_fb;
-                    cnt.iter_max = max(cnt.iter_max, (unsigned)o.iters);
-                } else if (linear) {
-                    exchange_linear_fp64(g, chat, dt, gc.kP, U[0], Tn);
-                }
-                cnt.fix += realize64(U, g.E_floor, g.f_E_floor);
-                const bool bad = !(finite_d(U[0]) && finite_d(U[1]) && finite_d(U[2]) && finite_d(U[3]) &&
-                                   (!(full || linear) || finite_d(Tn)));
-                cnt.nonfinite += bad;
-                a.Eo[li] = U[0];
-                a.Go[0][li] = U[1];
-                a.Go[1][li] = U[2];
-                a.Go[2][li] = U[3];
-                if (full || linear) a.T[li] = Tn;
+                finish_cell64(g, a, gc, chat, dt, Uhk, U, Tn, has_j, full, linear, li, cnt);
             }
         }
         __syncthreads();

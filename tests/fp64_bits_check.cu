@@ -21,7 +21,7 @@ __global__ void check_kernel(const double* x, const double* y, double* out, int 
     out[5 * i + 1] = rhd::min0_d(x[i], y[i]);
     out[5 * i + 2] = rhd::minmod_d(x[i], y[i]);
     out[5 * i + 3] = rhd::reaches1_d(x[i]) ? 1.0 : 0.0;
-    out[5 * i + 4] = rhd::sqrt_fast(x[i]);
+    out[5 * i + 4] = rhd::sqrt3(x[i]);
 }
 
 static int64_t bits(double v)
