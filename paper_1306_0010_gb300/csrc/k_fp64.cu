@@ -74,10 +74,59 @@ bool tile_supported(int precision, int nact, int tx, int ty)
     return (tx == 32 && ty == 16) || (tx == 64 && ty == 8);
 }
 
+// 1D grids.  Two threads per cell and up to eight subcycles per launch (a tile of 64 - 6 x 8 = 16 cells of the
+// 64 a CTA holds) while the tiles find an SM each (split: a quarter, the FP32 pipes take several warps);
+// the longest run of subcycles that does, since the halo's redone work is on idle SMs.  Beyond that (8816
+// cells in FP64, 35264 split) one thread per cell and one subcycle per launch, where the cells beyond a
+// tile cost a twentieth and not three quarters of the work.  A line with one periodic end alone has ghost cells
+// from its far end, which only the state in memory holds: one subcycle per launch.
+LinePlan line_plan(const GridParams& g, bool split, int n_sms)
+{
+    const long long most = (long long)n_sms * (split ? 4 : 1);
+    const bool half_periodic = (g.bc_lo[0] == BC_PERIODIC) != (g.bc_hi[0] == BC_PERIODIC);
+    for (int steps = half_periodic ? 1 : 8; steps >= 1; --steps) {
+        const int tile = LINE_NT / 2 - 6 * steps;
+        if ((g.n[0] + tile - 1) / tile <= most) return {2, steps};
+    }
+    return {1, 1};
+}
+
+LineParams line_params(const StepParams& p, int steps, int tpc, double* To)
+{
+    LineParams l;
+    l.g = p.g;
+    l.a = p.a;
+    l.To = To;
+    l.chat = p.chat;
+    l.dt = p.dt;
+    l.f_chat = p.f_chat;
+    l.f_dt = p.f_dt;
+    l.steps = steps;
+    l.tile = LINE_NT / tpc - 6 * steps;
+    l.stats = p.stats;
+    return l;
+}
+
+cudaError_t launch_line_fp64(const LineParams& p, int tpc, cudaStream_t s)
+{
+    const unsigned nb = (unsigned)((p.g.n[0] + p.tile - 1) / p.tile);
+    if (tpc == 2) line_kernel<double, 2><<<nb, LINE_NT, 0, s>>>(p);
+    else line_kernel<double, 1><<<nb, LINE_NT, 0, s>>>(p);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_line(const LineParams& p, bool split, int tpc, cudaStream_t s)
+{
+    return split ? launch_line_split(p, tpc, s) : launch_line_fp64(p, tpc, s);
+}
+
 cudaError_t launch_subcycle_fp64(const StepParams& p, cudaStream_t s)
 {
     switch (p.g.nact) {
-    case 1: return launch_tile_kernel<double, 122, 1, 1, false>(p, s);
+    case 1: {  // one subcycle, T in place
+        const int tpc = line_plan(p.g, false, 152).tpc;
+        return launch_line_fp64(line_params(p, 1, tpc, p.a.T), tpc, s);
+    }
     case 2: return launch_tile_kernel<double, 16, 16, 2, false>(p, s);
     default: return launch_tile_kernel<double, 16, 16, 3, false>(p, s);
     }

@@ -42,10 +42,21 @@ static int ens_occupancy()
 }
 
 
+cudaError_t launch_line_split(const LineParams& p, int tpc, cudaStream_t s)
+{
+    const unsigned nb = (unsigned)((p.g.n[0] + p.tile - 1) / p.tile);
+    if (tpc == 2) line_kernel<float, 2><<<nb, LINE_NT, 0, s>>>(p);
+    else line_kernel<float, 1><<<nb, LINE_NT, 0, s>>>(p);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_subcycle_split(const StepParams& p, cudaStream_t s)
 {
     switch (p.g.nact) {
-    case 1: return launch_tile_kernel<float, 122, 1, 1, true>(p, s);
+    case 1: {  // one subcycle, T in place
+        const int tpc = line_plan(p.g, true, 152).tpc;
+        return launch_line_split(line_params(p, 1, tpc, p.a.T), tpc, s);
+    }
     case 2: return launch_tile_kernel<float, 32, 8, 2, true>(p, s);
     default:
         if (p.ty == 16) return launch_tile_kernel<float, 32, 16, 3, true>(p, s);

@@ -60,6 +60,8 @@ struct GridState {
     int tx = 0, ty = 0, tiles_x = 0, tiles_y = 0, z_chunk = 1;
     double* U[2][4] = {{nullptr}};
     double* T = nullptr;
+    double* T2 = nullptr;         // 1D grids: T between two launches of a call (LinePlan.steps > 1)
+    LinePlan line = {0, 0};       // 1D grids: threads per cell, subcycles per launch
     double* rho = nullptr;
     double* v[3] = {nullptr, nullptr, nullptr};
     double* kP = nullptr;
@@ -331,6 +333,7 @@ void free_grid(GridState& gs)
     for (int b = 0; b < 2; ++b)
         for (int q = 0; q < 4; ++q) dfree(gs.U[b][q]);
     dfree(gs.T);
+    dfree(gs.T2);
     dfree(gs.rho);
     for (int d = 0; d < 3; ++d) {
         dfree(gs.v[d]);
@@ -427,6 +430,10 @@ rhd_status alloc_grid(rhd_ctx* ctx, GridState& gs)
         if (st) return st;
     }
     if (gs.variant == RHD_VARIANT_TWOPASS) return alloc_twopass(ctx, gs);
+    if (gs.gp.nact == 1) {
+        gs.line = line_plan(gs.gp, gs.desc.precision == RHD_SPLIT, ctx->num_sms);
+        if (gs.line.steps > 1 && (st = dalloc(ctx, (void**)&gs.T2, bytes))) return st;
+    }
     alloc_pair64(ctx, gs);
     plan_pair64(ctx, gs, gs.desc.z_chunk);
     return RHD_OK;
@@ -786,13 +793,44 @@ rhd_status launch_one(rhd_ctx* ctx, GridState& gs, int src, double chat, double 
                         [&] { return launch_twopass_corrector(p, s); });
 }
 
-// Run n_sub steps: replay a cached graph (or issue the launches directly).
-template <typename LaunchFn>
-rhd_status run_steps(rhd_ctx* ctx, int n_sub, double chat, double dt, bool use_graph, LaunchFn&& launch)
+// 1D grids: n_sub subcycles as line_launches(gs, n_sub) launches of up to gs.line.steps subcycles each.  Their
+// number is even beyond one, so T ends where it began (a launch of several subcycles reads its neighbours'
+// T, so it writes to the other buffer).
+int line_launches(const GridState& gs, int n_sub)
 {
-    if (!use_graph) {
-        for (int s = 0; s < n_sub; ++s) {
-            rhd_status st = launch((ctx->cur + s) & 1);
+    if (gs.line.steps <= 1 || n_sub <= 1) return n_sub;
+    const int n = (n_sub + gs.line.steps - 1) / gs.line.steps;
+    return n + (n & 1);
+}
+
+// launch i of them, reading buffer src
+rhd_status launch_line_part(rhd_ctx* ctx, GridState& gs, int n_sub, int i, int src, double chat, double dt)
+{
+    const int L = line_launches(gs, n_sub), base = n_sub / L, more = n_sub % L;
+    const int first = i * base + std::min(i, more);
+    const bool split = gs.desc.precision == RHD_SPLIT;
+    StepParams p = step_params(ctx, gs, src, chat, dt);
+    double* To = p.a.T;
+    if (gs.line.steps > 1 && L > 1) {
+        p.a.T = (i & 1) ? gs.T2 : gs.T;
+        To = (i & 1) ? gs.T : gs.T2;
+        if (gs.gp.exchange != RHD_EX_FULL && gs.gp.exchange != RHD_EX_LINEAR) p.a.T = gs.T;  // T is not written
+    }
+    if (p.a.dir_dev) p.a.dir_dev += 4 * (size_t)first;
+    const LineParams lp = line_params(p, base + (i < more), gs.line.tpc, To);
+    const int k = split ? K_FUSED_SPLIT : K_FUSED_FP64;
+    return timed_launch(ctx, k, (double)gs.ncell * alg_bytes_per_cell(gs, k),
+                        [&] { return launch_line(lp, split, gs.line.tpc, ctx->stream); });
+}
+
+// Run the n_launch launches of n_sub subcycles: replay a cached graph (or issue the launches directly).  A few
+// launches are issued faster than a graph is looked up and, for a time step not seen before, captured.
+template <typename LaunchFn>
+rhd_status run_steps(rhd_ctx* ctx, int n_sub, int n_launch, double chat, double dt, bool use_graph, LaunchFn&& launch)
+{
+    if (!use_graph || n_launch <= 4) {
+        for (int s = 0; s < n_launch; ++s) {
+            rhd_status st = launch(s, (ctx->cur + s) & 1);
             if (st) return st;
         }
         return RHD_OK;
@@ -806,7 +844,7 @@ rhd_status run_steps(rhd_ctx* ctx, int n_sub, double chat, double dt, bool use_g
     cudaGraph_t graph = nullptr;
     RHD_CUDA(ctx, cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
     rhd_status st = RHD_OK;
-    for (int s = 0; s < n_sub && st == RHD_OK; ++s) st = launch((ctx->cur + s) & 1);
+    for (int s = 0; s < n_launch && st == RHD_OK; ++s) st = launch(s, (ctx->cur + s) & 1);
     cudaError_t ce = cudaStreamEndCapture(ctx->stream, &graph);
     if (st) {
         if (graph) cudaGraphDestroy(graph);
@@ -1473,9 +1511,13 @@ rhd_status rhd_radiation_subcycle(rhd_ctx* ctx, int n_sub, double chat, double d
     if ((st = enter(ctx))) return st;
     if ((st = prepare_twopass(ctx, gs))) return st;
     bool use_graph = !(gs.desc.flags & RHD_FLAG_NO_GRAPH) && !ctx->ktiming;
-    st = run_steps(ctx, n_sub, chat, dt, use_graph, [&](int src) { return launch_one(ctx, gs, src, chat, dt); });
+    const bool line = gs.gp.nact == 1;
+    const int n_launch = line ? line_launches(gs, n_sub) : n_sub;
+    st = run_steps(ctx, n_sub, n_launch, chat, dt, use_graph, [&](int i, int src) {
+        return line ? launch_line_part(ctx, gs, n_sub, i, src, chat, dt) : launch_one(ctx, gs, src, chat, dt);
+    });
     if (st) return st;
-    ctx->cur = (ctx->cur + n_sub) & 1;
+    ctx->cur = (ctx->cur + n_launch) & 1;
     ctx->n_subcycles += n_sub;
     return leave(ctx);
 }
@@ -1509,13 +1551,16 @@ rhd_status rhd_marshak_advance(rhd_ctx* ctx, int n_sub, double chat, double dt, 
     // every subcycle's boundary state at once (one block each), then the subcycles, each reading its own
     RHD_CUDA(ctx, launch_marshak_boundary(t0, dt, tau_rate, eps, F_inc, gs.desc.c, n_quad, n_sub, ctx->marshak_state,
                                           ctx->stream));
-    for (int m = 0; m < n_sub && !st; ++m) {
-        gs.dir_dev = ctx->marshak_state + 4 * (size_t)m;
-        st = launch_one(ctx, gs, (ctx->cur + m) & 1, chat, dt);
+    const bool line = gs.gp.nact == 1;
+    const int n_launch = line ? line_launches(gs, n_sub) : n_sub;
+    for (int m = 0; m < n_launch && !st; ++m) {
+        gs.dir_dev = ctx->marshak_state + (line ? 0 : 4 * (size_t)m);
+        st = line ? launch_line_part(ctx, gs, n_sub, m, (ctx->cur + m) & 1, chat, dt)
+                  : launch_one(ctx, gs, (ctx->cur + m) & 1, chat, dt);
     }
     gs.dir_dev = nullptr;
     if (st) return st;
-    ctx->cur = (ctx->cur + n_sub) & 1;
+    ctx->cur = (ctx->cur + n_launch) & 1;
     ctx->n_subcycles += n_sub;
     return leave(ctx);
 }
@@ -2120,7 +2165,7 @@ rhd_status rhd_ensemble_subcycle(rhd_ctx* ctx, int n_sub, double chat, const dou
     double dt_sig = 0.0;
     if ((st = ens_prepare(ctx, chat, dt_per_grid, &dt_sig))) return st;
     bool use_graph = !(ctx->grids[0].desc.flags & RHD_FLAG_NO_GRAPH) && !ctx->ktiming;
-    st = run_steps(ctx, n_sub, chat, dt_sig, use_graph, [&](int src) { return ens_launch(ctx, chat, src); });
+    st = run_steps(ctx, n_sub, n_sub, chat, dt_sig, use_graph, [&](int, int src) { return ens_launch(ctx, chat, src); });
     if (st) return st;
     ctx->cur = (ctx->cur + n_sub) & 1;
     ctx->n_subcycles += n_sub;

@@ -100,6 +100,22 @@ struct StepParams {
     CUtensorMap uh_map;         // staging 1: tensor map of uhalf as floats {4 (n0+4), n1+4, n2+4}, box {4 (32+4), 8+4, 1}
 };
 
+// `steps` subcycles of a 1D grid in one launch (subcycle_1d.cuh): `tile` cells per CTA, a.E, a.G and a.T in,
+// a.Eo, a.Go and To out (To may be a.T when steps is 1); a.dir_dev, if given, holds one state per subcycle.
+struct LineParams {
+    GridParams g;
+    GridArrays a;
+    double* To;
+    double chat, dt;
+    float f_chat, f_dt;
+    int steps, tile;
+    DevStats* stats;
+};
+// threads per cell (1 or 2) and the most subcycles per launch for a 1D grid on n_sms SMs
+struct LinePlan {
+    int tpc, steps;
+};
+
 // The exchange once per gas step (rhd_gas_exchange): the current state and the gas, updated in place.
 struct GasExchangeParams {
     GridParams g;               // exchange parameters (theta_E, a_rad, gamma, mu_over_kB, E_floor, kappa law)
@@ -172,6 +188,11 @@ struct SmemLimitOnce {
 // Launch wrappers (defined in the kernel translation units).
 cudaError_t launch_subcycle_fp64(const StepParams& p, cudaStream_t s);
 cudaError_t launch_subcycle_split(const StepParams& p, cudaStream_t s);
+LinePlan line_plan(const GridParams& g, bool split, int n_sms);
+LineParams line_params(const StepParams& p, int steps, int tpc, double* To);
+cudaError_t launch_line(const LineParams& p, bool split, int tpc, cudaStream_t s);
+cudaError_t launch_line_fp64(const LineParams& p, int tpc, cudaStream_t s);
+cudaError_t launch_line_split(const LineParams& p, int tpc, cudaStream_t s);
 cudaError_t launch_twopass_split(const StepParams& p, cudaStream_t s);
 cudaError_t launch_twopass_predictor(const StepParams& p, cudaStream_t s);
 cudaError_t launch_twopass_corrector(const StepParams& p, cudaStream_t s);

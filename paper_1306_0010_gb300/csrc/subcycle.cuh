@@ -103,12 +103,16 @@ __device__ __forceinline__ double to_r<double>(double x) { return x; }
 template <>
 __device__ __forceinline__ float to_r<float>(double x) { return d2f_trunc(x); }
 
-__device__ __forceinline__ double rmax(double a, double b) { return fmax(a, b); }
-__device__ __forceinline__ float rmax(float a, float b) { return fmaxf(a, b); }
-__device__ __forceinline__ double rmin(double a, double b) { return fmin(a, b); }
-__device__ __forceinline__ float rmin(float a, float b) { return fminf(a, b); }
-__device__ __forceinline__ double rabs(double a) { return fabs(a); }
-__device__ __forceinline__ float rabs(float a) { return fabsf(a); }
+// comparisons of the formulas below in either precision (FP64: by bits, off the FP64 pipe): max(a, b, 0),
+// min(a, b, 0), x > 0 and x > 1
+__device__ __forceinline__ double rmax0(double a, double b) { return max0_d(a, b); }
+__device__ __forceinline__ float rmax0(float a, float b) { return fmaxf(fmaxf(a, b), 0.0f); }
+__device__ __forceinline__ double rmin0(double a, double b) { return min0_d(a, b); }
+__device__ __forceinline__ float rmin0(float a, float b) { return fminf(fminf(a, b), 0.0f); }
+__device__ __forceinline__ bool rpos(double x) { return pos_d(x); }
+__device__ __forceinline__ bool rpos(float x) { return x > 0.0f; }
+__device__ __forceinline__ bool rabove1(double x) { return above1_d(x); }
+__device__ __forceinline__ bool rabove1(float x) { return x > 1.0f; }
 
 // ------------------------------------------------------------------------------------------------
 // closure, wave speeds, HLL
@@ -128,7 +132,7 @@ __device__ __forceinline__ ClosureScalars<R> closure_scalars(R E, R gx, R gy, R 
     R invE = rcp(E);
     R f2 = xmul(xfma(gz, gz, xfma(gy, gy, xmul(gx, gx))), xmul(invE, invE));
     R invEb = invE;
-    if (f2 > R(1)) {
+    if (rabove1(f2)) {
         // |G| > E (a state outside the realizable set, e.g. an input U^m): the closure is that of
         // f = 1 along n = G/|G|, i.e. of the state (E, G/f), so mu f = gd/(E f) in the wave speeds and
         // b G G^T = E n n^T with b = 1/(E f^2).  Face states of the corrector have passed the
@@ -174,7 +178,7 @@ __device__ __forceinline__ void wave_speeds(const ClosureScalars<R>& k, R gd, R 
     }
     const R fd = xmul(gd, k.invE);
     R rad = xmul(xmul(R(2.0 / 3.0), xadd(k.s, R(-1))), xfma(-xmul(xmul(R(3), fd), fd), k.inv2ps, k.s));
-    rad = rmax(rad, R(0));
+    rad = rmax0(rad, R(0));
     const R sr = sqrt_fast(rad);
     l1 = xmul(xadd(fd, -sr), k.cs);
     l3 = xmul(xadd(fd, sr), k.cs);
@@ -196,10 +200,9 @@ template <typename R>
 __device__ __forceinline__ void hll(const R UL[4], const R UR[4], const R FL[4], const R FR[4], R l1L, R l3L,
                                     R l1R, R l3R, R out[4])
 {
-    R SR = rmax(l3L, l3R), SL = rmin(l1L, l1R);
-    R SRp = rmax(SR, R(0)), SLm = rmin(SL, R(0));
+    const R SRp = rmax0(l3L, l3R), SLm = rmin0(l1L, l1R);
     R den = xadd(SRp, -SLm);
-    if (den > R(0)) {
+    if (rpos(den)) {
         R inv = rcp(den);
         R pr = xmul(SRp, SLm);
 #pragma unroll
@@ -211,21 +214,37 @@ __device__ __forceinline__ void hll(const R UL[4], const R UR[4], const R FL[4],
     }
 }
 
-template <typename R>
-__device__ __forceinline__ R limited(R dl, R dr, int lim)
+__device__ __forceinline__ float limited(float dl, float dr, int lim)
 {
-    if (lim == LIM_NONE) return R(0.5) * (dl + dr);
-    bool same = (dl > R(0) && dr > R(0)) || (dl < R(0) && dr < R(0));
-    if (!same) return R(0);
-    R a = rabs(dl), b = rabs(dr);
-    R m = rmin(a, b);
-    if (lim == LIM_MC) m = rmin(R(2) * m, R(0.5) * rabs(dl + dr));
-    return dl > R(0) ? m : -m;
+    if (lim == LIM_NONE) return 0.5f * (dl + dr);
+    bool same = (dl > 0.0f && dr > 0.0f) || (dl < 0.0f && dr < 0.0f);
+    if (!same) return 0.0f;
+    float a = fabsf(dl), b = fabsf(dr);
+    float m = fminf(a, b);
+    if (lim == LIM_MC) m = fminf(2.0f * m, 0.5f * fabsf(dl + dr));
+    return dl > 0.0f ? m : -m;
 }
+__device__ __forceinline__ double limited(double dl, double dr, int lim)
+{
+    if (lim == LIM_NONE) return 0.5 * (dl + dr);
+    const double m = minmod_d(dl, dr);
+    return lim == LIM_MC ? minmod_d(2.0 * m, 0.5 * (dl + dr)) : m;
+}
+
+// FP64: is the state inside the light cone with room to spare (E well inside the FP32 range, |G|^2 <= 0.9999
+// E^2 in FP32)?  False sends the caller to the FP64 test.
+__device__ __forceinline__ bool surely_realizable(const double U[4])
+{
+    const float e = d2f_trunc(U[0]), x = d2f_trunc(U[1]), y = d2f_trunc(U[2]), z = d2f_trunc(U[3]);
+    return e > 1e-15f && e < 1e18f && x * x + y * y + z * z <= 0.9999f * (e * e);
+}
+__device__ __forceinline__ bool surely_realizable(const float[4]) { return false; }
 
 template <typename R>
 __device__ __forceinline__ bool face_unrealizable(R E, R gx, R gy, R gz)
 {
+    const R U[4] = {E, gx, gy, gz};
+    if (surely_realizable(U)) return false;
     const R g2 = xfma(gz, gz, xfma(gy, gy, xmul(gx, gx)));
     return !(E > R(0)) || (g2 > xmul(R(1) + Tol<R>::face, xmul(E, E)));
 }
@@ -454,6 +473,7 @@ __device__ __forceinline__ void theta_updates(const GridParams& g, const GasCell
 template <typename R>
 __device__ __forceinline__ int realize(R U[4], R E_floor)
 {
+    if (surely_realizable(U) && d2f_trunc(U[0]) > d2f_trunc(E_floor) * 1.001f) return 0;
     if (U[0] < E_floor) U[0] = E_floor;
     R g2 = U[1] * U[1] + U[2] * U[2] + U[3] * U[3];
     if (g2 > U[0] * U[0]) {
@@ -632,9 +652,9 @@ __device__ __forceinline__ ExchangeOut exchange_fp64(const GridParams& g, double
     {
         ExchangeOut o32;
         float q32;
-        const float d32 = exchange_delta_fp32(g, (float)chat, (float)dt, (float)rho, (float)kP, (float)E, (float)T,
+        const float d32 = exchange_delta_fp32(g, d2f_rn(chat), d2f_rn(dt), d2f_rn(rho), d2f_rn(kP), d2f_rn(E), d2f_rn(T),
                                               o32, q32);
-        if (isfinite(d32) && !o32.newton_fb) d = fmin(fmax((double)d32, dlo), dhi);
+        if (isfinite(d32) && !o32.newton_fb) d = fmin(fmax(f2d_exact(d32), dlo), dhi);
     }
     bool conv = false;
     int it;
@@ -767,26 +787,20 @@ __device__ __forceinline__ float exchange_delta_fp32(const GridParams& g, float 
 // ------------------------------------------------------------------------------------------------
 template <int TX, int TY, int DIM>
 struct Geo {
-    // threads of the CTA: one per tile cell in 2D and 3D; in 1D one per cell of the widest per-phase set
-    // (the 3-cell halo on each side: TX + 6 predictor cells, TX + 5 faces), so no phase takes a second
-    // round.  A 1D subcycle on a short grid is bound by its longest dependent chain, and each FP64
-    // instruction occupies a warp's pipe for as long with 2 active lanes as with 32, so a second round
-    // for the halo would nearly double the kernel's time.
-    static constexpr int NT = DIM == 1 ? ((TX + 6 + 31) / 32) * 32 : TX * TY;
-    static constexpr int HY = DIM >= 2 ? 1 : 0;
-    static constexpr int W3 = TX + 6, H3 = TY + 6 * HY;
-    static constexpr int W2 = TX + 4, H2 = TY + 4 * HY;
+    static constexpr int NT = TX * TY;  // one thread per tile cell
+    static constexpr int W3 = TX + 6, H3 = TY + 6;
+    static constexpr int W2 = TX + 4, H2 = TY + 4;
     static constexpr int N3 = W3 * H3, N2 = W2 * H2;
     static constexpr int NR2 = (N2 + NT - 1) / NT;
     static constexpr int NR3 = (N3 + NT - 1) / NT;
     // predictor faces
     static constexpr int NFX = (W2 + 1) * H2;
-    static constexpr int NFY = HY ? W2 * (H2 + 1) : 0;
+    static constexpr int NFY = W2 * (H2 + 1);
     // corrector: cells with face states, and faces
     static constexpr int NSX = (TX + 2) * TY;
-    static constexpr int NSY = HY ? TX * (TY + 2) : 0;
+    static constexpr int NSY = TX * (TY + 2);
     static constexpr int NCX = (TX + 1) * TY;
-    static constexpr int NCY = HY ? TX * (TY + 1) : 0;
+    static constexpr int NCY = TX * (TY + 1);
     static constexpr int RING = DIM == 3 ? 3 : 1;
     // shared memory (units of R): predictor buffers and corrector buffers share one region
     static constexpr int P_UM = 0;                 // 4 x N3 U^m
@@ -810,22 +824,17 @@ struct Geo {
     __host__ __device__ static constexpr size_t r_bytes(size_t rsize) { return ((END_R * rsize + 15) / 16) * 16; }
     __host__ __device__ static constexpr size_t bytes(size_t rsize) { return r_bytes(rsize) + 8 * (size_t)ST_END; }
 
-    __device__ static __forceinline__ int i3(int lx, int ly) { return (lx + 3) + W3 * (ly + 3 * HY); }
-    __device__ static __forceinline__ int i2(int lx, int ly) { return (lx + 2) + W2 * (ly + 2 * HY); }
+    __device__ static __forceinline__ int i3(int lx, int ly) { return (lx + 3) + W3 * (ly + 3); }
+    __device__ static __forceinline__ int i2(int lx, int ly) { return (lx + 2) + W2 * (ly + 2); }
     // enumeration of R3 cells: the R2 cells first, then the outer ring
     __device__ static __forceinline__ void cell_of(int c, int& lx, int& ly)
     {
         if (c < N2) {
             lx = c % W2 - 2;
-            ly = c / W2 - 2 * HY;
+            ly = c / W2 - 2;
             return;
         }
         int o = c - N2;
-        if (!HY) {
-            lx = o == 0 ? -3 : TX + 2;
-            ly = 0;
-            return;
-        }
         if (o < H3) {
             lx = -3;
             ly = o - 3;
@@ -1114,8 +1123,7 @@ __device__ __forceinline__ void subcycle_tile(const GridParams& g, const GridArr
     // cells of the R3 region handled by this thread, fixed for all planes
     int c_i3[G::NR3], c_off[G::NR3];
     // the tile's halo lies inside the domain in x and y: loads need no boundary remap there
-    const bool xy_inside = x0 - 3 >= 0 && x0 + TX + 3 <= g.n[0] &&
-                           (G::HY == 0 || (y0 - 3 >= 0 && y0 + TY + 3 <= g.n[1]));
+    const bool xy_inside = x0 - 3 >= 0 && x0 + TX + 3 <= g.n[0] && y0 - 3 >= 0 && y0 + TY + 3 <= g.n[1];
 #pragma unroll
     for (int r = 0; r < G::NR3; ++r) {
         int c = t + r * G::NT;
@@ -1207,7 +1215,7 @@ __device__ __forceinline__ void subcycle_tile(const GridParams& g, const GridArr
                 R Pyy = k.a + k.b * U[2] * U[2], Pyz = k.b * U[2] * U[3];
                 R l1x, l3x, l1y = R(0), l3y = R(0);
                 wave_speeds(k, U[1], chat, fixed, l1x, l3x);
-                if (G::HY) wave_speeds(k, U[2], chat, fixed, l1y, l3y);
+                wave_speeds(k, U[2], chat, fixed, l1y, l3y);
                 Cc[0 * G::N3 + i] = Pxx;
                 Cc[1 * G::N3 + i] = Pxy;
                 Cc[2 * G::N3 + i] = Pxz;
@@ -1236,7 +1244,7 @@ __device__ __forceinline__ void subcycle_tile(const GridParams& g, const GridArr
             if (f < G::NFX) {
                 int row = f / (G::W2 + 1);
                 int lx = f % (G::W2 + 1) - 2;
-                int ly = row - 2 * G::HY;
+                int ly = row - 2;
                 int iL = G::i3(lx - 1, ly), iR = G::i3(lx, ly);
 #pragma unroll
                 for (int qq = 0; qq < 4; ++qq) {
@@ -1287,12 +1295,12 @@ __device__ __forceinline__ void subcycle_tile(const GridParams& g, const GridArr
         for (int r = 0; r < G::NR2; ++r) {
             int c = t + r * G::NT;
             if (c < G::N2) {
-                int lx = c % G::W2 - 2, ly = c / G::W2 - 2 * G::HY;
+                int lx = c % G::W2 - 2, ly = c / G::W2 - 2;
                 R nd[4];
-                int fl = (ly + 2 * G::HY) * (G::W2 + 1) + (lx + 2);
+                int fl = (ly + 2) * (G::W2 + 1) + (lx + 2);
 #pragma unroll
                 for (int qq = 0; qq < 4; ++qq) nd[qq] = (Fx[qq * G::NFX + fl + 1] - Fx[qq * G::NFX + fl]) * idx;
-                if (G::HY) {
+                {
                     int fb = (ly + 2) * G::W2 + (lx + 2);
 #pragma unroll
                     for (int qq = 0; qq < 4; ++qq)
@@ -1476,7 +1484,7 @@ __device__ __forceinline__ void subcycle_tile(const GridParams& g, const GridArr
                 int fl = tly * (TX + 1) + tlx;
 #pragma unroll
                 for (int qq = 0; qq < 4; ++qq) div[qq] = (Cx[qq * G::NCX + fl + 1] - Cx[qq * G::NCX + fl]) * idx;
-                if (G::HY) {
+                {
                     int fb = tly * TX + tlx;
 #pragma unroll
                     for (int qq = 0; qq < 4; ++qq)
@@ -1535,6 +1543,7 @@ __device__ __forceinline__ void subcycle_tile(const GridParams& g, const GridArr
 
 }  // namespace rhd
 
+#include "subcycle_1d.cuh"
 #include "subcycle_fp64.cuh"
 #include "subcycle_pair.cuh"
 #include "subcycle_twopass.cuh"

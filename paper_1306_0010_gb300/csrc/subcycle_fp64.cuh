@@ -97,19 +97,6 @@ __device__ __forceinline__ void hll64(const double UL[4], const double UR[4], co
     for (int q = 0; q < 4; ++q) out[q] = xfma(wU, xadd(UR[q], -UL[q]), xfma(wL, FL[q], xmul(wR, FR[q])));
 }
 
-// Is the state inside the light cone with room to spare (E well inside the FP32 range, |G|^2 <= 0.9999
-// E^2 in FP32)?  False sends the caller to the FP64 test.
-__device__ __forceinline__ bool surely_realizable(const double U[4])
-{
-    const float e = d2f_trunc(U[0]), x = d2f_trunc(U[1]), y = d2f_trunc(U[2]), z = d2f_trunc(U[3]);
-    return e > 1e-15f && e < 1e18f && x * x + y * y + z * z <= 0.9999f * (e * e);
-}
-__device__ __forceinline__ int realize64(double U[4], double E_floor, float f_E_floor)
-{
-    if (surely_realizable(U) && d2f_trunc(U[0]) > f_E_floor * 1.001f) return 0;
-    return realize(U, E_floor);
-}
-
 // Half the limited slope from the left and right differences (the reading of `limited`)
 __device__ __forceinline__ double half_slope64(double dl, double dr, int lim)
 {
@@ -141,9 +128,7 @@ __device__ __forceinline__ int face_values64(const double um[4], const double u0
         Sm[q] = xadd(u0[q], -h);
         Sp[q] = xadd(u0[q], h);
     }
-    int fb = 0;
-    if (!(surely_realizable(Sm) && surely_realizable(Sp)))
-        fb = face_unrealizable(Sm[0], Sm[1], Sm[2], Sm[3]) || face_unrealizable(Sp[0], Sp[1], Sp[2], Sp[3]);
+    const int fb = face_unrealizable(Sm[0], Sm[1], Sm[2], Sm[3]) || face_unrealizable(Sp[0], Sp[1], Sp[2], Sp[3]);
     if (fb) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) Sm[q] = Sp[q] = u0[q];
@@ -213,7 +198,7 @@ __device__ __forceinline__ void finish_cell64(const GridParams& g, const GridArr
     } else if (linear) {
         exchange_linear_fp64(g, chat, dt, gc.kP, U[0], Tn);
     }
-    cnt.fix += realize64(U, g.E_floor, g.f_E_floor);
+    cnt.fix += realize(U, g.E_floor);
     const bool bad = !(finite_d(U[0]) && finite_d(U[1]) && finite_d(U[2]) && finite_d(U[3]) &&
                        (!(full || linear) || finite_d(Tn)));
     cnt.nonfinite += bad;
@@ -255,8 +240,7 @@ __device__ __forceinline__ void subcycle_tile64(const GridParams& g, const GridA
     // cells of the R3 region handled by this thread, fixed for all planes
     int c_i3[G::NR3], c_off[G::NR3];
     // the tile's halo lies inside the domain in x and y: loads need no boundary remap there
-    const bool xy_inside = x0 - 3 >= 0 && x0 + TX + 3 <= g.n[0] &&
-                           (G::HY == 0 || (y0 - 3 >= 0 && y0 + TY + 3 <= g.n[1]));
+    const bool xy_inside = x0 - 3 >= 0 && x0 + TX + 3 <= g.n[0] && y0 - 3 >= 0 && y0 + TY + 3 <= g.n[1];
 #pragma unroll
     for (int r = 0; r < G::NR3; ++r) {
         int c = t + r * G::NT;
@@ -352,7 +336,7 @@ __device__ __forceinline__ void subcycle_tile64(const GridParams& g, const GridA
                 Cc[2 * G::N3 + i] = Pxz;
                 Cc[5 * G::N3 + i] = l1;
                 Cc[6 * G::N3 + i] = l3;
-                if (G::HY) {
+                {
                     speeds64(k, k.f[1], fixed, l1, l3);
                     Cc[3 * G::N3 + i] = xfma(ty, k.f[1], k.a);
                     Cc[4 * G::N3 + i] = Pyz;
@@ -377,7 +361,7 @@ __device__ __forceinline__ void subcycle_tile64(const GridParams& g, const GridA
             const bool isx = f < G::NFX;
             const int fy = f - G::NFX;
             const int lx = isx ? f % (G::W2 + 1) - 2 : fy % G::W2 - 2;
-            const int ly = isx ? f / (G::W2 + 1) - 2 * G::HY : fy / G::W2 - 2;
+            const int ly = isx ? f / (G::W2 + 1) - 2 : fy / G::W2 - 2;
             const int iR = G::i3(lx, ly), iL = iR - (isx ? 1 : G::W3);
             // rows of Cc: P_x. = 0, 1, 2; P_y. = 1, 3, 4; speeds 5, 6 and 7, 8
             const int r0 = isx ? 0 : 1, r1 = isx ? 1 : 3, r2 = isx ? 2 : 4, rl = isx ? 5 : 7, rg = isx ? 1 : 2;
@@ -404,13 +388,13 @@ __device__ __forceinline__ void subcycle_tile64(const GridParams& g, const GridA
         for (int r = 0; r < G::NR2; ++r) {
             int c = t + r * G::NT;
             if (c < G::N2) {
-                int lx = c % G::W2 - 2, ly = c / G::W2 - 2 * G::HY;
+                int lx = c % G::W2 - 2, ly = c / G::W2 - 2;
                 double nd[4];
-                const int fl = (ly + 2 * G::HY) * (G::W2 + 1) + (lx + 2);
+                const int fl = (ly + 2) * (G::W2 + 1) + (lx + 2);
 #pragma unroll
                 for (int qq = 0; qq < 4; ++qq)
                     nd[qq] = xfma(-hx, xadd(Fx[qq * G::NFX + fl + 1], -Fx[qq * G::NFX + fl]), nU[r][qq]);
-                if (G::HY) {
+                {
                     const int fb = (ly + 2) * G::W2 + (lx + 2);
 #pragma unroll
                     for (int qq = 0; qq < 4; ++qq)
@@ -431,7 +415,7 @@ __device__ __forceinline__ void subcycle_tile64(const GridParams& g, const GridA
                     }
                     const GasCell<double> gc = load_gas<double, false>(g, a, x0 + lx, y0 + ly, p, needT_pred, false);
                     sources64(g, gc, U0, chat * hdt, chat * hdt * g.inv_c, has_j, U);
-                    const int fx_ = realize64(U, g.E_floor, g.f_E_floor);
+                    const int fx_ = realize(U, g.E_floor);
                     const bool owned = lx >= 0 && lx < TX && ly >= 0 && ly < TY && x0 + lx < g.n[0] &&
                                        y0 + ly < g.n[1] && p >= z0 && p < z1;
                     if (owned) cnt.fix += fx_;
@@ -552,7 +536,7 @@ __device__ __forceinline__ void subcycle_tile64(const GridParams& g, const GridA
                 for (int qq = 0; qq < 4; ++qq) {
                     Uhk[qq] = Uk[qq * G::N2 + ih];
                     U[qq] = xfma(-cx, xadd(Cx[qq * G::NCX + fl + 1], -Cx[qq * G::NCX + fl]), stC[qq * G::NT + t]);
-                    if (G::HY) U[qq] = xfma(-cy, xadd(Cy[qq * G::NCY + fb + TX], -Cy[qq * G::NCY + fb]), U[qq]);
+                    U[qq] = xfma(-cy, xadd(Cy[qq * G::NCY + fb + TX], -Cy[qq * G::NCY + fb]), U[qq]);
                     if (DIM == 3) U[qq] = xfma(-cz, dz[qq], U[qq]);
                 }
                 double Tn = needT_corr ? stC[4 * G::NT + t] : 0.0;

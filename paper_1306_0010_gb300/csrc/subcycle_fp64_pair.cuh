@@ -259,7 +259,7 @@ __device__ __forceinline__ void predictor_tile64(const GridParams& g, const Grid
                     U[qq] = DIM == 3 ? xfma(-hz, xadd(zfh[qq], -zfl[qq]), acc[qq]) : nd[qq];
                 }
                 sources64(g, gc, U0, chat * hdt, chat * hdt * g.inv_c, has_j, U);
-                const int fx_ = realize64(U, g.E_floor, g.f_E_floor);
+                const int fx_ = realize(U, g.E_floor);
                 if (own_interior && p >= 0 && p < g.n[2]) cnt.fix += fx_;
                 const long long po = chk((long long)(gx + g.pad[0]) +
                                              (long long)upad_extent(g, 0) * ((long long)(gy + g.pad[1]) +
