@@ -74,8 +74,9 @@ cudaError_t launch_ensemble_split(const EnsembleParams& p, int n_ctas, cudaStrea
 cudaError_t launch_twopass_predictor(const StepParams& p, cudaStream_t s)
 {
     constexpr int TX = 32, TY = 8;
-    const int zc = p.z_chunk;
+    const int zc = p.p_chunk;
     StepParams pp = p;
+    pp.z_chunk = zc;
     pp.tiles_x = (upad_extent(p.g, 0) + TX - 1) / TX;
     pp.tiles_y = (upad_extent(p.g, 1) + TY - 1) / TY;
     auto k = predictor_kernel<TX, TY>;

@@ -58,6 +58,7 @@ struct GridState {
     GridParams gp;
     long long ncell = 0;
     int tx = 0, ty = 0, tiles_x = 0, tiles_y = 0, z_chunk = 1;
+    int p_chunk = 0;              // two-pass predictor: planes per CTA where they differ from z_chunk (0: they do not)
     double* U[2][4] = {{nullptr}};
     double* T = nullptr;
     double* T2 = nullptr;         // 1D grids: T between two launches of a call (LinePlan.steps > 1)
@@ -301,6 +302,78 @@ void fill_params(GridState& gs)
         while (zc > 32 && tiles * ((d.n[2] + zc - 1) / zc) < 152LL * 8) zc = (zc + 1) / 2;
     }
     gs.z_chunk = std::max(1, std::min(zc, d.n[2]));
+}
+
+// Planes per CTA of the split two-pass kernels.  A CTA marches its column tile through z; t0 + t1 k is the time
+// (us) of one plane with k CTAs on an SM, t_full that with k_max of them in a long queue, and `start` the
+// planes' worth of work that a chunk adds (the predictor's two halo planes, the corrector's first face).  A
+// launch of more CTAs than fit at once ends with half a CTA's time on average.  Fitted to 3 .. 128 planes on
+// 97x61x45, 64^3, 128^3, 200x150x120, 256^3, 300x250x200 and 512^3: a lone corrector CTA takes 3.7 us a plane
+// and three on an SM 5.9, so a small grid wants enough chunks to put two or three CTAs on every SM (97x61x45:
+// 4 planes, 39 us against 129 us with 32 planes everywhere) and a large one long chunks (512^3: 64 planes, 6.99
+// ms against 7.08).
+struct MarchCost {
+    double start, t0, t1, t_full;
+    int k_max;
+};
+constexpr MarchCost kMarchPred = {2.2, 1.45, 0.52, 3.2, 4}, kMarchCorr = {1.2, 2.6, 1.2, 5.9, 3};
+
+// ctas CTAs of at most `chunk` planes, `planes` in all
+double march_time(const MarchCost& m, long long ctas, long long planes, int chunk, int n_sms)
+{
+    const long long slots = (long long)n_sms * m.k_max;
+    const double longest = chunk + m.start;
+    if (ctas <= slots) return longest * (m.t0 + m.t1 * (double)((ctas + n_sms - 1) / n_sms));
+    return m.t_full * (((double)planes + m.start * (double)ctas) / (double)slots + 0.5 * longest);
+}
+
+int march_chunk(const MarchCost& m, long long tiles, int planes, int n_sms)
+{
+    int best = planes;
+    double best_t = -1.0;
+    for (int n = 1; n == 1 || 2 * n <= planes; ++n) {
+        const int c = (planes + n - 1) / n;
+        const double t = march_time(m, tiles * ((planes + c - 1) / c), tiles * planes, c, n_sms);
+        if (best_t < 0.0 || t < best_t) {
+            best_t = t;
+            best = c;
+        }
+    }
+    return best;
+}
+
+// the two-pass kernels' own choice of chunks for a grid (32 x 8 tiles)
+void plan_twopass(rhd_ctx* ctx, GridState& gs)
+{
+    const int ex = upad_extent(gs.gp, 0), ey = upad_extent(gs.gp, 1);
+    gs.p_chunk = march_chunk(kMarchPred, (long long)((ex + 31) / 32) * ((ey + 7) / 8), upad_extent(gs.gp, 2), ctx->num_sms);
+    gs.z_chunk = march_chunk(kMarchCorr, (long long)((gs.desc.n[0] + 31) / 32) * ((gs.desc.n[1] + 7) / 8), gs.desc.n[2],
+                             ctx->num_sms);
+}
+
+// ... and for a split ensemble, whose grids share the launches and one chunk length
+int plan_ensemble_chunk(rhd_ctx* ctx)
+{
+    int best = 32;
+    double best_t = -1.0;
+    for (int c : {128, 96, 64, 48, 32, 24, 16, 12, 8, 6, 4, 3, 2}) {
+        long long pc = 0, pp = 0, cc = 0, cp = 0;  // CTA items and planes of the predictor and the corrector
+        for (auto& gs : ctx->grids) {
+            const int ex = upad_extent(gs.gp, 0), ey = upad_extent(gs.gp, 1), ez = upad_extent(gs.gp, 2);
+            const long long pt = (long long)((ex + 31) / 32) * ((ey + 7) / 8);
+            const long long ct = (long long)((gs.desc.n[0] + 31) / 32) * ((gs.desc.n[1] + 7) / 8);
+            pc += pt * ((ez + c - 1) / c);
+            pp += pt * ez;
+            cc += ct * ((gs.desc.n[2] + c - 1) / c);
+            cp += ct * gs.desc.n[2];
+        }
+        const double t = march_time(kMarchPred, pc, pp, c, ctx->num_sms) + march_time(kMarchCorr, cc, cp, c, ctx->num_sms);
+        if (best_t < 0.0 || t < best_t) {
+            best_t = t;
+            best = c;
+        }
+    }
+    return best;
 }
 
 rhd_status dalloc(rhd_ctx* ctx, void** p, size_t bytes)
@@ -660,6 +733,7 @@ StepParams step_params(rhd_ctx* ctx, GridState& gs, int src, double chat, double
     p.wait_polls = ctx->wait_polls;
     if (gs.staging == RHD_STAGING_TMA) p.uh_map = gs.uh_map;
     p.z_chunk = gs.z_chunk;
+    p.p_chunk = gs.p_chunk > 0 ? gs.p_chunk : gs.z_chunk;
     p.tx = gs.tx;
     p.ty = gs.ty;
     p.tiles_x = gs.tiles_x;
@@ -1051,6 +1125,7 @@ rhd_status apply_config(rhd_ctx* ctx, GridState& gs, const rhd_launch_config& c)
     gs.tiles_x = (gs.desc.n[0] + gs.tx - 1) / gs.tx;
     gs.tiles_y = (gs.desc.n[1] + gs.ty - 1) / gs.ty;
     gs.z_chunk = std::max(1, std::min(c.z_chunk, gs.desc.n[2]));
+    gs.p_chunk = 0;
     plan_pair64(ctx, gs, gs.z_chunk);
     clear_graphs(ctx);
     return RHD_OK;
@@ -1425,9 +1500,7 @@ rhd_status rhd_init_grid(rhd_ctx** out, const rhd_grid_desc* d)
         if (d->precision == RHD_SPLIT && gs.gp.nact == 3 && d->exchange != RHD_EX_LINEAR) {
             gs.variant = (d->flags & RHD_FLAG_SPLIT_FUSED) ? 0 : 1;
             if (const char* v = std::getenv("RHD_VARIANT")) gs.variant = std::strcmp(v, "fused") == 0 ? 0 : 1;
-            // the two kernels recompute nothing across z chunks but two predictor planes: short chunks
-            // cost little and fill the GPU evenly
-            if (gs.variant == 1 && d->z_chunk == 0) gs.z_chunk = std::min(32, d->n[2]);
+            if (gs.variant == 1 && d->z_chunk == 0) plan_twopass(ctx, gs);
         }
         st = alloc_grid(ctx, gs);
     }
@@ -2051,6 +2124,7 @@ rhd_status rhd_ensemble_create(rhd_ctx** out, int n_grids, const rhd_grid_desc* 
         }
         // one z chunk for all grids (the largest grid's automatic choice)
         int zc = descs[0].z_chunk > 0 ? descs[0].z_chunk : 32;
+        if (!st && descs[0].z_chunk == 0 && ctx->grids[0].variant == RHD_VARIANT_TWOPASS) zc = plan_ensemble_chunk(ctx);
         if (!st && descs[0].precision == RHD_FP64) {
             ctx->ens_pair64 = true;
             for (auto& gs : ctx->grids) ctx->ens_pair64 = ctx->ens_pair64 && gs.uhalf64;

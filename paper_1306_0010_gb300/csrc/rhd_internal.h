@@ -92,6 +92,7 @@ struct StepParams {
     double* uhalf64;            // FP64 pair: U^{m+1/2}, 4 doubles per cell of the same extent
     Tile64 t64;
     int z_chunk;                // planes per CTA
+    int p_chunk;                // the two-pass predictor's
     int tx, ty;                 // tile shape (selects the kernel instantiation)
     int tiles_x, tiles_y;       // tile grid in x, y
     int staging;                // two-pass corrector: 0 per-thread cp.async, 1 one TMA tile copy per plane

@@ -140,11 +140,13 @@ struct GeoPred {
     static_assert(NH <= NT && TX + TY <= NT, "one extra item per thread at most");
     static constexpr int NFX = (TX + 1) * TY, NFY = TX * (TY + 1);
     // float4 units: U^m of the tile + 1 region (two plane buffers), closure data, fluxes, and three
-    // per-thread slots for the own cell's gas (rho, vx, vy, vz): plane p's gas is copied when plane p
-    // is staged and read at the end of plane p + 1, after plane p + 2 has been issued
+    // per-thread slots for the own cell's gas (rho, vx, vy, vz) and its optional per-cell inputs (kP, kF, j):
+    // plane p's gas is copied when plane p is staged and read at the end of plane p + 1, after plane p + 2
+    // has been issued
     static constexpr int UM = 0, CXo = UM + 2 * N1, CYo = CXo + N1, L3o = CYo + N1;
     static constexpr int FXo = L3o + (N1 + 1) / 2, FYo = FXo + NFX, GSo = FYo + NFY, END4 = GSo + 3 * NT;
-    __host__ __device__ static constexpr size_t bytes() { return 16 * (size_t)END4; }
+    static constexpr int NOPT = 3;
+    __host__ __device__ static constexpr size_t bytes() { return 16 * (size_t)END4 + 4 * (size_t)(3 * NOPT * NT); }
     __device__ static __forceinline__ int i1(int lx, int ly) { return (lx + 1) + W1 * (ly + 1); }
     // the h-th halo cell: rows ly = -1 and ly = TY with lx from -1 to TX, then columns lx = -1, TX
     __device__ static __forceinline__ void halo(int h, int& lx, int& ly)
@@ -175,6 +177,10 @@ __device__ __forceinline__ void predictor_tile(const GridParams& g, const GridAr
     float4* Fx = sm + G::FXo;
     float4* Fy = sm + G::FYo;
     float4* gsl = sm + G::GSo + t;  // gsl[(p % 3) NT]: the own cell's (rho, vx, vy, vz) of plane p
+    // osl[((p % 3) 3 + k) NT]: kP (k = 0), kF (1) and j (2) of plane p, where the arrays are given.  Read from
+    // memory where they are used, at the end of the plane, they cost the whole latency of a load per plane
+    // (256^3 with j: 582 us a launch; staged: 470 us)
+    float* osl = reinterpret_cast<float*>(sm + G::END4) + t;
     const float hdt = 0.5f * dt;
     const float idx = g.f_inv_dx[0], idy = g.f_inv_dx[1], idz = g.f_inv_dx[2];
     const int p1 = g.closure == 1, fixed = g.speeds == 1;
@@ -243,9 +249,13 @@ __device__ __forceinline__ void predictor_tile(const GridParams& g, const GridAr
         if (own_in_pad && !needT) {
             int fl = gx_fl, df = -1;
             const int qr = ghost1(g, 2, q, false, fl, df);
-            cp_async16(gsl + ((q + 3) % 3) * G::NT,
-                       a.gas4 + chk((own_interior && (unsigned)q < (unsigned)g.n[2]) ? zoff + off_own : lin(g, gxr, gyr, qr),
-                                    n_cells(g)));
+            const long long ig = chk((own_interior && (unsigned)q < (unsigned)g.n[2]) ? zoff + off_own : lin(g, gxr, gyr, qr),
+                                     n_cells(g));
+            const int slot = (q + 3) % 3;
+            cp_async16(gsl + slot * G::NT, a.gas4 + ig);
+            if (a.kP32) cp_async4(osl + (3 * slot + 0) * G::NT, a.kP32 + ig);
+            if (a.kF32) cp_async4(osl + (3 * slot + 1) * G::NT, a.kF32 + ig);
+            if (a.j32) cp_async4(osl + (3 * slot + 2) * G::NT, a.j32 + ig);
         }
     };
     auto closure_xy = [&](int i, const float4& U, const ClosureScalars<float>& k) {
@@ -349,15 +359,13 @@ __device__ __forceinline__ void predictor_tile(const GridParams& g, const GridAr
             }
             const int p = q - 1;
             if (emit) {
-                // gas of the own cell of plane q - 1; zoff is (q + 1) nxy here, so that cell is at
-                // off_own + zoff - 2 nxy in the interior arrays
+                // gas of the own cell of plane q - 1
                 GasCell<float> gc;
-                const bool opt = a.kP32 || a.kF32 || a.j32;  // optional per-cell opacity / emissivity arrays
-                const bool inner = own_interior && (unsigned)(q - 1) < (unsigned)g.n[2];
-                if (!needT && (!opt || inner)) {
+                if (!needT) {
                     // staged when plane q - 1 was issued (the boundary rule's source cell for ghost cells,
                     // whose mirrored velocity components are negated here)
-                    const float4 gv = gsl[((q - 1 + 3) % 3) * G::NT];
+                    const int slot = (q - 1 + 3) % 3;
+                    const float4 gv = gsl[slot * G::NT];
                     int fl = gx_fl, df = -1;
                     ghost1(g, 2, q - 1, false, fl, df);
                     gc.T = 0.0;
@@ -366,11 +374,9 @@ __device__ __forceinline__ void predictor_tile(const GridParams& g, const GridAr
                     gc.v[0] = (fl & 1) ? -gv.y : gv.y;
                     gc.v[1] = (fl & 2) ? -gv.z : gv.z;
                     gc.v[2] = (fl & 4) ? -gv.w : gv.w;
-                    // read only with the optional arrays, which take this branch for interior cells alone
-                    const long long li = (long long)off_own + zoff - 2 * nxy;
-                    gc.kP = a.kP32 ? __ldg(a.kP32 + chk(li, n_cells(g))) : kappa_law_f(g.f_kappa_P, g.kpow, gv.x);
-                    gc.kF = a.kF32 ? __ldg(a.kF32 + chk(li, n_cells(g))) : kappa_law_f(g.f_kappa_F, g.kpow, gv.x);
-                    gc.j = a.j32 ? __ldg(a.j32 + chk(li, n_cells(g))) : 0.0f;
+                    gc.kP = a.kP32 ? osl[(3 * slot + 0) * G::NT] : kappa_law_f(g.f_kappa_P, g.kpow, gv.x);
+                    gc.kF = a.kF32 ? osl[(3 * slot + 1) * G::NT] : kappa_law_f(g.f_kappa_F, g.kpow, gv.x);
+                    gc.j = a.j32 ? osl[(3 * slot + 2) * G::NT] : 0.0f;
                 } else {
                     gc = load_gas<float, true>(g, a, gx, gy, q - 1, needT, false);
                 }
