@@ -136,6 +136,12 @@ __device__ __forceinline__ bool reaches1_d(double x)
     const long long b = __double_as_longlong(x);
     return b > 0x3ff0000000000000ll - 8 && b <= 0x7ff0000000000000ll;
 }
+// a < b (neither NaN)
+__device__ __forceinline__ bool less_d(double a, double b)
+{
+    const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+    return (x ^ ((x >> 63) & 0x7fffffffffffffffll)) < (y ^ ((y >> 63) & 0x7fffffffffffffffll));
+}
 // minmod(a, b): the one nearer zero if both have the same sign, else 0 (and 0 if either is NaN)
 __device__ __forceinline__ double minmod_d(double a, double b)
 {

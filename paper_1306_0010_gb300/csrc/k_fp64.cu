@@ -252,7 +252,7 @@ cudaError_t launch_ensemble_fp64(const EnsembleParams& p, int n_ctas, cudaStream
 int ensemble_ctas_per_sm_fp64() { return ens_occupancy<double, 16, 16, false>(); }
 
 // The stiff exchange integrated once per gas step (Section 3.1 step 2, the paper's placement of S_i): in
-// every cell, E floored at E_floor, then the FULL quartic theta scheme of the subcycles (exchange64,
+// every cell, E floored at E_floor, then the FULL quartic theta scheme of the subcycles (exchange_fp64,
 // Eqs. source:energyupdate - source:polynomial) over dt = Delta t_gas, then |G| <= E by rescaling G.
 // FP64 on every grid: it runs once per gas step, not per subcycle.  One thread per cell, grid-stride.
 __global__ void __launch_bounds__(256) gas_exchange_kernel(const __grid_constant__ GasExchangeParams P)
@@ -263,19 +263,22 @@ __global__ void __launch_bounds__(256) gas_exchange_kernel(const __grid_constant
         double E = P.E[i], T = P.T[i];
         const double rho = P.rho[i];
         const double kP = P.kP ? P.kP[i] : kappa_law(g.kappa_P, g.kpow, rho);
-        if (E < g.E_floor) E = g.E_floor;
-        const ExchangeOut o = exchange64(g, P.chat, P.dt, rho, kP, E, T);
+        if (!(d2f_trunc(E) > g.f_E_floor * 1.001f) && E < g.E_floor) E = g.E_floor;
+        const ExchangeOut o = exchange_fp64(g, P.chat, P.dt, rho, kP, E, T);
         cnt.theta += o.theta_fb;
         cnt.newton_fb += o.newton_fb;
         cnt.iter_max = max(cnt.iter_max, (unsigned)o.iters);
         double G[3] = {P.G[0][i], P.G[1][i], P.G[2][i]};
-        const double g2 = G[0] * G[0] + G[1] * G[1] + G[2] * G[2];
-        if (g2 > E * E) {
-            const double sc = E / sqrt(g2);
-            G[0] *= sc;
-            G[1] *= sc;
-            G[2] *= sc;
-            cnt.fix += 1;
+        const double U[4] = {E, G[0], G[1], G[2]};
+        if (!surely_realizable(U)) {
+            const double g2 = G[0] * G[0] + G[1] * G[1] + G[2] * G[2];
+            if (g2 > E * E) {
+                const double sc = E / sqrt(g2);
+                G[0] *= sc;
+                G[1] *= sc;
+                G[2] *= sc;
+                cnt.fix += 1;
+            }
         }
         cnt.nonfinite += !(finite_d(E) && finite_d(T) && finite_d(G[0]) && finite_d(G[1]) && finite_d(G[2]));
         P.E[i] = E;

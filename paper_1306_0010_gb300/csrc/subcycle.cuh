@@ -616,9 +616,10 @@ __device__ __forceinline__ ExchangeOut exchange64(const GridParams& g, double ch
     return o;
 }
 
-// 1D grids: the clamped iteration from the FP32 seed, FP64 throughout.
-__device__ __forceinline__ ExchangeOut exchange_fp64(const GridParams& g, double chat, double dt, double rho,
-                                                     double kP, double& E, double& T)
+// The clamped iteration from the FP32 seed, FP64 throughout: 1D grids and the exchange once per gas step, whose
+// results split grids carry into FP32 transport, where a last-bit change of E can move an FP32 value.
+static __device__ __noinline__ ExchangeOut exchange_fp64_general(const GridParams& g, double chat, double dt, double rho,
+                                                                 double kP, double& E, double& T)
 {
     ExchangeOut o = {0, 0, 0};
     // divisions as Newton-refined reciprocals times the numerator (within an ulp or two; the iteration
@@ -692,6 +693,57 @@ __device__ __forceinline__ ExchangeOut exchange_fp64(const GridParams& g, double
     return o;
 }
 
+// The same solve, to the bit, for theta_E = 1 and cells whose iterates keep clear of the bracket (tested in FP32
+// with a margin of 1e-4, far beyond its error): then neither the bracket (two reciprocals, two square roots) nor
+// c0 is needed, and the comparisons are bitwise.  About 65 FP64 instructions against about 220.
+__device__ __forceinline__ ExchangeOut exchange_fp64(const GridParams& g, double chat, double dt, double rho,
+                                                     double kP, double& E, double& T)
+{
+    const double c = g.c;
+    const double q = g.gm1_mu * rcp(rho);
+    const double e = rho * T * g.inv_gm1_mu;
+    const double alpha = g.a_rad * (q * q) * (q * q);
+    const double eta = c * kP * dt;
+    const double r = chat * g.inv_c;
+    // with theta_E = 1 the general expressions reduce exactly to these
+    const double A = eta * alpha, B = xadd(1.0, xmul(r, eta)), C = -(eta * E);
+    const float E32 = d2f_rn(E), e32 = d2f_trunc(e), A32 = d2f_trunc(A), B32 = d2f_trunc(B), r32 = d2f_trunc(r);
+    if (is_one_d(g.theta_E) && E32 >= 0.0f && e32 >= 0.0f && A32 > 1e-37f) {
+        ExchangeOut o32;
+        float q32;
+        const float d32 = exchange_delta_fp32(g, d2f_rn(chat), d2f_rn(dt), d2f_rn(rho), d2f_rn(kP), E32, d2f_rn(T), o32, q32);
+        // the paper's bracket x <= min(|c0|/B, (|c0|/A)^(1/4)) in FP32
+        const float c0 = e32 + d2f_trunc(eta) * (r32 * e32 + E32);
+        const float lim = 0.9999f * fminf(c0 * rcp(B32), sqrt_fast(sqrt_fast(c0 * rcp(A32))));
+        if (isfinite(d32) && !o32.newton_fb && !o32.theta_fb && lim < 1e37f) {
+            double d = f2d_exact(d32);
+            float x32 = d2f_trunc(e + d);
+            bool clear = x32 > 0.0f && x32 < lim, conv = false;
+            int it;
+            for (it = 0; it < 100 && clear; ++it) {
+                const double x = e + d;
+                const double x2 = x * x;
+                const double gv = A * x2 * x2 + B * d + C;
+                const double gp = 4.0 * A * x2 * x + B;
+                const double dn = d - gv * rcp(gp);
+                x32 = d2f_trunc(e + dn);
+                clear = x32 > 0.0f && x32 < lim;
+                if (it > 0 && !less_d(dn, d)) {
+                    conv = true;
+                    break;
+                }
+                d = dn;
+            }
+            if (conv && clear) {
+                E = E - r * d;
+                T = (e + d) * q;
+                return {0, 0, it};
+            }
+        }
+    }
+    return exchange_fp64_general(g, chat, dt, rho, kP, E, T);
+}
+
 // Linear exchange of the Pomraning material (c_v = alpha T^3, Section 4.1.4): Eqs. (marshak:update)
 // in v = a_R T^4 with dtau = eps c kP dt, dv = -(v - E) dtau / (1 + theta (1 + chat/(eps c)) dtau),
 // dE = -(chat / (eps c)) dv (the paper's chat = c gives 1 + 1/eps and -dv/eps), so v/(eps c) + E/chat
@@ -702,13 +754,13 @@ __device__ __forceinline__ void exchange_linear_fp64(const GridParams& g, double
     const double eps = g.linear_eps, c = g.c;
     const double T2 = T * T;
     double v = g.a_rad * T2 * T2;
-    const double dtau = (eps * c * dt) * kP;
+    const double dtau = eps * c * kP * dt;
     const double r = chat * g.inv_eps_c;  // chat / (eps c), 1/(eps c) from the host
     const double dv = -(v - E) * dtau * rcp(1.0 + g.theta_E * (1.0 + r) * dtau);
     E = E + (-r * dv);
     v = v + dv;
     v = max0_d(v, 0.0);
-    T = sqrt3(sqrt3(v * g.inv_a_rad));
+    T = sqrt(sqrt(v * g.inv_a_rad));
 }
 
 // FP32 Newton for delta with the same iteration, which also stops once a step is small enough that

