@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include "dfloat.cuh"
 #include "rhd_internal.h"
 
 namespace rhd {
@@ -25,19 +26,182 @@ cudaError_t launch_scale_copy(double* dst, const double* src, double scale, long
     return cudaGetLastError();
 }
 
+// (float)x, round to nearest, by integer operations: the conversion instruction runs on the FP64 pipe.  Values
+// outside the FP32 normal range (rare), infinities and NaN take it all the same.
+__device__ __forceinline__ float to_f32(double x)
+{
+    const unsigned m = (unsigned)__double2hiint(x) & 0x7fffffffu;
+    return m != 0u && (m < 0x38100000u || m >= 0x47f00000u) ? (float)x : d2f_rn(x);
+}
+// x / c, c > 0, for y = 1/c correctly rounded (0: always divide): one multiplication and one correction by the exact residual (the
+// correctly rounded quotient, by Markstein's theorem, where nothing under- or overflows: three FP64
+// instructions against CUDA's ten or so), the division itself elsewhere
+__device__ __forceinline__ double div_by(double x, double c, double y)
+{
+    const unsigned m = (unsigned)__double2hiint(x) & 0x7fffffffu;
+    if (m - 0x10000000u > 0x60000000u || y == 0.0)  // |x| outside about [1e-231, 1e231], inf, NaN
+        return (m | (unsigned)__double2loint(x)) == 0u ? x : x / c;
+    const double q = __dmul_rn(x, y);
+    return __fma_rn(__fma_rn(-q, c, x), y, q);
+}
+
+// What a caller hands over and takes back, each in one pass over memory: every array read once, and every
+// copy the kernels use (FP64, FP32, the two-pass path's interleaved forms) written once.  Bound by memory; at
+// 512^3 on a split grid (device arrays, velocity, no optional arrays) the state in takes 2.1 + 2.1 ms and the
+// moments out 1.4 ms, 5.9 with T, against 12.2 ms for the copies, conversions and interleavings as launches of their own,
+// whose F / c, 134 million FP64 divisions a component, was bound by the FP64 pipe.
+// V = 2: two cells per thread by 16-byte accesses (arrays 16-byte aligned); 1: one.
+template <int V>
+struct Cells;
+template <>
+struct Cells<1> {
+    double x[1];
+    __device__ __forceinline__ void get(const double* p, long long i) { x[0] = p[i]; }
+    __device__ __forceinline__ void put(double* p, long long i) const { p[i] = x[0]; }
+    __device__ __forceinline__ void put32(float* p, long long i) const { p[i] = to_f32(x[0]); }
+};
+template <>
+struct Cells<2> {
+    double x[2];
+    __device__ __forceinline__ void get(const double* p, long long i)
+    {
+        const double2 v = reinterpret_cast<const double2*>(p)[i];
+        x[0] = v.x;
+        x[1] = v.y;
+    }
+    __device__ __forceinline__ void put(double* p, long long i) const { reinterpret_cast<double2*>(p)[i] = make_double2(x[0], x[1]); }
+    __device__ __forceinline__ void put32(float* p, long long i) const
+    {
+        reinterpret_cast<float2*>(p)[i] = make_float2(to_f32(x[0]), to_f32(x[1]));
+    }
+};
+
+template <int V>
+__global__ void __launch_bounds__(256) gas_in_kernel(const __grid_constant__ GasIn g, long long n)
+{
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+        Cells<V> c[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            if (g.src[k]) c[k].get(g.src[k], i);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            if (!g.src[k]) continue;
+            if (g.dst[k] != g.src[k]) c[k].put(g.dst[k], i);
+            if (g.dst32[k]) c[k].put32(g.dst32[k], i);
+        }
+        if (g.gas4) {
+#pragma unroll
+            for (int e = 0; e < V; ++e)
+                g.gas4[V * i + e] = make_float4(to_f32(c[0].x[e]), g.src[2] ? to_f32(c[2].x[e]) : 0.0f,
+                                                g.src[3] ? to_f32(c[3].x[e]) : 0.0f, g.src[4] ? to_f32(c[4].x[e]) : 0.0f);
+        }
+    }
+}
+
+// F = true: src holds F and dst G = F / c
+template <int V, bool F>
+__global__ void __launch_bounds__(256) moments_in_kernel(const __grid_constant__ MomentsIn m, long long n)
+{
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+        Cells<V> c[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) c[k].get(m.src[k], i);
+        if (F) {
+#pragma unroll
+            for (int k = 1; k < 4; ++k)
+#pragma unroll
+                for (int e = 0; e < V; ++e) c[k].x[e] = div_by(c[k].x[e], m.c, m.inv_c);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (m.dst[k] != m.src[k] || (F && k > 0)) c[k].put(m.dst[k], i);
+        if (m.um32) {
+#pragma unroll
+            for (int e = 0; e < V; ++e)
+                m.um32[V * i + e] = make_float4(d2f_trunc(c[0].x[e]), d2f_trunc(c[1].x[e]), d2f_trunc(c[2].x[e]),
+                                                d2f_trunc(c[3].x[e]));
+        }
+    }
+}
+
+// dst = (E, c G); a NULL dst[0] leaves E out
+template <int V>
+__global__ void __launch_bounds__(256) moments_out_kernel(const __grid_constant__ MomentsIn m, long long n)
+{
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+        Cells<V> c[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (m.dst[k]) c[k].get(m.src[k], i);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (!m.dst[k]) continue;
+            if (k > 0) {
+#pragma unroll
+                for (int e = 0; e < V; ++e) c[k].x[e] = c[k].x[e] * m.c;
+            }
+            c[k].put(m.dst[k], i);
+        }
+    }
+}
+
+namespace {
+bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
+unsigned copy_blocks(long long n)
+{
+    const long long b = (n + 255) / 256;
+    return (unsigned)(b < 152 * 16 ? b : 152 * 16);
+}
+}  // namespace
+
+cudaError_t launch_gas_in(const GasIn& g, long long n, cudaStream_t s)
+{
+    if (n <= 0) return cudaSuccess;
+    bool two = n % 2 == 0;
+    for (int k = 0; k < 8; ++k) two = two && aligned16(g.src[k]) && aligned16(g.dst[k]) && ((uintptr_t)g.dst32[k] & 7u) == 0;
+    if (two) gas_in_kernel<2><<<copy_blocks(n / 2), 256, 0, s>>>(g, n / 2);
+    else gas_in_kernel<1><<<copy_blocks(n), 256, 0, s>>>(g, n);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_moments_in(const MomentsIn& m, bool conserved, long long n, cudaStream_t s)
+{
+    if (n <= 0) return cudaSuccess;
+    bool two = n % 2 == 0;
+    for (int k = 0; k < 4; ++k) two = two && aligned16(m.src[k]) && aligned16(m.dst[k]);
+    const unsigned nb = copy_blocks(two ? n / 2 : n);
+    if (two && conserved) moments_in_kernel<2, false><<<nb, 256, 0, s>>>(m, n / 2);
+    else if (two) moments_in_kernel<2, true><<<nb, 256, 0, s>>>(m, n / 2);
+    else if (conserved) moments_in_kernel<1, false><<<nb, 256, 0, s>>>(m, n);
+    else moments_in_kernel<1, true><<<nb, 256, 0, s>>>(m, n);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_moments_out(const MomentsIn& m, long long n, cudaStream_t s)
+{
+    if (n <= 0) return cudaSuccess;
+    bool two = n % 2 == 0;
+    for (int k = 0; k < 4; ++k) two = two && aligned16(m.src[k]) && aligned16(m.dst[k]);
+    if (two) moments_out_kernel<2><<<copy_blocks(n / 2), 256, 0, s>>>(m, n / 2);
+    else moments_out_kernel<1><<<copy_blocks(n), 256, 0, s>>>(m, n);
+    return cudaGetLastError();
+}
+
 __global__ void to_float_kernel(float* dst, const double* src, long long n)
 {
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     long long stride = (long long)gridDim.x * blockDim.x;
-    for (; i < n; i += stride) dst[i] = (float)src[i];
+    for (; i < n; i += stride) dst[i] = to_f32(src[i]);
 }
 
 cudaError_t launch_to_float(float* dst, const double* src, long long n, cudaStream_t s)
 {
     if (n <= 0) return cudaSuccess;
-    int blocks = (int)((n + 255) / 256);
-    if (blocks > 152 * 16) blocks = 152 * 16;
-    to_float_kernel<<<blocks, 256, 0, s>>>(dst, src, n);
+    to_float_kernel<<<copy_blocks(n), 256, 0, s>>>(dst, src, n);
     return cudaGetLastError();
 }
 

@@ -563,31 +563,6 @@ rhd_status put(rhd_ctx* ctx, double* dst, const double* src, long long n, int on
     return RHD_OK;
 }
 
-rhd_status set_optional(rhd_ctx* ctx, GridState& gs, double*& buf, float*& buf32, bool& has, const double* src,
-                        int on_device)
-{
-    if (!src) {
-        has = false;
-        return RHD_OK;
-    }
-    size_t bytes = sizeof(double) * (size_t)gs.ncell;
-    if (!buf) {
-        rhd_status st = dalloc(ctx, (void**)&buf, bytes);
-        if (st) return st;
-    }
-    rhd_status st = put(ctx, buf, src, gs.ncell, on_device);
-    if (st) return st;
-    if (gs.desc.precision == RHD_SPLIT) {
-        if (!buf32) {
-            st = dalloc(ctx, (void**)&buf32, sizeof(float) * (size_t)gs.ncell);
-            if (st) return st;
-        }
-        RHD_CUDA(ctx, launch_to_float(buf32, buf, gs.ncell, ctx->stream));
-    }
-    has = true;
-    return RHD_OK;
-}
-
 rhd_status set_gas(rhd_ctx* ctx, GridState& gs, const double* rho, const double* T, const double* vx,
                    const double* vy, const double* vz, const double* kP, const double* kF, const double* j,
                    int on_device)
@@ -595,6 +570,10 @@ rhd_status set_gas(rhd_ctx* ctx, GridState& gs, const double* rho, const double*
     if (!rho || !T) return fail(ctx, RHD_ERR_ARG, "rho and T are required");
     rhd_status st = enter(ctx);
     if (st) return st;
+    const bool split = gs.desc.precision == RHD_SPLIT;
+    const double* src[8] = {rho, T, vx, vy, vz, kP, kF, j};
+    double** buf[8] = {&gs.rho, &gs.T, &gs.v[0], &gs.v[1], &gs.v[2], &gs.kP, &gs.kF, &gs.j};
+    float** buf32[8] = {&gs.rho32, nullptr, &gs.v32[0], &gs.v32[1], &gs.v32[2], &gs.kP32, &gs.kF32, &gs.j32};
     // the arrays the captured subcycle graphs point at, and which of them are present: the graphs stay
     // valid when a new state arrives in the same arrays
     auto layout = [&gs] {
@@ -604,25 +583,35 @@ rhd_status set_gas(rhd_ctx* ctx, GridState& gs, const double* rho, const double*
                                                                  gs.has_j << 3 | gs.has_gas << 4)};
     };
     const std::vector<const void*> before = layout();
-    if ((st = put(ctx, gs.rho, rho, gs.ncell, on_device))) return st;
-    if ((st = put(ctx, gs.T, T, gs.ncell, on_device))) return st;
-    if (gs.desc.precision == RHD_SPLIT) RHD_CUDA(ctx, launch_to_float(gs.rho32, gs.rho, gs.ncell, ctx->stream));
-    const double* vin[3] = {vx, vy, vz};
-    bool hv[3];
-    for (int d = 0; d < 3; ++d)
-        if ((st = set_optional(ctx, gs, gs.v[d], gs.v32[d], hv[d], vin[d], on_device))) return st;
-    gs.has_v = hv[0] || hv[1] || hv[2];
-    // velocity components that were not given are zero: keep them as absent
-    for (int d = 0; d < 3; ++d)
-        if (!hv[d]) {
-            dfree(gs.v[d]);
-            dfree(gs.v32[d]);
+    const size_t bytes = sizeof(double) * (size_t)gs.ncell;
+    GasIn in;
+    std::memset(&in, 0, sizeof(in));
+    for (int k = 0; k < 8; ++k) {
+        if (!src[k]) {
+            // velocity components that were not given are zero: keep them as absent
+            if (k >= 2 && k <= 4) {
+                dfree(*buf[k]);
+                dfree(*buf32[k]);
+            }
+            continue;
         }
-    if ((st = set_optional(ctx, gs, gs.kP, gs.kP32, gs.has_kP, kP, on_device))) return st;
-    if ((st = set_optional(ctx, gs, gs.kF, gs.kF32, gs.has_kF, kF, on_device))) return st;
-    if ((st = set_optional(ctx, gs, gs.j, gs.j32, gs.has_j, j, on_device))) return st;
+        if (!*buf[k] && (st = dalloc(ctx, (void**)buf[k], bytes))) return st;
+        if (split && buf32[k] && !*buf32[k] && (st = dalloc(ctx, (void**)buf32[k], bytes / 2))) return st;
+        // host arrays land in the library's own first; the conversions then run in place
+        if (!on_device && (st = put(ctx, *buf[k], src[k], gs.ncell, 0))) return st;
+        in.src[k] = on_device ? src[k] : *buf[k];
+        in.dst[k] = *buf[k];
+        in.dst32[k] = split && buf32[k] ? *buf32[k] : nullptr;
+    }
+    const bool twopass = gs.variant == RHD_VARIANT_TWOPASS && gs.gas4;
+    in.gas4 = twopass ? gs.gas4 : nullptr;
+    if (on_device || split) RHD_CUDA(ctx, launch_gas_in(in, gs.ncell, ctx->stream));
+    gs.has_v = vx || vy || vz;
+    gs.has_kP = kP != nullptr;
+    gs.has_kF = kF != nullptr;
+    gs.has_j = j != nullptr;
     gs.has_gas = true;
-    gs.gas4_ok = false;
+    gs.gas4_ok = twopass;
     gs.gas_pending = false;  // a pending source correction belongs to the replaced state
     if (layout() != before) clear_graphs(ctx);  // the kernels' array pointers changed
     return leave(ctx);
@@ -636,20 +625,20 @@ rhd_status set_moments(rhd_ctx* ctx, GridState& gs, const double* E, const doubl
     rhd_status st = enter(ctx);
     if (st) return st;
     double** U = gs.U[ctx->cur];
-    if ((st = put(ctx, U[0], E, gs.ncell, on_device))) return st;
-    const double* F[3] = {Fx, Fy, Fz};
-    for (int d = 0; d < 3; ++d) {
-        if (conserved) {
-            if ((st = put(ctx, U[1 + d], F[d], gs.ncell, on_device))) return st;
-        } else if (on_device) {
-            RHD_CUDA(ctx, launch_scale_copy(U[1 + d], F[d], gs.desc.c, gs.ncell, ctx->stream));
-        } else {
-            if ((st = put(ctx, U[1 + d], F[d], gs.ncell, 0))) return st;
-            RHD_CUDA(ctx, launch_scale_copy(U[1 + d], U[1 + d], gs.desc.c, gs.ncell, ctx->stream));
-        }
+    const double* src[4] = {E, Fx, Fy, Fz};
+    MomentsIn in;
+    for (int q = 0; q < 4; ++q) {
+        if (!on_device && (st = put(ctx, U[q], src[q], gs.ncell, 0))) return st;
+        in.src[q] = on_device ? src[q] : U[q];
+        in.dst[q] = U[q];
     }
+    const bool twopass = gs.variant == RHD_VARIANT_TWOPASS && gs.um32;
+    in.um32 = twopass ? gs.um32 : nullptr;
+    in.c = gs.desc.c;
+    in.inv_c = gs.desc.c > 1e-60 && gs.desc.c < 1e60 ? 1.0 / gs.desc.c : 0.0;
+    if (on_device || !conserved || twopass) RHD_CUDA(ctx, launch_moments_in(in, conserved, gs.ncell, ctx->stream));
     gs.has_moments = true;
-    gs.um32_ok = false;
+    gs.um32_ok = twopass;
     return leave(ctx);
 }
 
@@ -669,13 +658,20 @@ rhd_status get_moments(rhd_ctx* ctx, GridState& gs, double* E, double* Fx, doubl
         const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
         for (int q = 0; q < 4; ++q)
             RHD_CUDA(ctx, cudaMemcpyAsync(q ? F[q - 1] : E, U[q], bytes, kind, ctx->stream));
-    } else if (on_device) {
-        RHD_CUDA(ctx, cudaMemcpyAsync(E, U[0], bytes, cudaMemcpyDeviceToDevice, ctx->stream));
-        for (int d = 0; d < 3; ++d) RHD_CUDA(ctx, launch_scale_copy(F[d], U[1 + d], -gs.desc.c, gs.ncell, ctx->stream));
     } else {
-        for (int d = 0; d < 3; ++d) RHD_CUDA(ctx, launch_scale_copy(W[1 + d], U[1 + d], -gs.desc.c, gs.ncell, ctx->stream));
-        RHD_CUDA(ctx, cudaMemcpyAsync(E, U[0], bytes, cudaMemcpyDeviceToHost, ctx->stream));
-        for (int d = 0; d < 3; ++d) RHD_CUDA(ctx, cudaMemcpyAsync(F[d], W[1 + d], bytes, cudaMemcpyDeviceToHost, ctx->stream));
+        MomentsIn out;
+        out.um32 = nullptr;
+        out.c = gs.desc.c;
+        out.inv_c = 0.0;
+        for (int q = 0; q < 4; ++q) {
+            out.src[q] = U[q];
+            out.dst[q] = on_device ? (q ? F[q - 1] : E) : (q ? W[q] : nullptr);
+        }
+        RHD_CUDA(ctx, launch_moments_out(out, gs.ncell, ctx->stream));
+        if (!on_device) {
+            RHD_CUDA(ctx, cudaMemcpyAsync(E, U[0], bytes, cudaMemcpyDeviceToHost, ctx->stream));
+            for (int d = 0; d < 3; ++d) RHD_CUDA(ctx, cudaMemcpyAsync(F[d], W[1 + d], bytes, cudaMemcpyDeviceToHost, ctx->stream));
+        }
     }
     if ((st = leave(ctx))) return st;
     RHD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));

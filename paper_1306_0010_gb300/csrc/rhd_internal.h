@@ -232,6 +232,24 @@ bool tile_supported(int precision, int nact, int tx, int ty);
 
 // Auxiliary kernels (k_aux.cu).
 cudaError_t launch_scale_copy(double* dst, const double* src, double scale, long long n, cudaStream_t s);
+// the gas state in: rho, T, vx, vy, vz, kP, kF, j (NULL: absent) copied to dst (skipped where dst is src), their
+// FP32 copies to dst32 where given, and (rho, v) interleaved to gas4 if given
+struct GasIn {
+    const double* src[8];
+    double* dst[8];
+    float* dst32[8];
+    float4* gas4;
+};
+cudaError_t launch_gas_in(const GasIn& g, long long n, cudaStream_t s);
+// the moments in (E, F or G) to (E, G), with the FP32 mirror if given; and out, (E, G) to (E, F)
+struct MomentsIn {
+    const double* src[4];
+    double* dst[4];
+    float4* um32;
+    double c, inv_c;
+};
+cudaError_t launch_moments_in(const MomentsIn& m, bool conserved, long long n, cudaStream_t s);
+cudaError_t launch_moments_out(const MomentsIn& m, long long n, cudaStream_t s);
 cudaError_t launch_to_float(float* dst, const double* src, long long n, cudaStream_t s);
 cudaError_t launch_reduce_state(const double* E, const double* G0, const double* G1, const double* G2,
                                 long long n, double* partials, int n_blocks, cudaStream_t s);
