@@ -36,11 +36,15 @@ __device__ __forceinline__ float to_f32(double x)
 // x / c, c > 0, for y = 1/c correctly rounded (0: always divide): one multiplication and one correction by the exact residual (the
 // correctly rounded quotient, by Markstein's theorem, where nothing under- or overflows: three FP64
 // instructions against CUDA's ten or so), the division itself elsewhere
+static __device__ __noinline__ double div_slow(double x, double c) { return x / c; }
 __device__ __forceinline__ double div_by(double x, double c, double y)
 {
     const unsigned m = (unsigned)__double2hiint(x) & 0x7fffffffu;
-    if (m - 0x10000000u > 0x60000000u || y == 0.0)  // |x| outside about [1e-231, 1e231], inf, NaN
-        return (m | (unsigned)__double2loint(x)) == 0u ? x : x / c;
+    if (m - 0x10000000u > 0x60000000u || y == 0.0) {  // |x| outside about [1e-231, 1e231], inf, NaN; zero
+        // out of line: inlined, the division's instructions ran in every cell
+        if ((m | (unsigned)__double2loint(x)) != 0u) return div_slow(x, c);
+        return x;
+    }
     const double q = __dmul_rn(x, y);
     return __fma_rn(__fma_rn(-q, c, x), y, q);
 }
