@@ -70,6 +70,14 @@ cudaError_t launch_ensemble_split(const EnsembleParams& p, int n_ctas, cudaStrea
     return launch_ens_kernel<float, 32, 8, true>(p, n_ctas, s);
 }
 
+// The grids whose modes the two-pass kernels know at compile time (see predictor_tile, corrector_tile)
+static bool common_predictor(const GridParams& g)
+{
+    return g.closure == 0 && g.speeds == 0 && g.theta_F == 1.0 && (g.exchange == EX_FULL || g.exchange == EX_EQUILIBRIUM);
+}
+static bool common_corrector(const GridParams& g) { return common_predictor(g) && g.theta_E == 1.0; }
+bool twopass_common(const GridParams& g) { return common_corrector(g); }
+
 // Two-pass split subcycle (3D): predictor over the grid and its stored ghost layers, then corrector.
 cudaError_t launch_twopass_predictor(const StepParams& p, cudaStream_t s)
 {
@@ -79,7 +87,7 @@ cudaError_t launch_twopass_predictor(const StepParams& p, cudaStream_t s)
     pp.z_chunk = zc;
     pp.tiles_x = (upad_extent(p.g, 0) + TX - 1) / TX;
     pp.tiles_y = (upad_extent(p.g, 1) + TY - 1) / TY;
-    auto k = predictor_kernel<TX, TY>;
+    auto k = common_predictor(p.g) ? predictor_kernel<TX, TY, true> : predictor_kernel<TX, TY, false>;
     const size_t smem = GeoPred<TX, TY>::bytes();
     static SmemLimitOnce smem_once;
     cudaError_t e = smem_once.set(k, smem);
@@ -96,14 +104,20 @@ cudaError_t launch_twopass_corrector(const StepParams& p, cudaStream_t s)
     StepParams pc = p;
     pc.tiles_x = (p.g.n[0] + TX - 1) / TX;
     pc.tiles_y = (p.g.n[1] + TY - 1) / TY;
-    // one instantiation per staging and limiter (the limiter is a compile-time constant in the kernel)
-    auto pick = [&](auto tma) {
+    // one instantiation per limiter and exchange mode (compile-time constants in the kernel); TMA staging, a
+    // tuner's candidate, with the general one only
+    auto pick = [&](auto tma, auto exk) {
         constexpr bool T = decltype(tma)::value;
-        return p.g.limiter == LIM_MC ? corrector_kernel<TX, TY, T, LIM_MC>
-               : p.g.limiter == LIM_NONE ? corrector_kernel<TX, TY, T, LIM_NONE>
-                                         : corrector_kernel<TX, TY, T, LIM_MINMOD>;
+        constexpr int X = decltype(exk)::value;
+        return p.g.limiter == LIM_MC ? corrector_kernel<TX, TY, T, LIM_MC, X>
+               : p.g.limiter == LIM_NONE ? corrector_kernel<TX, TY, T, LIM_NONE, X>
+                                         : corrector_kernel<TX, TY, T, LIM_MINMOD, X>;
     };
-    auto k = p.staging == 1 ? pick(std::true_type{}) : pick(std::false_type{});
+    using Any = std::integral_constant<int, -1>;
+    auto k = p.staging == 1              ? pick(std::true_type{}, Any{})
+             : !common_corrector(p.g)    ? pick(std::false_type{}, Any{})
+             : p.g.exchange == EX_FULL   ? pick(std::false_type{}, std::integral_constant<int, EX_FULL>{})
+                                         : pick(std::false_type{}, std::integral_constant<int, EX_EQUILIBRIUM>{});
     const size_t smem = GeoCorr<TX, TY>::bytes() + 128;  // + alignment slack for TMA destinations
     static SmemLimitOnce smem_once;
     cudaError_t e = smem_once.set(k, smem);
@@ -199,7 +213,7 @@ static int occupancy_of(K k, size_t smem, int threads)
 
 cudaError_t launch_ensemble_predictor(const EnsembleParams& p, int n_ctas, cudaStream_t s)
 {
-    auto k = predictor_ens_kernel<32, 8>;
+    auto k = p.common ? predictor_ens_kernel<32, 8, true> : predictor_ens_kernel<32, 8, false>;
     const size_t smem = GeoPred<32, 8>::bytes();
     static SmemLimitOnce smem_once;
     cudaError_t e = smem_once.set(k, smem);
@@ -210,11 +224,15 @@ cudaError_t launch_ensemble_predictor(const EnsembleParams& p, int n_ctas, cudaS
 
 cudaError_t launch_ensemble_corrector(const EnsembleParams& p, int n_ctas, cudaStream_t s)
 {
-    // all grids of an ensemble share the limiter: one instantiation per limiter
+    // all grids of an ensemble share the limiter and the exchange mode; common FULL ones have their own kernels
     const int lim = p.n_grids > 0 ? p.limiter : LIM_MINMOD;
-    auto k = lim == LIM_MC     ? corrector_ens_kernel<32, 8, LIM_MC>
-             : lim == LIM_NONE ? corrector_ens_kernel<32, 8, LIM_NONE>
-                               : corrector_ens_kernel<32, 8, LIM_MINMOD>;
+    auto pick = [&](auto exk) {
+        constexpr int X = decltype(exk)::value;
+        return lim == LIM_MC     ? corrector_ens_kernel<32, 8, LIM_MC, X>
+               : lim == LIM_NONE ? corrector_ens_kernel<32, 8, LIM_NONE, X>
+                                 : corrector_ens_kernel<32, 8, LIM_MINMOD, X>;
+    };
+    auto k = p.common ? pick(std::integral_constant<int, EX_FULL>{}) : pick(std::integral_constant<int, -1>{});
     const size_t smem = GeoCorr<32, 8>::bytes();
     static SmemLimitOnce smem_once;
     cudaError_t e = smem_once.set(k, smem);
@@ -223,10 +241,10 @@ cudaError_t launch_ensemble_corrector(const EnsembleParams& p, int n_ctas, cudaS
     return cudaGetLastError();
 }
 
-int ensemble_ctas_per_sm_predictor() { return occupancy_of(predictor_ens_kernel<32, 8>, GeoPred<32, 8>::bytes(), 256); }
+int ensemble_ctas_per_sm_predictor() { return occupancy_of(predictor_ens_kernel<32, 8, false>, GeoPred<32, 8>::bytes(), 256); }
 int ensemble_ctas_per_sm_corrector()
 {
-    return occupancy_of(corrector_ens_kernel<32, 8, LIM_MINMOD>, GeoCorr<32, 8>::bytes(), 256);
+    return occupancy_of(corrector_ens_kernel<32, 8, LIM_MINMOD, -1>, GeoCorr<32, 8>::bytes(), 256);
 }
 
 int ensemble_ctas_per_sm_split() { return ens_occupancy<float, 32, 8, true>(); }

@@ -1024,6 +1024,8 @@ rhd_status ens_launch(rhd_ctx* ctx, double chat, int src)
     ep.f_chat = (float)chat;
     ep.z_chunk = ctx->grids[0].z_chunk;
     ep.limiter = ctx->grids[0].desc.limiter;
+    ep.common = 1;
+    for (auto& gs : ctx->grids) ep.common = ep.common && twopass_common(gs.gp) && gs.gp.exchange == RHD_EX_FULL;
     ep.stats = ctx->dstats;
     if (ctx->ens_pair64) {
         double pb = 0.0, cb = 0.0;

@@ -156,6 +156,7 @@ struct EnsembleParams {
     float f_chat;
     int z_chunk;
     int limiter;                // shared by all grids (the two-pass corrector is instantiated per limiter)
+    int common;                 // 1: every grid is a common one (twopass_common) with the FULL exchange
     unsigned long long* counter;  // work-queue head, reset before each launch
     DevStats* stats;
 };
@@ -195,6 +196,7 @@ cudaError_t launch_line(const LineParams& p, bool split, int tpc, cudaStream_t s
 cudaError_t launch_line_fp64(const LineParams& p, int tpc, cudaStream_t s);
 cudaError_t launch_line_split(const LineParams& p, int tpc, cudaStream_t s);
 cudaError_t launch_twopass_split(const StepParams& p, cudaStream_t s);
+bool twopass_common(const GridParams& g);  // the modes the two-pass kernels have at compile time
 cudaError_t launch_twopass_predictor(const StepParams& p, cudaStream_t s);
 cudaError_t launch_twopass_corrector(const StepParams& p, cudaStream_t s);
 bool tma_available();  // tensor-map staging of the two-pass corrector can be used on this device

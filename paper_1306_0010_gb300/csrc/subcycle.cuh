@@ -991,10 +991,10 @@ __device__ __forceinline__ dfl split_x(const SplitStiffConsts& k, const float* k
     return p == 0 ? K : (p == 1 ? dmul(K, rho) : dmul(dmul(K, rho), rho));
 }
 __device__ __forceinline__ bool is_one(dfl t) { return t.hi == 1.0f && t.lo == 0.0f; }
-// (1 - (1 - theta) x)/(1 + theta x)
-__device__ __forceinline__ dfl theta_factor(dfl x, dfl th, dfl om)
+// (1 - (1 - theta) x)/(1 + theta x); one: theta is known to be 1
+__device__ __forceinline__ dfl theta_factor(dfl x, dfl th, dfl om, bool one = false)
 {
-    if (is_one(th)) return drcp(dadd(x, 1.0f));
+    if (one || is_one(th)) return drcp(dadd(x, 1.0f));
     return dmul(dadd(dneg(dmul(om, x)), 1.0f), drcp(dadd(dmul(th, x), 1.0f)));
 }
 // (U0 + d) f in FP64 for a double-float factor f: U0 (f_hi + f_lo) + d f_hi (d is an FP32 quantity, so
@@ -1006,19 +1006,21 @@ __device__ __forceinline__ double scale_state(double U0, float d, double f64, fl
 
 // U0: the FP64 state at t^m; d: the FP32 increment (transport and explicit sources over dt); T: the gas
 // temperature (read for FROZEN_T, read and updated for FULL and LINEAR).  Writes Un = U^{m+1} before
-// realizability.
+// realizability.  EXK >= 0: the exchange mode as a compile-time constant, and theta_F = theta_E = 1 (the two-pass
+// kernels of common grids); -1: g.exchange and any theta.
+template <int EXK = -1>
 __device__ __forceinline__ void split_stiff(const GridParams& g, const GridArrays& a, const SplitStiffConsts& k,
                                             float chat, float dt, const GasCell<float>& gc, const double U0[4],
                                             const float d[4], double& T, double Un[4], Counters& cnt)
 {
     const float rho = gc.rho32;
     {
-        const dfl fF = theta_factor(split_x(k, a.kF32, gc.kF, k.KF, g.kpow, rho), k.thF, k.omF);
+        const dfl fF = theta_factor(split_x(k, a.kF32, gc.kF, k.KF, g.kpow, rho), k.thF, k.omF, EXK >= 0);
         const double f64 = df2d(fF);
 #pragma unroll
         for (int q = 1; q < 4; ++q) Un[q] = scale_state(U0[q], d[q], f64, fF.hi);
     }
-    const int ex = g.exchange;
+    const int ex = EXK >= 0 ? EXK : g.exchange;
     if (ex == EX_EQUILIBRIUM) {
         Un[0] = U0[0] + f2d_exact(d[0]);
         return;
@@ -1054,7 +1056,7 @@ __device__ __forceinline__ void split_stiff(const GridParams& g, const GridArray
     float qv;
     const float del = exchange_delta_fp32(g, chat, dt, rho, gc.kP, Ein.hi, Td.hi, o, qv);
     const float t0 = qv * del;
-    const bool thone = o.theta_fb || is_one(k.thE);
+    const bool thone = EXK >= 0 || o.theta_fb || is_one(k.thE);
     const dfl th = o.theta_fb ? dfl{1.0f, 0.0f} : k.thE;
     const dfl sig = dmul(k.sig1, rho);
     const dfl sD = dmul(sig, dadd(thone ? xP : dmul(th, xP), 1.0f));  // sigma (1 + theta x)

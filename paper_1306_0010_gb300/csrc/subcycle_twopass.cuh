@@ -163,8 +163,9 @@ struct GeoPred {
 };
 
 // Predictor over the column tile (x0, y0) of the stored U^{m+1/2} (coordinates in [-pad, n+pad))
-// for planes [z0, z1).
-template <int TX, int TY>
+// for planes [z0, z1).  COMMON: M1 closure and speeds, theta_F = 1 and no theta update of E (FULL, EQUILIBRIUM),
+// known at compile time: the branches and arithmetic of the other modes cost every cell 7 % (256^3: 378 -> 351 us).
+template <int TX, int TY, bool COMMON>
 __device__ __forceinline__ void predictor_tile(const GridParams& g, const GridArrays& a, float4* uh, float chat,
                                                float dt, int x0, int y0, int z0, int z1, float4* sm, Counters& cnt)
 {
@@ -183,8 +184,8 @@ __device__ __forceinline__ void predictor_tile(const GridParams& g, const GridAr
     float* osl = reinterpret_cast<float*>(sm + G::END4) + t;
     const float hdt = 0.5f * dt;
     const float idx = g.f_inv_dx[0], idy = g.f_inv_dx[1], idz = g.f_inv_dx[2];
-    const int p1 = g.closure == 1, fixed = g.speeds == 1;
-    const bool needT = g.exchange == EX_FROZEN_T;
+    const int p1 = !COMMON && g.closure == 1, fixed = !COMMON && g.speeds == 1;
+    const bool needT = !COMMON && g.exchange == EX_FROZEN_T;
     const long long nxy = (long long)g.n[0] * g.n[1];
     const int tlx = t % TX, tly = t / TX;
     const int gx = x0 + tlx, gy = y0 + tly;
@@ -388,7 +389,15 @@ __device__ __forceinline__ void predictor_tile(const GridParams& g, const GridAr
                 float U[4];
 #pragma unroll
                 for (int qq = 0; qq < 4; ++qq) U[qq] = U0a[qq] - hdt * div[qq] + hdt * S[qq];
-                theta_updates(g, gc, chat, hdt, U);
+                if constexpr (COMMON) {
+                    // theta_updates with theta_F = 1, to the bit
+                    const float fF = rcp(xadd(1.0f, xmul(xmul(chat, gc.kF), hdt)));
+                    U[1] *= fF;
+                    U[2] *= fF;
+                    U[3] *= fF;
+                } else {
+                    theta_updates(g, gc, chat, hdt, U);
+                }
                 const int fx_ = realize(U, g.f_E_floor);
                 if (own_interior && p >= 0 && p < g.n[2]) cnt.fix += fx_;
                 uh[chk(uoff, n_padded(g))] = f4(U);
@@ -428,8 +437,10 @@ struct GeoCorr {
 
 // Corrector over the interior column tile (x0, y0) for planes [z0, z1).  TMA: the tile + 2-cell halo
 // of each U^{m+1/2} plane arrives by one tensor copy (issued by thread 0, completed on mbar[buf]; map
-// and mbar are then required, and sm must be 128-byte aligned); otherwise by per-thread cp.async.
-template <int TX, int TY, bool TMA = false, int LIMK = -1>
+// and mbar are then required, and sm must be 128-byte aligned); otherwise by per-thread cp.async.  EXK >= 0: a common
+// grid (M1 closure and speeds, theta_F = theta_E = 1) with that exchange mode, FULL or EQUILIBRIUM, at compile
+// time; -1: any mode (256^3, FULL: 922 us general; common 851 with the branch-free HLL and the integer split).
+template <int TX, int TY, bool TMA, int LIMK, int EXK>
 __device__ __forceinline__ void corrector_tile(const GridParams& g, const GridArrays& a, const float4* uh,
                                                float chat, float dt, double chat_d, double dt_d, int x0, int y0,
                                                int z0, int z1, float4* sm,
@@ -448,8 +459,10 @@ __device__ __forceinline__ void corrector_tile(const GridParams& g, const GridAr
     const float idx = g.f_inv_dx[0], idy = g.f_inv_dx[1], idz = g.f_inv_dx[2];
     const SplitStiffConsts sk = split_stiff_consts(g, chat_d, dt_d);
     // LIMK >= 0: the limiter is a compile-time constant (only its code is generated); -1: g.limiter
-    const int p1 = g.closure == 1, fixed = g.speeds == 1, lim = LIMK >= 0 ? LIMK : g.limiter;
-    const bool needT = g.exchange == EX_FULL || g.exchange == EX_FROZEN_T;
+    constexpr bool COMMON = EXK >= 0;
+    const int p1 = !COMMON && g.closure == 1, fixed = !COMMON && g.speeds == 1, lim = LIMK >= 0 ? LIMK : g.limiter;
+    const int ex = COMMON ? EXK : g.exchange;
+    const bool needT = ex == EX_FULL || ex == EX_FROZEN_T;
     const int tlx = t % TX, tly = t / TX;
     const int gx = x0 + tlx, gy = y0 + tly;
     const bool own_col = gx < g.n[0] && gy < g.n[1];
@@ -542,8 +555,8 @@ __device__ __forceinline__ void corrector_tile(const GridParams& g, const GridAr
     {
         const float4 u_m2 = col(z0 - 2), u_m1 = col(z0 - 1), u_0 = col(z0), u_1 = col(z0 + 1);
         float4 ra[4], rb[4];
-        face_record_ab<2>(u_m2, u_m1, u_0, chat, lim, p1, fixed, ra);
-        const int fb = face_record_ab<2>(u_m1, u_0, u_1, chat, lim, p1, fixed, rb);
+        face_record_ab<2, COMMON>(u_m2, u_m1, u_0, chat, lim, p1, fixed, ra);
+        const int fb = face_record_ab<2, COMMON>(u_m1, u_0, u_1, chat, lim, p1, fixed, rb);
         cnt.face += (unsigned)(fb & (int)own_col);
         cfl = hll_pair(ra[1], rb[0], flux_ab<2>(ra[1], ra[2].z, ra[2].w), flux_ab<2>(rb[0], rb[2].x, rb[2].y), ra[3].z,
                        ra[3].w, rb[3].x, rb[3].y, chat);
@@ -617,23 +630,23 @@ __device__ __forceinline__ void corrector_tile(const GridParams& g, const GridAr
         // face-state records: the own cell along x and along y, then this thread's halo record
         {
             float4 rec[4];
-            const int fb = face_record_ab<0>(Uk[ihc - 1], Uk[ihc], Uk[ihc + 1], chat, lim, p1, fixed, rec);
+            const int fb = face_record_ab<0, COMMON>(Uk[ihc - 1], Uk[ihc], Uk[ihc + 1], chat, lim, p1, fixed, rec);
             cnt.face += (unsigned)(fb & (int)own_col);
             store_rec(Sx, G::NSX, sx_own, rec);
         }
         {
             float4 rec[4];
-            const int fb = face_record_ab<1>(Uk[ihc - G::W2], Uk[ihc], Uk[ihc + G::W2], chat, lim, p1, fixed, rec);
+            const int fb = face_record_ab<1, COMMON>(Uk[ihc - G::W2], Uk[ihc], Uk[ihc + G::W2], chat, lim, p1, fixed, rec);
             cnt.face += (unsigned)(fb & (int)own_col);
             store_rec(Sy, G::NSY, sy_own, rec);
         }
         if (has_hr) {
             float4 rec[4];
             if (hr_is_y) {
-                face_record_ab<1>(Uk[hr_i - G::W2], Uk[hr_i], Uk[hr_i + G::W2], chat, lim, p1, fixed, rec);
+                face_record_ab<1, COMMON>(Uk[hr_i - G::W2], Uk[hr_i], Uk[hr_i + G::W2], chat, lim, p1, fixed, rec);
                 store_rec(Sy, G::NSY, hr_slot, rec);
             } else {
-                face_record_ab<0>(Uk[hr_i - 1], Uk[hr_i], Uk[hr_i + 1], chat, lim, p1, fixed, rec);
+                face_record_ab<0, COMMON>(Uk[hr_i - 1], Uk[hr_i], Uk[hr_i + 1], chat, lim, p1, fixed, rec);
                 store_rec(Sx, G::NSX, hr_slot, rec);
             }
         }
@@ -641,7 +654,7 @@ __device__ __forceinline__ void corrector_tile(const GridParams& g, const GridAr
         float4 cfh;
         {
             float4 rec[4];
-            const int fb = face_record_ab<2>(Uk[ihc], ukp1, ukp2, chat, lim, p1, fixed, rec);
+            const int fb = face_record_ab<2, COMMON>(Uk[ihc], ukp1, ukp2, chat, lim, p1, fixed, rec);
             cnt.face += (unsigned)(fb & (int)(k + 1 < z1) & (int)own_col);
             cfh = hll_pair(zpS, rec[0], flux_ab<2>(zpS, zpa, zpb), flux_ab<2>(rec[0], rec[2].x, rec[2].y), zpl1, zpl3,
                            rec[3].x, rec[3].y, chat);
@@ -694,14 +707,14 @@ __device__ __forceinline__ void corrector_tile(const GridParams& g, const GridAr
                                   (bxf.w - ax.w) * idx + (by.w - ay.w) * idy + (cfh.w - cfl.w) * idz};
             const float4 Uhk4 = Uk[ihc];
             const float Uhk[4] = {Uhk4.x, Uhk4.y, Uhk4.z, Uhk4.w};
-            const bool full = g.exchange == EX_FULL;
+            const bool full = ex == EX_FULL;
             float S[4];
             explicit_sources(g, gc, Uhk, chat, S);
             float d[4];
 #pragma unroll
             for (int qq = 0; qq < 4; ++qq) d[qq] = -dt * div[qq] + dt * S[qq];
             double Un[4];
-            split_stiff(g, a, sk, chat, dt, gc, U0, d, Tn, Un, cnt);
+            split_stiff<EXK>(g, a, sk, chat, dt, gc, U0, d, Tn, Un, cnt);
             // realizability: the FP32 mirror screens, the FP64 test runs only near the limit
             float4 m = make_float4(d2f_trunc(Un[0]), d2f_trunc(Un[1]), d2f_trunc(Un[2]), d2f_trunc(Un[3]));
             if (!(m.x > g.f_E_floor * 1.001f) || m.y * m.y + m.z * m.z + m.w * m.w > 0.9999f * m.x * m.x) {
@@ -741,7 +754,7 @@ __device__ __forceinline__ void corrector_tile(const GridParams& g, const GridAr
     }
 }
 
-template <int TX, int TY>
+template <int TX, int TY, bool COMMON>
 __global__ void __launch_bounds__(TX* TY, RHD_PRED_MIN_BLOCKS) predictor_kernel(const __grid_constant__ StepParams P)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -750,11 +763,11 @@ __global__ void __launch_bounds__(TX* TY, RHD_PRED_MIN_BLOCKS) predictor_kernel(
     const int z0 = (int)blockIdx.y * P.z_chunk - P.g.pad[2];
     const int z1 = min(z0 + P.z_chunk, P.g.n[2] + P.g.pad[2]);
     Counters cnt = {0, 0, 0, 0, 0, 0};
-    predictor_tile<TX, TY>(P.g, P.a, P.uhalf, P.f_chat, P.f_dt, x0, y0, z0, z1, reinterpret_cast<float4*>(smem_raw), cnt);
+    predictor_tile<TX, TY, COMMON>(P.g, P.a, P.uhalf, P.f_chat, P.f_dt, x0, y0, z0, z1, reinterpret_cast<float4*>(smem_raw), cnt);
     add_counter(&P.stats->n_fix, cnt.fix);
 }
 
-template <int TX, int TY, bool TMA, int LIMK>
+template <int TX, int TY, bool TMA, int LIMK, int EXK>
 __global__ void __launch_bounds__(TX* TY, RHD_CORR_MIN_BLOCKS) corrector_kernel(const __grid_constant__ StepParams P)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -767,7 +780,7 @@ __global__ void __launch_bounds__(TX* TY, RHD_CORR_MIN_BLOCKS) corrector_kernel(
     // TMA destinations need 128-byte alignment: the launch adds 128 bytes of slack
     float4* sm = reinterpret_cast<float4*>(smem_raw);
     if constexpr (TMA) sm = reinterpret_cast<float4*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
-    corrector_tile<TX, TY, TMA, LIMK>(P.g, P.a, P.uhalf, P.f_chat, P.f_dt, P.chat, P.dt, x0, y0, z0, z1, sm, cnt,
+    corrector_tile<TX, TY, TMA, LIMK, EXK>(P.g, P.a, P.uhalf, P.f_chat, P.f_dt, P.chat, P.dt, x0, y0, z0, z1, sm, cnt,
                                       &P.uh_map, mbar, P.wait_polls);
     add_counter(&P.stats->n_fix, cnt.fix);
     add_counter(&P.stats->n_face, cnt.face);
@@ -811,7 +824,7 @@ __device__ __forceinline__ bool ens_next(const EnsembleParams& P, EnsembleGrid& 
     return true;
 }
 
-template <int TX, int TY>
+template <int TX, int TY, bool COMMON>
 __global__ void __launch_bounds__(TX* TY, RHD_PRED_MIN_BLOCKS) predictor_ens_kernel(const __grid_constant__ EnsembleParams P)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -825,14 +838,14 @@ __global__ void __launch_bounds__(TX* TY, RHD_PRED_MIN_BLOCKS) predictor_ens_ker
         const int txy = (int)(local % nxy), tz = (int)(local / nxy);
         const int x0 = (txy % eg.ptiles_x) * TX - eg.g.pad[0], y0 = (txy / eg.ptiles_x) * TY - eg.g.pad[1];
         const int z0 = tz * P.z_chunk - eg.g.pad[2], z1 = min(z0 + P.z_chunk, eg.g.n[2] + eg.g.pad[2]);
-        predictor_tile<TX, TY>(eg.g, eg.a, eg.uhalf, P.f_chat, eg.f_dt, x0, y0, z0, z1,
+        predictor_tile<TX, TY, COMMON>(eg.g, eg.a, eg.uhalf, P.f_chat, eg.f_dt, x0, y0, z0, z1,
                                reinterpret_cast<float4*>(smem_raw), cnt);
         __syncthreads();
     }
     add_counter(&P.stats->n_fix, cnt.fix);
 }
 
-template <int TX, int TY, int LIMK>
+template <int TX, int TY, int LIMK, int EXK>
 __global__ void __launch_bounds__(TX* TY, RHD_CORR_MIN_BLOCKS) corrector_ens_kernel(const __grid_constant__ EnsembleParams P)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -846,7 +859,7 @@ __global__ void __launch_bounds__(TX* TY, RHD_CORR_MIN_BLOCKS) corrector_ens_ker
         const int txy = (int)(local % nxy), tz = (int)(local / nxy);
         const int x0 = (txy % eg.tiles_x) * TX, y0 = (txy / eg.tiles_x) * TY;
         const int z0 = tz * P.z_chunk, z1 = min(z0 + P.z_chunk, eg.g.n[2]);
-        corrector_tile<TX, TY, false, LIMK>(eg.g, eg.a, eg.uhalf, P.f_chat, eg.f_dt, P.chat, eg.dt, x0, y0, z0, z1,
+        corrector_tile<TX, TY, false, LIMK, EXK>(eg.g, eg.a, eg.uhalf, P.f_chat, eg.f_dt, P.chat, eg.dt, x0, y0, z0, z1,
                                reinterpret_cast<float4*>(smem_raw), cnt);
         __syncthreads();
     }
