@@ -101,6 +101,14 @@ __device__ __forceinline__ float d2f_rn(double x)
     r = a >= 0x47f00000u ? (sign | 0x7f800000u) : r;
     return __uint_as_float(r);
 }
+
+// (float)x, round to nearest, by integer operations: the conversion instruction runs on the FP64 pipe.  Values
+// outside the FP32 normal range (rare), infinities and NaN take it all the same.
+__device__ __forceinline__ float to_f32(double x)
+{
+    const unsigned m = (unsigned)__double2hiint(x) & 0x7fffffffu;
+    return m != 0u && (m < 0x38100000u || m >= 0x47f00000u) ? (float)x : d2f_rn(x);
+}
 // x as a double-float (one FP64 subtraction, exact: x - hi is representable); relative error u^2
 __device__ __forceinline__ dfl d2df(double x)
 {

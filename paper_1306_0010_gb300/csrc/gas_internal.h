@@ -36,24 +36,38 @@ struct GasArrays {
     double* rho;              // gas at t^n (read), overwritten with t^{n+1} by the corrector
     double* T;
     double* v[3];             // all three components present
-    const float* rho32;       // split grids: FP32 copies of rho and v (current with the FP64 state)
-    const float* v32[3];
+    float* rho32;             // split grids: FP32 copies of rho and v (current with the FP64 state; the corrector
+    float* v32[3];            // and the correction keep them so)
+    float4* gas4;             // the two-pass subcycles' interleaved copy, rewritten likewise, or NULL
     const double* kF;         // NULL: the opacity law
     const double* E;          // radiation at t^n (step) or t^{n+1} (correction), G = F/c
     const double* G[3];
-    double* wh[5];            // W^{n+1/2} = (rho, vx, vy, vz, P) on the extended grid m[0] x m[1] x m[2]
-                              // (FP64 grids; NULL on split grids)
-    float* wh32[5];           // split grids: W^{n+1/2} in FP32 (an intermediate of the step, like the
-                              // radiation's U^{m+1/2})
-    double* flux[3][5];       // face fluxes of direction d (predictor layout (m_d + 1) x m_e, corrector
-                              // layout (n_d + 1) x n_e), components (rho, Mx, My, Mz, E_gas); FP32 values
-                              // (the first half of each buffer) on split grids
-    double* pend[8];          // kept for the correction: k_F(rho^{n+1/2}), v^{n+1/2} (3), E^n, G^n (3)
+    const float4* um32;       // split grids: E and G in FP32 where the two-pass mirror is current, else NULL
+    double* wh[5];            // FP64 grids: W^{n+1/2} = (rho, vx, vy, vz, P) on the extended grid m[0] x m[1] x m[2]
+    float4* wh4;              // split grids: the same in FP32, (rho, v) and P (an intermediate of the step, like
+    float* whP;               // the radiation's U^{m+1/2})
+    double* flux[3][5];       // FP64 grids in 2D and 3D: face fluxes of direction d (predictor layout
+                              // (m_d + 1) x m_e, corrector layout (n_d + 1) x n_e), components (rho, Mx, My, Mz,
+                              // E_gas)
+    double* pend[8];          // FP64 grids, for the correction: k_F(rho^{n+1/2}), v^{n+1/2} (3), E^n, G^n (3)
+    float4* rad4;             // split grids, for the correction: E^n and G^n in FP32 (k_F and v^{n+1/2}: from wh4)
     unsigned long long* counters;  // [0] cells whose internal energy was floored to 0, [1] non-finite cells
 };
 
-// one gas step over p.dt is: launch_gas_pred_flux for each active direction, launch_gas_pred_update,
-// launch_gas_corr_flux for each active direction, launch_gas_corr_update (all on one stream)
+// How the marching kernels split a grid: tiles in x and y, planes a CTA marches
+struct GasMarch {
+    int tiles_x, planes;
+    long long tiles;
+};
+
+// Split grids, and FP64 grids in 1D, take a gas step in two launches, predictor and corrector.  FP64 grids in 2D
+// and 3D, which the FP64 pipe bounds and the fluxes' way through memory does not, compute each face once: a
+// launch for each direction's fluxes, then an update.
+bool gas_marched(const GasParams& p);
+cudaError_t launch_gas_predictor(const GasParams& p, const GasArrays& a, int num_sms, cudaStream_t s);
+cudaError_t launch_gas_corrector(const GasParams& p, const GasArrays& a, int num_sms, cudaStream_t s);
+// the others: launch_gas_pred_flux for each active direction, launch_gas_pred_update, launch_gas_corr_flux for
+// each active direction, launch_gas_corr_update
 cudaError_t launch_gas_pred_flux(const GasParams& p, const GasArrays& a, int d, cudaStream_t s);
 cudaError_t launch_gas_pred_update(const GasParams& p, const GasArrays& a, cudaStream_t s);
 cudaError_t launch_gas_corr_flux(const GasParams& p, const GasArrays& a, int d, cudaStream_t s);

@@ -26,13 +26,6 @@ cudaError_t launch_scale_copy(double* dst, const double* src, double scale, long
     return cudaGetLastError();
 }
 
-// (float)x, round to nearest, by integer operations: the conversion instruction runs on the FP64 pipe.  Values
-// outside the FP32 normal range (rare), infinities and NaN take it all the same.
-__device__ __forceinline__ float to_f32(double x)
-{
-    const unsigned m = (unsigned)__double2hiint(x) & 0x7fffffffu;
-    return m != 0u && (m < 0x38100000u || m >= 0x47f00000u) ? (float)x : d2f_rn(x);
-}
 // x / c, c > 0, for y = 1/c correctly rounded (0: always divide): one multiplication and one correction by the exact residual (the
 // correctly rounded quotient, by Markstein's theorem, where nothing under- or overflows: three FP64
 // instructions against CUDA's ten or so), the division itself elsewhere
@@ -192,20 +185,6 @@ cudaError_t launch_moments_out(const MomentsIn& m, long long n, cudaStream_t s)
     for (int k = 0; k < 4; ++k) two = two && aligned16(m.src[k]) && aligned16(m.dst[k]);
     if (two) moments_out_kernel<2><<<copy_blocks(n / 2), 256, 0, s>>>(m, n / 2);
     else moments_out_kernel<1><<<copy_blocks(n), 256, 0, s>>>(m, n);
-    return cudaGetLastError();
-}
-
-__global__ void to_float_kernel(float* dst, const double* src, long long n)
-{
-    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    long long stride = (long long)gridDim.x * blockDim.x;
-    for (; i < n; i += stride) dst[i] = to_f32(src[i]);
-}
-
-cudaError_t launch_to_float(float* dst, const double* src, long long n, cudaStream_t s)
-{
-    if (n <= 0) return cudaSuccess;
-    to_float_kernel<<<copy_blocks(n), 256, 0, s>>>(dst, src, n);
     return cudaGetLastError();
 }
 

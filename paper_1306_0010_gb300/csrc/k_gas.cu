@@ -9,8 +9,9 @@
 //              then the full step (sources from the gas at t^{n+1/2} and the radiation at t^n);
 //   correction (after the subcycles): dt/2 [S_e,gas(W^{n+1/2}, U_rad^{n+1}) - S_e,gas(W^{n+1/2}, U_rad^n)].
 //
-// Each face flux is computed once, by one thread, and stored (the face arrays of one direction); the
-// update kernels take the flux differences.  The HLLC solver (Toro, Riemann Solvers and Numerical
+// Split grids, and FP64 grids in 1D, take each half of the step in one launch, whose face fluxes stay in
+// shared memory; FP64 grids in 2D and 3D store them (each computed once, by one thread) for an update launch.
+// The HLLC solver (Toro, Riemann Solvers and Numerical
 // Methods for Fluid Dynamics, Sec. 10.4) uses the Davis wave-speed estimates; the left star state when
 // S* = 0; HLL where the contact speed's denominator is not negative.
 //
@@ -28,6 +29,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include "dfloat.cuh"
 #include "fp_convert.cuh"
 #include "gas_index.h"
 #include "gas_internal.h"
@@ -75,25 +77,6 @@ __device__ __forceinline__ Prim<double> load_prim(const GasParams& p, const GasA
     w.r = a.rho[i];
     for (int d = 0; d < 3; ++d) w.v[d] = flip(a.v[d][i], s[d]);
     w.P = w.r * a.T[i] * p.inv_mu;
-    return w;
-}
-
-template <typename R>
-__device__ __forceinline__ Prim<R> load_prim_t(const GasParams& p, const GasArrays& a, long long i, const int s[3]);
-template <>
-__device__ __forceinline__ Prim<double> load_prim_t<double>(const GasParams& p, const GasArrays& a, long long i,
-                                                            const int s[3])
-{
-    return load_prim(p, a, i, s);
-}
-template <>
-__device__ __forceinline__ Prim<float> load_prim_t<float>(const GasParams& p, const GasArrays& a, long long i,
-                                                          const int s[3])
-{
-    Prim<float> w;
-    w.r = a.rho32[i];
-    for (int d = 0; d < 3; ++d) w.v[d] = flip(a.v32[d][i], s[d]);
-    w.P = w.r * d2f_trunc(a.T[i]) * p.f_inv_mu;
     return w;
 }
 
@@ -264,13 +247,9 @@ __device__ __forceinline__ bool finite_prim(const Prim<double>& w)
 __device__ __forceinline__ long long first_index() { return (long long)blockIdx.x * blockDim.x + threadIdx.x; }
 __device__ __forceinline__ long long index_stride() { return (long long)gridDim.x * blockDim.x; }
 
-// minus the divergence of the stored FP64 face fluxes (FP64 grids)
-template <typename R>
+// minus the divergence of the stored face fluxes
 __device__ __forceinline__ void flux_divergence(const GasParams& p, const GasArrays& a, const long long lo[3],
-                                                const long long hi[3], double dU[5]);
-template <>
-__device__ __forceinline__ void flux_divergence<double>(const GasParams& p, const GasArrays& a, const long long lo[3],
-                                                        const long long hi[3], double dU[5])
+                                                const long long hi[3], double dU[5])
 {
     for (int q = 0; q < 5; ++q) dU[q] = 0.0;
     for (int d = 0; d < 3; ++d) {
@@ -279,242 +258,499 @@ __device__ __forceinline__ void flux_divergence<double>(const GasParams& p, cons
     }
 }
 
-// split grids: minus the divergence of the stored FP32 face fluxes, in FP32
-__device__ __forceinline__ void flux_divergence32(const GasParams& p, const GasArrays& a, const long long lo[3],
-                                                  const long long hi[3], float dU[5])
+// ---------------------------------------------------------------------------------------- a cell's steps
+
+// half step of extended cell i (interior cell k mirrored with the signs s): W^{n+1/2} from minus the flux
+// divergence dU and the sources at t^n; true if the internal energy was floored
+__device__ __forceinline__ bool pred_update(const GasParams& p, const GasArrays& a, long long i, long long k,
+                                            const int s[3], const double dU[5])
 {
-    for (int q = 0; q < 5; ++q) dU[q] = 0.0f;
-    for (int d = 0; d < 3; ++d) {
-        if (p.n[d] <= 1) continue;
-        for (int q = 0; q < 5; ++q) {
-            const float* F = reinterpret_cast<const float*>(a.flux[d][q]);
-            dU[q] -= (F[hi[d]] - F[lo[d]]) * p.f_inv_dx[d];
-        }
-    }
+    const double hdt = 0.5 * p.dt;
+    const Prim<double> W = load_prim(p, a, k, s);
+    double U[5];
+    to_cons(p, W, U);
+    const double G[3] = {flip(a.G[0][k], s[0]), flip(a.G[1][k], s[1]), flip(a.G[2][k], s[2])};
+    double S[5];
+    gas_source(p, absorption(p, a.kF, k, W.r), W.v, a.E[k], G, S);
+    double Uh[5], inv_r;
+    for (int q = 0; q < 5; ++q) Uh[q] = U[q] + hdt * dU[q] + hdt * S[q];
+    Prim<double> Wh;
+    const bool neg = to_prim(p, Uh, Wh, inv_r);
+    const double w5[5] = {Wh.r, Wh.v[0], Wh.v[1], Wh.v[2], Wh.P};
+    for (int q = 0; q < 5; ++q) a.wh[q][i] = w5[q];
+    return neg;
 }
 
-// ---------------------------------------------------------------------------------------- predictor
+// full step of interior cell i (extended cell x), and the record the source correction needs
+__device__ __forceinline__ void corr_update(const GasParams& p, const GasArrays& a, long long i, long long x,
+                                            const double dU[5], unsigned long long& floors, unsigned long long& bad)
+{
+    const int one[3] = {1, 1, 1};
+    const Prim<double> W = load_prim(p, a, i, one);
+    double U[5];
+    to_cons(p, W, U);
+    const double rh = a.wh[0][x];
+    const double vh[3] = {a.wh[1][x], a.wh[2][x], a.wh[3][x]};
+    const double kh = absorption(p, a.kF, i, rh);
+    const double E = a.E[i];
+    const double G[3] = {a.G[0][i], a.G[1][i], a.G[2][i]};
+    double S[5];
+    gas_source(p, kh, vh, E, G, S);
+    double U1[5], inv_r;
+    for (int q = 0; q < 5; ++q) U1[q] = U[q] + p.dt * dU[q] + p.dt * S[q];
+    Prim<double> W1;
+    if (to_prim(p, U1, W1, inv_r)) ++floors;
+    if (!finite_prim(W1)) ++bad;
+    a.rho[i] = W1.r;
+    for (int d = 0; d < 3; ++d) a.v[d][i] = W1.v[d];
+    a.T[i] = W1.P * p.mu_over_kB * inv_r;
+    a.pend[0][i] = kh;
+    for (int d = 0; d < 3; ++d) a.pend[1 + d][i] = vh[d];
+    a.pend[4][i] = E;
+    for (int d = 0; d < 3; ++d) a.pend[5 + d][i] = G[d];
+}
 
-template <typename R, int D>
+// limited slopes of a cell; a slope whose face values have rho <= 0 or P <= 0 is zeroed (all components)
+template <typename R>
+__device__ __forceinline__ void cell_slopes(const R wm[5], const R w0[5], const R wp[5], int lim, R sl[5])
+{
+    for (int q = 0; q < 5; ++q) sl[q] = limited_slope<R>(w0[q] - wm[q], wp[q] - w0[q], lim);
+    bool bad = false;
+    for (int hs = 0; hs < 2; ++hs) {
+        const R sg = hs ? R(0.5) : R(-0.5);
+        bad = bad || !(w0[0] + sg * sl[0] > R(0)) || !(w0[4] + sg * sl[4] > R(0));
+    }
+    if (bad)
+        for (int q = 0; q < 5; ++q) sl[q] = R(0);
+}
+
+// the cell's state at its high (h = 1/2) or low (h = -1/2) face
+template <typename R>
+__device__ __forceinline__ Prim<R> face_state(const R w0[5], const R sl[5], R h)
+{
+    Prim<R> W;
+    W.r = w0[0] + h * sl[0];
+    for (int q = 0; q < 3; ++q) W.v[q] = w0[1 + q] + h * sl[1 + q];
+    W.P = w0[4] + h * sl[4];
+    return W;
+}
+
+// ------------------------------------------------------------- FP64 grids in 2D and 3D: a launch per direction
+
+template <int D>
 __global__ void __launch_bounds__(GAS_THREADS) gas_pred_flux_kernel(GasParams p, GasArrays a)
 {
     int fe[3];
     gas_pred_faces(p, D, fe);
     const long long nf = gas_count(fe);
-    const Consts<R> k = consts<R>(p);
+    const Consts<double> k = consts<double>(p);
     for (long long f = first_index(); f < nf; f += index_stride()) {
         long long iL, iR;
         int sL[3], sR[3];
         gas_pred_flux_cells(p, D, f, &iL, sL, &iR, sR);
-        const Prim<R> WL = load_prim_t<R>(p, a, iL, sL), WR = load_prim_t<R>(p, a, iR, sR);
-        R F[5];
-        hllc<R, D>(k, WL, WR, F);
-        for (int q = 0; q < 5; ++q) reinterpret_cast<R*>(a.flux[D][q])[f] = F[q];
+        const Prim<double> WL = load_prim(p, a, iL, sL), WR = load_prim(p, a, iR, sR);
+        double F[5];
+        hllc<double, D>(k, WL, WR, F);
+        for (int q = 0; q < 5; ++q) a.flux[D][q][f] = F[q];
     }
 }
 
-// split grids (R = float): memory-bound, so more resident warps (6 and 5 CTAs of 256 per SM) keep more loads
-// in flight than the few registers they cost; FP64 grids: bound by the FP64 pipe
-template <typename R>
-__global__ void __launch_bounds__(GAS_THREADS, sizeof(R) == 4 ? 6 : 1) gas_pred_update_kernel(GasParams p, GasArrays a)
+__global__ void __launch_bounds__(GAS_THREADS) gas_pred_update_kernel(GasParams p, GasArrays a)
 {
     const long long ne = gas_count(p.m);
-    const double hdt = 0.5 * p.dt;
     unsigned long long floors = 0;
-    if constexpr (sizeof(R) == 4) {
-        // split grids: W^{n+1/2} in FP32 from the FP32 copies of W^n and FP32 increments
-        const float fh = (float)hdt;
-        for (long long i = first_index(); i < ne; i += index_stride()) {
-            long long k, lo[3], hi[3];
-            int s[3];
-            bool inside;
-            gas_pred_update_cells(p, i, &k, s, &inside, lo, hi);
-            const float r = a.rho32[k], T = d2f_trunc(a.T[k]);
-            const float v[3] = {flip(a.v32[0][k], s[0]), flip(a.v32[1][k], s[1]), flip(a.v32[2][k], s[2])};
-            float dU[5], S[5];
-            flux_divergence32(p, a, lo, hi, dU);
-            const float G[3] = {flip(d2f_trunc(a.G[0][k]), s[0]), flip(d2f_trunc(a.G[1][k]), s[1]),
-                                flip(d2f_trunc(a.G[2][k]), s[2])};
-            gas_source32(p, absorption32(p, a.kF, k, r), v, d2f_trunc(a.E[k]), G, S);
-            float D[5];
-            for (int q = 0; q < 5; ++q) D[q] = fh * (dU[q] + S[q]);
-            const PrimInc o = prim_increment(p, r, v, T, D);
-            float Th = T + o.dT;
-            if (Th < 0.0f) {
-                Th = 0.0f;
-                if (inside) ++floors;
-            }
-            a.wh32[0][i] = o.r1;
-            for (int d = 0; d < 3; ++d) a.wh32[1 + d][i] = v[d] + o.dv[d];
-            a.wh32[4][i] = o.r1 * Th * p.f_inv_mu;
-        }
-        if (floors) atomicAdd(&a.counters[0], floors);
-    } else {
-        for (long long i = first_index(); i < ne; i += index_stride()) {
-            long long k, lo[3], hi[3];
-            int s[3];
-            bool inside;
-            gas_pred_update_cells(p, i, &k, s, &inside, lo, hi);
-            const Prim<double> W = load_prim(p, a, k, s);
-            double U[5], dU[5];
-            to_cons(p, W, U);
-            flux_divergence<R>(p, a, lo, hi, dU);
-            const double G[3] = {flip(a.G[0][k], s[0]), flip(a.G[1][k], s[1]), flip(a.G[2][k], s[2])};
-            double S[5];
-            gas_source(p, absorption(p, a.kF, k, W.r), W.v, a.E[k], G, S);
-            double Uh[5], inv_r;
-            for (int q = 0; q < 5; ++q) Uh[q] = U[q] + hdt * dU[q] + hdt * S[q];
-            Prim<double> Wh;
-            if (to_prim(p, Uh, Wh, inv_r) && inside) ++floors;
-            const double w5[5] = {Wh.r, Wh.v[0], Wh.v[1], Wh.v[2], Wh.P};
-            for (int q = 0; q < 5; ++q) a.wh[q][i] = w5[q];
-        }
-        if (floors) atomicAdd(&a.counters[0], floors);
+    for (long long i = first_index(); i < ne; i += index_stride()) {
+        long long k, lo[3], hi[3];
+        int s[3];
+        bool inside;
+        gas_pred_update_cells(p, i, &k, s, &inside, lo, hi);
+        double dU[5];
+        flux_divergence(p, a, lo, hi, dU);
+        if (pred_update(p, a, i, k, s, dU) && inside) ++floors;
     }
+    if (floors) atomicAdd(&a.counters[0], floors);
 }
 
-// ---------------------------------------------------------------------------------------- corrector
-
-template <typename R>
-__device__ __forceinline__ R load_half(const GasArrays& a, int q, long long x);
-template <>
-__device__ __forceinline__ double load_half<double>(const GasArrays& a, int q, long long x)
-{
-    return a.wh[q][x];
-}
-template <>
-__device__ __forceinline__ float load_half<float>(const GasArrays& a, int q, long long x)
-{
-    return a.wh32[q][x];
-}
-
-template <typename R, int D>
+template <int D>
 __global__ void __launch_bounds__(GAS_THREADS) gas_corr_flux_kernel(GasParams p, GasArrays a)
 {
     int fe[3];
     gas_corr_faces(p, D, fe);
     const long long nf = gas_count(fe);
-    const Consts<R> k = consts<R>(p);
+    const Consts<double> k = consts<double>(p);
     for (long long f = first_index(); f < nf; f += index_stride()) {
         // W^{n+1/2} of the cells f - 2 e_D .. f + e_D
         long long x[4];
         gas_corr_flux_cells(p, D, f, x);
-        R w[4][5];
+        double w[4][5], sl[5];
         for (int j = 0; j < 4; ++j)
-            for (int q = 0; q < 5; ++q) w[j][q] = load_half<R>(a, q, x[j]);
-        // limited slopes of the cells on each side of the face; a slope whose face values have
-        // rho <= 0 or P <= 0 is zeroed (all components)
-        Prim<R> WL, WR;
-        for (int side = 0; side < 2; ++side) {
-            const R* wm = w[side];
-            const R* w0 = w[side + 1];
-            const R* wp = w[side + 2];
-            R sl[5];
-            for (int q = 0; q < 5; ++q) sl[q] = limited_slope<R>(w0[q] - wm[q], wp[q] - w0[q], p.limiter);
-            bool bad = false;
-            for (int hs = 0; hs < 2; ++hs) {
-                const R sg = hs ? R(0.5) : R(-0.5);
-                bad = bad || !(w0[0] + sg * sl[0] > R(0)) || !(w0[4] + sg * sl[4] > R(0));
-            }
-            if (bad)
-                for (int q = 0; q < 5; ++q) sl[q] = R(0);
-            Prim<R>& W = side ? WR : WL;
-            const R h = side ? R(-0.5) : R(0.5);  // cell f - e_D: its high face; cell f: its low face
-            W.r = w0[0] + h * sl[0];
-            for (int q = 0; q < 3; ++q) W.v[q] = w0[1 + q] + h * sl[1 + q];
-            W.P = w0[4] + h * sl[4];
-        }
-        R F[5];
-        hllc<R, D>(k, WL, WR, F);
-        for (int q = 0; q < 5; ++q) reinterpret_cast<R*>(a.flux[D][q])[f] = F[q];
+            for (int q = 0; q < 5; ++q) w[j][q] = a.wh[q][x[j]];
+        cell_slopes(w[0], w[1], w[2], p.limiter, sl);
+        const Prim<double> WL = face_state(w[1], sl, 0.5);
+        cell_slopes(w[1], w[2], w[3], p.limiter, sl);
+        const Prim<double> WR = face_state(w[2], sl, -0.5);
+        double F[5];
+        hllc<double, D>(k, WL, WR, F);
+        for (int q = 0; q < 5; ++q) a.flux[D][q][f] = F[q];
     }
 }
 
-template <typename R>
-__global__ void __launch_bounds__(GAS_THREADS, sizeof(R) == 4 ? 5 : 1) gas_corr_update_kernel(GasParams p, GasArrays a)
+__global__ void __launch_bounds__(GAS_THREADS) gas_corr_update_kernel(GasParams p, GasArrays a)
 {
     const long long nc = gas_count(p.n);
     unsigned long long floors = 0, bad = 0;
-    if constexpr (sizeof(R) == 4) {
-        // split grids: FP32 increments (fluxes, sources at W^{n+1/2}) accumulated into the FP64 state
-        const float fdt = (float)p.dt;
-        for (long long i = first_index(); i < nc; i += index_stride()) {
-            long long x, lo[3], hi[3];
-            gas_corr_update_cells(p, i, &x, lo, hi);
-            const double rho = a.rho[i], T = a.T[i];
-            const double v[3] = {a.v[0][i], a.v[1][i], a.v[2][i]};
-            const float v32[3] = {d2f_trunc(v[0]), d2f_trunc(v[1]), d2f_trunc(v[2])};
-            float dU[5], S[5];
-            flux_divergence32(p, a, lo, hi, dU);
-            const float rh = a.wh32[0][x];
-            const float vh[3] = {a.wh32[1][x], a.wh32[2][x], a.wh32[3][x]};
-            const float kh = absorption32(p, a.kF, i, rh);
-            const double E = a.E[i];
-            const double G[3] = {a.G[0][i], a.G[1][i], a.G[2][i]};
-            const float G32[3] = {d2f_trunc(G[0]), d2f_trunc(G[1]), d2f_trunc(G[2])};
-            gas_source32(p, kh, vh, d2f_trunc(E), G32, S);
-            float D[5];
-            for (int q = 0; q < 5; ++q) D[q] = fdt * (dU[q] + S[q]);
-            const PrimInc o = prim_increment(p, d2f_trunc(rho), v32, d2f_trunc(T), D);
-            const double rho1 = rho + f2d_exact(D[0]);
-            double T1 = T + f2d_exact(o.dT);
-            if (below_zero_bits(T1)) {
-                T1 = 0.0;
-                ++floors;
-            }
-            double v1[3];
-            for (int d = 0; d < 3; ++d) v1[d] = v[d] + f2d_exact(o.dv[d]);
-            if (!(finite_bits(rho1) && finite_bits(v1[0]) && finite_bits(v1[1]) && finite_bits(v1[2]) &&
-                  finite_bits(T1)))
-                ++bad;
-            a.rho[i] = rho1;
-            for (int d = 0; d < 3; ++d) a.v[d][i] = v1[d];
-            a.T[i] = T1;
-            a.pend[0][i] = f2d_exact(kh);
-            for (int d = 0; d < 3; ++d) a.pend[1 + d][i] = f2d_exact(vh[d]);
-            a.pend[4][i] = E;
-            for (int d = 0; d < 3; ++d) a.pend[5 + d][i] = G[d];
-        }
-        if (floors) atomicAdd(&a.counters[0], floors);
-        if (bad) atomicAdd(&a.counters[1], bad);
-    } else {
-        for (long long i = first_index(); i < nc; i += index_stride()) {
-            long long x, lo[3], hi[3];
-            gas_corr_update_cells(p, i, &x, lo, hi);
-            const int one[3] = {1, 1, 1};
-            const Prim<double> W = load_prim(p, a, i, one);
-            double U[5], dU[5];
-            to_cons(p, W, U);
-            flux_divergence<R>(p, a, lo, hi, dU);
-            const double rh = a.wh[0][x];
-            const double vh[3] = {a.wh[1][x], a.wh[2][x], a.wh[3][x]};
-            const double kh = absorption(p, a.kF, i, rh);
-            const double E = a.E[i];
-            const double G[3] = {a.G[0][i], a.G[1][i], a.G[2][i]};
-            double S[5];
-            gas_source(p, kh, vh, E, G, S);
-            double U1[5], inv_r;
-            for (int q = 0; q < 5; ++q) U1[q] = U[q] + p.dt * dU[q] + p.dt * S[q];
-            Prim<double> W1;
-            if (to_prim(p, U1, W1, inv_r)) ++floors;
-            if (!finite_prim(W1)) ++bad;
-            a.rho[i] = W1.r;
-            for (int d = 0; d < 3; ++d) a.v[d][i] = W1.v[d];
-            a.T[i] = W1.P * p.mu_over_kB * inv_r;
-            a.pend[0][i] = kh;
-            for (int d = 0; d < 3; ++d) a.pend[1 + d][i] = vh[d];
-            a.pend[4][i] = E;
-            for (int d = 0; d < 3; ++d) a.pend[5 + d][i] = G[d];
-        }
-        if (floors) atomicAdd(&a.counters[0], floors);
-        if (bad) atomicAdd(&a.counters[1], bad);
+    for (long long i = first_index(); i < nc; i += index_stride()) {
+        long long x, lo[3], hi[3];
+        gas_corr_update_cells(p, i, &x, lo, hi);
+        double dU[5];
+        flux_divergence(p, a, lo, hi, dU);
+        corr_update(p, a, i, x, dU, floors, bad);
     }
+    if (floors) atomicAdd(&a.counters[0], floors);
+    if (bad) atomicAdd(&a.counters[1], bad);
+}
+
+// ------------------------------------------- split grids, and FP64 grids in 1D: one launch for a half of the step
+//
+// A CTA takes a tile of x and y and marches its planes in z.  Each face's flux is computed by the thread of the
+// cell above it (x and y: passed to the cell below through shared memory; z: kept in registers for the next
+// plane), the faces that close the tile by two more warps (one for the row above it, one for the column).
+// Nothing but the half step's result goes through memory: a launch for each direction that stored its faces' five
+// components, and an update that read them back, moved 20 B a cell and direction there and again 20 B back.
+// Same arithmetic, operation for operation.  Bound by instruction issue (HLLC and the limiter; the launches per
+// direction were bound by memory): the step and its correction with the copies the subcycles read, 256^3 split,
+// 3.5 -> 2.5 ms; 300 x 250 x 200 3.2 -> 2.6 ms; FP64, 512 cells, 64 -> 38 us.
+
+// the FP32 radiation state of interior cell i: the two-pass subcycles' mirror where it is current
+__device__ __forceinline__ float4 load_rad32(const GasArrays& a, long long i)
+{
+    if (a.um32) return a.um32[i];
+    return make_float4(d2f_trunc(a.E[i]), d2f_trunc(a.G[0][i]), d2f_trunc(a.G[1][i]), d2f_trunc(a.G[2][i]));
+}
+
+// split grids: the new velocity and the FP32 copies the subcycles read
+__device__ __forceinline__ void store_velocity(const GasArrays& a, long long i, float r32, const double v1[3])
+{
+    const float f[3] = {to_f32(v1[0]), to_f32(v1[1]), to_f32(v1[2])};
+    for (int d = 0; d < 3; ++d) {
+        a.v[d][i] = v1[d];
+        a.v32[d][i] = f[d];
+    }
+    if (a.gas4) a.gas4[i] = make_float4(r32, f[0], f[1], f[2]);
+}
+
+// a cell of W^n as it lies in memory (split grids: the FP32 copies), its mirrored normal components flipped
+template <typename R>
+struct GasCell {
+    R r, v[3], T;
+};
+template <typename R>
+__device__ __forceinline__ GasCell<R> load_cell(const GasArrays& a, long long k, int s0, int s1, int s2)
+{
+    if constexpr (sizeof(R) == 4)
+        return {a.rho32[k], {flip(a.v32[0][k], s0), flip(a.v32[1][k], s1), flip(a.v32[2][k], s2)}, d2f_trunc(a.T[k])};
+    else
+        return {a.rho[k], {flip(a.v[0][k], s0), flip(a.v[1][k], s1), flip(a.v[2][k], s2)}, a.T[k]};
+}
+template <typename R>
+__device__ __forceinline__ Prim<R> prim_of(const GasParams& p, const GasCell<R>& c)
+{
+    Prim<R> w;
+    w.r = c.r;
+    for (int d = 0; d < 3; ++d) w.v[d] = c.v[d];
+    if constexpr (sizeof(R) == 4) w.P = c.r * c.T * p.f_inv_mu;
+    else w.P = c.r * c.T * p.inv_mu;
+    return w;
+}
+
+// W^{n+1/2} of extended cell x
+template <typename R>
+struct GasHalf {
+    R w[5];
+};
+template <typename R>
+__device__ __forceinline__ GasHalf<R> load_half(const GasArrays& a, long long x)
+{
+    if constexpr (sizeof(R) == 4) {
+        const float4 h = a.wh4[x];
+        return {{h.x, h.y, h.z, h.w, a.whP[x]}};
+    } else {
+        return {{a.wh[0][x], a.wh[1][x], a.wh[2][x], a.wh[3][x], a.wh[4][x]}};
+    }
+}
+
+// dU -= (hi - lo) / dx, the difference rounded by itself (as of values that come from memory)
+__device__ __forceinline__ void add_divergence(const GasParams& p, int d, float lo, float hi, float& dU)
+{
+    dU -= __fsub_rn(hi, lo) * p.f_inv_dx[d];
+}
+__device__ __forceinline__ void add_divergence(const GasParams& p, int d, double lo, double hi, double& dU)
+{
+    dU -= __dsub_rn(hi, lo) * p.inv_dx[d];
+}
+
+// The threads of a tile of TX x TY cells: one per cell (its low faces), then a warp for the y faces above the
+// top row (2D, 3D), then one for the x faces beyond the last column.
+template <int DIM, int TX, int TY>
+struct GasTile {
+    static constexpr int MAIN = TX * TY, ROW = DIM > 1 ? TX : 0, NT = MAIN + ROW + 32;
+    int tx, ty;
+    bool cell, fx, fy;
+    __device__ __forceinline__ GasTile()
+    {
+        const int t = threadIdx.x;
+        cell = t < MAIN;
+        fx = cell;
+        fy = DIM > 1 && t < MAIN + ROW;
+        tx = t % TX;
+        ty = t / TX;
+        if (t >= MAIN + ROW) {
+            tx = TX;
+            ty = t - (MAIN + ROW);
+            fx = ty < TY;
+        }
+    }
+};
+
+// faces of one plane, for the cells below them
+template <typename R, int DIM, int TX, int TY>
+struct GasFaces {
+    R x[5][TY][TX + 1];
+    R y[DIM > 1 ? 5 : 1][DIM > 1 ? TY + 1 : 1][DIM > 1 ? TX : 1];
+};
+
+template <typename R, int DIM, int TX, int TY>
+__device__ __forceinline__ void tile_divergence(const GasParams& p, const GasFaces<R, DIM, TX, TY>& f, int tx, int ty,
+                                                const R zlo[5], const R zhi[5], R dU[5])
+{
+    for (int q = 0; q < 5; ++q) {
+        dU[q] = R(0);
+        if (p.n[0] > 1) add_divergence(p, 0, f.x[q][ty][tx], f.x[q][ty][tx + 1], dU[q]);
+        if constexpr (DIM > 1) add_divergence(p, 1, f.y[q][ty][tx], f.y[q][ty + 1][tx], dU[q]);
+        if constexpr (DIM > 2) add_divergence(p, 2, zlo[q], zhi[q], dU[q]);
+    }
+}
+
+template <typename R, int DIM, int TX, int TY>
+__global__ void __launch_bounds__((GasTile<DIM, TX, TY>::NT)) gas_predictor_kernel(const __grid_constant__ GasParams p,
+                                                                                 const __grid_constant__ GasArrays a,
+                                                                                 const GasMarch t)
+{
+    __shared__ GasFaces<R, DIM, TX, TY> faces[DIM > 2 ? 2 : 1];
+    const GasTile<DIM, TX, TY> me;
+    const Consts<R> kc = consts<R>(p);
+    const int b = (int)(blockIdx.x % t.tiles), zc = (int)(blockIdx.x / t.tiles) * t.planes;
+    const int ze = zc + t.planes < p.m[2] ? zc + t.planes : p.m[2];
+    const int X = (b % t.tiles_x) * TX + me.tx, Y = (b / t.tiles_x) * TY + me.ty;
+    const bool cell = me.cell && X < p.m[0] && Y < p.m[1];
+    const bool fx = me.fx && p.n[0] > 1 && X <= p.m[0] && Y < p.m[1];
+    const bool fy = me.fy && X < p.m[0] && Y <= p.m[1];
+    // the interior cell under the thread's own, and under its low neighbours in x and y
+    int sx = 1, sy = 1, sxl = 1, syl = 1;
+    const int qx = gas_axis(X - p.g[0], p.n[0], p.bc_lo[0], p.bc_hi[0], sx);
+    const int qy = gas_axis(Y - p.g[1], p.n[1], p.bc_lo[1], p.bc_hi[1], sy);
+    const int qxl = gas_axis(X - p.g[0] - 1, p.n[0], p.bc_lo[0], p.bc_hi[0], sxl);
+    const int qyl = gas_axis(Y - p.g[1] - 1, p.n[1], p.bc_lo[1], p.bc_hi[1], syl);
+    const long long row = p.n[0], plane = row * p.n[1];
+    const long long own = qx + row * qy, left = qxl + row * qy, low = qx + row * qyl;
+    const bool in_xy = X >= p.g[0] && X < p.g[0] + p.n[0] && Y >= p.g[1] && Y < p.g[1] + p.n[1];
+    unsigned long long floors = 0;
+
+    int sz = 1, szn = 1;
+    int z = DIM > 2 ? zc - 1 : 0;  // 3D: the plane below the chunk gives the flux through its lowest face
+    long long base = DIM > 2 ? plane * gas_axis(z - p.g[2], p.n[2], p.bc_lo[2], p.bc_hi[2], sz) : 0, base_n = 0;
+    GasCell<R> cur = load_cell<R>(a, own + base, sx, sy, sz), nxt = cur;
+    R zlo[5], zhi[5];
+    for (int q = 0; q < 5; ++q) zlo[q] = zhi[q] = R(0);
+    for (; z < ze; ++z) {
+        const bool on = DIM < 3 || z >= zc;
+        GasFaces<R, DIM, TX, TY>& f = faces[DIM > 2 ? z & 1 : 0];
+        if constexpr (DIM > 2) {
+            szn = 1;
+            base_n = plane * gas_axis(z + 1 - p.g[2], p.n[2], p.bc_lo[2], p.bc_hi[2], szn);
+            if (cell || z + 1 < ze) nxt = load_cell<R>(a, own + base_n, sx, sy, szn);
+        }
+        float4 u = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        float kf = 0.0f;
+        if (on) {
+            if constexpr (sizeof(R) == 4)
+                if (cell) {
+                    u = load_rad32(a, own + base);
+                    kf = absorption32(p, a.kF, own + base, cur.r);
+                }
+            if (fx) {
+                const GasCell<R> l = load_cell<R>(a, left + base, sxl, sy, sz);
+                R F[5];
+                hllc<R, 0>(kc, prim_of(p, l), prim_of(p, cur), F);
+                for (int q = 0; q < 5; ++q) f.x[q][me.ty][me.tx] = F[q];
+            }
+            if constexpr (DIM > 1)
+                if (fy) {
+                    const GasCell<R> l = load_cell<R>(a, low + base, sx, syl, sz);
+                    R F[5];
+                    hllc<R, 1>(kc, prim_of(p, l), prim_of(p, cur), F);
+                    for (int q = 0; q < 5; ++q) f.y[q][me.ty][me.tx] = F[q];
+                }
+        }
+        if constexpr (DIM > 2)
+            if (cell) hllc<R, 2>(kc, prim_of(p, cur), prim_of(p, nxt), zhi);
+        if (on) {
+            __syncthreads();
+            if (cell) {
+                R dU[5];
+                tile_divergence(p, f, me.tx, me.ty, zlo, zhi, dU);
+                const long long i = X + (long long)p.m[0] * (Y + (long long)p.m[1] * z);
+                const bool inside = in_xy && (DIM < 3 || (z >= p.g[2] && z < p.g[2] + p.n[2]));
+                if constexpr (sizeof(R) == 4) {
+                    // W^{n+1/2} in FP32 from the FP32 copies of W^n and FP32 increments
+                    const float fh = (float)(0.5 * p.dt);
+                    float S[5], D[5];
+                    const float G[3] = {flip(u.y, sx), flip(u.z, sy), flip(u.w, sz)};
+                    gas_source32(p, kf, cur.v, u.x, G, S);
+                    for (int q = 0; q < 5; ++q) D[q] = fh * (dU[q] + S[q]);
+                    const PrimInc o = prim_increment(p, cur.r, cur.v, cur.T, D);
+                    float Th = cur.T + o.dT;
+                    if (Th < 0.0f) {
+                        Th = 0.0f;
+                        if (inside) ++floors;
+                    }
+                    a.wh4[i] = make_float4(o.r1, cur.v[0] + o.dv[0], cur.v[1] + o.dv[1], cur.v[2] + o.dv[2]);
+                    a.whP[i] = o.r1 * Th * p.f_inv_mu;
+                } else {
+                    const int s[3] = {sx, sy, sz};
+                    if (pred_update(p, a, i, own + base, s, dU) && inside) ++floors;
+                }
+            }
+        }
+        cur = nxt;
+        base = base_n;
+        sz = szn;
+        for (int q = 0; q < 5; ++q) zlo[q] = zhi[q];
+    }
+    if (floors) atomicAdd(&a.counters[0], floors);
+}
+
+template <typename R, int DIM, int TX, int TY>
+__global__ void __launch_bounds__((GasTile<DIM, TX, TY>::NT)) gas_corrector_kernel(const __grid_constant__ GasParams p,
+                                                                                 const __grid_constant__ GasArrays a,
+                                                                                 const GasMarch t)
+{
+    __shared__ GasFaces<R, DIM, TX, TY> faces[DIM > 2 ? 2 : 1];
+    const GasTile<DIM, TX, TY> me;
+    const Consts<R> kc = consts<R>(p);
+    const int b = (int)(blockIdx.x % t.tiles), zc = (int)(blockIdx.x / t.tiles) * t.planes;
+    const int ze = zc + t.planes < p.n[2] ? zc + t.planes : p.n[2];
+    const int X = (b % t.tiles_x) * TX + me.tx, Y = (b / t.tiles_x) * TY + me.ty;
+    const bool cell = me.cell && X < p.n[0] && Y < p.n[1];
+    const bool fx = me.fx && p.n[0] > 1 && X <= p.n[0] && Y < p.n[1];
+    const bool fy = me.fy && X < p.n[0] && Y <= p.n[1];
+    const bool any = cell || fx || fy;
+    const long long row = p.m[0], plane = row * p.m[1];
+    // the thread's extended cell in plane z is own + plane * z
+    const long long own = X + p.g[0] + row * (Y + p.g[1]) + plane * p.g[2];
+    unsigned long long floors = 0, bad = 0;
+
+    // 3D: cells z, z + 1 and z + 2 of the thread's column; the slope of z + 1 gives its states at the faces z + 1
+    // and z + 2, the flux through face z + 1 closes cell z.  Two planes below the chunk start the chain.
+    int z = DIM > 2 ? zc - 2 : 0;
+    GasHalf<R> w0{}, w1{}, w2{};
+    Prim<R> up{};  // state of cell z at its high z face
+    R zlo[5], zhi[5];
+    for (int q = 0; q < 5; ++q) zlo[q] = zhi[q] = R(0);
+    if (any) {
+        w0 = load_half<R>(a, own + plane * z);
+        if constexpr (DIM > 2) w1 = load_half<R>(a, own + plane * (z + 1));
+    }
+    for (; z < ze; ++z) {
+        const bool on = DIM < 3 || z >= zc;
+        GasFaces<R, DIM, TX, TY>& f = faces[DIM > 2 ? z & 1 : 0];
+        const long long x = own + plane * z;
+        R sl[5];
+        if constexpr (DIM > 2)
+            if (cell || (any && z + 2 < ze)) w2 = load_half<R>(a, x + 2 * plane);
+        if (on) {
+            if (fx) {
+                const GasHalf<R> a0 = load_half<R>(a, x - 2), a1 = load_half<R>(a, x - 1), a3 = load_half<R>(a, x + 1);
+                cell_slopes(a0.w, a1.w, w0.w, p.limiter, sl);
+                const Prim<R> L = face_state(a1.w, sl, R(0.5));
+                cell_slopes(a1.w, w0.w, a3.w, p.limiter, sl);
+                R F[5];
+                hllc<R, 0>(kc, L, face_state(w0.w, sl, R(-0.5)), F);
+                for (int q = 0; q < 5; ++q) f.x[q][me.ty][me.tx] = F[q];
+            }
+            if constexpr (DIM > 1)
+                if (fy) {
+                    const GasHalf<R> a0 = load_half<R>(a, x - 2 * row), a1 = load_half<R>(a, x - row),
+                                     a3 = load_half<R>(a, x + row);
+                    cell_slopes(a0.w, a1.w, w0.w, p.limiter, sl);
+                    const Prim<R> L = face_state(a1.w, sl, R(0.5));
+                    cell_slopes(a1.w, w0.w, a3.w, p.limiter, sl);
+                    R F[5];
+                    hllc<R, 1>(kc, L, face_state(w0.w, sl, R(-0.5)), F);
+                    for (int q = 0; q < 5; ++q) f.y[q][me.ty][me.tx] = F[q];
+                }
+        }
+        if constexpr (DIM > 2)
+            if (cell) {
+                cell_slopes(w0.w, w1.w, w2.w, p.limiter, sl);
+                if (z >= zc - 1) hllc<R, 2>(kc, up, face_state(w1.w, sl, R(-0.5)), zhi);
+                up = face_state(w1.w, sl, R(0.5));
+            }
+        if (on) {
+            __syncthreads();
+            if (cell) {
+                R dU[5];
+                tile_divergence(p, f, me.tx, me.ty, zlo, zhi, dU);
+                const long long i = X + (long long)p.n[0] * (Y + (long long)p.n[1] * z);
+                if constexpr (sizeof(R) == 4) {
+                    // FP32 increments (fluxes, sources at W^{n+1/2}) accumulated into the FP64 state
+                    const float fdt = (float)p.dt;
+                    const double rho = a.rho[i], T = a.T[i];
+                    const double v[3] = {a.v[0][i], a.v[1][i], a.v[2][i]};
+                    const float v32[3] = {d2f_trunc(v[0]), d2f_trunc(v[1]), d2f_trunc(v[2])};
+                    const float vh[3] = {w0.w[1], w0.w[2], w0.w[3]};
+                    const float kh = absorption32(p, a.kF, i, w0.w[0]);
+                    const float4 u = load_rad32(a, i);
+                    const float G[3] = {u.y, u.z, u.w};
+                    float S[5], D[5];
+                    gas_source32(p, kh, vh, u.x, G, S);
+                    for (int q = 0; q < 5; ++q) D[q] = fdt * (dU[q] + S[q]);
+                    const PrimInc o = prim_increment(p, d2f_trunc(rho), v32, d2f_trunc(T), D);
+                    const double rho1 = rho + f2d_exact(D[0]);
+                    double T1 = T + f2d_exact(o.dT);
+                    if (below_zero_bits(T1)) {
+                        T1 = 0.0;
+                        ++floors;
+                    }
+                    double v1[3];
+                    for (int d = 0; d < 3; ++d) v1[d] = v[d] + f2d_exact(o.dv[d]);
+                    if (!(finite_bits(rho1) && finite_bits(v1[0]) && finite_bits(v1[1]) && finite_bits(v1[2]) &&
+                          finite_bits(T1)))
+                        ++bad;
+                    const float r32 = to_f32(rho1);
+                    a.rho[i] = rho1;
+                    a.rho32[i] = r32;
+                    a.T[i] = T1;
+                    store_velocity(a, i, r32, v1);
+                    a.rad4[i] = u;  // the radiation at t^n, for the correction (k_F and v^{n+1/2}: from W^{n+1/2})
+                } else {
+                    corr_update(p, a, i, x, dU, floors, bad);
+                }
+            }
+        }
+        w0 = w1;
+        w1 = w2;
+        for (int q = 0; q < 5; ++q) zlo[q] = zhi[q];
+    }
+    if (floors) atomicAdd(&a.counters[0], floors);
+    if (bad) atomicAdd(&a.counters[1], bad);
 }
 
 // ---------------------------------------------------------------------------------------- correction
 
 template <bool SPLIT>
-__global__ void __launch_bounds__(GAS_THREADS) gas_correct_kernel(GasParams p, GasArrays a)
+__global__ void __launch_bounds__(GAS_THREADS) gas_correct_kernel(const __grid_constant__ GasParams p,
+                                                                  const __grid_constant__ GasArrays a)
 {
     const long long nc = gas_count(p.n);
     const double hdt = 0.5 * p.dt;
@@ -525,15 +761,19 @@ __global__ void __launch_bounds__(GAS_THREADS) gas_correct_kernel(GasParams p, G
         // increments accumulated into the FP64 state
         const float fh = (float)hdt;
         for (long long i = first_index(); i < nc; i += index_stride()) {
+            int c[3];
+            gas_unravel(i, p.n, c);
+            for (int d = 0; d < 3; ++d) c[d] += p.g[d];
+            const float4 h = a.wh4[gas_ravel(c, p.m)];
             const double rho = a.rho[i], T = a.T[i];
             const double v[3] = {a.v[0][i], a.v[1][i], a.v[2][i]};
             const float v32[3] = {d2f_trunc(v[0]), d2f_trunc(v[1]), d2f_trunc(v[2])};
-            const float kh = d2f_trunc(a.pend[0][i]);
-            const float vh[3] = {d2f_trunc(a.pend[1][i]), d2f_trunc(a.pend[2][i]), d2f_trunc(a.pend[3][i])};
-            float dG[3];
-            for (int d = 0; d < 3; ++d) dG[d] = d2f_trunc(a.G[d][i]) - d2f_trunc(a.pend[5 + d][i]);
+            const float vh[3] = {h.y, h.z, h.w};
+            const float kh = absorption32(p, a.kF, i, h.x);
+            const float4 u0 = a.rad4[i], u1 = load_rad32(a, i);
+            const float dG[3] = {u1.y - u0.y, u1.z - u0.z, u1.w - u0.w};
             float dS[5];
-            gas_source32(p, kh, vh, d2f_trunc(a.E[i]) - d2f_trunc(a.pend[4][i]), dG, dS);
+            gas_source32(p, kh, vh, u1.x - u0.x, dG, dS);
             const float D[5] = {0.0f, fh * dS[1], fh * dS[2], fh * dS[3], fh * dS[4]};
             const PrimInc o = prim_increment(p, d2f_trunc(rho), v32, d2f_trunc(T), D);
             double T1 = T + f2d_exact(o.dT);
@@ -544,8 +784,8 @@ __global__ void __launch_bounds__(GAS_THREADS) gas_correct_kernel(GasParams p, G
             double v1[3];
             for (int d = 0; d < 3; ++d) v1[d] = v[d] + f2d_exact(o.dv[d]);
             if (!(finite_bits(v1[0]) && finite_bits(v1[1]) && finite_bits(v1[2]) && finite_bits(T1))) ++bad;
-            for (int d = 0; d < 3; ++d) a.v[d][i] = v1[d];
             a.T[i] = T1;
+            store_velocity(a, i, to_f32(rho), v1);
         }
         if (floors) atomicAdd(&a.counters[0], floors);
         if (bad) atomicAdd(&a.counters[1], bad);
@@ -581,39 +821,79 @@ int blocks_for(long long n)
     return (int)(b < 1 ? 1 : (b > (1LL << 30) ? (1LL << 30) : b));
 }
 
-template <typename R>
-void pred_flux(const GasParams& p, const GasArrays& a, int d, int nb, cudaStream_t s)
+// The work split of a march over a grid of e cells: a tile per CTA, and in 3D so many planes that some four waves
+// of CTAs fill the chip (three resident ones on each multiprocessor), at least eight (a chunk starts with one
+// plane's z faces, the corrector's with another plane's slopes).
+GasMarch march_of(const int e[3], int tx, int ty, int num_sms, long long* blocks)
 {
-    if (d == 0) gas_pred_flux_kernel<R, 0><<<nb, GAS_THREADS, 0, s>>>(p, a);
-    else if (d == 1) gas_pred_flux_kernel<R, 1><<<nb, GAS_THREADS, 0, s>>>(p, a);
-    else gas_pred_flux_kernel<R, 2><<<nb, GAS_THREADS, 0, s>>>(p, a);
+    GasMarch t;
+    t.tiles_x = (e[0] + tx - 1) / tx;
+    t.tiles = (long long)t.tiles_x * ((e[1] + ty - 1) / ty);
+    long long chunks = (12LL * num_sms + t.tiles - 1) / t.tiles;
+    const long long most = (e[2] + 7) / 8;
+    if (chunks > most) chunks = most;
+    t.planes = (int)((e[2] + chunks - 1) / chunks);
+    *blocks = t.tiles * ((e[2] + t.planes - 1) / t.planes);
+    return t;
+}
+
+template <typename R, int DIM, int TX, int TY>
+void launch_half(const GasParams& p, const GasArrays& a, bool predictor, int num_sms, cudaStream_t s)
+{
+    long long nb;
+    const GasMarch t = march_of(predictor ? p.m : p.n, TX, TY, num_sms, &nb);
+    constexpr int NT = GasTile<DIM, TX, TY>::NT;
+    if (predictor) gas_predictor_kernel<R, DIM, TX, TY><<<(unsigned)nb, NT, 0, s>>>(p, a, t);
+    else gas_corrector_kernel<R, DIM, TX, TY><<<(unsigned)nb, NT, 0, s>>>(p, a, t);
 }
 
 template <typename R>
-void corr_flux(const GasParams& p, const GasArrays& a, int d, int nb, cudaStream_t s)
+void launch_half_1d(const GasParams& p, const GasArrays& a, bool predictor, int num_sms, cudaStream_t s)
 {
-    if (d == 0) gas_corr_flux_kernel<R, 0><<<nb, GAS_THREADS, 0, s>>>(p, a);
-    else if (d == 1) gas_corr_flux_kernel<R, 1><<<nb, GAS_THREADS, 0, s>>>(p, a);
-    else gas_corr_flux_kernel<R, 2><<<nb, GAS_THREADS, 0, s>>>(p, a);
+    // three warps of cells and one for the last face: a warp on each of the multiprocessor's partitions, while
+    // that gives every multiprocessor at most two CTAs; long lines take tiles with a smaller share of extra warps
+    if (p.m[0] <= 2LL * 96 * num_sms) launch_half<R, 1, 96, 1>(p, a, predictor, num_sms, s);
+    else launch_half<R, 1, 480, 1>(p, a, predictor, num_sms, s);
+}
+
+void launch_marched(const GasParams& p, const GasArrays& a, bool predictor, int num_sms, cudaStream_t s)
+{
+    if (!p.split) launch_half_1d<double>(p, a, predictor, num_sms, s);
+    else if (p.n[2] > 1) launch_half<float, 3, 32, 8>(p, a, predictor, num_sms, s);
+    else if (p.n[1] > 1) launch_half<float, 2, 32, 8>(p, a, predictor, num_sms, s);
+    else launch_half_1d<float>(p, a, predictor, num_sms, s);
 }
 
 }  // namespace
+
+bool gas_marched(const GasParams& p) { return p.split || p.n[1] <= 1; }
+
+cudaError_t launch_gas_predictor(const GasParams& p, const GasArrays& a, int num_sms, cudaStream_t s)
+{
+    launch_marched(p, a, true, num_sms, s);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_gas_corrector(const GasParams& p, const GasArrays& a, int num_sms, cudaStream_t s)
+{
+    launch_marched(p, a, false, num_sms, s);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_gas_pred_flux(const GasParams& p, const GasArrays& a, int d, cudaStream_t s)
 {
     int e[3];
     gas_pred_faces(p, d, e);
     const int nb = blocks_for(gas_count(e));
-    if (p.split) pred_flux<float>(p, a, d, nb, s);
-    else pred_flux<double>(p, a, d, nb, s);
+    if (d == 0) gas_pred_flux_kernel<0><<<nb, GAS_THREADS, 0, s>>>(p, a);
+    else if (d == 1) gas_pred_flux_kernel<1><<<nb, GAS_THREADS, 0, s>>>(p, a);
+    else gas_pred_flux_kernel<2><<<nb, GAS_THREADS, 0, s>>>(p, a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_gas_pred_update(const GasParams& p, const GasArrays& a, cudaStream_t s)
 {
-    const int nb = blocks_for(gas_count(p.m));
-    if (p.split) gas_pred_update_kernel<float><<<nb, GAS_THREADS, 0, s>>>(p, a);
-    else gas_pred_update_kernel<double><<<nb, GAS_THREADS, 0, s>>>(p, a);
+    gas_pred_update_kernel<<<blocks_for(gas_count(p.m)), GAS_THREADS, 0, s>>>(p, a);
     return cudaGetLastError();
 }
 
@@ -622,16 +902,15 @@ cudaError_t launch_gas_corr_flux(const GasParams& p, const GasArrays& a, int d, 
     int e[3];
     gas_corr_faces(p, d, e);
     const int nb = blocks_for(gas_count(e));
-    if (p.split) corr_flux<float>(p, a, d, nb, s);
-    else corr_flux<double>(p, a, d, nb, s);
+    if (d == 0) gas_corr_flux_kernel<0><<<nb, GAS_THREADS, 0, s>>>(p, a);
+    else if (d == 1) gas_corr_flux_kernel<1><<<nb, GAS_THREADS, 0, s>>>(p, a);
+    else gas_corr_flux_kernel<2><<<nb, GAS_THREADS, 0, s>>>(p, a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_gas_corr_update(const GasParams& p, const GasArrays& a, cudaStream_t s)
 {
-    const int nb = blocks_for(gas_count(p.n));
-    if (p.split) gas_corr_update_kernel<float><<<nb, GAS_THREADS, 0, s>>>(p, a);
-    else gas_corr_update_kernel<double><<<nb, GAS_THREADS, 0, s>>>(p, a);
+    gas_corr_update_kernel<<<blocks_for(gas_count(p.n)), GAS_THREADS, 0, s>>>(p, a);
     return cudaGetLastError();
 }
 

@@ -89,11 +89,13 @@ struct GridState {
     bool tuned = false;           // RHD_FLAG_AUTOTUNE handled
     double tuned_ms = -1.0;       // time per subcycle measured by the last tuning
     // gas step scratch (allocated by the first rhd_gas_step): W^{n+1/2} on the extended grid, the face
-    // fluxes of each active direction, and what rhd_gas_correct needs
+    // fluxes of each active direction (FP64 grids in 2D and 3D), and what rhd_gas_correct needs
     double* gas_wh[5] = {nullptr};
-    float* gas_wh32[5] = {nullptr};  // split grids: FP32 copy of W^{n+1/2}
-    double* gas_flux[3][5] = {{nullptr}};  // FP32 values on split grids
+    float4* gas_wh4 = nullptr;    // split grids: W^{n+1/2} in FP32
+    float* gas_whP = nullptr;
+    double* gas_flux[3][5] = {{nullptr}};
     double* gas_pend[8] = {nullptr};
+    float4* gas_rad4 = nullptr;   // split grids: the radiation at t^n in FP32
     bool gas_pending = false;     // a gas step waits for its source correction
     double gas_dt = 0.0;
 };
@@ -423,10 +425,10 @@ void free_grid(GridState& gs)
     dfree(gs.uhalf64);
     dfree(gs.um32);
     dfree(gs.gas4);
-    for (int q = 0; q < 5; ++q) {
-        dfree(gs.gas_wh[q]);
-        dfree(gs.gas_wh32[q]);
-    }
+    for (int q = 0; q < 5; ++q) dfree(gs.gas_wh[q]);
+    dfree(gs.gas_wh4);
+    dfree(gs.gas_whP);
+    dfree(gs.gas_rad4);
     for (int d = 0; d < 3; ++d)
         for (int q = 0; q < 5; ++q) dfree(gs.gas_flux[d][q]);
     for (int q = 0; q < 8; ++q) dfree(gs.gas_pend[q]);
@@ -754,14 +756,14 @@ rhd_status check_dt(rhd_ctx* ctx, const GridState& gs, double chat, double dt)
 // kernels reported by the kernel timer
 enum KernelId {
     K_FUSED_FP64 = 0, K_FUSED_SPLIT, K_PREDICTOR, K_CORRECTOR, K_ENS_FP64, K_ENS_SPLIT, K_ENS_PRED, K_ENS_CORR,
-    K_GAS_PRED_FLUX, K_GAS_PRED_UPDATE, K_GAS_CORR_FLUX, K_GAS_CORR_UPDATE, K_GAS_CORRECT, K_GAS_EXCHANGE,
+    K_GAS_PRED, K_GAS_CORR, K_GAS_PRED_FLUX, K_GAS_PRED_UPDATE, K_GAS_CORR_FLUX, K_GAS_CORR_UPDATE, K_GAS_CORRECT, K_GAS_EXCHANGE,
     K_PRED64, K_CORR64, K_ENS_PRED64, K_ENS_CORR64,
     K_COUNT
 };
 const char* const kKernelNames[K_COUNT] = {"subcycle_fused_fp64", "subcycle_fused_split", "twopass_predictor_split",
                                            "twopass_corrector_split", "ensemble_fp64", "ensemble_split",
                                            "ensemble_predictor_split", "ensemble_corrector_split",
-                                           "gas_predictor_flux", "gas_predictor_update", "gas_corrector_flux",
+                                           "gas_predictor", "gas_corrector", "gas_predictor_flux", "gas_predictor_update", "gas_corrector_flux",
                                            "gas_corrector_update", "gas_source_correction", "gas_step_exchange",
                                            "predictor_fp64", "corrector_fp64", "ensemble_predictor_fp64",
                                            "ensemble_corrector_fp64"};
@@ -1680,10 +1682,12 @@ GasArrays gas_arrays(rhd_ctx* ctx, GridState& gs)
     a.kF = gs.has_kF ? gs.kF : nullptr;
     a.E = gs.U[ctx->cur][0];
     for (int d = 0; d < 3; ++d) a.G[d] = gs.U[ctx->cur][1 + d];
-    for (int q = 0; q < 5; ++q) {
-        a.wh[q] = gs.gas_wh[q];
-        a.wh32[q] = gs.gas_wh32[q];
-    }
+    for (int q = 0; q < 5; ++q) a.wh[q] = gs.gas_wh[q];
+    a.wh4 = gs.gas_wh4;
+    a.whP = gs.gas_whP;
+    a.rad4 = gs.gas_rad4;
+    a.gas4 = gs.variant == RHD_VARIANT_TWOPASS ? gs.gas4 : nullptr;
+    a.um32 = gs.variant == RHD_VARIANT_TWOPASS && gs.um32_ok ? gs.um32 : nullptr;
     for (int d = 0; d < 3; ++d)
         for (int q = 0; q < 5; ++q) a.flux[d][q] = gs.gas_flux[d][q];
     for (int q = 0; q < 8; ++q) a.pend[q] = gs.gas_pend[q];
@@ -1696,21 +1700,23 @@ GasArrays gas_arrays(rhd_ctx* ctx, GridState& gs)
 rhd_status gas_prepare(rhd_ctx* ctx, GridState& gs, const GasParams& p)
 {
     rhd_status st;
-    if (!gs.gas_wh[0] && !gs.gas_wh32[0]) {
-        const size_t fb = p.split ? sizeof(float) : sizeof(double);
-        for (int q = 0; q < 5; ++q) {
-            if (!p.split && (st = dalloc(ctx, (void**)&gs.gas_wh[q], sizeof(double) * (size_t)gas_count(p.m))))
-                return st;
-            if (p.split && (st = dalloc(ctx, (void**)&gs.gas_wh32[q], sizeof(float) * (size_t)gas_count(p.m))))
-                return st;
-        }
-        for (int d = 0; d < 3; ++d) {
+    const size_t next = (size_t)gas_count(p.m), nc = (size_t)gs.ncell;
+    if (p.split) {
+        if (!gs.gas_wh4 && (st = dalloc(ctx, (void**)&gs.gas_wh4, sizeof(float4) * next))) return st;
+        if (!gs.gas_whP && (st = dalloc(ctx, (void**)&gs.gas_whP, sizeof(float) * next))) return st;
+        if (!gs.gas_rad4 && (st = dalloc(ctx, (void**)&gs.gas_rad4, sizeof(float4) * nc))) return st;
+    } else {
+        for (int q = 0; q < 5; ++q)
+            if (!gs.gas_wh[q] && (st = dalloc(ctx, (void**)&gs.gas_wh[q], sizeof(double) * next))) return st;
+        for (int d = 0; d < 3 && !gas_marched(p); ++d) {
             if (gs.desc.n[d] <= 1) continue;
             for (int q = 0; q < 5; ++q)
-                if ((st = dalloc(ctx, (void**)&gs.gas_flux[d][q], fb * (size_t)gas_face_capacity(p, d)))) return st;
+                if (!gs.gas_flux[d][q] &&
+                    (st = dalloc(ctx, (void**)&gs.gas_flux[d][q], sizeof(double) * (size_t)gas_face_capacity(p, d))))
+                    return st;
         }
         for (int q = 0; q < 8; ++q)
-            if ((st = dalloc(ctx, (void**)&gs.gas_pend[q], sizeof(double) * (size_t)gs.ncell))) return st;
+            if (!gs.gas_pend[q] && (st = dalloc(ctx, (void**)&gs.gas_pend[q], sizeof(double) * nc))) return st;
     }
     bool added = false;
     for (int d = 0; d < 3; ++d) {
@@ -1730,31 +1736,22 @@ rhd_status gas_prepare(rhd_ctx* ctx, GridState& gs, const GasParams& p)
     return RHD_OK;
 }
 
-// After the gas changed: the FP32 copies the split subcycles read
-rhd_status gas_refresh_copies(rhd_ctx* ctx, GridState& gs)
-{
-    if (gs.desc.precision == RHD_SPLIT) {
-        RHD_CUDA(ctx, launch_to_float(gs.rho32, gs.rho, gs.ncell, ctx->stream));
-        for (int d = 0; d < 3; ++d) RHD_CUDA(ctx, launch_to_float(gs.v32[d], gs.v[d], gs.ncell, ctx->stream));
-    }
-    gs.gas4_ok = false;
-    return RHD_OK;
-}
-
-// bytes per cell of each gas kernel (each array read or written once per launch): the gas state is
-// 40 B (rho, T, v; on split grids the predictor reads the FP32 rho, v and the FP64 T, 24 B), W^{n+1/2}
-// 40 B (20 B in FP32 on split grids), one face-flux array 40 B per cell (20 B split), the radiation
-// 32 B, the correction's record 64 B
+// bytes per cell of each gas kernel (each array read or written once per launch).  FP64 grids: the gas state is
+// 40 B (rho, T, v), W^{n+1/2} 40 B, one face-flux array 40 B, the radiation 32 B, the correction's record 64 B.
+// Split grids: the predictor reads the FP32 rho, v and the FP64 T (24 B), W^{n+1/2} is 20 B, the radiation 32 B
+// (16 B from the two-pass mirror), the record 16 B, and the new state's FP32 copies 16 B (32 B with gas4).
 double gas_alg_bytes(const GridState& gs, int k, int nact)
 {
     const bool split = gs.desc.precision == RHD_SPLIT;
-    const double kf = gs.has_kF ? 8.0 : 0.0, fl = split ? 20.0 : 40.0;
+    const double kf = gs.has_kF ? 8.0 : 0.0, rad = split && gs.um32 ? 16.0 : 32.0, copies = gs.gas4 ? 32.0 : 16.0;
     switch (k) {
-    case K_GAS_PRED_FLUX: return (split ? 24.0 : 40.0) + fl;
-    case K_GAS_PRED_UPDATE: return (split ? 24.0 : 40.0) + 32.0 + kf + fl * nact + (split ? 20.0 : 40.0);
-    case K_GAS_CORR_FLUX: return (split ? 20.0 : 40.0) + fl;
-    case K_GAS_CORR_UPDATE: return 40.0 + fl * nact + (split ? 16.0 : 32.0) + 32.0 + kf + 40.0 + 64.0;
-    default: return 40.0 + 64.0 + 32.0 + 32.0;  // K_GAS_CORRECT
+    case K_GAS_PRED: return split ? 24.0 + rad + kf + 20.0 : 40.0 + rad + kf + 40.0;
+    case K_GAS_CORR: return split ? 20.0 + 40.0 + rad + kf + 40.0 + copies + 16.0 : 40.0 + 40.0 + rad + kf + 40.0 + 64.0;
+    case K_GAS_PRED_FLUX: return 40.0 + 40.0;
+    case K_GAS_PRED_UPDATE: return 40.0 + 32.0 + kf + 40.0 * nact + 40.0;
+    case K_GAS_CORR_FLUX: return 40.0 + 40.0;
+    case K_GAS_CORR_UPDATE: return 40.0 + 40.0 * nact + 32.0 + 32.0 + kf + 40.0 + 64.0;
+    default: return split ? 36.0 + 16.0 + 16.0 + kf + rad + 32.0 + copies - 4.0 : 40.0 + 64.0 + 32.0 + 32.0;  // K_GAS_CORRECT
     }
 }
 
@@ -1784,25 +1781,34 @@ rhd_status rhd_gas_step(rhd_ctx* ctx, double dt_gas)
     int nact = 0;
     for (int d = 0; d < 3; ++d) nact += gs.desc.n[d] > 1;
     cudaStream_t s = ctx->stream;
-    for (int d = 0; d < 3; ++d) {
-        if (gs.desc.n[d] <= 1) continue;
-        if ((st = timed_launch(ctx, K_GAS_PRED_FLUX, ext * gas_alg_bytes(gs, K_GAS_PRED_FLUX, nact),
-                               [&] { return launch_gas_pred_flux(p, a, d, s); })))
+    if (gas_marched(p)) {
+        if ((st = timed_launch(ctx, K_GAS_PRED, ext * gas_alg_bytes(gs, K_GAS_PRED, nact),
+                               [&] { return launch_gas_predictor(p, a, ctx->num_sms, s); })))
+            return st;
+        if ((st = timed_launch(ctx, K_GAS_CORR, nc * gas_alg_bytes(gs, K_GAS_CORR, nact),
+                               [&] { return launch_gas_corrector(p, a, ctx->num_sms, s); })))
+            return st;
+    } else {
+        for (int d = 0; d < 3; ++d) {
+            if (gs.desc.n[d] <= 1) continue;
+            if ((st = timed_launch(ctx, K_GAS_PRED_FLUX, ext * gas_alg_bytes(gs, K_GAS_PRED_FLUX, nact),
+                                   [&] { return launch_gas_pred_flux(p, a, d, s); })))
+                return st;
+        }
+        if ((st = timed_launch(ctx, K_GAS_PRED_UPDATE, ext * gas_alg_bytes(gs, K_GAS_PRED_UPDATE, nact),
+                               [&] { return launch_gas_pred_update(p, a, s); })))
+            return st;
+        for (int d = 0; d < 3; ++d) {
+            if (gs.desc.n[d] <= 1) continue;
+            if ((st = timed_launch(ctx, K_GAS_CORR_FLUX, nc * gas_alg_bytes(gs, K_GAS_CORR_FLUX, nact),
+                                   [&] { return launch_gas_corr_flux(p, a, d, s); })))
+                return st;
+        }
+        if ((st = timed_launch(ctx, K_GAS_CORR_UPDATE, nc * gas_alg_bytes(gs, K_GAS_CORR_UPDATE, nact),
+                               [&] { return launch_gas_corr_update(p, a, s); })))
             return st;
     }
-    if ((st = timed_launch(ctx, K_GAS_PRED_UPDATE, ext * gas_alg_bytes(gs, K_GAS_PRED_UPDATE, nact),
-                           [&] { return launch_gas_pred_update(p, a, s); })))
-        return st;
-    for (int d = 0; d < 3; ++d) {
-        if (gs.desc.n[d] <= 1) continue;
-        if ((st = timed_launch(ctx, K_GAS_CORR_FLUX, nc * gas_alg_bytes(gs, K_GAS_CORR_FLUX, nact),
-                               [&] { return launch_gas_corr_flux(p, a, d, s); })))
-            return st;
-    }
-    if ((st = timed_launch(ctx, K_GAS_CORR_UPDATE, nc * gas_alg_bytes(gs, K_GAS_CORR_UPDATE, nact),
-                           [&] { return launch_gas_corr_update(p, a, s); })))
-        return st;
-    if ((st = gas_refresh_copies(ctx, gs))) return st;
+    gs.gas4_ok = a.gas4 != nullptr;
     gs.gas_pending = true;
     gs.gas_dt = dt_gas;
     return leave(ctx);
@@ -1821,7 +1827,7 @@ rhd_status rhd_gas_correct(rhd_ctx* ctx)
     if ((st = timed_launch(ctx, K_GAS_CORRECT, (double)gs.ncell * gas_alg_bytes(gs, K_GAS_CORRECT, 0),
                            [&] { return launch_gas_correct(p, a, ctx->stream); })))
         return st;
-    if ((st = gas_refresh_copies(ctx, gs))) return st;
+    gs.gas4_ok = a.gas4 != nullptr;
     gs.gas_pending = false;
     return leave(ctx);
 }

@@ -252,7 +252,6 @@ struct MomentsIn {
 };
 cudaError_t launch_moments_in(const MomentsIn& m, bool conserved, long long n, cudaStream_t s);
 cudaError_t launch_moments_out(const MomentsIn& m, long long n, cudaStream_t s);
-cudaError_t launch_to_float(float* dst, const double* src, long long n, cudaStream_t s);
 cudaError_t launch_reduce_state(const double* E, const double* G0, const double* G1, const double* G2,
                                 long long n, double* partials, int n_blocks, cudaStream_t s);
 cudaError_t launch_reduce_finish(const double* partials, int n_blocks, double* out5, cudaStream_t s);
