@@ -42,36 +42,76 @@ __device__ __forceinline__ void block_max(double v, double* out)
 }
 
 // v_max over the cells: |v| + sqrt((gamma P + (4/9) E (1 - exp(-k_F dx))) / rho) with P = rho T / (mu/k_B).
-// The FP64 value (the result) costs an exponential, two square roots and two divisions on the FP64
-// pipe; only the maximum matters, so each cell is first screened in FP32 (inputs truncated, relative
-// error about 1e-6) and evaluated in FP64 only if its FP32 value is not below the thread's running FP32
-// maximum by more than 2^-12, or is NaN or inf.  The cell holding the FP64 maximum always passes the
-// screen, so the result is the FP64 maximum itself; FP32 underflow or overflow only sends more cells
-// to the FP64 evaluation.
+// The FP64 value (the result) costs an exponential, two square roots and two divisions on the FP64 pipe, about
+// ten times what reading the cell takes; only the maximum matters, so few cells are evaluated in FP64: those
+// whose FP32 value cannot be told from the maximum.  The FP32 value has a relative error below 2^-20 (truncated
+// inputs and some ten roundings of 2^-24 under a square root); two values are told apart where they differ by
+// 2^-18.  Each thread keeps the inputs of its largest cell so far: a cell that is clearly below it or below the
+// block's maximum is passed over, one clearly above it takes its place, and one that cannot be told from it is
+// evaluated at once, unless its inputs are the same.  At the end the kept cell is evaluated if it cannot be told
+// from the block's maximum.  The cell with the FP64 maximum is never passed over, so the result is the FP64
+// maximum itself, whatever the timing.  NaN, infinities and values small enough to lose bits to FP32 underflow
+// are evaluated at once.
+struct SignalCell {
+    double r, T, E, v[3], k;
+};
+__device__ __forceinline__ double signal_speed(const GridParams& g, const SignalCell& s, double dx_min)
+{
+    const double P = s.r * s.T / g.mu_over_kB;
+    const double rad = (4.0 / 9.0) * s.E * (-expm1(-s.k * dx_min));
+    return sqrt(s.v[0] * s.v[0] + s.v[1] * s.v[1] + s.v[2] * s.v[2]) + sqrt((g.gamma * P + rad) / s.r);
+}
+__device__ __forceinline__ unsigned long long differs(double a, double b)
+{
+    return (unsigned long long)(__double_as_longlong(a) ^ __double_as_longlong(b));
+}
+
 __global__ void __launch_bounds__(RS_THREADS) signal_speed_kernel(GridParams g, const double* rho, const double* T,
                                                                   const double* E, const double* v0, const double* v1,
                                                                   const double* v2, const double* kF, double dx_min,
                                                                   long long n, double* partial)
 {
+    constexpr float kClear = 1.0f - 0x1p-18f;
+    __shared__ unsigned block_bits;  // the block's largest finite FP32 value so far (its bits: they order like it)
+    if (threadIdx.x == 0) block_bits = 0;
+    __syncthreads();
     const float gam = (float)g.gamma, inv_mu = (float)(1.0 / g.mu_over_kB), dxf = (float)dx_min;
     double m = 0.0;
-    float m32 = 0.0f;
-    for (long long i = (long long)blockIdx.x * RS_THREADS + threadIdx.x; i < n; i += (long long)gridDim.x * RS_THREADS) {
-        const double r = rho[i], Ti = T[i], Ei = E[i], kFi = kF ? kF[i] : 0.0;
-        const double a = v0 ? v0[i] : 0.0, b = v1 ? v1[i] : 0.0, c = v2 ? v2[i] : 0.0;
-        const float rf = d2f_trunc(r), af = d2f_trunc(a), bf = d2f_trunc(b), cf = d2f_trunc(c);
-        const float kf = kF ? d2f_trunc(kFi) : (g.kpow == 0 ? g.f_kappa_F : (g.kpow == 1 ? g.f_kappa_F * rf : (g.f_kappa_F * rf) * rf));
-        const float Pf = rf * d2f_trunc(Ti) * inv_mu;
-        const float radf = (4.0f / 9.0f) * d2f_trunc(Ei) * (-expm1f(-kf * dxf));
-        const float s32 = sqrtf(af * af + bf * bf + cf * cf) + sqrtf((gam * Pf + radf) / rf);
-        if (!(s32 < m32 * 0.999755859375f)) {
-            m32 = fmaxf(m32, s32);
-            const double k = kF ? kFi : flux_absorption(g, nullptr, rho, i);
-            const double P = r * Ti / g.mu_over_kB;
-            const double rad = (4.0 / 9.0) * Ei * (-expm1(-k * dx_min));
-            m = max_nan(m, sqrt(a * a + b * b + c * c) + sqrt((g.gamma * P + rad) / r));
+    float top = -1.0f;  // FP32 value of the kept cell; -1: none yet
+    SignalCell keep{};
+    const long long stride = (long long)gridDim.x * RS_THREADS;
+    for (long long i = (long long)blockIdx.x * RS_THREADS + threadIdx.x; i < n; i += stride) {
+        SignalCell c;
+        c.r = rho[i];
+        c.T = T[i];
+        c.E = E[i];
+        c.v[0] = v0 ? v0[i] : 0.0;
+        c.v[1] = v1 ? v1[i] : 0.0;
+        c.v[2] = v2 ? v2[i] : 0.0;
+        const float rf = d2f_trunc(c.r), af = d2f_trunc(c.v[0]), bf = d2f_trunc(c.v[1]), cf = d2f_trunc(c.v[2]);
+        c.k = kF ? kF[i] : 0.0;
+        const float kf = kF ? d2f_trunc(c.k) : (g.kpow == 0 ? g.f_kappa_F : (g.kpow == 1 ? g.f_kappa_F * rf : (g.f_kappa_F * rf) * rf));
+        const float Pf = rf * d2f_trunc(c.T) * inv_mu;
+        const float radf = (4.0f / 9.0f) * d2f_trunc(c.E) * (-expm1f(-kf * dxf));
+        const float q = gam * Pf + radf, s32 = sqrtf(af * af + bf * bf + cf * cf) + sqrtf(q / rf);
+        const float seen = __uint_as_float(*(volatile unsigned*)&block_bits);
+        if (s32 < seen * kClear && q > 1e-30f) continue;
+        const bool plain = s32 < 3e38f && s32 > 1e-15f && q > 1e-30f;
+        if (plain && s32 > seen) atomicMax(&block_bits, __float_as_uint(s32));
+        if (plain && s32 < top * kClear) continue;
+        if (!kF) c.k = flux_absorption(g, nullptr, rho, i);
+        if (plain && s32 * kClear > top) {
+            top = s32;
+            keep = c;
+            continue;
         }
+        if (plain && (differs(c.r, keep.r) | differs(c.T, keep.T) | differs(c.E, keep.E) | differs(c.v[0], keep.v[0]) |
+                      differs(c.v[1], keep.v[1]) | differs(c.v[2], keep.v[2]) | differs(c.k, keep.k)) == 0)
+            continue;
+        m = max_nan(m, signal_speed(g, c, dx_min));
     }
+    __syncthreads();
+    if (top >= 0.0f && !(top < __uint_as_float(block_bits) * kClear)) m = max_nan(m, signal_speed(g, keep, dx_min));
     block_max(m, partial);
 }
 
@@ -90,6 +130,7 @@ __global__ void __launch_bounds__(RS_THREADS) line_depth_kernel(GridParams g, co
         const long long nwarps = ((long long)gridDim.x * RS_THREADS) >> 5;
         for (long long l = warp0; l < lines; l += nwarps) {
             double s = 0.0;
+#pragma unroll 8
             for (long long x = lane; x < nx; x += 32) s += flux_absorption(g, kF, rho, l * nx + x);
             for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
             m = max_nan(m, s * dx);
@@ -102,6 +143,7 @@ __global__ void __launch_bounds__(RS_THREADS) line_depth_kernel(GridParams g, co
             const long long x = l % nx, o = l / nx;  // o: z (axis y) or y (axis z)
             long long i = axis == 1 ? x + nx * ny * o : x + nx * o;
             double s = 0.0;
+#pragma unroll 8
             for (long long k = 0; k < len; ++k, i += step) s += flux_absorption(g, kF, rho, i);
             m = max_nan(m, s * dx);
         }
