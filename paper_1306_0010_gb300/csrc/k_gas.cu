@@ -119,31 +119,56 @@ __device__ __forceinline__ void euler_flux(const Consts<R>& k, const Prim<R>& w,
     F[4] = (E + w.P) * u;
 }
 
+// HLL, where the contact speed's denominator is not negative (inlined: a call's stack and registers cost the
+// marching kernels 20 to 30 %, though it all but never runs)
 template <typename R, int D>
-__device__ void hllc(const Consts<R>& k, const Prim<R>& L, const Prim<R>& Rt, R F[5])
+__device__ __forceinline__ void hll_flux(const Consts<R>& k, const Prim<R>& L, const Prim<R>& Rt, R SL, R SR, R F[5])
+{
+    R FL[5], FR[5], EL, ER;
+    euler_flux<R, D>(k, L, FL, EL);
+    euler_flux<R, D>(k, Rt, FR, ER);
+    const R UL[5] = {L.r, L.r * L.v[0], L.r * L.v[1], L.r * L.v[2], EL};
+    const R UR[5] = {Rt.r, Rt.r * Rt.v[0], Rt.r * Rt.v[1], Rt.r * Rt.v[2], ER};
+    const R iw = rcp(SR - SL);
+    for (int q = 0; q < 5; ++q) F[q] = (SR * FL[q] - SL * FR[q] + SL * SR * (UR[q] - UL[q])) * iw;
+}
+
+// products and sums that the compiler does not contract any further
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+
+// The flux through a face between L and Rt.  Only one side's flux is needed wherever the contact speed exists: the
+// side is chosen first (supersonic: the upwind one; else the contact's), its flux formed, and the star state's jump
+// added.  The products that the jump is added to are rounded by themselves.
+template <typename R, int D>
+__device__ __forceinline__ void hllc(const Consts<R>& k, const Prim<R>& L, const Prim<R>& Rt, R F[5])
 {
     const R irL = rcp(L.r), irR = rcp(Rt.r);
     const R aL = sqrt_fast(k.gamma * L.P * irL), aR = sqrt_fast(k.gamma * Rt.P * irR);
     const R uL = L.v[D], uR = Rt.v[D];
     const R SL = fmin(uL - aL, uR - aR), SR = fmax(uL + aL, uR + aR);
-    R FL[5], FR[5], EL, ER;
-    if (SL >= R(0)) {
-        euler_flux<R, D>(k, L, F, EL);
-        return;
-    }
-    if (SR <= R(0)) {
-        euler_flux<R, D>(k, Rt, F, ER);
-        return;
-    }
-    euler_flux<R, D>(k, L, FL, EL);
-    euler_flux<R, D>(k, Rt, FR, ER);
     const R den = L.r * (SL - uL) - Rt.r * (SR - uR);
-    if (den < R(0)) {
-        const R Ss = (Rt.P - L.P + L.r * uL * (SL - uL) - Rt.r * uR * (SR - uR)) * rcp(den);
-        const bool left = Ss >= R(0);
-        const Prim<R>& K = left ? L : Rt;
-        const R S = left ? SL : SR, EK = left ? EL : ER, uK = K.v[D], irK = left ? irL : irR;
-        const R* FK = left ? FL : FR;
+    const bool supL = SL >= R(0), supR = SR <= R(0);
+    if (!(supL || supR || den < R(0))) {
+        hll_flux<R, D>(k, L, Rt, SL, SR, F);
+        return;
+    }
+    const R Ss = (Rt.P - L.P + L.r * uL * (SL - uL) - Rt.r * uR * (SR - uR)) * rcp(den);
+    const bool left = supL || (!supR && Ss >= R(0));
+    Prim<R> K;
+    K.r = left ? L.r : Rt.r;
+    for (int q = 0; q < 3; ++q) K.v[q] = left ? L.v[q] : Rt.v[q];
+    K.P = left ? L.P : Rt.P;
+    const R S = left ? SL : SR, irK = left ? irL : irR, uK = K.v[D];
+    R EK, M[3];
+    for (int q = 0; q < 3; ++q) M[q] = mul_rn(K.r, K.v[q]);
+    EK = K.P * k.inv_gm1 + R(0.5) * K.r * kin2(K);
+    F[0] = M[D];
+    for (int q = 0; q < 3; ++q) F[1 + q] = q == D ? fma_rn(M[q], uK, K.P) : mul_rn(M[q], uK);
+    F[4] = mul_rn(EK + K.P, uK);
+    if (!(supL || supR)) {
         const R chi = K.r * (S - uK) * rcp(S - Ss);
         R Us[5];
         Us[0] = chi;
@@ -151,12 +176,7 @@ __device__ void hllc(const Consts<R>& k, const Prim<R>& L, const Prim<R>& Rt, R 
         Us[1 + D] = chi * Ss;
         Us[4] = chi * (EK * irK + (Ss - uK) * (Ss + K.P * irK * rcp(S - uK)));
         const R UK[5] = {K.r, K.r * K.v[0], K.r * K.v[1], K.r * K.v[2], EK};
-        for (int q = 0; q < 5; ++q) F[q] = FK[q] + S * (Us[q] - UK[q]);
-    } else {
-        const R UL[5] = {L.r, L.r * L.v[0], L.r * L.v[1], L.r * L.v[2], EL};
-        const R UR[5] = {Rt.r, Rt.r * Rt.v[0], Rt.r * Rt.v[1], Rt.r * Rt.v[2], ER};
-        const R iw = rcp(SR - SL);
-        for (int q = 0; q < 5; ++q) F[q] = (SR * FL[q] - SL * FR[q] + SL * SR * (UR[q] - UL[q])) * iw;
+        for (int q = 0; q < 5; ++q) F[q] = F[q] + S * (Us[q] - UK[q]);
     }
 }
 
@@ -165,10 +185,9 @@ __device__ __forceinline__ R limited_slope(R dl, R dr, int lim)
 {
     if (lim == 2) return R(0.5) * (dl + dr);  // no limiter
     if (dl * dr <= R(0)) return R(0);
-    const R s = dl > R(0) ? R(1) : R(-1);
-    const R m = fmin(fabs(dl), fabs(dr));
-    if (lim == 0) return s * m;                          // minmod
-    return s * fmin(R(2) * m, R(0.5) * fabs(dl + dr));  // monotonized central
+    R m = fmin(fabs(dl), fabs(dr));                                   // minmod
+    if (lim != 0) m = fmin(R(2) * m, R(0.5) * fabs(dl + dr));  // monotonized central
+    return dl > R(0) ? m : -m;
 }
 
 __device__ __forceinline__ double absorption(const GasParams& p, const double* kF, long long i, double rho)
@@ -512,6 +531,16 @@ struct GasTile {
     }
 };
 
+// Resident CTAs asked of the compiler.  The fluxes' chains leave half of the issue slots empty at the two CTAs that
+// the unbounded kernels' registers allow; a few spilled values cost less.  256^3 and 300 x 250 x 200, us:
+// predictor (95 registers unbounded) 633 and 688 at two, 575 and 586 at three, 560 and 547 at four; corrector (113)
+// 955 and 1089 at two, 1013 and 1057 at three, 1211 and 1333 at four.
+template <typename R, int DIM>
+constexpr int gas_min_blocks(int n)
+{
+    return sizeof(R) == 4 && DIM > 1 ? n : 1;
+}
+
 // faces of one plane, for the cells below them
 template <typename R, int DIM, int TX, int TY>
 struct GasFaces {
@@ -532,7 +561,7 @@ __device__ __forceinline__ void tile_divergence(const GasParams& p, const GasFac
 }
 
 template <typename R, int DIM, int TX, int TY>
-__global__ void __launch_bounds__((GasTile<DIM, TX, TY>::NT)) gas_predictor_kernel(const __grid_constant__ GasParams p,
+__global__ void __launch_bounds__((GasTile<DIM, TX, TY>::NT), gas_min_blocks<R, DIM>(4)) gas_predictor_kernel(const __grid_constant__ GasParams p,
                                                                                  const __grid_constant__ GasArrays a,
                                                                                  const GasMarch t)
 {
@@ -630,8 +659,9 @@ __global__ void __launch_bounds__((GasTile<DIM, TX, TY>::NT)) gas_predictor_kern
     if (floors) atomicAdd(&a.counters[0], floors);
 }
 
-template <typename R, int DIM, int TX, int TY>
-__global__ void __launch_bounds__((GasTile<DIM, TX, TY>::NT)) gas_corrector_kernel(const __grid_constant__ GasParams p,
+// LIM: the limiter, -1: p.limiter
+template <typename R, int DIM, int TX, int TY, int LIM>
+__global__ void __launch_bounds__((GasTile<DIM, TX, TY>::NT), gas_min_blocks<R, DIM>(3)) gas_corrector_kernel(const __grid_constant__ GasParams p,
                                                                                  const __grid_constant__ GasArrays a,
                                                                                  const GasMarch t)
 {
@@ -645,6 +675,7 @@ __global__ void __launch_bounds__((GasTile<DIM, TX, TY>::NT)) gas_corrector_kern
     const bool fx = me.fx && p.n[0] > 1 && X <= p.n[0] && Y < p.n[1];
     const bool fy = me.fy && X < p.n[0] && Y <= p.n[1];
     const bool any = cell || fx || fy;
+    const int lim = LIM >= 0 ? LIM : p.limiter;
     const long long row = p.m[0], plane = row * p.m[1];
     // the thread's extended cell in plane z is own + plane * z
     const long long own = X + p.g[0] + row * (Y + p.g[1]) + plane * p.g[2];
@@ -671,9 +702,9 @@ __global__ void __launch_bounds__((GasTile<DIM, TX, TY>::NT)) gas_corrector_kern
         if (on) {
             if (fx) {
                 const GasHalf<R> a0 = load_half<R>(a, x - 2), a1 = load_half<R>(a, x - 1), a3 = load_half<R>(a, x + 1);
-                cell_slopes(a0.w, a1.w, w0.w, p.limiter, sl);
+                cell_slopes(a0.w, a1.w, w0.w, lim, sl);
                 const Prim<R> L = face_state(a1.w, sl, R(0.5));
-                cell_slopes(a1.w, w0.w, a3.w, p.limiter, sl);
+                cell_slopes(a1.w, w0.w, a3.w, lim, sl);
                 R F[5];
                 hllc<R, 0>(kc, L, face_state(w0.w, sl, R(-0.5)), F);
                 for (int q = 0; q < 5; ++q) f.x[q][me.ty][me.tx] = F[q];
@@ -682,9 +713,9 @@ __global__ void __launch_bounds__((GasTile<DIM, TX, TY>::NT)) gas_corrector_kern
                 if (fy) {
                     const GasHalf<R> a0 = load_half<R>(a, x - 2 * row), a1 = load_half<R>(a, x - row),
                                      a3 = load_half<R>(a, x + row);
-                    cell_slopes(a0.w, a1.w, w0.w, p.limiter, sl);
+                    cell_slopes(a0.w, a1.w, w0.w, lim, sl);
                     const Prim<R> L = face_state(a1.w, sl, R(0.5));
-                    cell_slopes(a1.w, w0.w, a3.w, p.limiter, sl);
+                    cell_slopes(a1.w, w0.w, a3.w, lim, sl);
                     R F[5];
                     hllc<R, 1>(kc, L, face_state(w0.w, sl, R(-0.5)), F);
                     for (int q = 0; q < 5; ++q) f.y[q][me.ty][me.tx] = F[q];
@@ -692,7 +723,7 @@ __global__ void __launch_bounds__((GasTile<DIM, TX, TY>::NT)) gas_corrector_kern
         }
         if constexpr (DIM > 2)
             if (cell) {
-                cell_slopes(w0.w, w1.w, w2.w, p.limiter, sl);
+                cell_slopes(w0.w, w1.w, w2.w, lim, sl);
                 if (z >= zc - 1) hllc<R, 2>(kc, up, face_state(w1.w, sl, R(-0.5)), zhi);
                 up = face_state(w1.w, sl, R(0.5));
             }
@@ -844,7 +875,11 @@ void launch_half(const GasParams& p, const GasArrays& a, bool predictor, int num
     const GasMarch t = march_of(predictor ? p.m : p.n, TX, TY, num_sms, &nb);
     constexpr int NT = GasTile<DIM, TX, TY>::NT;
     if (predictor) gas_predictor_kernel<R, DIM, TX, TY><<<(unsigned)nb, NT, 0, s>>>(p, a, t);
-    else gas_corrector_kernel<R, DIM, TX, TY><<<(unsigned)nb, NT, 0, s>>>(p, a, t);
+    else if (DIM == 3 && p.limiter == 0)
+        gas_corrector_kernel<R, DIM, TX, TY, DIM == 3 ? 0 : -1><<<(unsigned)nb, NT, 0, s>>>(p, a, t);
+    else if (DIM == 3 && p.limiter == 1)
+        gas_corrector_kernel<R, DIM, TX, TY, DIM == 3 ? 1 : -1><<<(unsigned)nb, NT, 0, s>>>(p, a, t);
+    else gas_corrector_kernel<R, DIM, TX, TY, -1><<<(unsigned)nb, NT, 0, s>>>(p, a, t);
 }
 
 template <typename R>
