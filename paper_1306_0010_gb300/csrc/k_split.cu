@@ -76,6 +76,10 @@ static bool common_predictor(const GridParams& g)
     return g.closure == 0 && g.speeds == 0 && g.theta_F == 1.0 && (g.exchange == EX_FULL || g.exchange == EX_EQUILIBRIUM);
 }
 static bool common_corrector(const GridParams& g) { return common_predictor(g) && g.theta_E == 1.0; }
+static bool theta_one(const GridParams& g)
+{
+    return g.closure == 0 && g.speeds == 0 && g.theta_F == 1.0 && g.theta_E == 1.0;
+}
 bool twopass_common(const GridParams& g) { return common_corrector(g); }
 
 // Two-pass split subcycle (3D): predictor over the grid and its stored ghost layers, then corrector.
@@ -94,6 +98,41 @@ cudaError_t launch_twopass_predictor(const StepParams& p, cudaStream_t s)
     if (e != cudaSuccess) return e;
     dim3 grid((unsigned)(pp.tiles_x * pp.tiles_y), (unsigned)((upad_extent(p.g, 2) + zc - 1) / zc));
     k<<<grid, TX * TY, smem, s>>>(pp);
+    return cudaGetLastError();
+}
+
+// The 2D pair (uhalf given): predictor over the grid and its stored ghost layers, then corrector
+cudaError_t launch_predictor2d(const StepParams& p, cudaStream_t s)
+{
+    StepParams pp = p;
+    pp.tiles_x = (upad_extent(p.g, 0) + S2_TX - 1) / S2_TX;
+    pp.tiles_y = (upad_extent(p.g, 1) + S2_TY - 1) / S2_TY;
+    auto k = common_predictor(p.g) ? predictor2d_kernel<true> : predictor2d_kernel<false>;
+    k<<<(unsigned)((long long)pp.tiles_x * pp.tiles_y), S2_NT, 0, s>>>(pp);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_corrector2d(const StepParams& p, cudaStream_t s)
+{
+    StepParams pc = p;
+    pc.tiles_x = (p.g.n[0] + S2_TX - 1) / S2_TX;
+    pc.tiles_y = (p.g.n[1] + S2_TY - 1) / S2_TY;
+    auto pick = [&](auto exk) {
+        constexpr int X = decltype(exk)::value;
+        return p.g.limiter == LIM_MC     ? corrector2d_kernel<LIM_MC, X>
+               : p.g.limiter == LIM_NONE ? corrector2d_kernel<LIM_NONE, X>
+                                         : corrector2d_kernel<LIM_MINMOD, X>;
+    };
+    auto k = !theta_one(p.g)                    ? corrector2d_kernel<-1, -1>
+             : p.g.exchange == EX_FULL        ? pick(std::integral_constant<int, EX_FULL>{})
+             : p.g.exchange == EX_EQUILIBRIUM ? pick(std::integral_constant<int, EX_EQUILIBRIUM>{})
+             : p.g.exchange == EX_ABSORB      ? pick(std::integral_constant<int, EX_ABSORB>{})
+             : p.g.exchange == EX_FROZEN_T    ? pick(std::integral_constant<int, EX_FROZEN_T>{})
+                                              : corrector2d_kernel<-1, -1>;
+    static SmemLimitOnce smem_once;
+    cudaError_t e = smem_once.set(k, corrector2d_smem());
+    if (e != cudaSuccess) return e;
+    k<<<(unsigned)((long long)pc.tiles_x * pc.tiles_y), S2_NT, corrector2d_smem(), s>>>(pc);
     return cudaGetLastError();
 }
 

@@ -83,6 +83,7 @@ struct GridState {
     bool um32_ok = false, gas4_ok = false;
     double* uhalf64 = nullptr;    // FP64 pair (2D, 3D): U^{m+1/2} with its ghost layers; NULL: the fused kernel
     Tile64 t64 = {};              // its work split for the current z chunk
+    float4* uhalf2d = nullptr;    // split 2D pair: U^{m+1/2} with its ghost layers; NULL: the fused kernel
     CUtensorMap uh_map;           // its tensor map (staging RHD_STAGING_TMA), valid when uh_map_ok
     bool uh_map_ok = false;
     const double* dir_dev = nullptr;  // low x Dirichlet state in device memory (rhd_marshak_advance only)
@@ -423,6 +424,7 @@ void free_grid(GridState& gs)
     dfree(gs.j32);
     dfree(gs.uhalf);
     dfree(gs.uhalf64);
+    dfree(gs.uhalf2d);
     dfree(gs.um32);
     dfree(gs.gas4);
     for (int q = 0; q < 5; ++q) dfree(gs.gas_wh[q]);
@@ -469,15 +471,18 @@ void free_twopass(GridState& gs)
     gs.um32_ok = gs.gas4_ok = false;
 }
 
-// FP64 grids of two or three dimensions: U^{m+1/2} of the kernel pair (32 bytes per stored cell).  A grid
-// that leaves no room for it runs the fused kernel, which needs none.
-void alloc_pair64(rhd_ctx* ctx, GridState& gs)
+// U^{m+1/2} of the kernel pair: FP64 grids of two or three dimensions (32 bytes per stored cell), split grids of
+// two (16 bytes).  A grid that leaves no room for it runs the fused kernel, which needs none.
+void alloc_pair(rhd_ctx* ctx, GridState& gs)
 {
-    if (gs.desc.precision != RHD_FP64 || gs.gp.nact < 2) return;
+    const bool split = gs.desc.precision == RHD_SPLIT;
+    if (split ? gs.gp.nact != 2 : gs.gp.nact < 2) return;
     size_t np = (size_t)upad_extent(gs.gp, 0) * upad_extent(gs.gp, 1);
     if (gs.gp.nact == 3) np *= (size_t)upad_extent(gs.gp, 2);
     const std::string err = ctx->err;
-    if (dalloc(ctx, (void**)&gs.uhalf64, 4 * sizeof(double) * np)) ctx->err = err;
+    if (split ? dalloc(ctx, (void**)&gs.uhalf2d, sizeof(float4) * np)
+              : dalloc(ctx, (void**)&gs.uhalf64, 4 * sizeof(double) * np))
+        ctx->err = err;
 }
 
 // The pair's work split: z_chunk planes per CTA, or its own choice (0), which then is the grid's z chunk
@@ -509,7 +514,7 @@ rhd_status alloc_grid(rhd_ctx* ctx, GridState& gs)
         gs.line = line_plan(gs.gp, gs.desc.precision == RHD_SPLIT, ctx->num_sms);
         if (gs.line.steps > 1 && (st = dalloc(ctx, (void**)&gs.T2, bytes))) return st;
     }
-    alloc_pair64(ctx, gs);
+    alloc_pair(ctx, gs);
     plan_pair64(ctx, gs, gs.desc.z_chunk);
     return RHD_OK;
 }
@@ -724,7 +729,7 @@ StepParams step_params(rhd_ctx* ctx, GridState& gs, int src, double chat, double
     p.dt = dt;
     p.f_chat = (float)chat;
     p.f_dt = (float)dt;
-    p.uhalf = gs.uhalf;
+    p.uhalf = gs.uhalf2d ? gs.uhalf2d : gs.uhalf;
     p.uhalf64 = gs.uhalf64;
     p.t64 = gs.t64;
     p.staging = gs.staging;
@@ -756,17 +761,19 @@ rhd_status check_dt(rhd_ctx* ctx, const GridState& gs, double chat, double dt)
 // kernels reported by the kernel timer
 enum KernelId {
     K_FUSED_FP64 = 0, K_FUSED_SPLIT, K_PREDICTOR, K_CORRECTOR, K_ENS_FP64, K_ENS_SPLIT, K_ENS_PRED, K_ENS_CORR,
-    K_GAS_PRED, K_GAS_CORR, K_GAS_PRED_FLUX, K_GAS_PRED_UPDATE, K_GAS_CORR_FLUX, K_GAS_CORR_UPDATE, K_GAS_CORRECT, K_GAS_EXCHANGE,
-    K_PRED64, K_CORR64, K_ENS_PRED64, K_ENS_CORR64,
+    K_GAS_PRED, K_GAS_CORR, K_GAS_PRED_FLUX, K_GAS_PRED_UPDATE, K_GAS_CORR_FLUX, K_GAS_CORR_UPDATE, K_GAS_CORRECT,
+    K_GAS_EXCHANGE,
+    K_PRED64, K_CORR64, K_ENS_PRED64, K_ENS_CORR64, K_PRED2D, K_CORR2D,
     K_COUNT
 };
 const char* const kKernelNames[K_COUNT] = {"subcycle_fused_fp64", "subcycle_fused_split", "twopass_predictor_split",
                                            "twopass_corrector_split", "ensemble_fp64", "ensemble_split",
                                            "ensemble_predictor_split", "ensemble_corrector_split",
-                                           "gas_predictor", "gas_corrector", "gas_predictor_flux", "gas_predictor_update", "gas_corrector_flux",
-                                           "gas_corrector_update", "gas_source_correction", "gas_step_exchange",
+                                           "gas_predictor", "gas_corrector", "gas_predictor_flux",
+                                           "gas_predictor_update", "gas_corrector_flux", "gas_corrector_update",
+                                           "gas_source_correction", "gas_step_exchange",
                                            "predictor_fp64", "corrector_fp64", "ensemble_predictor_fp64",
-                                           "ensemble_corrector_fp64"};
+                                           "ensemble_corrector_fp64", "predictor_split_2d", "corrector_split_2d"};
 
 // Algorithmic bytes per interior cell of one launch of kernel k: every array the kernel reads, read
 // once, and every array it writes, written once.  Fused kernels: U^m and U^{m+1} (4 FP64 each), the
@@ -788,6 +795,9 @@ double alg_bytes_per_cell(const GridState& gs, int k)
     // the FP64 pair: U^{m+1/2} in FP64 (32 B) written by the predictor and read by the corrector
     case K_PRED64: return 32.0 + gas + (ex == RHD_EX_FROZEN_T ? 8.0 : 0.0) + 32.0;
     case K_CORR64: return 32.0 + 32.0 + gas + Tr + 32.0 + Tw;
+    // the split 2D pair: U^{m+1/2} in FP32 (16 B)
+    case K_PRED2D: return 32.0 + gas + (ex == RHD_EX_FROZEN_T ? 8.0 : 0.0) + 16.0;
+    case K_CORR2D: return 16.0 + 32.0 + gas + Tr + 32.0 + Tw;
     default: return 32.0 + gas + Tr + 32.0 + Tw;
     }
 }
@@ -849,6 +859,13 @@ rhd_status launch_one(rhd_ctx* ctx, GridState& gs, int src, double chat, double 
         if (st) return st;
         return timed_launch(ctx, K_CORR64, nc * alg_bytes_per_cell(gs, K_CORR64),
                             [&] { return launch_corrector64(p, s); });
+    }
+    if (gs.uhalf2d) {
+        rhd_status st = timed_launch(ctx, K_PRED2D, nc * alg_bytes_per_cell(gs, K_PRED2D),
+                                     [&] { return launch_predictor2d(p, s); });
+        if (st) return st;
+        return timed_launch(ctx, K_CORR2D, nc * alg_bytes_per_cell(gs, K_CORR2D),
+                            [&] { return launch_corrector2d(p, s); });
     }
     if (gs.desc.precision != RHD_SPLIT)
         return timed_launch(ctx, K_FUSED_FP64, nc * alg_bytes_per_cell(gs, K_FUSED_FP64),

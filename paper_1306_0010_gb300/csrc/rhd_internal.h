@@ -198,6 +198,9 @@ cudaError_t launch_line_split(const LineParams& p, int tpc, cudaStream_t s);
 cudaError_t launch_twopass_split(const StepParams& p, cudaStream_t s);
 bool twopass_common(const GridParams& g);  // the modes the two-pass kernels have at compile time
 cudaError_t launch_twopass_predictor(const StepParams& p, cudaStream_t s);
+// split 2D grids with U^{m+1/2}: predictor, corrector
+cudaError_t launch_predictor2d(const StepParams& p, cudaStream_t s);
+cudaError_t launch_corrector2d(const StepParams& p, cudaStream_t s);
 cudaError_t launch_twopass_corrector(const StepParams& p, cudaStream_t s);
 bool tma_available();  // tensor-map staging of the two-pass corrector can be used on this device
 // FP32 mirror of the FP64 state (E, G): dst[i] = truncation toward zero of each component

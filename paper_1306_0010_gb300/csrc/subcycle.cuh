@@ -1601,6 +1601,7 @@ __device__ __forceinline__ void subcycle_tile(const GridParams& g, const GridArr
 #include "subcycle_fp64.cuh"
 #include "subcycle_pair.cuh"
 #include "subcycle_twopass.cuh"
+#include "subcycle_split2d.cuh"
 #include "subcycle_fp64_pair.cuh"
 
 namespace rhd {

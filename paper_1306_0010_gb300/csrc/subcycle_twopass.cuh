@@ -457,7 +457,14 @@ __device__ __forceinline__ void corrector_tile(const GridParams& g, const GridAr
     double* oD = reinterpret_cast<double*>(sm + G::END4) + t;                       // oD[q NT]: E, Gx, Gy, Gz, T
     float4* oG = reinterpret_cast<float4*>(reinterpret_cast<double*>(sm + G::END4) + G::OD * G::NT) + t;  // gas
     const float idx = g.f_inv_dx[0], idy = g.f_inv_dx[1], idz = g.f_inv_dx[2];
-    const SplitStiffConsts sk = split_stiff_consts(g, chat_d, dt_d);
+    // In shared memory, formed by one thread (some thirty FP64 operations): in registers they pushed others out
+    // (256^3, FULL: 851 -> 832 us; 97x61x45, whose CTAs take 5 planes: 38.9 -> 36.3).  EQUILIBRIUM uses few of them
+    // and has registers to spare (300x250x200: 603 us in registers, 634 in shared memory).
+    constexpr bool SKREG = EXK == EX_EQUILIBRIUM;
+    __shared__ SplitStiffConsts sk_shared;
+    SplitStiffConsts sk_own;
+    if constexpr (SKREG) sk_own = split_stiff_consts(g, chat_d, dt_d);
+    const SplitStiffConsts& sk = SKREG ? sk_own : sk_shared;
     // LIMK >= 0: the limiter is a compile-time constant (only its code is generated); -1: g.limiter
     constexpr bool COMMON = EXK >= 0;
     const int p1 = !COMMON && g.closure == 1, fixed = !COMMON && g.speeds == 1, lim = LIMK >= 0 ? LIMK : g.limiter;
@@ -587,6 +594,8 @@ __device__ __forceinline__ void corrector_tile(const GridParams& g, const GridAr
     issue_plane(next_plane, 0, z0);
     next_plane += pz;
     cp_async_commit();
+    // while the first plane is under way; read after the barrier that the plane waits at
+    if (!SKREG && t == 0) sk_shared = split_stiff_consts(g, chat_d, dt_d);
     bool timed_out = false;
     int fail_buf = 0;
     unsigned fail_ph = 0;
