@@ -65,7 +65,7 @@ def parse():
                     help="write profiles/traffic.json from this ncu raw CSV (measured at --N, scaled to 512^3; "
                          "--launch names the configuration) and exit")
     ap.add_argument("--fp64-ops-from", default=None,
-                    help="write profiles/fp64_ops.json (FP64 instructions per cell-update of the FP64 fused "
+                    help="write profiles/fp64_ops.json (FP64 instructions per cell-update of the FP64 "
                          "kernel) from this ncu raw CSV of one launch at --N and exit")
     ap.add_argument("--ens-n-sub", type=int, default=50, help="subcycles per step of the ensemble workload")
     return ap.parse_args()
@@ -209,6 +209,7 @@ def record_traffic(csv_path, measured_N, target_N, launch_spec):
     """Write profiles/traffic.json from an `ncu --page raw --csv` export: DRAM bytes per launch of each
     split kernel, scaled from measured_N^3 to target_N^3 cells (traffic grows with the cell count)."""
     import csv
+    import re
 
     names = {"predictor_kernel": "twopass_predictor_split", "corrector_kernel": "twopass_corrector_split"}
     rows = list(csv.reader(open(csv_path)))
@@ -221,8 +222,8 @@ def record_traffic(csv_path, measured_N, target_N, launch_spec):
     unit_mult = {"byte": 1, "Kbyte": 1e3, "Mbyte": 1e6, "Gbyte": 1e9, "Tbyte": 1e12}
     for r in rows[2:]:
         kname = r[hdr.index("Kernel Name")]
-        key = next((v for k, v in names.items() if k in kname), None)
-        if key is None:
+        key = next((v for k, v in names.items() if re.search(rf"(?<![A-Za-z0-9_]){k}", kname)), None)
+        if key is None or key in out:
             continue
         b = 0.0
         for m in ("dram__bytes_read.sum", "dram__bytes_write.sum"):
@@ -237,27 +238,29 @@ def record_traffic(csv_path, measured_N, target_N, launch_spec):
     print(json.dumps(out, indent=1))
 
 
-# the sources the FP64 fused kernel is compiled from
+# the sources the FP64 kernel pair is compiled from
 FP64_KERNEL_SOURCES = ("dfloat.cuh", "fp_convert.cuh", "k_fp64.cu", "rhd_internal.h", "subcycle.cuh",
-                       "subcycle_pair.cuh", "subcycle_twopass.cuh")
+                       "subcycle_fp64.cuh", "subcycle_fp64_pair.cuh")
 # FP64 issue peak from unit counts and the maximum SM clock: 152 SMs x 2 FP64 operations per cycle (the
 # ncu peak of sm__sass_thread_inst_executed_op_dfma_pred_on is 304 per cycle) x 2.07 GHz
 FP64_PEAK_TOPS = 152 * 2 * 2.07e9 / 1e12
 
 
 def record_fp64_ops(csv_path, N):
-    """Write profiles/fp64_ops.json from an `ncu --page raw --csv` export of one FP64 fused-kernel launch
-    over N^3 cells: thread-level dadd + dfma + dmul instructions per cell-update."""
+    """Write profiles/fp64_ops.json from an `ncu --page raw --csv` export of one launch of each kernel of the FP64
+    pair over N^3 cells: thread-level dadd + dfma + dmul instructions per cell-update."""
     import csv
 
     rows = list(csv.reader(open(csv_path)))
     first = next(i for i, r in enumerate(rows) if "Kernel Name" in r)
     hdr, rows = rows[first], rows[first + 2:]
-    r = next(r for r in rows if "subcycle_kernel<double" in r[hdr.index("Kernel Name")])
-    ops = {}
-    for op in ("dadd", "dfma", "dmul"):
-        ops[op] = float(r[hdr.index(f"smsp__sass_thread_inst_executed_op_{op}_pred_on.sum")].replace(",", "")) / N ** 3
-    out = {"note": f"FP64 thread instructions per cell-update of the FP64 fused kernel, ncu at {N}^3 (one launch)",
+    ops = {"dadd": 0.0, "dfma": 0.0, "dmul": 0.0}
+    for kernel in ("predictor64_kernel", "corrector64_kernel"):
+        r = next(r for r in rows if kernel in r[hdr.index("Kernel Name")])
+        for op in ops:
+            name = f"smsp__sass_thread_inst_executed_op_{op}_pred_on.sum"
+            ops[op] += float(r[hdr.index(name)].replace(",", "")) / N ** 3
+    out = {"note": f"FP64 thread instructions per cell-update of the FP64 kernel pair, ncu at {N}^3 (one launch each)",
            "source_sha256": kernel_source_hash(FP64_KERNEL_SOURCES), "N": N, "per_cell_update": ops,
            "fp64_ops_per_cell_update": sum(ops.values())}
     with open(os.path.join(ROOT, "profiles", "fp64_ops.json"), "w") as f:
@@ -267,8 +270,8 @@ def record_fp64_ops(csv_path, N):
 
 
 def fp64_pipe_roofline(rate):
-    """The FP64 path against the FP64 issue peak: its kernel's FP64 instructions per cell-update (ncu,
-    profiles/fp64_ops.json, dropped when the kernel's sources have changed since) times the rate."""
+    """The FP64 path against the FP64 issue peak: its kernels' FP64 instructions per cell-update (ncu,
+    profiles/fp64_ops.json, dropped when the kernels' sources have changed since) times the rate."""
     path = os.path.join(ROOT, "profiles", "fp64_ops.json")
     if not os.path.exists(path):
         return None
@@ -789,7 +792,8 @@ def run_marshak(args):
             if N * n_sub <= args.marshak_cpu_cells:
                 row["cpu_s"] = marshak_oracle_seconds(case, n_sub)
             table.append(row)
-    # the kernels' own time per subcycle (events around each launch), against the wall clock per subcycle
+    # the kernels' own time per subcycle (events around each launch, which may take several), against the wall
+    # clock per subcycle
     kernel_us = {}
     for precision in ("fp64", "split"):
         case = wl.marshak_case(max(Ns), precision=precision)
@@ -801,7 +805,7 @@ def run_marshak(args):
         g.synchronize()
         kt = g.kernel_times()
         g.close()
-        kernel_us[precision] = {k: 1e3 * v["total_ms"] / v["launches"] for k, v in kt.items()}
+        kernel_us[precision] = {k: 1e3 * v["total_ms"] / n_sub for k, v in kt.items()}
     big = table[-1]
     line = {"metric": "non-equilibrium Marshak wave (Section 4.1.4): wall-clock time to reach tau", "value": big["gpu_s"],
             "unit": "s", "higher_is_better": False, "n_gpus": 1, "dtype": "f64", "data": "synthetic",

@@ -137,7 +137,7 @@ typedef struct {
     int speeds;                 /* rhd_speeds */
     int precision;              /* rhd_precision */
     int flags;                  /* RHD_FLAG_* bits */
-    int z_chunk;                /* z planes per CTA of the fused kernel; 0 chooses automatically */
+    int z_chunk;                /* z planes per CTA; 0 chooses automatically */
     double kappa_P, kappa_F;    /* opacity law used where kP / kF arrays are not given: */
     int kappa_rho_pow;          /*   k = kappa * rho^p, p in {0, 1, 2} (absorption coefficients) */
     void* cuda_stream;          /* cudaStream_t to run on (NULL: legacy default stream, see above) */
@@ -194,8 +194,8 @@ rhd_status rhd_set_dirichlet(rhd_ctx* ctx, int face, const double state[4]);
 
 /* Run n_sub >= 0 radiation subcycles of length dt with reduced speed of light chat (Section 3.1 steps
  * 4-5).  Requires chat <= c and dt <= cfl * min(dx) / chat (RHD_ERR_CFL otherwise).  The loop is
- * replayed from a cached CUDA graph of n_sub kernel launches on the context stream; the call returns
- * without synchronising.  Errors: RHD_ERR_ARG, RHD_ERR_STATE (moments or gas not set), RHD_ERR_CFL,
+ * replayed from a cached CUDA graph of its kernel launches on the context stream (a few launches are
+ * issued directly; 1D grids take several subcycles per launch); the call returns without synchronising.  Errors: RHD_ERR_ARG, RHD_ERR_STATE (moments or gas not set), RHD_ERR_CFL,
  * RHD_ERR_CUDA. */
 rhd_status rhd_radiation_subcycle(rhd_ctx* ctx, int n_sub, double chat, double dt);
 
@@ -216,9 +216,9 @@ rhd_status rhd_radiation_subcycle(rhd_ctx* ctx, int n_sub, double chat, double d
  * RHD_SPLIT grids compute the face fluxes (reconstruction, wave speeds, HLLC), their differences, the
  * sources, the half step and the increments of (rho, v, T) in FP32 and add the increments to the FP64
  * state in FP64 (rhd_gas_correct likewise).  Does not synchronise.  Scratch, allocated by the first
- * call, for n cells and m = (n0+4)(n1+4)(n2+4) (2D / 1D: no padding in inactive directions): 8 n
- * doubles; 5 m doubles and 15 m face doubles (FP64 grids) or 5 m floats and 15 m face floats
- * (RHD_SPLIT grids).  Single grids only.  Errors: RHD_ERR_ARG (dt_gas), RHD_ERR_STATE
+ * call, for n cells and m = (n0+4)(n1+4)(n2+4) (2D / 1D: no padding in inactive directions): 5 m floats
+ * and 4 n floats (RHD_SPLIT grids); 5 m and 8 n doubles, and in 2D and 3D 5 face doubles per active
+ * direction (FP64 grids).  Single grids only.  Errors: RHD_ERR_ARG (dt_gas), RHD_ERR_STATE
  * (ensemble, gas or moments not set), RHD_ERR_OOM, RHD_ERR_CUDA. */
 rhd_status rhd_gas_step(rhd_ctx* ctx, double dt_gas);
 
@@ -300,7 +300,9 @@ rhd_status rhd_ensemble_subcycle(rhd_ctx* ctx, int n_sub, double chat, const dou
  * pick how the subcycle kernels are laid out on the GPU, never what they compute: every candidate
  * gives results within the error bound of its precision.
  *   variant   RHD_VARIANT_FUSED: one kernel per subcycle; the predictor (U^{m+1/2}) is recomputed
- *             on the 2-cell halo of each x-y tile.  RHD_VARIANT_TWOPASS (RHD_SPLIT, 3D grids only):
+ *             on the 2-cell halo of each x-y tile.  FP64 grids of 2 and 3 dimensions and RHD_SPLIT grids of
+ *             2 run a predictor and a corrector under this name where the device has room for U^{m+1/2}
+ *             (32 and 16 bytes per cell, layers as below), and choose their tiles.  RHD_VARIANT_TWOPASS (RHD_SPLIT, 3D grids only):
  *             a predictor kernel writes U^{m+1/2} (FP32) for the grid plus 2 ghost layers per face
  *             in each direction that is not periodic on both faces, then a corrector kernel reads
  *             it back; extra device memory (n0+p0)(n1+p1)(n2+p2) x 16 bytes, p = 0 for a direction
@@ -453,7 +455,7 @@ rhd_status rhd_marshak_boundary(double tau, double eps, double F_inc, double c, 
 /* n_sub subcycles of the Marshak wave from time t0, the low x face's Dirichlet state of subcycle m
  * computed on the device by the same quadrature as rhd_marshak_boundary at tau = tau_rate (t0 + (m + 1/2) dt)
  * (the subcycle's midpoint; tau_rate = eps c rho kappa_0): one launch computes all n_sub states (one block
- * each, kept in a context buffer of 32 n_sub bytes), then one plain launch per subcycle reads its own.  Needs a single-grid context with
+ * each, kept in a context buffer of 32 n_sub bytes), then plain launches of the subcycles read theirs.  Needs a single-grid context with
  * a Dirichlet low x face, state set, and the fused kernels (FP64, or split with RHD_FLAG_SPLIT_FUSED or
  * fewer than 3 dimensions).  Returns without synchronising.  Errors: RHD_ERR_ARG, RHD_ERR_CFL,
  * RHD_ERR_STATE, RHD_ERR_UNSUPPORTED (two-pass split grid), RHD_ERR_OOM, RHD_ERR_CUDA. */
