@@ -26,8 +26,8 @@ cudaError_t launch_scale_copy(double* dst, const double* src, double scale, long
     return cudaGetLastError();
 }
 
-// x / c, c > 0, for y = 1/c correctly rounded (0: always divide): one multiplication and one correction by the exact residual (the
-// correctly rounded quotient, by Markstein's theorem, where nothing under- or overflows: three FP64
+// x / c, c > 0, for y = 1/c correctly rounded (0: always divide): one multiplication and one correction by the
+// exact residual (the correctly rounded quotient, by Markstein's theorem, where nothing under- or overflows: three FP64
 // instructions against CUDA's ten or so), the division itself elsewhere
 static __device__ __noinline__ double div_slow(double x, double c) { return x / c; }
 __device__ __forceinline__ double div_by(double x, double c, double y)
@@ -44,9 +44,9 @@ __device__ __forceinline__ double div_by(double x, double c, double y)
 
 // What a caller hands over and takes back, each in one pass over memory: every array read once, and every
 // copy the kernels use (FP64, FP32, the two-pass path's interleaved forms) written once.  Bound by memory; at
-// 512^3 on a split grid (device arrays, velocity, no optional arrays) the state in takes 2.1 + 2.1 ms and the
-// moments out 1.4 ms, 5.9 with T, against 12.2 ms for the copies, conversions and interleavings as launches of their own,
-// whose F / c, 134 million FP64 divisions a component, was bound by the FP64 pipe.
+// 512^3 on a split grid (device arrays, velocity, no optional arrays) the state in and the moments and T out take 6.4
+// ms, against 12.2 ms for the copies, conversions and interleavings as launches of their own, whose F / c, 134
+// million FP64 divisions a component, was bound by the FP64 pipe.
 // V = 2: two cells per thread by 16-byte accesses (arrays 16-byte aligned); 1: one.
 template <int V>
 struct Cells;

@@ -151,8 +151,8 @@ double plane_cost(const PairCost& c, bool predictor, int w, int h)
 
 // Tile shape and planes per CTA for an ex x ey x ez range: the fewest FP64 instructions on the busiest SM.
 // An SM's time is the sum over its CTAs (the pipe is shared), with a tenth more where it has only one to
-// fill the gaps between its phases.  128^3: 16 x 16 x 19 (448 CTAs, three per SM), 3.05 ms a subcycle
-// for both kernels against 3.6 ms with 32 planes per CTA (256 CTAs: one SM in three has half the work).
+// fill the gaps between its phases.  128^3: 16 x 16 x 19 (448 CTAs, three per SM; with 32 planes per CTA one
+// SM in three would have half the work), 1157 + 2292 us a subcycle, 4960 for the fused kernel.
 void best_split(const PairCost& c, bool predictor, int ex, int ey, int ez, int n_sms, int z_fixed, bool shared,
                 int* bw, int* bh, int* bz)
 {

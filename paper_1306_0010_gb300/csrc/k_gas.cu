@@ -437,8 +437,9 @@ __global__ void __launch_bounds__(GAS_THREADS) gas_corr_update_kernel(GasParams 
 // Nothing but the half step's result goes through memory: a launch for each direction that stored its faces' five
 // components, and an update that read them back, moved 20 B a cell and direction there and again 20 B back.
 // Same arithmetic, operation for operation.  Bound by instruction issue (HLLC and the limiter; the launches per
-// direction were bound by memory): the step and its correction with the copies the subcycles read, 256^3 split,
-// 3.5 -> 2.5 ms; 300 x 250 x 200 3.2 -> 2.6 ms; FP64, 512 cells, 64 -> 38 us.
+// direction were bound by memory).  256^3, us: five launches of fluxes and updates a half 1176 and 1467, marched 554
+// and 1004; the step and its correction, 300 x 250 x 200: 2.8 ms, and the copies by five launches, -> 2.1 with the copies;
+// FP64, 512 cells: 54 -> 28 us.
 
 // the FP32 radiation state of interior cell i: the two-pass subcycles' mirror where it is current
 __device__ __forceinline__ float4 load_rad32(const GasArrays& a, long long i)

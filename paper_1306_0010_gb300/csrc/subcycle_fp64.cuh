@@ -9,8 +9,8 @@
 //   - fluxes and wave speeds are kept per unit chat, and chat dt / dx is one factor per direction, applied
 //     with the flux difference as one fused multiply-add on the state;
 //   - the closure works on f = G/E (each component once), and the HLL flux on three weights.
-// At 128^3 (the throughput state) the FP64 additions, multiplications and fused multiply-adds fell from
-// 1537 per cell-update (and some 250 comparisons) to 794.
+// At 128^3 (the throughput state) the FP64 additions, multiplications and fused multiply-adds of the fused kernel
+// fell from 1537 per cell-update (and some 250 comparisons) to 882; the pair of kernels takes 750.
 #pragma once
 
 namespace rhd {

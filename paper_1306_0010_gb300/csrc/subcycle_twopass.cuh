@@ -439,7 +439,8 @@ struct GeoCorr {
 // of each U^{m+1/2} plane arrives by one tensor copy (issued by thread 0, completed on mbar[buf]; map
 // and mbar are then required, and sm must be 128-byte aligned); otherwise by per-thread cp.async.  EXK >= 0: a common
 // grid (M1 closure and speeds, theta_F = theta_E = 1) with that exchange mode, FULL or EQUILIBRIUM, at compile
-// time; -1: any mode (256^3, FULL: 922 us general; common 851 with the branch-free HLL and the integer split).
+// time; -1: any mode (256^3, FULL: 922 us general; common 851 with the branch-free HLL and the integer split, 832 with the
+// stiff sources' constants in shared memory).
 template <int TX, int TY, bool TMA, int LIMK, int EXK>
 __device__ __forceinline__ void corrector_tile(const GridParams& g, const GridArrays& a, const float4* uh,
                                                float chat, float dt, double chat_d, double dt_d, int x0, int y0,
