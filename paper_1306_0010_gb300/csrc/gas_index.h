@@ -1,7 +1,8 @@
 // gas_index.h -- index arithmetic of the gas-step kernels (k_gas.cu): the ghost rule, the layouts of
-// the extended grid and of the face-flux arrays.  Host-and-device code: the kernels compute every
-// array index through these functions, and a host test enumerates them over whole grids to check that
-// every index stays inside its array.
+// the extended grid and of the face-flux arrays.  Host-and-device code: the kernels of a launch per direction
+// compute every array index through these functions, and a host test enumerates them over whole grids to check
+// that every index stays inside its array.  The marching kernels take the ghost rule from here and step by
+// whole rows and planes of the two layouts; each access lies within the ghost layers (k_gas.cu).
 #pragma once
 
 #include "gas_internal.h"
