@@ -154,9 +154,13 @@ cudaError_t launch_twopass_corrector(const StepParams& p, cudaStream_t s)
     };
     using Any = std::integral_constant<int, -1>;
     auto k = p.staging == 1              ? pick(std::true_type{}, Any{})
-             : !common_corrector(p.g)    ? pick(std::false_type{}, Any{})
+             : !theta_one(p.g)           ? pick(std::false_type{}, Any{})
              : p.g.exchange == EX_FULL   ? pick(std::false_type{}, std::integral_constant<int, EX_FULL>{})
-                                         : pick(std::false_type{}, std::integral_constant<int, EX_EQUILIBRIUM>{});
+             : p.g.exchange == EX_ABSORB ? pick(std::false_type{}, std::integral_constant<int, EX_ABSORB>{})
+             : p.g.exchange == EX_FROZEN_T ? pick(std::false_type{}, std::integral_constant<int, EX_FROZEN_T>{})
+             : p.g.exchange == EX_EQUILIBRIUM
+                 ? pick(std::false_type{}, std::integral_constant<int, EX_EQUILIBRIUM>{})
+                 : pick(std::false_type{}, Any{});
     const size_t smem = GeoCorr<TX, TY>::bytes() + 128;  // + alignment slack for TMA destinations
     static SmemLimitOnce smem_once;
     cudaError_t e = smem_once.set(k, smem);

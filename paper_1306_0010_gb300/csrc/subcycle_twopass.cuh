@@ -438,9 +438,9 @@ struct GeoCorr {
 // Corrector over the interior column tile (x0, y0) for planes [z0, z1).  TMA: the tile + 2-cell halo
 // of each U^{m+1/2} plane arrives by one tensor copy (issued by thread 0, completed on mbar[buf]; map
 // and mbar are then required, and sm must be 128-byte aligned); otherwise by per-thread cp.async.  EXK >= 0: a common
-// grid (M1 closure and speeds, theta_F = theta_E = 1) with that exchange mode, FULL or EQUILIBRIUM, at compile
-// time; -1: any mode (256^3, FULL: 922 us general; common 851 with the branch-free HLL and the integer split, 832 with the
-// stiff sources' constants in shared memory).
+// grid (M1 closure and speeds, theta_F = theta_E = 1) with that exchange mode (not LINEAR) at compile time; -1: any
+// mode (256^3, ABSORB: 691 us general, 655 common; FROZEN_T: 766, 734; FULL: 922 us general; common 851 with the
+// branch-free HLL and the integer split, 832 with the stiff sources' constants in shared memory).
 template <int TX, int TY, bool TMA, int LIMK, int EXK>
 __device__ __forceinline__ void corrector_tile(const GridParams& g, const GridArrays& a, const float4* uh,
                                                float chat, float dt, double chat_d, double dt_d, int x0, int y0,

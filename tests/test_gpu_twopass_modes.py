@@ -1,6 +1,7 @@
-"""GPU: the two-pass split kernels' compile-time modes (M1 closure and speeds, theta = 1, FULL or EQUILIBRIUM) against
-their general instantiations, to the bit.  The general corrector runs with TMA staging; the general predictor and
-corrector run with ABSORB at k_P = 0, which is EQUILIBRIUM (its factor of E is exactly 1).  Grids: one tile and less,
+"""GPU: the two-pass split kernels' compile-time modes (M1 closure and speeds, theta = 1; predictor: FULL and
+EQUILIBRIUM; corrector: ABSORB and FROZEN_T too) against their general instantiations, to the bit.  The general
+corrector runs with TMA staging; the general predictor with ABSORB at k_P = 0, which is EQUILIBRIUM (its factor of E is
+exactly 1).  Grids: one tile and less,
 ragged tiles, every boundary rule, one plane more than a chunk; optional arrays on and off."""
 import numpy as np
 import pytest
@@ -41,7 +42,7 @@ def run(rhd, case, staging="cpasync", **kw):
 
 
 @pytest.mark.parametrize("limiter", ["minmod", "mc", "none"])
-@pytest.mark.parametrize("exchange", ["full", "equilibrium"])
+@pytest.mark.parametrize("exchange", ["full", "equilibrium", "absorb", "frozen_t"])
 @pytest.mark.parametrize("i", range(len(GRIDS)))
 def test_common_modes_are_the_general_ones(rhd, i, exchange, limiter):
     n, bc = GRIDS[i]
