@@ -506,7 +506,7 @@ __device__ __forceinline__ float exchange_delta_fp32(const GridParams& g, float 
                                                      float E, float T, ExchangeOut& o, float& qout);
 
 // The solve from delta = d0 with clamped FP64 Newton steps and the bisection fallback: the cells that the
-// two steps of exchange_fp64 do not settle (a seed outside the FP32 range).
+// two steps of exchange64 do not settle, or whose energy densities are outside the range of its test.
 struct ExchangeGeneral {
     double d;
     int newton_fb, iters;
@@ -560,7 +560,9 @@ static __device__ __noinline__ ExchangeGeneral exchange_general(double A, double
 // multiplies the error by the relative error of 1/g' (2^-22 and the seed's own) and squares what is left,
 // so the second step is about 2^-47 of x and the result is at the rounding level of g, where the clamped
 // iteration ends as well.  A second step above 2^-36 of x, or anything not finite, sends the cell to
-// exchange_general.  About 30 FP64 instructions with theta = 1, against about 110 when the bracket of the
+// exchange_general.  So does an x outside [1e-26, 1e26], where the test and g' would lose their FP32 operands:
+// below it 2^-36 x is no normal FP32 number (an unconverged step would read as 0 and pass), above it A x^2 may
+// flush to 0 while 4 A x^3 still counts beside B >= 1 (at x <= 1e26 what flushes is below 2^-35 of B).  About 30 FP64 instructions with theta = 1, against about 110 when the bracket of the
 // general solve was set up in every cell and each Newton step took its own FP64 reciprocal.
 __device__ __forceinline__ ExchangeOut exchange64(const GridParams& g, double chat, double dt, double rho,
                                                      double kP, double& E, double& T)
@@ -600,7 +602,9 @@ __device__ __forceinline__ ExchangeOut exchange64(const GridParams& g, double ch
     const double x2 = e + d, y2 = x2 * x2;
     const double gv = fma(A * y2, y2, fma(B, d, C));
     const float s2 = d2f_trunc(gv) * d2f_trunc(ig);
-    if (fabsf(s2) <= 1.4551915228366852e-11f * x32 && gp < 1e37f && !o32.newton_fb && o32.theta_fb == o.theta_fb) {
+    const bool in_range = x32 >= 1e-26f && x32 <= 1e26f;
+    if (in_range && fabsf(s2) <= 1.4551915228366852e-11f * x32 && gp < 1e37f && !o32.newton_fb &&
+        o32.theta_fb == o.theta_fb) {
         d = fma(-gv, ig, d);
     } else {
         double c0;
