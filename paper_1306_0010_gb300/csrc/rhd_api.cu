@@ -404,6 +404,14 @@ void dfree(T*& p)
     p = nullptr;
 }
 
+// ... and the context's account of its `bytes` credited, for memory that makes room for another array
+template <typename T>
+void dfree(rhd_ctx* ctx, T*& p, size_t bytes)
+{
+    if (p) ctx->mem_used -= bytes;
+    dfree(p);
+}
+
 void free_grid(GridState& gs)
 {
     for (int b = 0; b < 2; ++b)
@@ -591,19 +599,65 @@ rhd_status set_gas(rhd_ctx* ctx, GridState& gs, const double* rho, const double*
     };
     const std::vector<const void*> before = layout();
     const size_t bytes = sizeof(double) * (size_t)gs.ncell;
+    // every array that is missing, before anything of the old state is touched: a call that finds no room leaves
+    // the grid as it was
+    double* add[8] = {nullptr};
+    float* add32[8] = {nullptr};
+    auto allocate = [&]() -> rhd_status {
+        for (int k = 0; k < 8; ++k) {
+            if (!src[k]) continue;
+            rhd_status e;
+            if (!*buf[k] && !add[k] && (e = dalloc(ctx, (void**)&add[k], bytes))) return e;
+            if (split && buf32[k] && !*buf32[k] && !add32[k] && (e = dalloc(ctx, (void**)&add32[k], bytes / 2))) return e;
+        }
+        return RHD_OK;
+    };
+    // velocity components that are not given are zero and kept as absent
+    auto drop = [&] {
+        bool any = false;
+        for (int k = 2; k <= 4; ++k) {
+            if (src[k]) continue;
+            any = any || *buf[k] || *buf32[k];
+            dfree(ctx, *buf[k], bytes);
+            dfree(ctx, *buf32[k], bytes / 2);
+        }
+        return any;
+    };
+    st = allocate();
+    if (st == RHD_ERR_OOM) {
+        // the room of the components this call drops, whose state then is gone even if that does not suffice
+        RHD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+        if (drop()) {
+            clear_graphs(ctx);
+            gs.has_v = gs.v[0] || gs.v[1] || gs.v[2];
+            gs.has_gas = gs.gas4_ok = gs.gas_pending = false;
+            st = allocate();
+        }
+    }
+    if (st) {
+        for (int k = 0; k < 8; ++k) {
+            dfree(ctx, add[k], bytes);
+            dfree(ctx, add32[k], bytes / 2);
+        }
+        return st;
+    }
+    for (int k = 0; k < 8; ++k) {
+        if (add[k]) *buf[k] = add[k];
+        if (add32[k]) *buf32[k] = add32[k];
+    }
+    drop();
+    gs.has_v = vx || vy || vz;
+    gs.has_kP = kP != nullptr;
+    gs.has_kF = kF != nullptr;
+    gs.has_j = j != nullptr;
+    gs.has_gas = true;
+    gs.gas4_ok = false;
+    gs.gas_pending = false;  // a pending source correction belongs to the replaced state
+    if (layout() != before) clear_graphs(ctx);  // the kernels' array pointers changed
     GasIn in;
     std::memset(&in, 0, sizeof(in));
     for (int k = 0; k < 8; ++k) {
-        if (!src[k]) {
-            // velocity components that were not given are zero: keep them as absent
-            if (k >= 2 && k <= 4) {
-                dfree(*buf[k]);
-                dfree(*buf32[k]);
-            }
-            continue;
-        }
-        if (!*buf[k] && (st = dalloc(ctx, (void**)buf[k], bytes))) return st;
-        if (split && buf32[k] && !*buf32[k] && (st = dalloc(ctx, (void**)buf32[k], bytes / 2))) return st;
+        if (!src[k]) continue;
         // host arrays land in the library's own first; the conversions then run in place
         if (!on_device && (st = put(ctx, *buf[k], src[k], gs.ncell, 0))) return st;
         in.src[k] = on_device ? src[k] : *buf[k];
@@ -613,14 +667,7 @@ rhd_status set_gas(rhd_ctx* ctx, GridState& gs, const double* rho, const double*
     const bool twopass = gs.variant == RHD_VARIANT_TWOPASS && gs.gas4;
     in.gas4 = twopass ? gs.gas4 : nullptr;
     if (on_device || split) RHD_CUDA(ctx, launch_gas_in(in, gs.ncell, ctx->stream));
-    gs.has_v = vx || vy || vz;
-    gs.has_kP = kP != nullptr;
-    gs.has_kF = kF != nullptr;
-    gs.has_j = j != nullptr;
-    gs.has_gas = true;
     gs.gas4_ok = twopass;
-    gs.gas_pending = false;  // a pending source correction belongs to the replaced state
-    if (layout() != before) clear_graphs(ctx);  // the kernels' array pointers changed
     return leave(ctx);
 }
 
