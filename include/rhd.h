@@ -66,8 +66,8 @@ typedef enum {
 /* Environment (read by the library, none required):
  *   RHD_LOG=1                   print every error status and its message to stderr; 2: also the launch
  *                               configurations the autotuner chooses
- *   RHD_DEVICE_MEMORY_LIMIT=B   cap (bytes) on the cumulative device allocations of each context created
- *                               afterwards; allocations beyond it return RHD_ERR_OOM (a test hook for the
+ *   RHD_DEVICE_MEMORY_LIMIT=B   cap (bytes) on the device memory that each context created afterwards
+ *                               holds; allocations beyond it return RHD_ERR_OOM (a test hook for the
  *                               out-of-memory paths)
  * Every API call is also marked as an NVTX range of the same name for Nsight tools. */
 typedef enum { RHD_BC_PERIODIC = 0, RHD_BC_OUTFLOW = 1, RHD_BC_REFLECT = 2, RHD_BC_DIRICHLET = 3 } rhd_bc;

@@ -126,8 +126,8 @@ struct rhd_ctx {
     std::vector<GraphEntry> graphs;
     unsigned long long stamp = 0;
     std::string err;
-    // RHD_DEVICE_MEMORY_LIMIT (bytes, read at creation): cap on the context's cumulative device
-    // allocations, a test hook that forces RHD_ERR_OOM without exhausting the device
+    // RHD_DEVICE_MEMORY_LIMIT (bytes, read at creation): cap on the device memory that the
+    // context holds, a test hook that forces RHD_ERR_OOM without exhausting the device
     size_t mem_limit = 0, mem_used = 0;
     // kernel timing: events recorded around each kernel launch (plain launches while enabled)
     bool ktiming = false;
@@ -451,15 +451,18 @@ void clear_graphs(rhd_ctx* ctx)
     ctx->graphs.clear();
 }
 
+// U^{m+1/2} of the two-pass split path
+size_t uhalf_bytes(const GridState& gs)
+{
+    return sizeof(float4) * (size_t)upad_extent(gs.gp, 0) * upad_extent(gs.gp, 1) * upad_extent(gs.gp, 2);
+}
+
 // Buffers of the two-pass split path: U^{m+1/2} with its ghost layers, the FP32 state mirror and the
 // interleaved FP32 gas (allocated once, kept until the variant changes).
 rhd_status alloc_twopass(rhd_ctx* ctx, GridState& gs)
 {
     rhd_status st;
-    if (!gs.uhalf) {
-        size_t np = (size_t)upad_extent(gs.gp, 0) * upad_extent(gs.gp, 1) * upad_extent(gs.gp, 2);
-        if ((st = dalloc(ctx, (void**)&gs.uhalf, sizeof(float4) * np))) return st;
-    }
+    if (!gs.uhalf && (st = dalloc(ctx, (void**)&gs.uhalf, uhalf_bytes(gs)))) return st;
     if (!gs.um32) {
         if ((st = dalloc(ctx, (void**)&gs.um32, sizeof(float4) * (size_t)gs.ncell))) return st;
         gs.um32_ok = false;
@@ -471,11 +474,11 @@ rhd_status alloc_twopass(rhd_ctx* ctx, GridState& gs)
     return RHD_OK;
 }
 
-void free_twopass(GridState& gs)
+void free_twopass(rhd_ctx* ctx, GridState& gs)
 {
-    dfree(gs.uhalf);
-    dfree(gs.um32);
-    dfree(gs.gas4);
+    dfree(ctx, gs.uhalf, uhalf_bytes(gs));
+    dfree(ctx, gs.um32, sizeof(float4) * (size_t)gs.ncell);
+    dfree(ctx, gs.gas4, sizeof(float4) * (size_t)gs.ncell);
     gs.um32_ok = gs.gas4_ok = false;
 }
 
@@ -1006,13 +1009,13 @@ rhd_status ensure_reduce(rhd_ctx* ctx, long long n)
 {
     int nb = reduce_blocks_for(n);
     if (ctx->red_partials && ctx->red_blocks >= nb) return RHD_OK;
-    dfree(ctx->red_partials);
-    dfree(ctx->red_out);
+    dfree(ctx, ctx->red_partials, sizeof(double) * 5 * (size_t)ctx->red_blocks);
+    dfree(ctx, ctx->red_out, sizeof(double) * 5);
     rhd_status st = dalloc(ctx, (void**)&ctx->red_partials, sizeof(double) * 5 * (size_t)nb);
     if (st) return st;
+    ctx->red_blocks = nb;
     st = dalloc(ctx, (void**)&ctx->red_out, sizeof(double) * 5);
     if (st) return st;
-    ctx->red_blocks = nb;
     return RHD_OK;
 }
 
@@ -1173,7 +1176,7 @@ rhd_status apply_config(rhd_ctx* ctx, GridState& gs, const rhd_launch_config& c)
         rhd_status st = alloc_twopass(ctx, gs);
         if (st) return st;
     } else {
-        free_twopass(gs);
+        free_twopass(ctx, gs);
     }
     gs.um32_ok = false;
     if (c.staging == RHD_STAGING_TMA) {
@@ -1257,10 +1260,10 @@ rhd_status tune_restore(rhd_ctx* ctx, TuneBackup& b)
     return RHD_OK;
 }
 
-void tune_free(TuneBackup& b)
+void tune_free(rhd_ctx* ctx, TuneBackup& b)
 {
-    for (auto& p : b.T) dfree(p);
-    dfree(b.stats);
+    for (size_t i = 0; i < b.T.size(); ++i) dfree(ctx, b.T[i], sizeof(double) * (size_t)ctx->grids[i].ncell);
+    dfree(ctx, b.stats, sizeof(DevStats));
 }
 
 // Mean milliseconds per launch of reps launches of fn (after one warm-up), on the context's stream;
@@ -1329,7 +1332,7 @@ rhd_status grid_autotune(rhd_ctx* ctx, double chat, double dt, int reps, rhd_lau
     if (st) return st;
     TuneBackup b;
     if ((st = tune_backup(ctx, b))) {
-        tune_free(b);
+        tune_free(ctx, b);
         return st;
     }
     int best = -1;
@@ -1351,7 +1354,7 @@ rhd_status grid_autotune(rhd_ctx* ctx, double chat, double dt, int reps, rhd_lau
     if (!st) st2 = apply_config(ctx, gs, best >= 0 ? cand[best] : before);
     if (!st && !st2) st2 = tune_restore(ctx, b);
     cudaError_t ce = cudaStreamSynchronize(ctx->stream);
-    tune_free(b);
+    tune_free(ctx, b);
     if (st) return st;
     if (st2) return st2;
     if (ce != cudaSuccess) return fail(ctx, RHD_ERR_CUDA, std::string("autotune: ") + cudaGetErrorString(ce));
@@ -1404,7 +1407,7 @@ rhd_status ens_apply(rhd_ctx* ctx, int v, int zc)
         }
     }
     for (auto& gs : ctx->grids) {
-        if (v != RHD_VARIANT_TWOPASS) free_twopass(gs);
+        if (v != RHD_VARIANT_TWOPASS) free_twopass(ctx, gs);
         gs.um32_ok = false;
         gs.variant = v;
         gs.z_chunk = zc;  // one chunk length for all grids, as at creation
@@ -1435,7 +1438,7 @@ rhd_status ensemble_autotune(rhd_ctx* ctx, double chat, const double* dt_per_gri
     if (st) return st;
     TuneBackup b;
     if ((st = tune_backup(ctx, b))) {
-        tune_free(b);
+        tune_free(ctx, b);
         return st;
     }
     int best = -1;
@@ -1459,7 +1462,7 @@ rhd_status ensemble_autotune(rhd_ctx* ctx, double chat, const double* dt_per_gri
     if (!st) st2 = best >= 0 ? ens_apply(ctx, cand[best].variant, cand[best].z_chunk) : ens_apply(ctx, v_before, zc_before);
     if (!st && !st2) st2 = tune_restore(ctx, b);
     cudaError_t ce = cudaStreamSynchronize(ctx->stream);
-    tune_free(b);
+    tune_free(ctx, b);
     if (st) return st;
     if (st2) return st2;
     if (ce != cudaSuccess) return fail(ctx, RHD_ERR_CUDA, std::string("autotune: ") + cudaGetErrorString(ce));
@@ -1680,7 +1683,7 @@ rhd_status rhd_marshak_advance(rhd_ctx* ctx, int n_sub, double chat, double dt, 
     if (ctx->marshak_cap < n_sub) {
         // the stream may still read the old states: wait before replacing them
         RHD_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-        dfree(ctx->marshak_state);
+        dfree(ctx, ctx->marshak_state, 4 * sizeof(double) * (size_t)ctx->marshak_cap);
         ctx->marshak_cap = 0;
         if ((st = dalloc(ctx, (void**)&ctx->marshak_state, 4 * sizeof(double) * (size_t)n_sub))) return st;
         ctx->marshak_cap = n_sub;
@@ -1783,14 +1786,21 @@ rhd_status gas_prepare(rhd_ctx* ctx, GridState& gs, const GasParams& p)
             if (!gs.gas_pend[q] && (st = dalloc(ctx, (void**)&gs.gas_pend[q], sizeof(double) * nc))) return st;
     }
     bool added = false;
+    const size_t nv = sizeof(double) * nc;
     for (int d = 0; d < 3; ++d) {
         if (gs.v[d]) continue;
-        if ((st = dalloc(ctx, (void**)&gs.v[d], sizeof(double) * (size_t)gs.ncell))) return st;
-        RHD_CUDA(ctx, cudaMemsetAsync(gs.v[d], 0, sizeof(double) * (size_t)gs.ncell, ctx->stream));
-        if (gs.desc.precision == RHD_SPLIT) {
-            if (!gs.v32[d] && (st = dalloc(ctx, (void**)&gs.v32[d], sizeof(float) * (size_t)gs.ncell))) return st;
-            RHD_CUDA(ctx, cudaMemsetAsync(gs.v32[d], 0, sizeof(float) * (size_t)gs.ncell, ctx->stream));
+        // a component and its FP32 copy together, or neither: the kernels write both
+        double* v = nullptr;
+        float* v32 = nullptr;
+        if ((st = dalloc(ctx, (void**)&v, nv))) return st;
+        if (p.split && (st = dalloc(ctx, (void**)&v32, nv / 2))) {
+            dfree(ctx, v, nv);
+            return st;
         }
+        gs.v[d] = v;
+        gs.v32[d] = v32;
+        RHD_CUDA(ctx, cudaMemsetAsync(v, 0, nv, ctx->stream));
+        if (v32) RHD_CUDA(ctx, cudaMemsetAsync(v32, 0, nv / 2, ctx->stream));
         added = true;
     }
     if (added) {
