@@ -1008,7 +1008,7 @@ rhd_status run_steps(rhd_ctx* ctx, int n_sub, int n_launch, double chat, double 
 rhd_status ensure_reduce(rhd_ctx* ctx, long long n)
 {
     int nb = reduce_blocks_for(n);
-    if (ctx->red_partials && ctx->red_blocks >= nb) return RHD_OK;
+    if (ctx->red_partials && ctx->red_out && ctx->red_blocks >= nb) return RHD_OK;
     dfree(ctx, ctx->red_partials, sizeof(double) * 5 * (size_t)ctx->red_blocks);
     dfree(ctx, ctx->red_out, sizeof(double) * 5);
     rhd_status st = dalloc(ctx, (void**)&ctx->red_partials, sizeof(double) * 5 * (size_t)nb);

@@ -76,3 +76,25 @@ def test_dropped_velocities_make_room(rhd, monkeypatch):  # noqa: F811
     g.close()
     for k in ref:
         assert np.max(np.abs(out[k] - ref[k])) <= 1e-12 * case["desc"]["c"] * np.max(np.abs(ref[k])), k
+
+
+def test_statistics_without_room_for_their_result(rhd, monkeypatch):  # noqa: F811
+    """get_stats allocates the partial sums, then the result; where only the first fit, each call says so."""
+    case = wl.parity_case("stats_oom", (48, 1, 1), exchange="full", seed=13)
+    seen = set()
+    for limit in range(4000, 5200, 8):
+        monkeypatch.setenv("RHD_DEVICE_MEMORY_LIMIT", str(limit))
+        try:
+            g = rhd.Grid(case["desc"])
+            g.load_case(case)
+        except rhd.RhdError as e:
+            assert e.status == rhd.ERR_OOM
+            continue
+        for _ in range(3):
+            try:
+                seen.add(np.isfinite(g.get_stats()["sum_E"]))
+            except rhd.RhdError as e:
+                assert e.status == rhd.ERR_OOM
+                seen.add("oom")
+        g.close()
+    assert seen == {True, "oom"}
