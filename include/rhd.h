@@ -302,7 +302,9 @@ rhd_status rhd_ensemble_subcycle(rhd_ctx* ctx, int n_sub, double chat, const dou
  *   variant   RHD_VARIANT_FUSED: one kernel per subcycle; the predictor (U^{m+1/2}) is recomputed
  *             on the 2-cell halo of each x-y tile.  FP64 grids of 2 and 3 dimensions and RHD_SPLIT grids of
  *             2 run a predictor and a corrector under this name where the device has room for U^{m+1/2}
- *             (32 and 16 bytes per cell, layers as below), and choose their tiles.  RHD_VARIANT_TWOPASS (RHD_SPLIT, 3D grids only):
+ *             (32 and 16 bytes per cell, layers as below), and choose their tiles.  A context takes that
+ *             memory after all its grids' states and gives it back to an array of its own that finds no room
+ *             later (gas arrays, the gas step's scratch); the fused kernel runs from then on.  RHD_VARIANT_TWOPASS (RHD_SPLIT, 3D grids only):
  *             a predictor kernel writes U^{m+1/2} (FP32) for the grid plus 2 ghost layers per face
  *             in each direction that is not periodic on both faces, then a corrector kernel reads
  *             it back; extra device memory (n0+p0)(n1+p1)(n2+p2) x 16 bytes, p = 0 for a direction

@@ -58,6 +58,7 @@ struct GridState {
     GridParams gp;
     long long ncell = 0;
     int tx = 0, ty = 0, tiles_x = 0, tiles_y = 0, z_chunk = 1;
+    int z_fused = 1;              // the fused kernel's own z_chunk
     int p_chunk = 0;              // two-pass predictor: planes per CTA where they differ from z_chunk (0: they do not)
     double* U[2][4] = {{nullptr}};
     double* T = nullptr;
@@ -304,7 +305,7 @@ void fill_params(GridState& gs)
         zc = d.n[2];
         while (zc > 32 && tiles * ((d.n[2] + zc - 1) / zc) < 152LL * 8) zc = (zc + 1) / 2;
     }
-    gs.z_chunk = std::max(1, std::min(zc, d.n[2]));
+    gs.z_chunk = gs.z_fused = std::max(1, std::min(zc, d.n[2]));
 }
 
 // Planes per CTA of the split two-pass kernels.  A CTA marches its column tile through z; t0 + t1 k is the time
@@ -379,21 +380,22 @@ int plan_ensemble_chunk(rhd_ctx* ctx)
     return best;
 }
 
-rhd_status dalloc(rhd_ctx* ctx, void** p, size_t bytes)
+// One attempt: the status, and on failure its message in *why
+rhd_status try_alloc(rhd_ctx* ctx, void** p, size_t bytes, std::string* why)
 {
-    if (ctx && ctx->mem_limit && ctx->mem_used + bytes > ctx->mem_limit) {
-        *p = nullptr;
-        return fail(ctx, RHD_ERR_OOM, "RHD_DEVICE_MEMORY_LIMIT reached (" + std::to_string(ctx->mem_used + bytes) +
-                                          " bytes requested in total)");
+    *p = nullptr;
+    if (ctx->mem_limit && ctx->mem_used + bytes > ctx->mem_limit) {
+        *why = "RHD_DEVICE_MEMORY_LIMIT reached (" + std::to_string(ctx->mem_used + bytes) + " bytes requested in total)";
+        return RHD_ERR_OOM;
     }
-    cudaError_t e = cudaMalloc(p, bytes);
+    const cudaError_t e = cudaMalloc(p, bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
         *p = nullptr;
-        return fail(ctx, e == cudaErrorMemoryAllocation ? RHD_ERR_OOM : RHD_ERR_CUDA,
-                    std::string("cudaMalloc(") + std::to_string(bytes) + "): " + cudaGetErrorString(e));
+        *why = std::string("cudaMalloc(") + std::to_string(bytes) + "): " + cudaGetErrorString(e);
+        return e == cudaErrorMemoryAllocation ? RHD_ERR_OOM : RHD_ERR_CUDA;
     }
-    if (ctx) ctx->mem_used += bytes;
+    ctx->mem_used += bytes;
     return RHD_OK;
 }
 
@@ -451,6 +453,50 @@ void clear_graphs(rhd_ctx* ctx)
     ctx->graphs.clear();
 }
 
+// U^{m+1/2} of the kernel pair: FP64 grids of two or three dimensions (32 bytes per stored cell), split grids of
+// two (16 bytes); 0: the grid has no pair
+size_t pair_bytes(const GridState& gs)
+{
+    const bool split = gs.desc.precision == RHD_SPLIT;
+    if (split ? gs.gp.nact != 2 : gs.gp.nact < 2) return 0;
+    size_t np = (size_t)upad_extent(gs.gp, 0) * upad_extent(gs.gp, 1);
+    if (gs.gp.nact == 3) np *= (size_t)upad_extent(gs.gp, 2);
+    return np * (split ? sizeof(float4) : 4 * sizeof(double));
+}
+
+// Planes per CTA of the fused FP64 ensemble kernel where the caller leaves them to the library
+constexpr int kEnsembleChunk = 32;
+
+// Gives up what the grids run faster with and can do without, for an array that the context needs: the pair's
+// U^{m+1/2} (the fused kernels take over) and T's second buffer of 1D grids (one subcycle per launch).  False:
+// there was nothing to give.
+bool release_spare(rhd_ctx* ctx)
+{
+    bool any = false;
+    for (auto& gs : ctx->grids) any = any || gs.uhalf64 || gs.uhalf2d || gs.T2;
+    if (!any) return false;
+    cudaStreamSynchronize(ctx->stream);
+    clear_graphs(ctx);
+    for (auto& gs : ctx->grids) {
+        // the chunk length goes with the kernels unless the caller chose it
+        if (gs.uhalf64 && gs.desc.z_chunk == 0) gs.z_chunk = ctx->ensemble ? kEnsembleChunk : gs.z_fused;
+        dfree(ctx, gs.uhalf64, pair_bytes(gs));
+        dfree(ctx, gs.uhalf2d, pair_bytes(gs));
+        if (gs.T2) gs.line.steps = 1;
+        dfree(ctx, gs.T2, sizeof(double) * (size_t)gs.ncell);
+    }
+    ctx->ens_pair64 = false;
+    return true;
+}
+
+rhd_status dalloc(rhd_ctx* ctx, void** p, size_t bytes)
+{
+    std::string why;
+    rhd_status st = try_alloc(ctx, p, bytes, &why);
+    if (st == RHD_ERR_OOM && release_spare(ctx)) st = try_alloc(ctx, p, bytes, &why);
+    return st ? fail(ctx, st, why) : RHD_OK;
+}
+
 // U^{m+1/2} of the two-pass split path
 size_t uhalf_bytes(const GridState& gs)
 {
@@ -482,18 +528,13 @@ void free_twopass(rhd_ctx* ctx, GridState& gs)
     gs.um32_ok = gs.gas4_ok = false;
 }
 
-// U^{m+1/2} of the kernel pair: FP64 grids of two or three dimensions (32 bytes per stored cell), split grids of
-// two (16 bytes).  A grid that leaves no room for it runs the fused kernel, which needs none.
+// Takes the pair's U^{m+1/2} if there is room.  After every array that the grids must have (an ensemble's grids all
+// have theirs by then), and given back by dalloc to those that come later.
 void alloc_pair(rhd_ctx* ctx, GridState& gs)
 {
-    const bool split = gs.desc.precision == RHD_SPLIT;
-    if (split ? gs.gp.nact != 2 : gs.gp.nact < 2) return;
-    size_t np = (size_t)upad_extent(gs.gp, 0) * upad_extent(gs.gp, 1);
-    if (gs.gp.nact == 3) np *= (size_t)upad_extent(gs.gp, 2);
-    const std::string err = ctx->err;
-    if (split ? dalloc(ctx, (void**)&gs.uhalf2d, sizeof(float4) * np)
-              : dalloc(ctx, (void**)&gs.uhalf64, 4 * sizeof(double) * np))
-        ctx->err = err;
+    const size_t bytes = pair_bytes(gs);
+    std::string why;
+    if (bytes) try_alloc(ctx, gs.desc.precision == RHD_SPLIT ? (void**)&gs.uhalf2d : (void**)&gs.uhalf64, bytes, &why);
 }
 
 // The pair's work split: z_chunk planes per CTA, or its own choice (0), which then is the grid's z chunk
@@ -523,8 +564,11 @@ rhd_status alloc_grid(rhd_ctx* ctx, GridState& gs)
     if (gs.variant == RHD_VARIANT_TWOPASS) return alloc_twopass(ctx, gs);
     if (gs.gp.nact == 1) {
         gs.line = line_plan(gs.gp, gs.desc.precision == RHD_SPLIT, ctx->num_sms);
-        if (gs.line.steps > 1 && (st = dalloc(ctx, (void**)&gs.T2, bytes))) return st;
+        std::string why;
+        // without room for T's second buffer, one subcycle per launch
+        if (gs.line.steps > 1 && try_alloc(ctx, (void**)&gs.T2, bytes, &why)) gs.line.steps = 1;
     }
+    if (ctx->ensemble) return RHD_OK;
     alloc_pair(ctx, gs);
     plan_pair64(ctx, gs, gs.desc.z_chunk);
     return RHD_OK;
@@ -2200,14 +2244,21 @@ rhd_status rhd_ensemble_create(rhd_ctx** out, int n_grids, const rhd_grid_desc* 
                              : RHD_VARIANT_FUSED;
             st = alloc_grid(ctx, gs);
         }
+        if (!st) st = dalloc(ctx, (void**)&ctx->d_egrids[0], sizeof(EnsembleGrid) * (size_t)n_grids);
+        if (!st) st = dalloc(ctx, (void**)&ctx->d_egrids[1], sizeof(EnsembleGrid) * (size_t)n_grids);
+        if (!st) st = dalloc(ctx, (void**)&ctx->d_counter, 2 * sizeof(unsigned long long));
         // one z chunk for all grids (the largest grid's automatic choice)
-        int zc = descs[0].z_chunk > 0 ? descs[0].z_chunk : 32;
+        int zc = descs[0].z_chunk > 0 ? descs[0].z_chunk : kEnsembleChunk;
         if (!st && descs[0].z_chunk == 0 && ctx->grids[0].variant == RHD_VARIANT_TWOPASS) zc = plan_ensemble_chunk(ctx);
         if (!st && descs[0].precision == RHD_FP64) {
+            for (auto& gs : ctx->grids) gs.z_chunk = zc;
             ctx->ens_pair64 = true;
-            for (auto& gs : ctx->grids) ctx->ens_pair64 = ctx->ens_pair64 && gs.uhalf64;
-            if (!ctx->ens_pair64)
-                for (auto& gs : ctx->grids) dfree(gs.uhalf64);
+            for (auto& gs : ctx->grids) {
+                alloc_pair(ctx, gs);
+                ctx->ens_pair64 = ctx->ens_pair64 && gs.uhalf64;
+                if (!ctx->ens_pair64) break;
+            }
+            if (!ctx->ens_pair64) release_spare(ctx);
             // shorter chunks (each costs less than a plane more) until the items even out over the SMs
             while (ctx->ens_pair64 && descs[0].z_chunk == 0) {
                 long long n = 0;
@@ -2226,9 +2277,6 @@ rhd_status rhd_ensemble_create(rhd_ctx** out, int n_grids, const rhd_grid_desc* 
         for (auto& gs : ctx->grids)
             items += (long long)gs.tiles_x * gs.tiles_y * ((gs.desc.n[2] + zc - 1) / zc);
         ctx->n_items = items;
-        if (!st) st = dalloc(ctx, (void**)&ctx->d_egrids[0], sizeof(EnsembleGrid) * (size_t)n_grids);
-        if (!st) st = dalloc(ctx, (void**)&ctx->d_egrids[1], sizeof(EnsembleGrid) * (size_t)n_grids);
-        if (!st) st = dalloc(ctx, (void**)&ctx->d_counter, 2 * sizeof(unsigned long long));
         if (!st) {
             int per_sm = descs[0].precision == RHD_SPLIT ? ensemble_ctas_per_sm_split() : ensemble_ctas_per_sm_fp64();
             ctx->ens_ctas = per_sm * ctx->num_sms;

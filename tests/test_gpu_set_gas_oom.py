@@ -82,7 +82,7 @@ def test_statistics_without_room_for_their_result(rhd, monkeypatch):  # noqa: F8
     """get_stats allocates the partial sums, then the result; where only the first fit, each call says so."""
     case = wl.parity_case("stats_oom", (48, 1, 1), exchange="full", seed=13)
     seen = set()
-    for limit in range(4000, 5200, 8):
+    for limit in range(3000, 5200, 8):
         monkeypatch.setenv("RHD_DEVICE_MEMORY_LIMIT", str(limit))
         try:
             g = rhd.Grid(case["desc"])
