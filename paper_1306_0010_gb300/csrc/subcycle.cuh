@@ -331,12 +331,12 @@ __device__ __forceinline__ long long lin(const GridParams& g, int x, int y, int 
 #endif
     return (long long)x + (long long)g.n[0] * ((long long)y + (long long)g.n[1] * (long long)z);
 }
-// cells of the interior arrays and of the stored U^{m+1/2} of the two-pass path (grid plus its ghost
-// layers in the directions that are not periodic on both faces)
+// cells of the interior arrays and of the stored U^{m+1/2} (grid plus its ghost layers in the active directions
+// that are not periodic on both faces)
 __device__ __forceinline__ long long n_cells(const GridParams& g) { return (long long)g.n[0] * g.n[1] * g.n[2]; }
 __device__ __forceinline__ long long n_padded(const GridParams& g)
 {
-    return (long long)upad_extent(g, 0) * upad_extent(g, 1) * upad_extent(g, 2);
+    return (long long)upad_extent(g, 0) * upad_extent(g, 1) * (g.nact == 3 ? upad_extent(g, 2) : 1);
 }
 
 // U^m = (E, Gx, Gy, Gz) at any cell, ghosts by the boundary rule.

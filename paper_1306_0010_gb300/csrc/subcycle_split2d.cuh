@@ -11,6 +11,8 @@
 // instruction issue, the predictor by the latency of its first loads as well.
 #pragma once
 
+#include <type_traits>
+
 namespace rhd {
 
 // HLL flux of hll() with the weights chosen instead of the code: the average is weights 1, 1, 0 and 1/2
@@ -62,6 +64,7 @@ __global__ void __launch_bounds__(S2_NT, 4) predictor2d_kernel(const __grid_cons
         wave_speeds(k, U.z, chat, fixed, l1y, l3y);
         const float bx = xmul(k.b, U.y), bz = xmul(k.b, U.z);
         const float Pxy = xmul(chat, xmul(bx, U.z)), Pxz = xmul(chat, xmul(bx, U.w)), Pyz = xmul(chat, xmul(bz, U.w));
+        i = chk(i, G::N1);
         Um[i] = U;
         CX[i] = make_float4(xmul(chat, xfma(bx, U.y, k.a)), Pxy, Pxz, l1x);
         CY[i] = make_float4(Pxy, xmul(chat, xfma(bz, U.z, k.a)), Pyz, l1y);
@@ -79,24 +82,28 @@ __global__ void __launch_bounds__(S2_NT, 4) predictor2d_kernel(const __grid_cons
     if (has_h) closure(G::i1(hlx, hly), Uhalo);
     __syncthreads();
     auto xface = [&](int iL, int iR) {
+        iL = chk(iL, G::N1);
+        iR = chk(iR, G::N1);
         const float4 UL = Um[iL], UR = Um[iR], CL = CX[iL], CR = CX[iR];
         return hll2d(UL, UR, make_float4(xmul(chat, UL.y), CL.x, CL.y, CL.z), make_float4(xmul(chat, UR.y), CR.x, CR.y, CR.z),
                      CL.w, L3[iL].x, CR.w, L3[iR].x);
     };
     auto yface = [&](int iL, int iR) {
+        iL = chk(iL, G::N1);
+        iR = chk(iR, G::N1);
         const float4 UL = Um[iL], UR = Um[iR], CL = CY[iL], CR = CY[iR];
         return hll2d(UL, UR, make_float4(xmul(chat, UL.z), CL.x, CL.y, CL.z), make_float4(xmul(chat, UR.z), CR.x, CR.y, CR.z),
                      CL.w, L3[iL].y, CR.w, L3[iR].y);
     };
     const int fl = tly * (TX + 1) + tlx, fb = tly * TX + tlx;
-    Fx[fl] = xface(i_own - 1, i_own);
-    Fy[fb] = yface(i_own - G::W1, i_own);
+    Fx[chk(fl, G::NFX)] = xface(i_own - 1, i_own);
+    Fy[chk(fb, G::NFY)] = yface(i_own - G::W1, i_own);
     if (t < TX) {
         const int iL = G::i1(t, TY - 1);
-        Fy[TY * TX + t] = yface(iL, iL + G::W1);
+        Fy[chk(TY * TX + t, G::NFY)] = yface(iL, iL + G::W1);
     } else if (t < TX + TY) {
         const int ly = t - TX, iL = G::i1(TX - 1, ly);
-        Fx[ly * (TX + 1) + TX] = xface(iL, iL + 1);
+        Fx[chk(ly * (TX + 1) + TX, G::NFX)] = xface(iL, iL + 1);
     }
     __syncthreads();
     unsigned fix = 0;
@@ -124,7 +131,7 @@ __global__ void __launch_bounds__(S2_NT, 4) predictor2d_kernel(const __grid_cons
         }
         const int f = realize(Un, g.f_E_floor);
         if (interior) fix = f;
-        P.uhalf[(gx + g.pad[0]) + (long long)upad_extent(g, 0) * (gy + g.pad[1])] = f4(Un);
+        P.uhalf[chk((gx + g.pad[0]) + (long long)upad_extent(g, 0) * (gy + g.pad[1]), n_padded(g))] = f4(Un);
     }
     add_counter(&P.stats->n_fix, fix);
 }
@@ -245,15 +252,16 @@ __global__ void __launch_bounds__(S2_NT, 4) corrector2d_kernel(const __grid_cons
     const int x0 = (int)(blockIdx.x % P.tiles_x) * TX, y0 = (int)(blockIdx.x / P.tiles_x) * TY;
     const int gx = x0 + tlx, gy = y0 + tly;
     const bool cell = gx < g.n[0] && gy < g.n[1];
-    const long long li = cell ? gx + (long long)g.n[0] * gy : 0;
+    const long long li = chk(cell ? gx + (long long)g.n[0] * gy : 0ll, n_cells(g));
     Counters cnt = {0, 0, 0, 0, 0, 0};
     // U^{m+1/2} of the tile and two cells around it, at the stored positions (beyond ragged edges: values unused)
 #pragma unroll
     for (int r = 0; r < G::NR2; ++r) {
         const int c = t + r * G::NT;
         if (c < G::N2)
-            cp_async16(Uk + c, P.uhalf + upad_pos(g, 0, x0 + c % G::W2 - 2) +
-                                   (long long)upad_extent(g, 0) * upad_pos(g, 1, y0 + c / G::W2 - 2));
+            cp_async16(Uk + c, P.uhalf + chk(upad_pos(g, 0, x0 + c % G::W2 - 2) +
+                                                 (long long)upad_extent(g, 0) * upad_pos(g, 1, y0 + c / G::W2 - 2),
+                                             n_padded(g)));
     }
     cp_async_commit();
     GasCell<float> gc{};
@@ -272,43 +280,56 @@ __global__ void __launch_bounds__(S2_NT, 4) corrector2d_kernel(const __grid_cons
     const int i_own = G::i2(tlx, tly);
     const float4 uh = Uk[i_own];
     auto store_rec = [](float4* S, int n, int slot, const float4 (&rec)[4]) {
+        slot = chk(slot, n);
 #pragma unroll
         for (int v = 0; v < 4; ++v) S[v * n + slot] = rec[v];
     };
+    // the face states of the cell at i along x or y
+    const std::integral_constant<int, 0> along_x;
+    const std::integral_constant<int, 1> along_y;
+    auto record = [&](auto dir, int i, float4 (&rec)[4]) {
+        constexpr int D = decltype(dir)::value;
+        const int di = D == 0 ? 1 : G::W2;
+        return face_record2d<D>(Uk[chk(i - di, G::N2)], Uk[chk(i, G::N2)], Uk[chk(i + di, G::N2)], chat, lim, p1, fixed, rec);
+    };
     {
         float4 rec[4];
-        int fb = face_record2d<0>(Uk[i_own - 1], Uk[i_own], Uk[i_own + 1], chat, lim, p1, fixed, rec);
+        int fb = record(along_x, i_own, rec);
         cnt.face += (unsigned)(fb & (int)cell);
         store_rec(Sx, G::NSX, G::sx(tlx, tly), rec);
-        fb = face_record2d<1>(Uk[i_own - G::W2], Uk[i_own], Uk[i_own + G::W2], chat, lim, p1, fixed, rec);
+        fb = record(along_y, i_own, rec);
         cnt.face += (unsigned)(fb & (int)cell);
         store_rec(Sy, G::NSY, G::sy(tlx, tly), rec);
         if (t < 2 * TX) {
             const int ly = t < TX ? -1 : TY, lx = t % TX, i = G::i2(lx, ly);
-            face_record2d<1>(Uk[i - G::W2], Uk[i], Uk[i + G::W2], chat, lim, p1, fixed, rec);
+            record(along_y, i, rec);
             store_rec(Sy, G::NSY, G::sy(lx, ly), rec);
         } else if (t < G::NHR) {
             const int hh = t - 2 * TX, ly = hh >> 1, lx = (hh & 1) ? TX : -1, i = G::i2(lx, ly);
-            face_record2d<0>(Uk[i - 1], Uk[i], Uk[i + 1], chat, lim, p1, fixed, rec);
+            record(along_x, i, rec);
             store_rec(Sx, G::NSX, G::sx(lx, ly), rec);
         }
     }
     __syncthreads();
     auto hll_x = [&](int iL, int iR) {
+        iL = chk(iL, G::NSX);
+        iR = chk(iR, G::NSX);
         const float4 UL = Sx[G::NSX + iL], UR = Sx[iR], cL = Sx[2 * G::NSX + iL], cR = Sx[2 * G::NSX + iR];
         const float4 LL = Sx[3 * G::NSX + iL], LR = Sx[3 * G::NSX + iR];
         return hll2d(UL, UR, flux2d<0>(UL, cL.z, cL.w, chat), flux2d<0>(UR, cR.x, cR.y, chat), LL.z, LL.w, LR.x, LR.y);
     };
     auto hll_y = [&](int iL, int iR) {
+        iL = chk(iL, G::NSY);
+        iR = chk(iR, G::NSY);
         const float4 UL = Sy[G::NSY + iL], UR = Sy[iR], cL = Sy[2 * G::NSY + iL], cR = Sy[2 * G::NSY + iR];
         const float4 LL = Sy[3 * G::NSY + iL], LR = Sy[3 * G::NSY + iR];
         return hll2d(UL, UR, flux2d<1>(UL, cL.z, cL.w, chat), flux2d<1>(UR, cR.x, cR.y, chat), LL.z, LL.w, LR.x, LR.y);
     };
     const int fl = tly * (TX + 1) + tlx, fb = tly * TX + tlx;
-    Cx[fl] = hll_x(G::sx(tlx - 1, tly), G::sx(tlx, tly));
-    Cy[fb] = hll_y(G::sy(tlx, tly - 1), G::sy(tlx, tly));
-    if (t < TX) Cy[TY * TX + t] = hll_y(G::sy(t, TY - 1), G::sy(t, TY));
-    else if (t < TX + TY) Cx[(t - TX) * (TX + 1) + TX] = hll_x(G::sx(TX - 1, t - TX), G::sx(TX, t - TX));
+    Cx[chk(fl, G::NCX)] = hll_x(G::sx(tlx - 1, tly), G::sx(tlx, tly));
+    Cy[chk(fb, G::NCY)] = hll_y(G::sy(tlx, tly - 1), G::sy(tlx, tly));
+    if (t < TX) Cy[chk(TY * TX + t, G::NCY)] = hll_y(G::sy(t, TY - 1), G::sy(t, TY));
+    else if (t < TX + TY) Cx[chk((t - TX) * (TX + 1) + TX, G::NCX)] = hll_x(G::sx(TX - 1, t - TX), G::sx(TX, t - TX));
     cp_async_wait_all();
     __syncthreads();
     if (cell) {
