@@ -1,8 +1,7 @@
 // gas_index.h -- index arithmetic of the gas-step kernels (k_gas.cu): the ghost rule, the layouts of
-// the extended grid and of the face-flux arrays.  Host-and-device code: the kernels of a launch per direction
-// compute every array index through these functions, and a host test enumerates them over whole grids to check
-// that every index stays inside its array.  The marching kernels take the ghost rule from here and step by
-// whole rows and planes of the two layouts; each access lies within the ghost layers (k_gas.cu).
+// the extended grid and of the face-flux arrays.  Host-and-device code: the kernels compute every
+// array index through these functions, and host tests enumerate them over whole grids to check that
+// every index stays inside its array.
 #pragma once
 
 #include "gas_internal.h"
@@ -166,6 +165,86 @@ GAS_HD void gas_corr_update_cells(const GasParams& p, long long i, long long* x,
         lo[d] = gas_ravel(A, fe);
         hi[d] = gas_ravel(B, fe);
     }
+}
+
+// ---- the marching kernels: a CTA takes a tile of TX x TY cells and marches planes in z
+
+// The work split of a march over a grid of e cells: a tile per CTA, and in 3D so many planes that some four waves
+// of CTAs fill the chip (three resident ones on each multiprocessor), at least eight (a chunk starts with one
+// plane's z faces, the corrector's with another plane's slopes).
+inline GasMarch gas_march(const int e[3], int tx, int ty, int num_sms, long long* blocks)
+{
+    GasMarch t;
+    t.tiles_x = (e[0] + tx - 1) / tx;
+    t.tiles = (long long)t.tiles_x * ((e[1] + ty - 1) / ty);
+    long long chunks = (12LL * num_sms + t.tiles - 1) / t.tiles;
+    const long long most = (e[2] + 7) / 8;
+    if (chunks > most) chunks = most;
+    t.planes = (int)((e[2] + chunks - 1) / chunks);
+    *blocks = t.tiles * ((e[2] + t.planes - 1) / t.planes);
+    return t;
+}
+
+// The threads of a tile of TX x TY cells: one per cell (its low faces), then a warp for the y faces above the
+// top row (2D, 3D), then one for the x faces beyond the last column.
+template <int DIM, int TX, int TY>
+struct GasTile {
+    static constexpr int MAIN = TX * TY, ROW = DIM > 1 ? TX : 0, NT = MAIN + ROW + 32;
+    int tx, ty;
+    bool cell, fx, fy;
+    GAS_HD explicit GasTile(int t)
+    {
+        cell = t < MAIN;
+        fx = cell;
+        fy = DIM > 1 && t < MAIN + ROW;
+        tx = t % TX;
+        ty = t / TX;
+        if (t >= MAIN + ROW) {
+            tx = TX;
+            ty = t - (MAIN + ROW);
+            fx = ty < TY;
+        }
+    }
+};
+
+// Of a tile's threads, those whose cell, low x face and low y face lie in a range of e0 x e1 cells
+GAS_HD bool gas_cell_in(int X, int Y, int e0, int e1) { return X < e0 && Y < e1; }
+GAS_HD bool gas_xface_in(int X, int Y, int e0, int e1) { return X <= e0 && Y < e1; }
+GAS_HD bool gas_yface_in(int X, int Y, int e0, int e1) { return X < e0 && Y <= e1; }
+
+// predictor, extended column (X, Y): the interior cells of plane 0 under it and under its low neighbours in x and y,
+// with the signs of their normal components; any X and Y >= 0 give cells inside the plane
+struct GasPredColumn {
+    long long own, left, low;
+    int sx, sy, sxl, syl;
+};
+GAS_HD GasPredColumn gas_pred_column(const GasParams& p, int X, int Y)
+{
+    GasPredColumn c;
+    c.sx = c.sy = c.sxl = c.syl = 1;
+    const int qx = gas_axis(X - p.g[0], p.n[0], p.bc_lo[0], p.bc_hi[0], c.sx);
+    const int qy = gas_axis(Y - p.g[1], p.n[1], p.bc_lo[1], p.bc_hi[1], c.sy);
+    const int qxl = gas_axis(X - p.g[0] - 1, p.n[0], p.bc_lo[0], p.bc_hi[0], c.sxl);
+    const int qyl = gas_axis(Y - p.g[1] - 1, p.n[1], p.bc_lo[1], p.bc_hi[1], c.syl);
+    const long long row = p.n[0];
+    c.own = qx + row * qy;
+    c.left = qxl + row * qy;
+    c.low = qx + row * qyl;
+    return c;
+}
+// ... and what extended plane z adds to them (plane: the cells of an interior one)
+GAS_HD long long gas_pred_plane(const GasParams& p, long long plane, int z, int& s)
+{
+    s = 1;
+    return plane * gas_axis(z - p.g[2], p.n[2], p.bc_lo[2], p.bc_hi[2], s);
+}
+
+// corrector: the extended cell of interior column (X, Y) in interior plane 0; a row is m[0] and a plane m[0] m[1]
+// cells
+GAS_HD long long gas_corr_column(const GasParams& p, int X, int Y)
+{
+    const long long row = p.m[0];
+    return X + p.g[0] + row * (Y + p.g[1]) + row * p.m[1] * p.g[2];
 }
 
 }  // namespace rhd

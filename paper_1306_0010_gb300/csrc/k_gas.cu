@@ -509,29 +509,6 @@ __device__ __forceinline__ void add_divergence(const GasParams& p, int d, double
     dU -= __dsub_rn(hi, lo) * p.inv_dx[d];
 }
 
-// The threads of a tile of TX x TY cells: one per cell (its low faces), then a warp for the y faces above the
-// top row (2D, 3D), then one for the x faces beyond the last column.
-template <int DIM, int TX, int TY>
-struct GasTile {
-    static constexpr int MAIN = TX * TY, ROW = DIM > 1 ? TX : 0, NT = MAIN + ROW + 32;
-    int tx, ty;
-    bool cell, fx, fy;
-    __device__ __forceinline__ GasTile()
-    {
-        const int t = threadIdx.x;
-        cell = t < MAIN;
-        fx = cell;
-        fy = DIM > 1 && t < MAIN + ROW;
-        tx = t % TX;
-        ty = t / TX;
-        if (t >= MAIN + ROW) {
-            tx = TX;
-            ty = t - (MAIN + ROW);
-            fx = ty < TY;
-        }
-    }
-};
-
 // Resident CTAs asked of the compiler.  The fluxes' chains leave half of the issue slots empty at the two CTAs that
 // the unbounded kernels' registers allow; a few spilled values cost less.  256^3 and 300 x 250 x 200, us:
 // predictor (95 registers unbounded) 633 and 688 at two, 575 and 586 at three, 560 and 547 at four; corrector (113)
@@ -567,28 +544,24 @@ __global__ void __launch_bounds__((GasTile<DIM, TX, TY>::NT), gas_min_blocks<R, 
                                                                                  const GasMarch t)
 {
     __shared__ GasFaces<R, DIM, TX, TY> faces[DIM > 2 ? 2 : 1];
-    const GasTile<DIM, TX, TY> me;
+    const GasTile<DIM, TX, TY> me(threadIdx.x);
     const Consts<R> kc = consts<R>(p);
     const int b = (int)(blockIdx.x % t.tiles), zc = (int)(blockIdx.x / t.tiles) * t.planes;
     const int ze = zc + t.planes < p.m[2] ? zc + t.planes : p.m[2];
     const int X = (b % t.tiles_x) * TX + me.tx, Y = (b / t.tiles_x) * TY + me.ty;
-    const bool cell = me.cell && X < p.m[0] && Y < p.m[1];
-    const bool fx = me.fx && p.n[0] > 1 && X <= p.m[0] && Y < p.m[1];
-    const bool fy = me.fy && X < p.m[0] && Y <= p.m[1];
+    const bool cell = me.cell && gas_cell_in(X, Y, p.m[0], p.m[1]);
+    const bool fx = me.fx && p.n[0] > 1 && gas_xface_in(X, Y, p.m[0], p.m[1]);
+    const bool fy = me.fy && gas_yface_in(X, Y, p.m[0], p.m[1]);
     // the interior cell under the thread's own, and under its low neighbours in x and y
-    int sx = 1, sy = 1, sxl = 1, syl = 1;
-    const int qx = gas_axis(X - p.g[0], p.n[0], p.bc_lo[0], p.bc_hi[0], sx);
-    const int qy = gas_axis(Y - p.g[1], p.n[1], p.bc_lo[1], p.bc_hi[1], sy);
-    const int qxl = gas_axis(X - p.g[0] - 1, p.n[0], p.bc_lo[0], p.bc_hi[0], sxl);
-    const int qyl = gas_axis(Y - p.g[1] - 1, p.n[1], p.bc_lo[1], p.bc_hi[1], syl);
-    const long long row = p.n[0], plane = row * p.n[1];
-    const long long own = qx + row * qy, left = qxl + row * qy, low = qx + row * qyl;
+    const GasPredColumn col = gas_pred_column(p, X, Y);
+    const int sx = col.sx, sy = col.sy, sxl = col.sxl, syl = col.syl;
+    const long long own = col.own, left = col.left, low = col.low, plane = (long long)p.n[0] * p.n[1];
     const bool in_xy = X >= p.g[0] && X < p.g[0] + p.n[0] && Y >= p.g[1] && Y < p.g[1] + p.n[1];
     unsigned long long floors = 0;
 
     int sz = 1, szn = 1;
     int z = DIM > 2 ? zc - 1 : 0;  // 3D: the plane below the chunk gives the flux through its lowest face
-    long long base = DIM > 2 ? plane * gas_axis(z - p.g[2], p.n[2], p.bc_lo[2], p.bc_hi[2], sz) : 0, base_n = 0;
+    long long base = DIM > 2 ? gas_pred_plane(p, plane, z, sz) : 0, base_n = 0;
     GasCell<R> cur = load_cell<R>(a, own + base, sx, sy, sz), nxt = cur;
     R zlo[5], zhi[5];
     for (int q = 0; q < 5; ++q) zlo[q] = zhi[q] = R(0);
@@ -596,8 +569,7 @@ __global__ void __launch_bounds__((GasTile<DIM, TX, TY>::NT), gas_min_blocks<R, 
         const bool on = DIM < 3 || z >= zc;
         GasFaces<R, DIM, TX, TY>& f = faces[DIM > 2 ? z & 1 : 0];
         if constexpr (DIM > 2) {
-            szn = 1;
-            base_n = plane * gas_axis(z + 1 - p.g[2], p.n[2], p.bc_lo[2], p.bc_hi[2], szn);
+            base_n = gas_pred_plane(p, plane, z + 1, szn);
             if (cell || z + 1 < ze) nxt = load_cell<R>(a, own + base_n, sx, sy, szn);
         }
         float4 u = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
@@ -629,7 +601,8 @@ __global__ void __launch_bounds__((GasTile<DIM, TX, TY>::NT), gas_min_blocks<R, 
             if (cell) {
                 R dU[5];
                 tile_divergence(p, f, me.tx, me.ty, zlo, zhi, dU);
-                const long long i = X + (long long)p.m[0] * (Y + (long long)p.m[1] * z);
+                const int at[3] = {X, Y, z};
+                const long long i = gas_ravel(at, p.m);
                 const bool inside = in_xy && (DIM < 3 || (z >= p.g[2] && z < p.g[2] + p.n[2]));
                 if constexpr (sizeof(R) == 4) {
                     // W^{n+1/2} in FP32 from the FP32 copies of W^n and FP32 increments
@@ -667,19 +640,19 @@ __global__ void __launch_bounds__((GasTile<DIM, TX, TY>::NT), gas_min_blocks<R, 
                                                                                  const GasMarch t)
 {
     __shared__ GasFaces<R, DIM, TX, TY> faces[DIM > 2 ? 2 : 1];
-    const GasTile<DIM, TX, TY> me;
+    const GasTile<DIM, TX, TY> me(threadIdx.x);
     const Consts<R> kc = consts<R>(p);
     const int b = (int)(blockIdx.x % t.tiles), zc = (int)(blockIdx.x / t.tiles) * t.planes;
     const int ze = zc + t.planes < p.n[2] ? zc + t.planes : p.n[2];
     const int X = (b % t.tiles_x) * TX + me.tx, Y = (b / t.tiles_x) * TY + me.ty;
-    const bool cell = me.cell && X < p.n[0] && Y < p.n[1];
-    const bool fx = me.fx && p.n[0] > 1 && X <= p.n[0] && Y < p.n[1];
-    const bool fy = me.fy && X < p.n[0] && Y <= p.n[1];
+    const bool cell = me.cell && gas_cell_in(X, Y, p.n[0], p.n[1]);
+    const bool fx = me.fx && p.n[0] > 1 && gas_xface_in(X, Y, p.n[0], p.n[1]);
+    const bool fy = me.fy && gas_yface_in(X, Y, p.n[0], p.n[1]);
     const bool any = cell || fx || fy;
     const int lim = LIM >= 0 ? LIM : p.limiter;
     const long long row = p.m[0], plane = row * p.m[1];
     // the thread's extended cell in plane z is own + plane * z
-    const long long own = X + p.g[0] + row * (Y + p.g[1]) + plane * p.g[2];
+    const long long own = gas_corr_column(p, X, Y);
     unsigned long long floors = 0, bad = 0;
 
     // 3D: cells z, z + 1 and z + 2 of the thread's column; the slope of z + 1 gives its states at the faces z + 1
@@ -733,7 +706,8 @@ __global__ void __launch_bounds__((GasTile<DIM, TX, TY>::NT), gas_min_blocks<R, 
             if (cell) {
                 R dU[5];
                 tile_divergence(p, f, me.tx, me.ty, zlo, zhi, dU);
-                const long long i = X + (long long)p.n[0] * (Y + (long long)p.n[1] * z);
+                const int at[3] = {X, Y, z};
+                const long long i = gas_ravel(at, p.n);
                 if constexpr (sizeof(R) == 4) {
                     // FP32 increments (fluxes, sources at W^{n+1/2}) accumulated into the FP64 state
                     const float fdt = (float)p.dt;
@@ -853,27 +827,11 @@ int blocks_for(long long n)
     return (int)(b < 1 ? 1 : (b > (1LL << 30) ? (1LL << 30) : b));
 }
 
-// The work split of a march over a grid of e cells: a tile per CTA, and in 3D so many planes that some four waves
-// of CTAs fill the chip (three resident ones on each multiprocessor), at least eight (a chunk starts with one
-// plane's z faces, the corrector's with another plane's slopes).
-GasMarch march_of(const int e[3], int tx, int ty, int num_sms, long long* blocks)
-{
-    GasMarch t;
-    t.tiles_x = (e[0] + tx - 1) / tx;
-    t.tiles = (long long)t.tiles_x * ((e[1] + ty - 1) / ty);
-    long long chunks = (12LL * num_sms + t.tiles - 1) / t.tiles;
-    const long long most = (e[2] + 7) / 8;
-    if (chunks > most) chunks = most;
-    t.planes = (int)((e[2] + chunks - 1) / chunks);
-    *blocks = t.tiles * ((e[2] + t.planes - 1) / t.planes);
-    return t;
-}
-
 template <typename R, int DIM, int TX, int TY>
 void launch_half(const GasParams& p, const GasArrays& a, bool predictor, int num_sms, cudaStream_t s)
 {
     long long nb;
-    const GasMarch t = march_of(predictor ? p.m : p.n, TX, TY, num_sms, &nb);
+    const GasMarch t = gas_march(predictor ? p.m : p.n, TX, TY, num_sms, &nb);
     constexpr int NT = GasTile<DIM, TX, TY>::NT;
     if (predictor) gas_predictor_kernel<R, DIM, TX, TY><<<(unsigned)nb, NT, 0, s>>>(p, a, t);
     else if (DIM == 3 && p.limiter == 0)
