@@ -138,17 +138,17 @@ __device__ __forceinline__ int face_record_ab(float4 um, float4 u0, float4 up, f
 }
 
 // HLL flux (Eq. hyperbolic:hllflux2) with the four components as two FP32 pairs; FL, FR are the
-// states' fluxes per unit chat and the weights carry the factor chat.  S_R^+ = S_L^- = 0 gives the average: the
-// weights are chosen, not the code, since a branch here costs its instructions at every face (corrector 2.7 %,
-// predictor 5 % slower).
+// states' fluxes per unit chat and the weights carry the factor chat.  S_R^+ = S_L^- = 0 gives the average, (F_L +
+// F_R) chat / 2 rounded in that order: the weights are chosen, not the code, since a branch here costs its
+// instructions at every face (corrector 2.7 %, predictor 5 % slower).
 __device__ __forceinline__ float4 hll_pair(float4 UL, float4 UR, float4 FL, float4 FR, float l1L, float l3L,
                                            float l1R, float l3R, float chat)
 {
     const float SRp = fmaxf(fmaxf(l3L, l3R), 0.f), SLm = fminf(fminf(l1L, l1R), 0.f);
     const float den = SRp - SLm, h = 0.5f * chat;
     const bool two = den > 0.f;
-    const float2 a = p_s(two ? SRp * chat : h), b = p_s(two ? -SLm * chat : h), c = p_s(SRp * SLm);
-    const float2 iv = p_s(two ? rcp(den) : 1.f);
+    const float2 a = p_s(two ? SRp * chat : 1.f), b = p_s(two ? -SLm * chat : 1.f), c = p_s(SRp * SLm);
+    const float2 iv = p_s(two ? rcp(den) : h);
     const float2 lo = p_mul(p_fma(c, p_sub(p_lo(UR), p_lo(UL)), p_fma(b, p_lo(FR), p_mul(a, p_lo(FL)))), iv);
     const float2 hi = p_mul(p_fma(c, p_sub(p_hi(UR), p_hi(UL)), p_fma(b, p_hi(FR), p_mul(a, p_hi(FL)))), iv);
     return make_float4(lo.x, lo.y, hi.x, hi.y);
@@ -162,8 +162,8 @@ __device__ __forceinline__ float4 hll4(float4 UL, float4 UR, float4 FL, float4 F
     const float SRp = fmaxf(fmaxf(l3L, l3R), 0.f), SLm = fminf(fminf(l1L, l1R), 0.f);
     const float den = SRp - SLm, h = 0.5f * chat;
     const bool two = den > 0.f;
-    const float a = two ? xmul(SRp, chat) : h, b = two ? xmul(-SLm, chat) : h, c = xmul(SRp, SLm);
-    const float iv = two ? rcp(den) : 1.f;
+    const float a = two ? xmul(SRp, chat) : 1.f, b = two ? xmul(-SLm, chat) : 1.f, c = xmul(SRp, SLm);
+    const float iv = two ? rcp(den) : h;
     return make_float4(xmul(xfma(c, xadd(UR.x, -UL.x), xfma(b, FR.x, xmul(a, FL.x))), iv),
                        xmul(xfma(c, xadd(UR.y, -UL.y), xfma(b, FR.y, xmul(a, FL.y))), iv),
                        xmul(xfma(c, xadd(UR.z, -UL.z), xfma(b, FR.z, xmul(a, FL.z))), iv),

@@ -1,0 +1,44 @@
+// The HLL flux of the split kernels where both wave speeds are zero (fp32; subcycle_pair.cuh, subcycle_split2d.cuh): the
+// average (F_L + F_R) chat / 2, the sum rounded first, for random fluxes.  Prints the number of values that differ, per
+// function.  Built and run by tests/test_gpu_hll_average.py.
+#include <cstdio>
+#include <random>
+#include <vector>
+
+#include "subcycle.cuh"
+
+__global__ void check_kernel(const float4* v, float chat, float4* out, int n)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const float4 UL = v[4 * i], UR = v[4 * i + 1], FL = v[4 * i + 2], FR = v[4 * i + 3];
+    out[3 * i] = rhd::hll_pair(UL, UR, FL, FR, 0.0f, 0.0f, 0.0f, 0.0f, chat);
+    out[3 * i + 1] = rhd::hll4(UL, UR, FL, FR, 0.0f, 0.0f, 0.0f, 0.0f, chat);
+    out[3 * i + 2] = rhd::hll2d(UL, UR, FL, FR, 0.0f, 0.0f, 0.0f, 0.0f);  // fluxes with their factor chat
+}
+
+int main()
+{
+    const int n = 1 << 16;
+    const float chat = 0.3f;
+    std::vector<float> v(16 * n), o(12 * n);
+    std::mt19937 rng(5);
+    std::uniform_real_distribution<float> d(-1.0f, 1.0f);
+    for (auto& x : v) x = d(rng);
+    float4 *dv, *dout;
+    if (cudaMalloc(&dv, 64 * n) || cudaMalloc(&dout, 48 * n)) return 2;
+    cudaMemcpy(dv, v.data(), 64 * n, cudaMemcpyHostToDevice);
+    check_kernel<<<(n + 255) / 256, 256>>>(dv, chat, dout, n);
+    if (cudaMemcpy(o.data(), dout, 48 * n, cudaMemcpyDeviceToHost)) return 3;
+    long long off[3] = {0, 0, 0};
+    for (int i = 0; i < n; ++i)
+        for (int q = 0; q < 4; ++q) {
+            volatile float sum = v[16 * i + 8 + q] + v[16 * i + 12 + q];
+            volatile float h = 0.5f * chat;
+            off[0] += o[12 * i + q] != sum * h;
+            off[1] += o[12 * i + 4 + q] != sum * h;
+            off[2] += o[12 * i + 8 + q] != sum * 0.5f;
+        }
+    std::printf("%lld %lld %lld\n", off[0], off[1], off[2]);
+    return 0;
+}
