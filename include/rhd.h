@@ -304,13 +304,17 @@ rhd_status rhd_ensemble_subcycle(rhd_ctx* ctx, int n_sub, double chat, const dou
  *             2 run a predictor and a corrector under this name where the device has room for U^{m+1/2}
  *             (32 and 16 bytes per cell, layers as below), and choose their tiles.  A context takes that
  *             memory after all its grids' states and gives it back to an array of its own that finds no room
- *             later (gas arrays, the gas step's scratch); the fused kernel runs from then on.  RHD_VARIANT_TWOPASS (RHD_SPLIT, 3D grids only):
- *             a predictor kernel writes U^{m+1/2} (FP32) for the grid plus 2 ghost layers per face
+ *             later (gas arrays, the gas step's scratch); the fused kernel runs from then on.
+ *             RHD_VARIANT_TWOPASS (RHD_SPLIT, 3D grids only): a predictor kernel writes U^{m+1/2} (FP32) for the grid plus 2 ghost layers per face
  *             in each direction that is not periodic on both faces, then a corrector kernel reads
  *             it back; extra device memory (n0+p0)(n1+p1)(n2+p2) x 16 bytes, p = 0 for a direction
  *             periodic on both faces, else 4.
- *   tile_x, tile_y   cells per CTA tile in x and y (the supported shapes are those the tuner lists)
- *   z_chunk   planes per CTA along z (each CTA marches its tile through a chunk of planes)
+ *   tile_x, tile_y   cells per CTA tile in x and y (the supported shapes are those the tuner lists; 1D grids
+ *             have one configuration, named 122 x 1, and choose their tiles)
+ *   z_chunk   planes per CTA along z (each CTA marches its tile through a chunk of planes).  Grids created with
+ *             z_chunk = 0 plan the chunks of each kernel by themselves (and the FP64 pair's tiles); the plan's
+ *             value here, which rhd_get_launch_config reports, stands for all of it, so that a configuration
+ *             read from such a grid puts its plan back.  Other values hold for every kernel of the subcycle.
  *   staging   RHD_STAGING_CPASYNC: the tile and its halo are staged into shared memory with per-
  *             thread asynchronous copies.  RHD_STAGING_TMA (two-pass corrector): the tile + 2-cell
  *             halo of U^{m+1/2} is fetched with one tensor-memory-accelerator copy per plane.
@@ -326,14 +330,16 @@ typedef struct {
 
 /* Time every candidate configuration of a single-grid context on its current state (moments and
  * gas must be set; chat and dt as for rhd_radiation_subcycle) with reps >= 1 timed subcycles each
- * (plain launches, after one warm-up), then keep the fastest.  The grid's state (E, F, T) and the
+ * (plain launches, after one warm-up), then keep the fastest.  The configuration in use and the grid's own
+ * plan are among them (FP64 3D grids: timed like the others, without an entry in the table).  The grid's state (E, F, T) and the
  * statistics are left exactly as they were; captured graphs are dropped.  table (may be NULL)
  * receives up to capacity entries, *n_entries (may be NULL) the number of candidates, *chosen (may
  * be NULL) the configuration kept.  Synchronises the context's stream.  Errors: RHD_ERR_ARG,
  * RHD_ERR_STATE (state not set, or an ensemble context), RHD_ERR_OOM / RHD_ERR_CUDA. */
 rhd_status rhd_autotune(rhd_ctx* ctx, double chat, double dt, int reps, rhd_launch_config* table, int capacity,
                         int* n_entries, rhd_launch_config* chosen);
-/* The same for an ensemble context: candidates are the z_chunk values shared by all grids. */
+/* The same for an ensemble context: candidates are z_chunk values shared by all grids, the one in use and the
+ * ensemble's own plan among them. */
 rhd_status rhd_ensemble_autotune(rhd_ctx* ctx, double chat, const double* dt_per_grid, int reps,
                                  rhd_launch_config* table, int capacity, int* n_entries,
                                  rhd_launch_config* chosen);

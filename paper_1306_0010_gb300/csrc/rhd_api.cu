@@ -347,12 +347,15 @@ int march_chunk(const MarchCost& m, long long tiles, int planes, int n_sms)
 }
 
 // the two-pass kernels' own choice of chunks for a grid (32 x 8 tiles)
-void plan_twopass(rhd_ctx* ctx, GridState& gs)
+struct TwopassPlan {
+    int predictor, corrector;
+};
+TwopassPlan twopass_plan(rhd_ctx* ctx, const GridState& gs)
 {
     const int ex = upad_extent(gs.gp, 0), ey = upad_extent(gs.gp, 1);
-    gs.p_chunk = march_chunk(kMarchPred, (long long)((ex + 31) / 32) * ((ey + 7) / 8), upad_extent(gs.gp, 2), ctx->num_sms);
-    gs.z_chunk = march_chunk(kMarchCorr, (long long)((gs.desc.n[0] + 31) / 32) * ((gs.desc.n[1] + 7) / 8), gs.desc.n[2],
-                             ctx->num_sms);
+    return {march_chunk(kMarchPred, (long long)((ex + 31) / 32) * ((ey + 7) / 8), upad_extent(gs.gp, 2), ctx->num_sms),
+            march_chunk(kMarchCorr, (long long)((gs.desc.n[0] + 31) / 32) * ((gs.desc.n[1] + 7) / 8), gs.desc.n[2],
+                        ctx->num_sms)};
 }
 
 // ... and for a split ensemble, whose grids share the launches and one chunk length
@@ -1213,7 +1216,17 @@ bool config_supported(const GridState& gs, const rhd_launch_config& c)
     return tile_supported(prec, nact, c.tile_x, c.tile_y);
 }
 
-// Make c the configuration of gs (c must be supported); allocates or frees the U^{m+1/2} buffer.
+// The z chunk of the plan that a grid has from its creation, for a variant: the caller's, or the kernels' own choice
+int planned_chunk(rhd_ctx* ctx, const GridState& gs, int variant)
+{
+    if (gs.desc.z_chunk > 0) return std::min(gs.desc.z_chunk, gs.desc.n[2]);
+    if (variant == RHD_VARIANT_TWOPASS) return twopass_plan(ctx, gs).corrector;
+    return gs.uhalf64 ? pair64_plan(gs.gp, ctx->num_sms, 0, false).cz : gs.z_fused;
+}
+
+// Make c the configuration of gs (c must be supported); allocates or frees the U^{m+1/2} buffer.  The z chunk of
+// the grid's own plan stands for the whole plan (the predictor's chunk, the FP64 pair's tiles): a configuration that
+// was read from a grid puts it back.
 rhd_status apply_config(rhd_ctx* ctx, GridState& gs, const rhd_launch_config& c)
 {
     if (c.variant == RHD_VARIANT_TWOPASS) {
@@ -1236,13 +1249,17 @@ rhd_status apply_config(rhd_ctx* ctx, GridState& gs, const rhd_launch_config& c)
     gs.tiles_x = (gs.desc.n[0] + gs.tx - 1) / gs.tx;
     gs.tiles_y = (gs.desc.n[1] + gs.ty - 1) / gs.ty;
     gs.z_chunk = std::max(1, std::min(c.z_chunk, gs.desc.n[2]));
-    gs.p_chunk = 0;
-    plan_pair64(ctx, gs, gs.z_chunk);
+    const bool own = gs.desc.z_chunk == 0 && gs.z_chunk == planned_chunk(ctx, gs, gs.variant);
+    gs.p_chunk = own && gs.variant == RHD_VARIANT_TWOPASS ? twopass_plan(ctx, gs).predictor : 0;
+    plan_pair64(ctx, gs, own ? 0 : gs.z_chunk);
     clear_graphs(ctx);
     return RHD_OK;
 }
 
-std::vector<rhd_launch_config> grid_candidates(const GridState& gs)
+// What the tuner times: the configuration in place and the grid's own plan, so that tuning never ends with a slower
+// one, and fixed chunk lengths.  FP64 grids, whose rows are the fixed lengths, run the first two without a row: the
+// first *n_rows are reported.
+std::vector<rhd_launch_config> grid_candidates(rhd_ctx* ctx, const GridState& gs, int* n_rows)
 {
     std::vector<rhd_launch_config> v;
     auto add = [&](int variant, int tx, int ty, int zc, int staging) {
@@ -1254,18 +1271,25 @@ std::vector<rhd_launch_config> grid_candidates(const GridState& gs)
                 return;
         v.push_back(c);
     };
-    if (gs.gp.nact < 3) {
-        rhd_launch_config c = current_config(gs);
-        add(c.variant, c.tile_x, c.tile_y, c.z_chunk, c.staging);
-    } else if (gs.desc.precision == RHD_FP64) {
+    const rhd_launch_config now = current_config(gs);
+    auto add_now = [&] { add(now.variant, now.tile_x, now.tile_y, now.z_chunk, now.staging); };
+    if (gs.gp.nact == 3 && gs.desc.precision == RHD_FP64) {
         for (int zc : {8, 16, 32, 64, 128, 256, 512}) add(RHD_VARIANT_FUSED, 16, 16, zc, RHD_STAGING_CPASYNC);
-    } else {
+        *n_rows = (int)v.size();
+        add_now();
+        add(RHD_VARIANT_FUSED, 16, 16, planned_chunk(ctx, gs, RHD_VARIANT_FUSED), RHD_STAGING_CPASYNC);
+        return v;
+    }
+    add_now();
+    if (gs.gp.nact == 3) {
+        add(RHD_VARIANT_TWOPASS, 32, 8, planned_chunk(ctx, gs, RHD_VARIANT_TWOPASS), RHD_STAGING_CPASYNC);
         for (int stg : {RHD_STAGING_CPASYNC, RHD_STAGING_TMA})
             for (int zc : {16, 32, 64, 128}) add(RHD_VARIANT_TWOPASS, 32, 8, zc, stg);
         const int tiles[3][2] = {{32, 8}, {32, 16}, {64, 8}};
         for (auto& t : tiles)
             for (int zc : {32, 64, 128}) add(RHD_VARIANT_FUSED, t[0], t[1], zc, RHD_STAGING_CPASYNC);
     }
+    *n_rows = (int)v.size();
     return v;
 }
 
@@ -1370,7 +1394,8 @@ rhd_status grid_autotune(rhd_ctx* ctx, double chat, double dt, int reps, rhd_lau
                          int* n_entries, rhd_launch_config* chosen)
 {
     GridState& gs = ctx->grids[0];
-    std::vector<rhd_launch_config> cand = grid_candidates(gs);
+    int n_rows = 0;
+    std::vector<rhd_launch_config> cand = grid_candidates(ctx, gs, &n_rows);
     const rhd_launch_config before = current_config(gs);
     rhd_status st = enter(ctx);
     if (st) return st;
@@ -1404,6 +1429,7 @@ rhd_status grid_autotune(rhd_ctx* ctx, double chat, double dt, int reps, rhd_lau
     if (ce != cudaSuccess) return fail(ctx, RHD_ERR_CUDA, std::string("autotune: ") + cudaGetErrorString(ce));
     gs.tuned = true;
     gs.tuned_ms = best >= 0 ? cand[best].ms_per_subcycle : -1.0;
+    cand.resize(n_rows);
     report(cand, current_config(gs), table, capacity, n_entries, chosen);
     if (log_level() >= 2) {
         const rhd_launch_config c = current_config(gs);
@@ -1469,13 +1495,19 @@ rhd_status ensemble_autotune(rhd_ctx* ctx, double chat, const double* dt_per_gri
     int max_nz = 1;
     for (auto& gs : ctx->grids) max_nz = std::max(max_nz, gs.desc.n[2]);
     std::vector<rhd_launch_config> cand;
-    auto add = [&](int v, int zc) {
-        if (zc > max_nz && zc != 8) return;
+    auto add = [&](int v, int zc, bool always = false) {
+        if (zc > max_nz && zc != 8 && !always) return;
+        for (auto& o : cand)
+            if (o.variant == v && o.z_chunk == zc) return;
         if (v == RHD_VARIANT_TWOPASS) cand.push_back({v, 32, 8, zc, RHD_STAGING_CPASYNC, -1.0});
         else cand.push_back({v, g0.tx, g0.ty, zc, RHD_STAGING_CPASYNC, -1.0});
     };
-    if (split && g0.desc.exchange != RHD_EX_LINEAR)
+    // the configuration in place and the ensemble's own plan first, as for single grids
+    add(g0.variant, g0.z_chunk, true);
+    if (split && g0.desc.exchange != RHD_EX_LINEAR) {
+        add(RHD_VARIANT_TWOPASS, g0.desc.z_chunk > 0 ? g0.desc.z_chunk : plan_ensemble_chunk(ctx), true);
         for (int zc : {16, 32, 64}) add(RHD_VARIANT_TWOPASS, zc);
+    }
     for (int zc : {8, 16, 32, 64, 128}) add(RHD_VARIANT_FUSED, zc);
     const int v_before = g0.variant, zc_before = g0.z_chunk;
     rhd_status st = enter(ctx);
@@ -1611,7 +1643,11 @@ rhd_status rhd_init_grid(rhd_ctx** out, const rhd_grid_desc* d)
         if (d->precision == RHD_SPLIT && gs.gp.nact == 3 && d->exchange != RHD_EX_LINEAR) {
             gs.variant = (d->flags & RHD_FLAG_SPLIT_FUSED) ? 0 : 1;
             if (const char* v = std::getenv("RHD_VARIANT")) gs.variant = std::strcmp(v, "fused") == 0 ? 0 : 1;
-            if (gs.variant == 1 && d->z_chunk == 0) plan_twopass(ctx, gs);
+            if (gs.variant == 1 && d->z_chunk == 0) {
+                const TwopassPlan plan = twopass_plan(ctx, gs);
+                gs.p_chunk = plan.predictor;
+                gs.z_chunk = plan.corrector;
+            }
         }
         st = alloc_grid(ctx, gs);
     }
