@@ -1413,7 +1413,14 @@ rhd_status grid_autotune(rhd_ctx* ctx, double chat, double dt, int reps, rhd_lau
         }
         double ms = -1.0;
         st = prepare_twopass(ctx, gs);
-        if (!st) st = time_launches(ctx, reps, [&] { return launch_one(ctx, gs, ctx->cur, chat, dt); }, &ms);
+        // 1D grids: the first of two launches of as many subcycles as one takes
+        const int n_sub = gs.gp.nact == 1 ? gs.line.steps : 1;
+        auto launch = [&] {
+            return gs.gp.nact == 1 ? launch_line_part(ctx, gs, 2 * n_sub, 0, ctx->cur, chat, dt)
+                                   : launch_one(ctx, gs, ctx->cur, chat, dt);
+        };
+        if (!st) st = time_launches(ctx, reps, launch, &ms);
+        if (ms >= 0.0) ms /= n_sub;
         gs.um32_ok = false;  // the timed correctors rewrote the mirror with the next state
         if (!st) st = tune_restore(ctx, b);
         cand[i].ms_per_subcycle = ms;

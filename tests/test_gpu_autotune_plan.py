@@ -1,5 +1,5 @@
-"""GPU: the tuner's candidates include what an untuned grid runs, and a configuration that was read from a grid can be
-put back."""
+"""GPU: the tuner's candidates include what an untuned grid runs, a configuration that was read from a grid can be put
+back, and a 1D grid's tuned time is that of the launches it makes."""
 import numpy as np
 import pytest
 
@@ -69,3 +69,17 @@ def test_split_ensemble_plan_is_a_candidate(rhd):  # noqa: F811
     assert (before["variant"], before["z_chunk"]) in [(c["variant"], c["z_chunk"]) for c in table]
     assert chosen["ms_per_subcycle"] == min(c["ms_per_subcycle"] for c in table)
 
+
+@pytest.mark.parametrize("precision", ["fp64", "split"])
+def test_tuned_time_of_a_1d_grid(rhd, precision):  # noqa: F811
+    g, case = grid(rhd, (512, 1, 1), precision)
+    T = np.array(g.get_gas_state())
+    chosen, _ = g.autotune(case["chat"], case["dt"], reps=50)
+    assert np.array_equal(g.get_gas_state(), T)
+    g.set_kernel_timing(True)
+    g.radiation_subcycle(160, case["chat"], case["dt"])
+    (kt,) = g.kernel_times().values()
+    g.close()
+    assert kt["launches"] < 160  # several subcycles a launch
+    # one launch of one subcycle takes 1.7 times as long per subcycle
+    assert chosen["ms_per_subcycle"] <= 1.3 * kt["total_ms"] / 160
