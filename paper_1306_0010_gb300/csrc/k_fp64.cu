@@ -44,7 +44,7 @@ static int ens_occupancy()
 void tile_shape(int precision, int nact, int* tx, int* ty)
 {
     if (nact == 1) {
-        *tx = 122;  // 128 threads: the tile and its 3-cell halo on each side
+        *tx = 122;  // the name of 1D grids' one configuration, in files too (their tiles: line_plan)
         *ty = 1;
     } else if (precision == 0) {
         // one CTA of 256 threads per SM (255 registers each): against 16x8 tiles (two CTAs of 128) it
@@ -123,10 +123,7 @@ cudaError_t launch_line(const LineParams& p, bool split, int tpc, cudaStream_t s
 cudaError_t launch_subcycle_fp64(const StepParams& p, cudaStream_t s)
 {
     switch (p.g.nact) {
-    case 1: {  // one subcycle, T in place
-        const int tpc = line_plan(p.g, false, 152).tpc;
-        return launch_line_fp64(line_params(p, 1, tpc, p.a.T), tpc, s);
-    }
+    case 1: return cudaErrorInvalidValue;  // 1D grids: launch_line
     case 2: return launch_tile_kernel<double, 16, 16, 2, false>(p, s);
     default: return launch_tile_kernel<double, 16, 16, 3, false>(p, s);
     }

@@ -170,12 +170,6 @@ cudaError_t launch_twopass_corrector(const StepParams& p, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_twopass_split(const StepParams& p, cudaStream_t s)
-{
-    cudaError_t e = launch_twopass_predictor(p, s);
-    return e != cudaSuccess ? e : launch_twopass_corrector(p, s);
-}
-
 // cuTensorMapEncodeTiled from the driver, found at run time (the library does not link libcuda)
 static decltype(&cuTensorMapEncodeTiled) tensor_map_encoder()
 {

@@ -188,6 +188,7 @@ struct SmemLimitOnce {
 };
 
 // Launch wrappers (defined in the kernel translation units).
+// the fused kernels (2D, 3D), and the 1D kernel
 cudaError_t launch_subcycle_fp64(const StepParams& p, cudaStream_t s);
 cudaError_t launch_subcycle_split(const StepParams& p, cudaStream_t s);
 LinePlan line_plan(const GridParams& g, bool split, int n_sms);
@@ -195,7 +196,6 @@ LineParams line_params(const StepParams& p, int steps, int tpc, double* To);
 cudaError_t launch_line(const LineParams& p, bool split, int tpc, cudaStream_t s);
 cudaError_t launch_line_fp64(const LineParams& p, int tpc, cudaStream_t s);
 cudaError_t launch_line_split(const LineParams& p, int tpc, cudaStream_t s);
-cudaError_t launch_twopass_split(const StepParams& p, cudaStream_t s);
 bool twopass_common(const GridParams& g);  // the modes the two-pass kernels have at compile time
 cudaError_t launch_twopass_predictor(const StepParams& p, cudaStream_t s);
 // split 2D grids with U^{m+1/2}: predictor, corrector

@@ -142,6 +142,12 @@ extern "C" rhd_status rhd_subcycle_noalloc(const rhd_grid_desc* d, const double 
     a.kP = kP;
     a.kF = kF;
     a.j = j;
+    int tpc = 1;
+    if (gp.nact == 1) {
+        int n_sms = 0;
+        NA_CUDA(cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev));
+        tpc = line_plan(gp, false, n_sms).tpc;
+    }
     // ping-pong between the scratch state (A) and the caller's outputs (B, holding G until the end)
     for (int step = 0; step < n_sub; ++step) {
         double** src = (step & 1) ? B : A;
@@ -152,7 +158,8 @@ extern "C" rhd_status rhd_subcycle_noalloc(const rhd_grid_desc* d, const double 
             a.G[q] = src[1 + q];
             a.Go[q] = dst[1 + q];
         }
-        NA_CUDA(launch_subcycle_fp64(p, s));
+        // 1D: one subcycle per launch, T in place
+        NA_CUDA(gp.nact == 1 ? launch_line(line_params(p, 1, tpc, a.T), false, tpc, s) : launch_subcycle_fp64(p, s));
     }
     if ((n_sub & 1) == 0) {
         NA_CUDA(cudaMemcpyAsync(E_out, A[0], bytes, cudaMemcpyDeviceToDevice, s));
