@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 
 #include <mutex>
+#include <utility>
+#include <vector>
 
 namespace rhd {
 
@@ -165,24 +167,18 @@ struct EnsembleParams {
 // launch).  One instance per launch site, which may choose among a few kernels of one size.
 struct SmemLimitOnce {
     std::mutex m;
-    const void* fn[16] = {};
-    int dev_of[16] = {};
-    int n = 0;
+    std::vector<std::pair<const void*, int>> raised;  // (kernel, device), as many as the site has
     template <typename K>
     cudaError_t set(K k, size_t smem)
     {
         int dev = 0;
         if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
-        const void* f = reinterpret_cast<const void*>(k);
+        const std::pair<const void*, int> key(reinterpret_cast<const void*>(k), dev);
         std::lock_guard<std::mutex> lock(m);
-        for (int i = 0; i < n; ++i)
-            if (fn[i] == f && dev_of[i] == dev) return cudaSuccess;
+        for (const auto& r : raised)
+            if (r == key) return cudaSuccess;
         const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess && dev >= 0 && n < 16) {
-            fn[n] = f;
-            dev_of[n] = dev;
-            ++n;
-        }
+        if (e == cudaSuccess && dev >= 0) raised.push_back(key);
         return e;
     }
 };
