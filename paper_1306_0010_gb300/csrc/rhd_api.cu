@@ -21,6 +21,7 @@
 #include "rhd_internal.h"
 #include "gas_index.h"
 #include "gas_internal.h"
+#include "march_plan.h"
 
 using namespace rhd;
 
@@ -306,44 +307,6 @@ void fill_params(GridState& gs)
         while (zc > 32 && tiles * ((d.n[2] + zc - 1) / zc) < 152LL * 8) zc = (zc + 1) / 2;
     }
     gs.z_chunk = gs.z_fused = std::max(1, std::min(zc, d.n[2]));
-}
-
-// Planes per CTA of the split two-pass kernels.  A CTA marches its column tile through z; t0 + t1 k is the time
-// (us) of one plane with k CTAs on an SM, t_full that with k_max of them in a long queue, and `start` the
-// planes' worth of work that a chunk adds (the predictor's two halo planes, the corrector's first face).  A
-// launch of more CTAs than fit at once ends with half a CTA's time on average.  Fitted to 3 .. 128 planes on
-// 97x61x45, 64^3, 128^3, 200x150x120, 256^3, 300x250x200 and 512^3: a lone corrector CTA takes 3.7 us a plane
-// and three on an SM 5.9, so a small grid wants enough chunks to put two or three CTAs on every SM (97x61x45:
-// 4 planes, 39 us against 129 us with 32 planes everywhere) and a large one long chunks (512^3: 64 planes, 6.99
-// ms against 7.08).
-struct MarchCost {
-    double start, t0, t1, t_full;
-    int k_max;
-};
-constexpr MarchCost kMarchPred = {2.2, 1.45, 0.52, 3.2, 4}, kMarchCorr = {1.2, 2.6, 1.2, 5.9, 3};
-
-// ctas CTAs of at most `chunk` planes, `planes` in all
-double march_time(const MarchCost& m, long long ctas, long long planes, int chunk, int n_sms)
-{
-    const long long slots = (long long)n_sms * m.k_max;
-    const double longest = chunk + m.start;
-    if (ctas <= slots) return longest * (m.t0 + m.t1 * (double)((ctas + n_sms - 1) / n_sms));
-    return m.t_full * (((double)planes + m.start * (double)ctas) / (double)slots + 0.5 * longest);
-}
-
-int march_chunk(const MarchCost& m, long long tiles, int planes, int n_sms)
-{
-    int best = planes;
-    double best_t = -1.0;
-    for (int n = 1; n == 1 || 2 * n <= planes; ++n) {
-        const int c = (planes + n - 1) / n;
-        const double t = march_time(m, tiles * ((planes + c - 1) / c), tiles * planes, c, n_sms);
-        if (best_t < 0.0 || t < best_t) {
-            best_t = t;
-            best = c;
-        }
-    }
-    return best;
 }
 
 // the two-pass kernels' own choice of chunks for a grid (32 x 8 tiles)
