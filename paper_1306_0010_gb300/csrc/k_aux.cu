@@ -27,8 +27,10 @@ cudaError_t launch_scale_copy(double* dst, const double* src, double scale, long
 }
 
 // x / c, c > 0, for y = 1/c correctly rounded (0: always divide): one multiplication and one correction by the
-// exact residual (the correctly rounded quotient, by Markstein's theorem, where nothing under- or overflows: three FP64
-// instructions against CUDA's ten or so), the division itself elsewhere
+// residual (three FP64 instructions against CUDA's ten or so), the division itself where something under- or
+// overflows.  q = x y may be 1.5 ulp off where x's mantissa is below c's, beyond the premise of Markstein's theorem (q
+// within an ulp), so that it is the correctly rounded quotient is tested instead: on the quotients nearest to a
+// halfway point, where a correction could go wrong, and over all operands in arithmetic of 4 to 11 bits.
 static __device__ __noinline__ double div_slow(double x, double c) { return x / c; }
 __device__ __forceinline__ double div_by(double x, double c, double y)
 {
