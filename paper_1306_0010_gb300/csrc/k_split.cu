@@ -53,10 +53,7 @@ cudaError_t launch_line_split(const LineParams& p, int tpc, cudaStream_t s)
 cudaError_t launch_subcycle_split(const StepParams& p, cudaStream_t s)
 {
     switch (p.g.nact) {
-    case 1: {  // one subcycle, T in place
-        const int tpc = line_plan(p.g, true, 152).tpc;
-        return launch_line_split(line_params(p, 1, tpc, p.a.T), tpc, s);
-    }
+    case 1: return cudaErrorInvalidValue;  // 1D grids: launch_line
     case 2: return launch_tile_kernel<float, 32, 8, 2, true>(p, s);
     default:
         if (p.ty == 16) return launch_tile_kernel<float, 32, 16, 3, true>(p, s);
