@@ -545,7 +545,7 @@ __device__ __forceinline__ void corrector_tile(const GridParams& g, const GridAr
         const float4 UL = Sx[G::NSX + iL], UR = Sx[iR];
         const float4 cL = Sx[2 * G::NSX + iL], cR = Sx[2 * G::NSX + iR];
         const float4 LL = Sx[3 * G::NSX + iL], LR = Sx[3 * G::NSX + iR];
-        return hll_pair(UL, UR, flux_ab<0>(UL, cL.z, cL.w), flux_ab<0>(UR, cR.x, cR.y), LL.z, LL.w, LR.x, LR.y, chat);
+        return hll_pair<COMMON>(UL, UR, flux_ab<0>(UL, cL.z, cL.w), flux_ab<0>(UR, cR.x, cR.y), LL.z, LL.w, LR.x, LR.y, chat);
     };
     auto hll_y = [&](int iL, int iR) {
         iL = chk(iL, G::NSY);
@@ -553,7 +553,7 @@ __device__ __forceinline__ void corrector_tile(const GridParams& g, const GridAr
         const float4 UL = Sy[G::NSY + iL], UR = Sy[iR];
         const float4 cL = Sy[2 * G::NSY + iL], cR = Sy[2 * G::NSY + iR];
         const float4 LL = Sy[3 * G::NSY + iL], LR = Sy[3 * G::NSY + iR];
-        return hll_pair(UL, UR, flux_ab<1>(UL, cL.z, cL.w), flux_ab<1>(UR, cR.x, cR.y), LL.z, LL.w, LR.x, LR.y, chat);
+        return hll_pair<COMMON>(UL, UR, flux_ab<1>(UL, cL.z, cL.w), flux_ab<1>(UR, cR.x, cR.y), LL.z, LL.w, LR.x, LR.y, chat);
     };
 
     // lower z face of the first plane: face states of cells z0-1 and z0 from U^{m+1/2} at z0-2 .. z0+1
@@ -566,7 +566,7 @@ __device__ __forceinline__ void corrector_tile(const GridParams& g, const GridAr
         face_record_ab<2, COMMON>(u_m2, u_m1, u_0, chat, lim, p1, fixed, ra);
         const int fb = face_record_ab<2, COMMON>(u_m1, u_0, u_1, chat, lim, p1, fixed, rb);
         cnt.face += (unsigned)(fb & (int)own_col);
-        cfl = hll_pair(ra[1], rb[0], flux_ab<2>(ra[1], ra[2].z, ra[2].w), flux_ab<2>(rb[0], rb[2].x, rb[2].y), ra[3].z,
+        cfl = hll_pair<COMMON>(ra[1], rb[0], flux_ab<2>(ra[1], ra[2].z, ra[2].w), flux_ab<2>(rb[0], rb[2].x, rb[2].y), ra[3].z,
                        ra[3].w, rb[3].x, rb[3].y, chat);
         zpS = rb[1];
         zpa = rb[2].z;
@@ -666,7 +666,7 @@ __device__ __forceinline__ void corrector_tile(const GridParams& g, const GridAr
             float4 rec[4];
             const int fb = face_record_ab<2, COMMON>(Uk[ihc], ukp1, ukp2, chat, lim, p1, fixed, rec);
             cnt.face += (unsigned)(fb & (int)(k + 1 < z1) & (int)own_col);
-            cfh = hll_pair(zpS, rec[0], flux_ab<2>(zpS, zpa, zpb), flux_ab<2>(rec[0], rec[2].x, rec[2].y), zpl1, zpl3,
+            cfh = hll_pair<COMMON>(zpS, rec[0], flux_ab<2>(zpS, zpa, zpb), flux_ab<2>(rec[0], rec[2].x, rec[2].y), zpl1, zpl3,
                            rec[3].x, rec[3].y, chat);
             zpS = rec[1];
             zpa = rec[2].z;
