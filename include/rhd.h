@@ -156,7 +156,8 @@ typedef struct {
     int64_t n_nonfinite;         /* interior cells that produced a non-finite value (split grids: also a
                                     state beyond the FP32 range of their transport) */
     int32_t newton_iter_max;     /* largest Newton iteration count of one solve (split path: the FP32
-                                    iterations plus the double-float step) */
+                                    iterations plus the double-float step; FP64 in 2D and 3D: 2, the FP64
+                                    steps after the FP32 iterations, or the count of a cell they do not settle) */
     int32_t wait_timeouts;       /* bounded device-side waits that ran out; nonzero makes rhd_get_stats
                                     return RHD_ERR_TIMEOUT (the affected tiles were not updated) */
     double sum_E;                /* sum of E over the interior (current state), FP64, fixed order */

@@ -32,12 +32,12 @@ __device__ __forceinline__ double f2d_exact(float f)
 }
 
 // Square root and reciprocal.  Split path: the hardware approximations (MUFU, about 1-2 ulp), well
-// inside the FP32 error budget of the fluxes.  FP64 path: IEEE square root; the reciprocal is the
-// hardware FP64 approximation refined by two Newton-Raphson steps r <- r + r (1 - x r), each of which
-// squares the relative error (from below 2^-20 to below 2^-40, then to rounding): within an ulp or
-// two of 1/x, not the correctly rounded quotient, which the FP64 path does not need (its bound
-// against the oracle is 1e-12) and which costs several more FP64 operations.  x = 0, +-inf and FP64
-// denormals (flushed) give NaN.
+// inside the FP32 error budget of the fluxes.  FP64, 1D grids and the gas step (2D and 3D grids: rcp3,
+// rsqrt3 and sqrt3 below): IEEE square root; the reciprocal is the hardware FP64 approximation refined by
+// two Newton-Raphson steps r <- r + r (1 - x r), each of which squares the relative error (from below
+// 2^-20 to below 2^-40, then to rounding): within an ulp or two of 1/x, not the correctly rounded
+// quotient, which the FP64 path does not need (its bound against the oracle is 1e-12) and which costs
+// several more FP64 operations.  x = 0, +-inf and FP64 denormals (flushed) give NaN.
 __device__ __forceinline__ double sqrt_fast(double x) { return sqrt(x); }
 __device__ __forceinline__ float sqrt_fast(float x)
 {

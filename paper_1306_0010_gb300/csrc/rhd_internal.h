@@ -75,7 +75,7 @@ struct GridArrays {
                                 // rewritten with U^{m+1} by the corrector
     const float4* gas4;         // (rho, vx, vy, vz) as FP32 per cell (the FP32 gas copies interleaved)
     const double* dir_dev;      // non-NULL: the low x face's Dirichlet state (E, Gx, Gy, Gz) in device memory,
-                                // written by a kernel before each subcycle (fused kernels; else NULL)
+                                // written by a kernel before the subcycles (not with the two-pass kernels; else NULL)
 };
 
 // Work split of the FP64 kernel pair (subcycle_fp64_pair.cuh): tile width and height, planes per CTA and

@@ -17,8 +17,8 @@
 // Every stage follows the order of the CPU oracle; the readings of the paper (limiter, face-state
 // fallback, split order, ghost rule) are the same.
 //
-// Precision: R = double gives the FP64 path.  R = float with SPLIT gives the split path: closure,
-// wave speeds, reconstruction and fluxes (and so U^{m+1/2}) in FP32; the update of the FP64 state is
+// Precision: the FP64 kernels take subcycle_tile64 (subcycle_fp64.cuh), the same stages in FP64.  Here,
+// R = float with SPLIT, the split path: closure, wave speeds, reconstruction and fluxes (and so U^{m+1/2}) in FP32; the update of the FP64 state is
 // formed as an FP32 increment (transport + sources + theta terms + exchange change) added once in FP64.
 #pragma once
 
