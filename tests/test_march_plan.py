@@ -14,7 +14,7 @@ PLANS = {(97, 61, 45, 2): (5, 5), (64, 64, 64, 2): (5, 4), (256, 256, 256, 2): (
 
 
 @pytest.fixture(scope="module")
-def checker():
+def plan_exe():
     cxx = shutil.which("g++") or shutil.which("c++")
     if not cxx:
         pytest.skip("no host C++ compiler")
@@ -26,13 +26,13 @@ def checker():
     return exe
 
 
-def test_plans_of_known_grids(checker):
+def test_plans_of_known_grids(plan_exe):
     lines = "\n".join(" ".join(map(str, k)) for k in PLANS)
-    out = subprocess.run([checker], input=lines, capture_output=True, text=True, check=True).stdout
+    out = subprocess.run([plan_exe], input=lines, capture_output=True, text=True, check=True).stdout
     assert [tuple(map(int, x.split())) for x in out.splitlines()] == list(PLANS.values())
 
 
-def test_every_plan_lies_within_the_grid(checker):
-    out = subprocess.run([checker, "sweep"], capture_output=True, text=True, check=True, timeout=300).stdout
+def test_every_plan_lies_within_the_grid(plan_exe):
+    out = subprocess.run([plan_exe, "sweep"], capture_output=True, text=True, check=True, timeout=300).stdout
     bad, n = map(int, out.split())
     assert bad == 0 and n > 10000
